@@ -406,7 +406,7 @@ template <typename T> class BatchEngine final : public BatchBase {
         for (E* e : order) {
             f.push_back(ForwardArgs<T>{e->rho_fx_, e->Zxy_, e->tw_, e->density_scale(), 1, e->counters_});
             if (e->refresh_tables()) return fail_from(e);
-            z.push_back(ZArgs<T>{e->Zxy_, e->H_, e->tw_, e->spectral_params(), nullptr, nullptr});
+            z.push_back(ZArgs<T>{e->Zxy_, e->H_, e->tw_, e->spectral_params(), nullptr});
             inv.push_back(InverseArgs<T>{e->H_, e->grad_, e->tw_, e->two_pi_L(), 0});
             const int n = e->n_, C = persistent_zcols<T>(n);
             nn.push_back(n);
@@ -452,7 +452,7 @@ template <typename T> class BatchEngine final : public BatchBase {
         plan_.status = plan_.bar_count + 2;
         plan_.R = R;
         // shared memory: the largest stage body (bead tile, plane or z tile of 64^3)
-        const size_t plane64 = (64 + 64 * 65) * sizeof(V);
+        const size_t plane64 = (64 + 64 * row_pitch(64)) * sizeof(V);
         const size_t z64 = (64 + 4 * 64 * persistent_zcols<T>(64)) * sizeof(V);
         p_smem_ = std::max(bead_smem_bytes<2, T>(), std::max(plane64, z64));
         int sms = 0, dev = 0;
@@ -546,7 +546,7 @@ template <typename T> class BatchEngine final : public BatchBase {
             f.push_back(ForwardArgs<T>{e->rho_fx_, e->Zxy_, e->tw_, e->density_scale(), 1, e->counters_});
             // the z pass needs the kernel tables of the replica's current a (and a_e)
             if (e->refresh_tables()) return fail_from(e);
-            z.push_back(ZArgs<T>{e->Zxy_, e->H_, e->tw_, e->spectral_params(), nullptr, nullptr});
+            z.push_back(ZArgs<T>{e->Zxy_, e->H_, e->tw_, e->spectral_params(), nullptr});
             inv.push_back(InverseArgs<T>{e->H_, e->grad_, e->tw_, e->two_pi_L(), 0});
         }
         tild_status st;
@@ -577,7 +577,7 @@ template <typename T> class BatchEngine final : public BatchBase {
         E* e0 = g.reps[0];
         return dispatch_group(g, [&](auto nn, auto pp) -> tild_status {
             constexpr int NN = decltype(nn)::value, PP = decltype(pp)::value;
-            if constexpr ((size_t)NN * (NN + 1) * sizeof(V) <= 200 * 1024) {
+            if constexpr (plane_fits(NN, sizeof(V))) {
                 constexpr int CC = E::zpass_cols(NN);
                 constexpr int CA = E::zpass_cols_alt(NN);
                 TILD_CUDA(cudaFuncSetAttribute(xy_forward_plane_batched<T, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -654,7 +654,7 @@ template <typename T> class BatchEngine final : public BatchBase {
             E* e0 = g.reps[0];
             tild_status st = dispatch_group(g, [&](auto nn, auto pp) -> tild_status {
                 constexpr int NN = decltype(nn)::value, PP = decltype(pp)::value;
-                if constexpr ((size_t)NN * (NN + 1) * sizeof(V) <= 200 * 1024) {
+                if constexpr (plane_fits(NN, sizeof(V))) {
                     constexpr int CC = E::zpass_cols(NN);
                     constexpr int CA = E::zpass_cols_alt(NN);
                     with_group_nt<NN>(g, [&](auto nt) {

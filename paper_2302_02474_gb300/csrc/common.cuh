@@ -17,8 +17,16 @@ template <typename T> using cplx_t = typename cplx_of<T>::type;
 
 template <class V> __device__ __forceinline__ V c_add(V a, V b) { return {a.x + b.x, a.y + b.y}; }
 template <class V> __device__ __forceinline__ V c_sub(V a, V b) { return {a.x - b.x, a.y - b.y}; }
+// Products rounded by themselves and fused multiply-adds, written out where a
+// sum has two products: left to the compiler, which of them is fused may differ
+// between two instantiations of the same code, and the launch shapes, the
+// batched and the single kernels have to give the same bits.
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
 template <class V> __device__ __forceinline__ V c_mul(V a, V b) {
-    return {a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x};
+    return {fma_rn(a.x, b.x, -mul_rn(a.y, b.y)), fma_rn(a.x, b.y, mul_rn(a.y, b.x))};
 }
 template <class V> __device__ __forceinline__ V c_conj(V a) { return {a.x, -a.y}; }
 template <class V, typename T> __device__ __forceinline__ V c_scale(V a, T s) { return {a.x * s, a.y * s}; }
@@ -56,8 +64,16 @@ template <> struct FixedPoint<double> {
     static __device__ __forceinline__ unsigned long long to_grid(double w) { return to_patch(w); }
 };
 // Fixed point -> density (scale = 2^-F / dV); no FP64 in the FP32 path.
-__device__ __forceinline__ float from_fixed(long long v, float scale) { return __ll2float_rn(v) * scale; }
-__device__ __forceinline__ double from_fixed(long long v, double scale) { return (double)v * scale; }
+__device__ __forceinline__ float from_fixed(long long v, float scale) { return mul_rn(__ll2float_rn(v), scale); }
+__device__ __forceinline__ double from_fixed(long long v, double scale) { return mul_rn((double)v, scale); }
+// The same for densities (v >= 0). A sum below 2^32 (a thousand beads on one
+// point) is converted from 32 bits: the 64-bit conversion runs at a small
+// fraction of that rate, and both round the same value to nearest.
+__device__ __forceinline__ float density_from_fixed(long long v, float scale) {
+    const float f = (v >> 32) == 0 ? __uint2float_rn((unsigned)v) : __ll2float_rn(v);
+    return mul_rn(f, scale);
+}
+__device__ __forceinline__ double density_from_fixed(long long v, double scale) { return from_fixed(v, scale); }
 
 // Tiles of the bead kernel: beads are binned by 8x8x8 grid cells.
 constexpr int kTile = 8;

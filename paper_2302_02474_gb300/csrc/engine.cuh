@@ -49,7 +49,7 @@ template <typename T> class Engine final : public EngineBase {
         M_ = (size_t)nz_ * n_ * n_;
         tiles_ = (n_ + kTile - 1) / kTile;
         P_ = cfg->pmeorder + 1;
-        plane_fits_ = plane_smem() <= 200 * 1024;
+        plane_fits_ = plane_fits(n_, sizeof(V));
         C_ = std::min(n_, (int)(128 / sizeof(V)));  // y-column tiles of the split passes
         CZ_ = zpass_cols(n_);                          // column tiles of the z pass
         TILD_CUDA(cudaGetDevice(&device_));
@@ -395,7 +395,7 @@ template <typename T> class Engine final : public EngineBase {
         const int el = c_el_on() ? 1 : 0;
         if ((st = dispatch_n([&](auto nn) -> tild_status {
                  constexpr int NN = decltype(nn)::value;
-                 if constexpr ((size_t)NN * (NN + 1) * sizeof(V) <= 200 * 1024) {
+                 if constexpr (plane_fits(NN, sizeof(V))) {
                      constexpr int CV = vjp_cols(NN);
                      xy_forward_cplx<T, NN><<<dim3(NN, 3), 512, plane_smem(), stream_>>>((const longlong2*)fx, bits, S, H_, tw_);
                      z_vjp<T, NN, CV><<<dim3(NN / CV, NN / 2 + 1), 256, vjp_smem(), stream_>>>(H_, Zxy_, tw_, sp, partials_, el);
@@ -1020,6 +1020,7 @@ template <typename T> class Engine final : public EngineBase {
     static unsigned blocks(size_t count) { return (unsigned)((count + 255) / 256); }
     static size_t dtype_size(int dtype) { return dtype == TILD_DTYPE_F32 ? 4 : 8; }
 
+    // the planes (and the rows) of the xy passes, with twiddles
     size_t plane_smem() const { return ((size_t)n_ + (size_t)n_ * row_pitch(n_)) * sizeof(V); }
     // two dimensions: z stays 0
     tild_status zero_z() {
@@ -1305,7 +1306,7 @@ template <typename T> class Engine final : public EngineBase {
 
     template <int NN> tild_status attrs_n() {
         if (plane_fits_) {
-            if constexpr ((size_t)NN * (NN + 1) * sizeof(V) <= 200 * 1024) {
+            if constexpr (plane_fits(NN, sizeof(V))) {
                 TILD_CUDA(cudaFuncSetAttribute(xy_forward_plane<T, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plane_smem()));
                 TILD_CUDA(cudaFuncSetAttribute(xy_inverse_plane<T, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plane_smem()));
                 if constexpr (plane_nt_ok(NN, 256)) {
@@ -1334,13 +1335,13 @@ template <typename T> class Engine final : public EngineBase {
         constexpr int C2 = zpass_cols2(NN);
         TILD_CUDA(cudaFuncSetAttribute(z_spectral_pairs<T, NN, C2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)zpass2_smem()));
         TILD_CUDA(cudaFuncSetAttribute(z_spectral_pairs<T, NN, C2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)zpass2_smem()));
-        TILD_CUDA(cudaFuncSetAttribute(z_spectral<T, NN, CC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)zpass_smem()));
-        if constexpr (zpass_cols_alt(NN) != CC)
-            TILD_CUDA(cudaFuncSetAttribute(z_spectral<T, NN, zpass_cols_alt(NN)>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)zpass_smem_cols(zpass_cols_alt(NN))));
-        TILD_CUDA(cudaFuncSetAttribute(z_spectral<T, NN, CC, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)zpass_smem()));
-        TILD_CUDA(cudaFuncSetAttribute(z_spectral<T, NN, CC, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)zpass_smem()));
-        TILD_CUDA(cudaFuncSetAttribute(z_spectral<T, NN, CC, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)zpass_smem()));
+        TILD_CUDA(cudaFuncSetAttribute(z_spectrum<T, NN, CC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)zpass_smem()));
+        tild_status st = with_z<NN>([&](auto cc, auto g, auto el, auto e) -> tild_status {
+            TILD_CUDA(cudaFuncSetAttribute(z_spectral<T, NN, decltype(cc)::value, decltype(g)::value != 0, decltype(el)::value != 0, decltype(e)::value != 0>,
+                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)zpass_smem_cols(decltype(cc)::value)));
+            return TILD_OK;
+        }, true);
+        if (st) return st;
         return TILD_OK;
     }
 
@@ -1413,7 +1414,7 @@ template <typename T> class Engine final : public EngineBase {
 
     template <int NN> tild_status forward_n(bool zero_after) {
         if (use_planes()) {
-            if constexpr ((size_t)NN * (NN + 1) * sizeof(V) <= 200 * 1024) {
+            if constexpr (plane_fits(NN, sizeof(V))) {
                 with_nt<NN>([&](auto nt) {
                     constexpr int NT = decltype(nt)::value;
                     xy_forward_plane<T, NN, NT><<<dim3(NN, NP_), NT, plane_smem(), stream_>>>(
@@ -1450,7 +1451,10 @@ template <typename T> class Engine final : public EngineBase {
     }
     size_t vjp_smem() const { return ((size_t)n_ + 8 * (size_t)n_ * vjp_cols(n_)) * sizeof(V); }
 
+    // At 256^3 half of that: 16 columns take 133 KB (one CTA per SM) and 177
+    // registers, 8 columns 67 KB and two CTAs per SM (z pass 148 against 114 us).
     static constexpr int zpass_cols(int n) {
+        if (n == 256) return (int)(64 / sizeof(V));
         int c = (int)(128 / sizeof(V));
         while (c > 1 && (n % c) != 0) c /= 2;
         return c < n ? c : n;
@@ -1480,7 +1484,7 @@ template <typename T> class Engine final : public EngineBase {
     }
     bool use_planes() const { return plane_fits_ && plane_nt_ != 0; }
     // runtime forms for the batch's groups
-    static bool plane_nt_allowed(int n, int nt) { return plane_nt_ok(n, nt) && n * (n + 1) * (int)sizeof(V) <= 200 * 1024; }
+    static bool plane_nt_allowed(int n, int nt) { return plane_nt_ok(n, nt) && plane_fits(n, sizeof(V)); }
     static int zpass_cols_n(int n) { return zpass_cols(n); }
     static int zpass_cols_alt_n(int n) { return zpass_cols_alt(n); }
     template <int NN, class F> void with_nt(F&& f) {
@@ -1521,41 +1525,53 @@ template <typename T> class Engine final : public EngineBase {
 
     template <int NN> tild_status zpass_n(double* partials, V* spec_out, bool g_only) {
         constexpr int CC = zpass_cols(NN);
-        const dim3 grid(NN / CC, NN / 2 + 1);
         const SpectralParams<T> sp = spectral_params();
         const bool el = c_el_on();
-        if (NP_ == 2) {
-            if (spec_out) {
-                // the spectra alone: each pair's forward z transform (no coupling)
-                for (int q = 0; q < 2; ++q)
-                    z_spectral<T, NN, CC><<<grid, 256, zpass_smem(), stream_>>>(Zxy_ + q * M_, H_, tw_, sp, nullptr,
-                                                                              spec_out + q * M_);
-            } else {
-                constexpr int C2 = zpass_cols2(NN);
-                const dim3 grid2(NN / C2, NN / 2 + 1);
-                if (g_only)
-                    z_spectral_pairs<T, NN, C2, true><<<grid2, 256, zpass2_smem(), stream_>>>(Zxy_, H_, tw_, sp, partials);
-                else
-                    z_spectral_pairs<T, NN, C2><<<grid2, 256, zpass2_smem(), stream_>>>(Zxy_, H_, tw_, sp, partials);
-            }
+        if (spec_out) {
+            // the spectra alone: each pair's forward z transform (no coupling)
+            for (int q = 0; q < NP_; ++q)
+                z_spectrum<T, NN, CC><<<dim3(NN / CC, NN), 256, zpass_smem(), stream_>>>(Zxy_ + q * M_, tw_, spec_out + q * M_);
             TILD_CUDA(cudaGetLastError());
             return TILD_OK;
         }
-        if (g_only && el)
-            z_spectral<T, NN, CC, true, true><<<grid, 256, zpass_smem(), stream_>>>(Zxy_, H_, tw_, sp, partials, spec_out);
-        else if (g_only)
-            z_spectral<T, NN, CC, true><<<grid, 256, zpass_smem(), stream_>>>(Zxy_, H_, tw_, sp, partials, spec_out);
-        else if (el)
-            z_spectral<T, NN, CC, false, true><<<grid, 256, zpass_smem(), stream_>>>(Zxy_, H_, tw_, sp, partials, spec_out);
-        else if (zalt_ && !partials && !spec_out) {
-            // the step's z pass with the alternative column tile (launch shapes)
-            constexpr int CA = zpass_cols_alt(NN);
-            z_spectral<T, NN, CA><<<dim3(NN / CA, NN / 2 + 1), 256, zpass_smem_cols(CA), stream_>>>(Zxy_, H_, tw_, sp,
-                                                                                                 nullptr, nullptr);
-        } else
-            z_spectral<T, NN, CC><<<grid, 256, zpass_smem(), stream_>>>(Zxy_, H_, tw_, sp, partials, spec_out);
-        TILD_CUDA(cudaGetLastError());
-        return TILD_OK;
+        if (NP_ == 2) {
+            constexpr int C2 = zpass_cols2(NN);
+            const dim3 grid2(NN / C2, NN / 2 + 1);
+            if (g_only)
+                z_spectral_pairs<T, NN, C2, true><<<grid2, 256, zpass2_smem(), stream_>>>(Zxy_, H_, tw_, sp, partials);
+            else
+                z_spectral_pairs<T, NN, C2><<<grid2, 256, zpass2_smem(), stream_>>>(Zxy_, H_, tw_, sp, partials);
+            TILD_CUDA(cudaGetLastError());
+            return TILD_OK;
+        }
+        return with_z<NN>([&](auto cc, auto g, auto e_l, auto e) -> tild_status {
+            constexpr int CZ = decltype(cc)::value;
+            z_spectral<T, NN, CZ, decltype(g)::value != 0, decltype(e_l)::value != 0, decltype(e)::value != 0>
+                <<<dim3(NN / CZ, NN / 2 + 1), 256, zpass_smem_cols(CZ), stream_>>>(Zxy_, H_, tw_, sp, partials);
+            TILD_CUDA(cudaGetLastError());
+            return TILD_OK;
+        }, false, g_only, el, partials != nullptr);
+    }
+    // f(columns, G alone, charges, energies) for the z pass to launch, or for
+    // every instantiation when `all`. The alternative column tile serves the
+    // plain step only (launch shapes).
+    template <int NN, class F>
+    tild_status with_z(F&& f, bool all, bool g_only = false, bool el = false, bool want_e = false) {
+        constexpr int CC = zpass_cols(NN), CA = zpass_cols_alt(NN);
+        tild_status st = TILD_OK;
+        auto pick = [&](bool take, auto cc, auto g, auto e_l, auto e) {
+            if (!st && (all || take)) st = f(cc, g, e_l, e);
+        };
+        if constexpr (CA != CC) pick(zalt_ && !g_only && !el && !want_e, ic<CA>{}, ic<0>{}, ic<0>{}, ic<0>{});
+        pick(!(zalt_ && CA != CC) && !g_only && !el && !want_e, ic<CC>{}, ic<0>{}, ic<0>{}, ic<0>{});
+        pick(g_only && !el && !want_e, ic<CC>{}, ic<1>{}, ic<0>{}, ic<0>{});
+        pick(!g_only && el && !want_e, ic<CC>{}, ic<0>{}, ic<1>{}, ic<0>{});
+        pick(g_only && el && !want_e, ic<CC>{}, ic<1>{}, ic<1>{}, ic<0>{});
+        pick(!g_only && !el && want_e, ic<CC>{}, ic<0>{}, ic<0>{}, ic<1>{});
+        pick(g_only && !el && want_e, ic<CC>{}, ic<1>{}, ic<0>{}, ic<1>{});
+        pick(!g_only && el && want_e, ic<CC>{}, ic<0>{}, ic<1>{}, ic<1>{});
+        pick(g_only && el && want_e, ic<CC>{}, ic<1>{}, ic<1>{}, ic<1>{});
+        return st;
     }
     // separable Gaussian tables exp(-s^2 k_m^2), k_m = 2 pi m / L, m in FFT
     // index order: the pair kernel's (s = a) and, with charges, the charge
@@ -1604,7 +1620,7 @@ template <typename T> class Engine final : public EngineBase {
         const unsigned nd = what == kInvGrad ? 3 : what == kInvGradPot ? 4 : 1;
         const int d0 = what == kInvPot ? 3 : 0;
         if (use_planes()) {
-            if constexpr ((size_t)NN * (NN + 1) * sizeof(V) <= 200 * 1024) {
+            if constexpr (plane_fits(NN, sizeof(V))) {
                 with_nt<NN>([&](auto nt) {
                     constexpr int NT = decltype(nt)::value;
                     xy_inverse_plane<T, NN, NT><<<dim3(NN, nd, NP_), NT, plane_smem(), stream_>>>(H_, grad_, tw_, two_pi_L(), d0);

@@ -63,7 +63,7 @@ template <int DIR, class V> __device__ __forceinline__ V w16_mul(int m, V v) {
         default: cr = c1; ci = s1; break;  // 15
     }
     if (DIR > 0) ci = -ci;
-    return {v.x * cr - v.y * ci, v.x * ci + v.y * cr};
+    return c_mul(v, V{cr, ci});
 }
 
 // In-register DFT of R points (R = 1, 2, 4, 8, 16 by radix-2 decimation in
@@ -97,8 +97,8 @@ template <int DIR, class V> struct reg_dft<3, DIR, V> {
         using T = decltype(v[0].x);
         const T c = T(-0.5), s = T(DIR) * T(0.86602540378443864676);  // DIR sin(2 pi / 3)
         const V t1 = c_add(v[1], v[2]), t3 = c_sub(v[1], v[2]);
-        const V m = {v[0].x + c * t1.x, v[0].y + c * t1.y};
-        const V it = {-s * t3.y, s * t3.x};  // i s (x1 - x2)
+        const V m = {fma_rn(c, t1.x, v[0].x), fma_rn(c, t1.y, v[0].y)};
+        const V it = {-mul_rn(s, t3.y), mul_rn(s, t3.x)};  // i s (x1 - x2)
         v[0] = c_add(v[0], t1);
         v[1] = c_add(m, it);
         v[2] = c_sub(m, it);
@@ -115,10 +115,10 @@ template <int DIR, class V> struct reg_dft<5, DIR, V> {
         const T s1 = T(DIR) * T(0.95105651629515357212), s2 = T(DIR) * T(0.58778525229247312917);
         const V t1 = c_add(v[1], v[4]), t2 = c_add(v[2], v[3]);
         const V t3 = c_sub(v[1], v[4]), t4 = c_sub(v[2], v[3]);
-        const V a = {v[0].x + c1 * t1.x + c2 * t2.x, v[0].y + c1 * t1.y + c2 * t2.y};
-        const V b = {v[0].x + c2 * t1.x + c1 * t2.x, v[0].y + c2 * t1.y + c1 * t2.y};
-        const V p = {s1 * t3.x + s2 * t4.x, s1 * t3.y + s2 * t4.y};
-        const V q = {s2 * t3.x - s1 * t4.x, s2 * t3.y - s1 * t4.y};
+        const V a = {fma_rn(c2, t2.x, fma_rn(c1, t1.x, v[0].x)), fma_rn(c2, t2.y, fma_rn(c1, t1.y, v[0].y))};
+        const V b = {fma_rn(c1, t2.x, fma_rn(c2, t1.x, v[0].x)), fma_rn(c1, t2.y, fma_rn(c2, t1.y, v[0].y))};
+        const V p = {fma_rn(s1, t3.x, mul_rn(s2, t4.x)), fma_rn(s1, t3.y, mul_rn(s2, t4.y))};
+        const V q = {fma_rn(s2, t3.x, -mul_rn(s1, t4.x)), fma_rn(s2, t3.y, -mul_rn(s1, t4.y))};
         const V ip = {-p.y, p.x}, iq = {-q.y, q.x};
         v[0] = {v[0].x + t1.x + t2.x, v[0].y + t1.y + t2.y};
         v[1] = c_add(a, ip);
@@ -216,41 +216,56 @@ template <int LS> struct StridedLines {
     __device__ __forceinline__ int operator()(int l) const { return l * LS; }
 };
 
-}  // namespace tild
-
-namespace tild {
-
-// smem_fft_lines whose second stage hands each output to out(l, k, X_l[k])
-// instead of writing it back to shared memory (the caller's last use of the
-// lines, e.g. a store to global memory); no barrier at the end. N2 > 1.
-template <int N, int DIR, int NLINES, int NTHR, class V, class Addr, class Out>
-__device__ __forceinline__ void smem_fft_lines_out(V* buf, Addr addr, int es, const V* tw, Out out) {
-    constexpr int N1 = fft_split<N>::N1;
-    constexpr int N2 = fft_split<N>::N2;
-    static_assert(N2 > 1, "two-stage lengths only");
-    constexpr int UPT = (NLINES * N1 + NTHR - 1) / NTHR;
-    smem_fft_stage_a<N, DIR, NLINES, NTHR>(buf, addr, es, tw);
-    V v[UPT][N2];
-#pragma unroll
-    for (int r = 0; r < UPT; ++r) {
-        const int u = threadIdx.x + r * NTHR;
-        if (u < NLINES * N1) {
-            const int l = u % NLINES, k1 = u / NLINES;
-            const V* p = buf + addr(l) + k1 * N2 * es;
-#pragma unroll
-            for (int j2 = 0; j2 < N2; ++j2) v[r][j2] = p[j2 * es];
-        }
+// ------------------------------------------------- register-first stages
+//
+// The passes of the step run each stage of a line transform as one visit of
+// shared memory: the first stage takes its inputs straight from global
+// memory (or from the registers of the stage before), and the last one hands
+// its outputs straight to global memory. Every stage works in place: unit
+// (line, j2) of stage A owns the slots k1 N2 + j2 and unit (line, k1) of stage
+// B the slots k1 N2 + j2, so a stage reads and writes its own slots only and
+// needs no barrier in between, its units can run one after the other (small
+// code, few registers), and one barrier separates two stages. The price is
+// that the transform is left in the order slot k1 N2 + k2 <-> X[k1 + N1 k2],
+// which the consumer of the lines undoes in its addressing.
+//
+// Rows of a plane keep slot i at i + (i / N2) (S2 - N2) with S2 odd and have a
+// pitch of N2 modulo 16 words of 8 bytes: lanes over (j2, row) and lanes over
+// k1 both fall into distinct banks.
+template <int N> struct LineSlots {
+    static constexpr int N1 = fft_split<N>::N1, N2 = fft_split<N>::N2;
+    static constexpr int S2 = N2 | 1;
+    static constexpr int make_pitch() {
+        int p = N1 * S2;
+        while (p % 16 != N2 % 16) ++p;
+        return p;
     }
+    static constexpr int pitch = make_pitch();
+    // padded position of slot i in a row
+    static __device__ __forceinline__ int at(int i) { return (i / N2) * S2 + i % N2; }
+    // the slot that holds X[k] after stage B, and its inverse
+    static __device__ __forceinline__ int slot_of(int k) { return (k % N1) * N2 + k / N1; }
+    static __device__ __forceinline__ int index_of(int slot) { return slot / N2 + N1 * (slot % N2); }
+};
+
+// v * s with each product rounded by itself: the same bits in every pass that
+// scales a field.
+template <class V, typename T> __device__ __forceinline__ V c_scale_rn(V v, T s) { return {mul_rn(v.x, s), mul_rn(v.y, s)}; }
+
+// Stage A of one unit in registers: the N1-point DFT over j1 and the twiddle
+// W_N^{j2 k1}.
+template <int N, int DIR, class V>
+__device__ __forceinline__ void stage_a_regs(V (&v)[fft_split<N>::N1], int j2, const V* tw) {
+    constexpr int N1 = fft_split<N>::N1;
+    reg_dft<N1, DIR, V>::run(v);
+    if (fft_split<N>::N2 > 1) {
 #pragma unroll
-    for (int r = 0; r < UPT; ++r) {
-        const int u = threadIdx.x + r * NTHR;
-        if (u < NLINES * N1) {
-            const int l = u % NLINES, k1 = u / NLINES;
-            reg_dft<N2, DIR, V>::run(v[r]);
-#pragma unroll
-            for (int k2 = 0; k2 < N2; ++k2) out(l, k1 + N1 * k2, v[r][k2]);
-        }
+        for (int k1 = 1; k1 < N1; ++k1) v[k1] = c_mul(v[k1], twiddle<DIR>(tw, j2 * k1));
     }
 }
+
+// Grid sizes whose xy-plane of values of `bytes` fits the shared memory of one
+// CTA (FP32 up to 128, FP64 up to 80).
+__host__ __device__ constexpr bool plane_fits(int n, int bytes) { return n * (n + 1) * bytes <= 200 * 1024; }
 
 }  // namespace tild

@@ -44,6 +44,7 @@ template <typename T> struct SpectralParams {
 };
 
 template <int N> __host__ __device__ __forceinline__ int kx_of_pos(int p);
+template <int N> __host__ __device__ __forceinline__ int pos_of_kx(int kx);
 template <int C, int STRIDE> struct TileAddr;
 
 // Wavenumber 2 pi m / L of FFT index i (m = i or i - n; the Nyquist index
@@ -63,17 +64,26 @@ template <typename T, int N> __device__ __forceinline__ T grad_k(int i, T two_pi
 __device__ __forceinline__ float recip(float x) { return __frcp_rn(x); }
 __device__ __forceinline__ double recip(double x) { return 1.0 / x; }
 
-// Pitch (in complex elements) of a row of n elements in shared memory: odd
-// so that threads on consecutive rows hit distinct banks.
-__host__ __device__ constexpr int row_pitch(int n) { return n + 1; }
+// Host side of LineSlots<n>::pitch: complex values of shared memory per row of
+// the xy passes (0: no hand-written transform of that length).
+inline int row_pitch(int n) {
+    switch (n) {
+        case 8: return LineSlots<8>::pitch;
+        case 16: return LineSlots<16>::pitch;
+        case 24: return LineSlots<24>::pitch;
+        case 32: return LineSlots<32>::pitch;
+        case 40: return LineSlots<40>::pitch;
+        case 48: return LineSlots<48>::pitch;
+        case 64: return LineSlots<64>::pitch;
+        case 80: return LineSlots<80>::pitch;
+        case 128: return LineSlots<128>::pitch;
+        case 256: return LineSlots<256>::pitch;
+    }
+    return 0;
+}
 
 template <class V> __device__ __forceinline__ void load_twiddles(V* s_tw, const V* g_tw, int n) {
     for (int i = threadIdx.x; i < n; i += blockDim.x) s_tw[i] = g_tw[i];
-}
-
-// Units of stage B per thread for `lines` lines of length N with THREADS threads.
-template <int N, int THREADS> __host__ __device__ constexpr int upt_for(int lines) {
-    return (lines * fft_split<N>::N1 + THREADS - 1) / THREADS;
 }
 
 // Copy COUNT elements from global to shared memory with up to 16
@@ -102,43 +112,189 @@ __device__ __forceinline__ void batched_load(Src src, Dst dst) {
     }
 }
 
-// Load ROWS rows of N fixed-point densities of both species (16-byte
-// vectors), optionally zero them, and store rho_A + i rho_B to shared rows of
-// pitch PITCH. Loads are issued in batches before any store so that the
-// zeroing stores do not serialise them.
-template <int N, int PITCH, int ROWS, int NTHR, class V, typename T>
-__device__ __forceinline__ void load_fixed_rows(unsigned long long* __restrict__ ga, unsigned long long* __restrict__ gb,
-                                                V* rows, T scale, int zero_after) {
-    constexpr int PAIRS = ROWS * N / 2;
-    constexpr int ITER = (PAIRS + NTHR - 1) / NTHR;
-    constexpr int BATCH = ITER < 8 ? ITER : 8;
-    constexpr bool kFull = PAIRS % NTHR == 0 && ITER % BATCH == 0;  // no partial batch
-    longlong2* pa = reinterpret_cast<longlong2*>(ga);
-    longlong2* pb = reinterpret_cast<longlong2*>(gb);
+// The N1 inputs of stage-A unit j2 of one row of fixed-point densities
+// (ga, gb: the row of either species): rho_A + i rho_B at x = j2 + N2 j1. Up to
+// eight loads of each species are in flight (the raw 64-bit values of more
+// would not leave registers for the transform). Lanes take consecutive j2,
+// so a warp reads whole sectors.
+template <int N, class V, typename T>
+__device__ __forceinline__ void load_fixed_unit(const long long* __restrict__ ga, const long long* __restrict__ gb, int j2,
+                                                T scale, V (&v)[fft_split<N>::N1]) {
+    constexpr int N1 = fft_split<N>::N1, N2 = fft_split<N>::N2;
+    constexpr int B = N1 < 8 ? N1 : 8;
+#pragma unroll
+    for (int h = 0; h < N1; h += B) {
+        long long a[B], b[B];
+#pragma unroll
+        for (int k = 0; k < B; ++k) {
+            a[k] = __ldcs(ga + j2 + N2 * (h + k));
+            b[k] = __ldcs(gb + j2 + N2 * (h + k));
+        }
+#pragma unroll
+        for (int k = 0; k < B; ++k) v[h + k] = V{density_from_fixed(a[k], scale), density_from_fixed(b[k], scale)};
+    }
+}
+
+// Zero `count` values (16-byte stores; count even, base 16-byte aligned).
+template <int NTHR> __device__ __forceinline__ void zero_fixed(unsigned long long* g, int count) {
+    longlong2* p = reinterpret_cast<longlong2*>(g);
+    for (int i = threadIdx.x; i < count / 2; i += NTHR) p[i] = make_longlong2(0, 0);
+}
+
+// --------------------------------------------------------------------------
+// Transforms of one whole xy-plane held in shared memory, [row][LineSlots],
+// four stages with three barriers: x stage A from the loader, x stage B, y
+// stage A, y stage B to global memory (forward), and the mirror image
+// (inverse). Bound by shared memory and latency (one CTA per SM at 128^3):
+// a stage visits shared memory once, in place, where a separate load, two
+// stages with their own barriers, a scaling pass and a store pass per
+// direction visited it ten to twelve times (inverse at 128^3, 512 threads:
+// 38.1 -> 34.9 us; at 80^3, 14.4 -> 12.3 us in the step).
+// --------------------------------------------------------------------------
+// load(y, j2, v): inputs x = j2 + N2 j1 of row y; after_load(): runs once all
+// rows have been loaded; dst: [ky][pos(kx)].
+template <typename T, int N, int NT, class Load, class After>
+__device__ __forceinline__ void plane_forward_xy(cplx_t<T>* plane, cplx_t<T>* tw, const cplx_t<T>* __restrict__ tw_g, Load load,
+                                                 After after_load, cplx_t<T>* __restrict__ dst) {
+    using V = cplx_t<T>;
+    using LS = LineSlots<N>;
+    constexpr int N1 = LS::N1, N2 = LS::N2, S2 = LS::S2, PITCH = LS::pitch;
+    {
+        // x stage A: unit (row, j2), lanes over j2 (the first loads are in
+        // flight while the twiddles are copied)
+        int u = threadIdx.x;
+        V v[N1];
+        if (u < N * N2) load(u / N2, u % N2, v);
+        load_twiddles(tw, tw_g, N);
+        __syncthreads();
 #pragma unroll 1
-    for (int k0 = 0; k0 < ITER; k0 += BATCH) {
-        longlong2 a[BATCH], b[BATCH];
+        while (u < N * N2) {
+            const int r = u / N2, j2 = u % N2;
+            stage_a_regs<N, -1>(v, j2, tw);
+            V* p = plane + r * PITCH + j2;
 #pragma unroll
-        for (int k = 0; k < BATCH; ++k) {
-            const int i = threadIdx.x + (k0 + k) * NTHR;
-            if (kFull || i < PAIRS) {
-                a[k] = __ldcs(pa + i);
-                b[k] = __ldcs(pb + i);
-            }
+            for (int k1 = 0; k1 < N1; ++k1) p[k1 * S2] = v[k1];
+            u += NT;
+            if (u < N * N2) load(u / N2, u % N2, v);
+        }
+    }
+    __syncthreads();
+    after_load();
+    // x stage B: unit (row, k1), lanes over k1
+#pragma unroll 1
+    for (int u = threadIdx.x; u < N * N1; u += NT) {
+        V* p = plane + (u / N1) * PITCH + (u % N1) * S2;
+        V v[N2];
+#pragma unroll
+        for (int j = 0; j < N2; ++j) v[j] = p[j];
+        reg_dft<N2, -1, V>::run(v);
+#pragma unroll
+        for (int j = 0; j < N2; ++j) p[j] = v[j];
+    }
+    __syncthreads();
+    // y stage A: unit (column slot, j2), lanes over columns
+#pragma unroll 1
+    for (int u = threadIdx.x; u < N * N2; u += NT) {
+        const int j2 = u / N;
+        V* p = plane + j2 * PITCH + LS::at(u % N);
+        V v[N1];
+#pragma unroll
+        for (int k = 0; k < N1; ++k) v[k] = p[k * N2 * PITCH];
+        stage_a_regs<N, -1>(v, j2, tw);
+#pragma unroll
+        for (int k = 0; k < N1; ++k) p[k * N2 * PITCH] = v[k];
+    }
+    __syncthreads();
+    // y stage B: unit (column position, k1), lanes over positions, to global memory
+#pragma unroll 1
+    for (int u = threadIdx.x; u < N * N1; u += NT) {
+        const int q = u % N, k1 = u / N;
+        const V* p = plane + k1 * N2 * PITCH + LS::at(LS::slot_of(kx_of_pos<N>(q)));
+        V v[N2];
+#pragma unroll
+        for (int j = 0; j < N2; ++j) v[j] = p[j * PITCH];
+        reg_dft<N2, -1, V>::run(v);
+#pragma unroll
+        for (int k2 = 0; k2 < N2; ++k2) dst[(k1 + N1 * k2) * N + q] = v[k2];
+    }
+}
+
+// load(ky, pos): the input at row ky, column position pos; scale(kx): the
+// factor of the columns between the two transforms (x_scale: apply it);
+// dst: [y][x].
+template <typename T, int N, int NT, class Load>
+__device__ __forceinline__ void plane_inverse_yx(cplx_t<T>* plane, cplx_t<T>* tw, const cplx_t<T>* __restrict__ tw_g, Load load,
+                                                 bool x_scale, T two_pi_over_L, cplx_t<T>* __restrict__ dst) {
+    using V = cplx_t<T>;
+    using LS = LineSlots<N>;
+    constexpr int N1 = LS::N1, N2 = LS::N2, S2 = LS::S2, PITCH = LS::pitch;
+    {
+        // y stage A: unit (column position, j2), lanes over positions
+        int u = threadIdx.x;
+        V v[N1];
+        auto fetch = [&]() {
+#pragma unroll
+            for (int k = 0; k < N1; ++k) v[k] = load(u / N + N2 * k, u % N);
+        };
+        if (u < N * N2) fetch();
+        load_twiddles(tw, tw_g, N);
+        __syncthreads();
+#pragma unroll 1
+        while (u < N * N2) {
+            const int j2 = u / N;
+            stage_a_regs<N, +1>(v, j2, tw);
+            // columns in slot order of their natural index kx
+            V* p = plane + j2 * PITCH + LS::at(kx_of_pos<N>(u % N));
+#pragma unroll
+            for (int k1 = 0; k1 < N1; ++k1) p[k1 * N2 * PITCH] = v[k1];
+            u += NT;
+            if (u < N * N2) fetch();
+        }
+    }
+    __syncthreads();
+    // y stage B: unit (column, k1), lanes over columns
+#pragma unroll 1
+    for (int u = threadIdx.x; u < N * N1; u += NT) {
+        const int kx = u % N;
+        V* p = plane + (u / N) * N2 * PITCH + LS::at(kx);
+        V v[N2];
+#pragma unroll
+        for (int j = 0; j < N2; ++j) v[j] = p[j * PITCH];
+        reg_dft<N2, +1, V>::run(v);
+        if (x_scale) {
+            const T s = grad_k<T, N>(kx, two_pi_over_L);
+#pragma unroll
+            for (int j = 0; j < N2; ++j) v[j] = c_scale_rn(v[j], s);
         }
 #pragma unroll
-        for (int k = 0; k < BATCH; ++k) {
-            const int i = threadIdx.x + (k0 + k) * NTHR;
-            if (kFull || i < PAIRS) {
-                if (zero_after) {
-                    pa[i] = make_longlong2(0, 0);
-                    pb[i] = make_longlong2(0, 0);
-                }
-                const int r = (2 * i) / N, x = (2 * i) % N;
-                rows[r * PITCH + x] = V{from_fixed(a[k].x, scale), from_fixed(b[k].x, scale)};
-                rows[r * PITCH + x + 1] = V{from_fixed(a[k].y, scale), from_fixed(b[k].y, scale)};
-            }
-        }
+        for (int j = 0; j < N2; ++j) p[j * PITCH] = v[j];
+    }
+    __syncthreads();
+    // x stage A: unit (row, j2), lanes over j2; row r holds y = index_of(r)
+#pragma unroll 1
+    for (int u = threadIdx.x; u < N * N2; u += NT) {
+        const int j2 = u % N2;
+        V* p = plane + (u / N2) * PITCH + j2;
+        V v[N1];
+#pragma unroll
+        for (int k = 0; k < N1; ++k) v[k] = p[k * S2];
+        stage_a_regs<N, +1>(v, j2, tw);
+#pragma unroll
+        for (int k = 0; k < N1; ++k) p[k * S2] = v[k];
+    }
+    __syncthreads();
+    // x stage B: unit (row, k1), lanes over k1, to global memory
+#pragma unroll 1
+    for (int u = threadIdx.x; u < N * N1; u += NT) {
+        const int r = u / N1, k1 = u % N1;
+        const V* p = plane + r * PITCH + k1 * S2;
+        V v[N2];
+#pragma unroll
+        for (int j = 0; j < N2; ++j) v[j] = p[j];
+        reg_dft<N2, +1, V>::run(v);
+        V* o = dst + LS::index_of(r) * N + k1;
+#pragma unroll
+        for (int k2 = 0; k2 < N2; ++k2) o[N1 * k2] = v[k2];
     }
 }
 
@@ -165,26 +321,26 @@ __device__ __forceinline__ void xy_forward_plane_body(const ForwardArgs<T>& args
     const T scale = args.scale;
     const int zero_after = args.zero_after;
     unsigned long long* step_ctr = args.step_ctr;
-    constexpr int PITCH = row_pitch(N);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V* tw = reinterpret_cast<V*>(smem_raw);
     V* plane = tw + N;
-    load_twiddles(tw, tw_g, N);
     // a step's first kernel advances the noise counter to n+1
     if (step_ctr && bx == 0 && threadIdx.x == 0) *step_ctr += 1ull;
 
-    const int z = bx;
     const size_t M = (size_t)N * N * N;
-    const size_t base = (size_t)z * N * N;
-    // load + convert: pairs of x so that global accesses are 16-byte vectors
-    load_fixed_rows<N, PITCH, N, NT>(rho_fx + base, rho_fx + M + base, plane, scale, zero_after);
-    __syncthreads();
-    smem_fft_lines<N, -1, N, NT>(plane, StridedLines<PITCH>{}, 1, tw);  // along x
-    smem_fft_lines<N, -1, N, NT>(plane, StridedLines<1>{}, PITCH, tw);  // along y
-    for (int i = threadIdx.x; i < N * N; i += NT) {
-        const int y = i / N, x = i % N;
-        Zxy[base + i] = plane[y * PITCH + kx_of_pos<N>(x)];  // mirror-paired column order
-    }
+    const size_t base = (size_t)bx * N * N;
+    const long long* ra = reinterpret_cast<const long long*>(rho_fx + base);
+    const long long* rb = ra + M;
+    plane_forward_xy<T, N, NT>(
+        plane, tw, tw_g,
+        [&](int y, int j2, V (&v)[fft_split<N>::N1]) { load_fixed_unit<N>(ra + y * N, rb + y * N, j2, scale, v); },
+        [&]() {
+            if (zero_after) {  // every density of the plane has been read
+                zero_fixed<NT>(rho_fx + base, N * N);
+                zero_fixed<NT>(rho_fx + M + base, N * N);
+            }
+        },
+        Zxy + base);
 }
 
 // grid = (n, NP): species pair blockIdx.y
@@ -224,35 +380,22 @@ __device__ __forceinline__ void xy_inverse_plane_body(const InverseArgs<T>& args
     cplx_t<T>* __restrict__ grad = args.grad;
     const cplx_t<T>* __restrict__ tw_g = args.tw;
     const T two_pi_over_L = args.two_pi_over_L;
-    constexpr int PITCH = row_pitch(N);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V* tw = reinterpret_cast<V*>(smem_raw);
     V* plane = tw + N;
-    load_twiddles(tw, tw_g, N);
 
     // direction d: x from i k_x G, y from i k_y G, z from G_z (field 2);
     // d = 3 (optional): the potentials themselves, i (w_A + i w_B), from G
     const int d = by + args.d0;
     const size_t M = (size_t)N * N * N;
-    const size_t src = (d == 2 ? 2 * M : 0) + (size_t)bx * N * N;
-    batched_load<N * N, NT, V>([&](int i) { return H[src + i]; },
-                                [&](int i, V v) {
-                                    const int ky = i / N;
-                                    if (d == 1) v = c_scale(v, grad_k<T, N>(ky, two_pi_over_L));
-                                    plane[ky * PITCH + kx_of_pos<N>(i % N)] = v;
-                                });
-    __syncthreads();
-    smem_fft_lines<N, +1, N, NT>(plane, StridedLines<1>{}, PITCH, tw);  // along y
-    if (d == 0) {
-        for (int i = threadIdx.x; i < N * N; i += NT) {
-            const int y = i / N, kx = i % N;
-            plane[y * PITCH + kx] = c_scale(plane[y * PITCH + kx], grad_k<T, N>(kx, two_pi_over_L));
-        }
-        __syncthreads();
-    }
-    smem_fft_lines<N, +1, N, NT>(plane, StridedLines<PITCH>{}, 1, tw);  // along x
-    const size_t dst = (size_t)d * M + (size_t)bx * N * N;
-    for (int i = threadIdx.x; i < N * N; i += NT) grad[dst + i] = plane[(i / N) * PITCH + i % N];
+    const V* src = H + (d == 2 ? 2 * M : 0) + (size_t)bx * N * N;
+    plane_inverse_yx<T, N, NT>(
+        plane, tw, tw_g,
+        [&](int ky, int q) {
+            const V v = src[ky * N + q];
+            return d == 1 ? c_scale_rn(v, grad_k<T, N>(ky, two_pi_over_L)) : v;
+        },
+        d == 0, two_pi_over_L, grad + (size_t)d * M + (size_t)bx * N * N);
 }
 
 // grid = (n, directions, NP): species pair blockIdx.z
@@ -282,49 +425,119 @@ __global__ void __launch_bounds__(256) x_forward_rows(unsigned long long* __rest
                                                        const cplx_t<T>* __restrict__ tw_g, T scale,
                                                        int zero_after, unsigned long long* step_ctr) {
     using V = cplx_t<T>;
-    constexpr int PITCH = row_pitch(N);
+    using LS = LineSlots<N>;
+    constexpr int N1 = LS::N1, N2 = LS::N2, S2 = LS::S2, PITCH = LS::pitch;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V* tw = reinterpret_cast<V*>(smem_raw);
     V* rows = tw + N;
-    load_twiddles(tw, tw_g, N);
     const size_t M = (size_t)N * N * N;
     const size_t base = (size_t)blockIdx.x * R * N;
     const int pr = blockIdx.y;  // species pair
     rho_fx += 2 * pr * M;
     Zxy += pr * M;
     if (step_ctr && blockIdx.x == 0 && pr == 0 && threadIdx.x == 0) *step_ctr += 1ull;
-    load_fixed_rows<N, PITCH, R, 256>(rho_fx + base, rho_fx + M + base, rows, scale, zero_after);
+    const long long* ra = reinterpret_cast<const long long*>(rho_fx + base);
+    const long long* rb = ra + M;
+    {
+        int u = threadIdx.x;  // stage A: unit (row, j2), lanes over j2
+        V v[N1];
+        auto fetch = [&]() { load_fixed_unit<N>(ra + (u / N2) * N, rb + (u / N2) * N, u % N2, scale, v); };
+        if (u < R * N2) fetch();
+        load_twiddles(tw, tw_g, N);
+        __syncthreads();
+#pragma unroll 1
+        while (u < R * N2) {
+            const int j2 = u % N2;
+            stage_a_regs<N, -1>(v, j2, tw);
+            V* p = rows + (u / N2) * PITCH + j2;
+#pragma unroll
+            for (int k1 = 0; k1 < N1; ++k1) p[k1 * S2] = v[k1];
+            u += 256;
+            if (u < R * N2) fetch();
+        }
+    }
     __syncthreads();
-    smem_fft_lines<N, -1, R, 256>(rows, StridedLines<PITCH>{}, 1, tw);
-    for (int i = threadIdx.x; i < R * N; i += blockDim.x) Zxy[base + i] = rows[(i / N) * PITCH + kx_of_pos<N>(i % N)];
+    if (zero_after) {
+        zero_fixed<256>(rho_fx + base, R * N);
+        zero_fixed<256>(rho_fx + M + base, R * N);
+    }
+    // stage B in place; the store below takes the columns in position order
+#pragma unroll 1
+    for (int u = threadIdx.x; u < R * N1; u += 256) {
+        V* p = rows + (u / N1) * PITCH + (u % N1) * S2;
+        V v[N2];
+#pragma unroll
+        for (int j = 0; j < N2; ++j) v[j] = p[j];
+        reg_dft<N2, -1, V>::run(v);
+#pragma unroll
+        for (int j = 0; j < N2; ++j) p[j] = v[j];
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < R * N; i += 256)
+        Zxy[base + i] = rows[(i / N) * PITCH + LS::at(LS::slot_of(kx_of_pos<N>(i % N)))];
 }
 
 template <typename T, int N, int R>
 __global__ void __launch_bounds__(256) x_inverse_rows(const cplx_t<T>* __restrict__ H, cplx_t<T>* __restrict__ grad,
                                                        const cplx_t<T>* __restrict__ tw_g, T two_pi_over_L, int d0) {
     using V = cplx_t<T>;
-    constexpr int PITCH = row_pitch(N);
+    using LS = LineSlots<N>;
+    constexpr int N1 = LS::N1, N2 = LS::N2, S2 = LS::S2, PITCH = LS::pitch;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V* tw = reinterpret_cast<V*>(smem_raw);
     V* rows = tw + N;
-    load_twiddles(tw, tw_g, N);
     const size_t M = (size_t)N * N * N;
     const int d = (int)blockIdx.y + d0;
     H += 3 * (size_t)blockIdx.z * M;  // species pair blockIdx.z
     grad += 4 * (size_t)blockIdx.z * M;
     const size_t base = (size_t)d * M + (size_t)blockIdx.x * R * N;
     // field 3 (optional, the potentials) is the plain transform of field 0
-    const size_t src = (size_t)(d == 3 ? 0 : d) * M + (size_t)blockIdx.x * R * N;
+    const V* src = H + (size_t)(d == 3 ? 0 : d) * M + (size_t)blockIdx.x * R * N;
     const bool kx_mult = d == 0;  // d_x: multiply by k_x before the x transform
-    batched_load<R * N, 256, V>([&](int i) { return H[src + i]; },
-                                [&](int i, V v) {
-                                    const int kx = kx_of_pos<N>(i % N);
-                                    if (kx_mult) v = c_scale(v, grad_k<T, N>(kx, two_pi_over_L));
-                                    rows[(i / N) * PITCH + kx] = v;
-                                });
+    {
+        // stage A: unit (row, j2), lanes over j2. Column kx lies at position
+        // 2 kx or 2 (n - kx) + 1, so lanes read every other value; the values
+        // between them are the mirror columns, which the same CTA reads with
+        // another j1 (from L1)
+        int u = threadIdx.x;
+        V v[N1];
+        auto fetch = [&]() {
+            const V* row = src + (u / N2) * N;
+#pragma unroll
+            for (int k = 0; k < N1; ++k) {
+                const int kx = u % N2 + N2 * k;
+                const V t = __ldg(row + pos_of_kx<N>(kx));
+                v[k] = kx_mult ? c_scale_rn(t, grad_k<T, N>(kx, two_pi_over_L)) : t;
+            }
+        };
+        if (u < R * N2) fetch();
+        load_twiddles(tw, tw_g, N);
+        __syncthreads();
+#pragma unroll 1
+        while (u < R * N2) {
+            const int j2 = u % N2;
+            stage_a_regs<N, +1>(v, j2, tw);
+            V* p = rows + (u / N2) * PITCH + j2;
+#pragma unroll
+            for (int k1 = 0; k1 < N1; ++k1) p[k1 * S2] = v[k1];
+            u += 256;
+            if (u < R * N2) fetch();
+        }
+    }
     __syncthreads();
-    smem_fft_lines<N, +1, R, 256>(rows, StridedLines<PITCH>{}, 1, tw);
-    for (int i = threadIdx.x; i < R * N; i += blockDim.x) grad[base + i] = rows[(i / N) * PITCH + i % N];
+    // stage B: unit (row, k1), lanes over k1, to global memory
+#pragma unroll 1
+    for (int u = threadIdx.x; u < R * N1; u += 256) {
+        const int r = u / N1, k1 = u % N1;
+        const V* p = rows + r * PITCH + k1 * S2;
+        V v[N2];
+#pragma unroll
+        for (int j = 0; j < N2; ++j) v[j] = p[j];
+        reg_dft<N2, +1, V>::run(v);
+        V* o = grad + base + r * N + k1;
+#pragma unroll
+        for (int k2 = 0; k2 < N2; ++k2) o[N1 * k2] = v[k2];
+    }
 }
 
 // Column pass along y: CTA (x tile, z plane, part) handles C columns.
@@ -333,15 +546,20 @@ __global__ void __launch_bounds__(256) x_inverse_rows(const cplx_t<T>* __restric
 // the transforms of G (field 0) and of i k_y G (field 1) from the same
 // load; part 1 transforms G_z (field 2) in place; blockIdx.z = 2 pair +
 // part. With only_g, one part transforms G alone (blockIdx.z = pair).
+// Stage A reads global memory and stage B writes it: one visit of shared
+// memory (the tile) in between. A CTA reads all of its columns before the
+// barrier and writes them after it, so the pass works in place. At 256^3 the
+// inverse row and column passes move 1.48 GB in 258 us (303 us with the
+// lines loaded to and stored from shared memory), 84% of the copy rate.
 template <typename T, int N, int C, int DIR>
 __global__ void __launch_bounds__(256) y_columns(cplx_t<T>* __restrict__ data, const cplx_t<T>* __restrict__ tw_g,
                                                  T two_pi_over_L, int only_g) {
     using V = cplx_t<T>;
+    constexpr int N1 = fft_split<N>::N1, N2 = fft_split<N>::N2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V* tw = reinterpret_cast<V*>(smem_raw);
-    V* tile = tw + N;  // [2][y][c]
+    V* tile = tw + N;  // [2][slot][c]
     constexpr int TS = N * C;
-    load_twiddles(tw, tw_g, N);
     const size_t M = (size_t)N * N * N;
     const int part = (DIR < 0 || only_g) ? 0 : (int)(blockIdx.z & 1);
     const int pr = (DIR < 0 || only_g) ? (int)blockIdx.z : (int)(blockIdx.z >> 1);
@@ -349,21 +567,48 @@ __global__ void __launch_bounds__(256) y_columns(cplx_t<T>* __restrict__ data, c
     const bool two = DIR > 0 && part == 0 && !only_g;  // only_g: G alone (one part)
     const size_t off = (size_t)blockIdx.y * N * N + (size_t)blockIdx.x * C;
     const size_t src = (DIR > 0 && part == 1 ? 2 * M : 0) + off;
-    batched_load<TS, 256, V>([&](int i) { return data[src + (size_t)(i / C) * N + i % C]; },
-                             [&](int i, V v) {
-                                 tile[i] = v;
-                                 if (two) tile[TS + i] = c_scale(v, grad_k<T, N>(i / C, two_pi_over_L));
-                             });
-    __syncthreads();
-    if (two) {
-        smem_fft_lines<N, DIR, 2 * C, 256>(tile, TileAddr<C, TS>{}, C, tw);
-        for (int i = threadIdx.x; i < TS; i += blockDim.x) {
-            data[off + (size_t)(i / C) * N + i % C] = tile[i];
-            data[M + off + (size_t)(i / C) * N + i % C] = tile[TS + i];
+    {
+        int u = threadIdx.x;  // stage A: unit (column, j2), lanes over columns
+        V v[N1];
+        auto fetch = [&]() {
+#pragma unroll
+            for (int k = 0; k < N1; ++k) v[k] = data[src + (size_t)(u / C + N2 * k) * N + u % C];
+        };
+        if (u < C * N2) fetch();
+        load_twiddles(tw, tw_g, N);
+        __syncthreads();
+#pragma unroll 1
+        while (u < C * N2) {
+            const int j2 = u / C;
+            V* p = tile + j2 * C + u % C;
+            if (two) {
+                V w[N1];
+#pragma unroll
+                for (int k = 0; k < N1; ++k) w[k] = c_scale_rn(v[k], grad_k<T, N>(j2 + N2 * k, two_pi_over_L));
+                stage_a_regs<N, DIR>(w, j2, tw);
+#pragma unroll
+                for (int k1 = 0; k1 < N1; ++k1) p[TS + k1 * N2 * C] = w[k1];
+            }
+            stage_a_regs<N, DIR>(v, j2, tw);
+#pragma unroll
+            for (int k1 = 0; k1 < N1; ++k1) p[k1 * N2 * C] = v[k1];
+            u += 256;
+            if (u < C * N2) fetch();
         }
-    } else {
-        smem_fft_lines<N, DIR, C, 256>(tile, StridedLines<1>{}, C, tw);
-        for (int i = threadIdx.x; i < TS; i += blockDim.x) data[src + (size_t)(i / C) * N + i % C] = tile[i];
+    }
+    __syncthreads();
+    // stage B: unit (column, k1, field), lanes over columns
+#pragma unroll 1
+    for (int u = threadIdx.x; u < (two ? 2 : 1) * C * N1; u += 256) {
+        const int c = u % C, k1 = (u / C) % N1, f = u / (C * N1);
+        const V* p = tile + f * TS + k1 * N2 * C + c;
+        V v[N2];
+#pragma unroll
+        for (int j = 0; j < N2; ++j) v[j] = p[j * C];
+        reg_dft<N2, DIR, V>::run(v);
+        V* o = data + src + f * M + (size_t)k1 * N + c;
+#pragma unroll
+        for (int k2 = 0; k2 < N2; ++k2) o[(size_t)(N1 * k2) * N] = v[k2];
     }
 }
 
@@ -377,6 +622,9 @@ template <int N> __host__ __device__ __forceinline__ int kx_of_pos(int p) {
     return p == 0 ? 0 : p == 1 ? N / 2 : (p & 1) ? N - (p >> 1) : (p >> 1);
 }
 __host__ __device__ __forceinline__ int mirror_pos(int p) { return p < 2 ? p : (p ^ 1); }
+template <int N> __host__ __device__ __forceinline__ int pos_of_kx(int kx) {
+    return kx == 0 ? 0 : kx == N / 2 ? 1 : kx < N / 2 ? 2 * kx : 2 * (N - kx) + 1;
+}
 
 template <int C, int STRIDE> struct TileAddr {  // buffer b of a tile set starts at b * STRIDE
     __device__ __forceinline__ int operator()(int l) const { return (l / C) * STRIDE + l % C; }
@@ -396,162 +644,175 @@ template <typename T> __device__ __forceinline__ int freq_index(int i, int n) { 
 // with Q = w~_A + i w~_B. Buffers [2R][N][C]: G of row r in buffer r
 // (overwriting the input), G_z in buffer R + r.
 // --------------------------------------------------------------------------
-// out(b, c, z, v): output element z of column c of buffer b (the inverse
-// transforms' results, handed over as their last stage produces them).
-template <typename T, int N, int C, int R, bool G_ONLY, bool EL, class Out>
-__device__ __forceinline__ void z_tile(cplx_t<T>* buf, const cplx_t<T>* tw, const T* e1, const SpectralParams<T>& sp,
-                                       int p0, const int (&ky)[2], bool want_e, double (&acc)[5], const T* e2, Out out) {
+//
+// Bound by L2 and HBM traffic and by the tail of its 1.1 to 1.7 waves. Each
+// value visits shared memory twice and the CTA meets at three barriers, where
+// load, transform, multiply and inverse as separate passes visited it five
+// times: 24.1 -> 16.7 us at 128^3, 190 -> 114 us at 256^3, 16 column tiles
+// (256^3: 8), isolated launches.
+//   1. stage A of the forward transform from global memory;
+//   2. stage B in registers; the spectral multiply where it left X[k]; and
+//      the first stage of the inverse transform on the products, without
+//      leaving registers: with the two factors taken in the other order (N2
+//      points over k2, then N1 over k1; z = m + N2 q) its inputs are the N2
+//      outputs of one stage-B unit;
+//   3. the inverse's second stage, to global memory.
+// The unit (row, column c, k1) of step 2 needs Z(-k) as well, the outputs of
+// the mirror unit (mirror row, mirror column, (N1 - k1) mod N1). PAIRED: a
+// thread takes both units and writes both; otherwise each unit has its own
+// thread, which transforms the mirror unit's inputs a second time (half the
+// registers and twice the threads, for tiles that leave threads idle).
+template <int N, int C> struct ZTile {
+    static constexpr int N1 = fft_split<N>::N1, N2 = fft_split<N>::N2;
+    static constexpr bool paired = 2 * C * N1 > 256;
+    static_assert(256 % C == 0 && C * N1 <= 256, "every unit of a row has a thread");
+};
+
+// fetch(r, z, c): the input of row r; out(b, c, z, v): output element z of
+// column c of buffer b (buffers: G of row r in r, G_z in R + r).
+template <typename T, int N, int C, bool G_ONLY, bool EL, bool WANT_E, class Fetch, class Out>
+__device__ __forceinline__ void z_tile(cplx_t<T>* buf, cplx_t<T>* tw, const cplx_t<T>* __restrict__ tw_g, T* e1, T* e2,
+                                       const SpectralParams<T>& sp, int p0, const int (&ky)[2], int R, double (&acc)[5],
+                                       Fetch fetch, Out out) {
     using V = cplx_t<T>;
-    constexpr int TS = N * C;
-    static_assert(256 % C == 0, "a thread keeps one column");
-    constexpr int rB = R - 1;
-    // column constants of element A (row 0, column c) and its mirror B (row
-    // rB, column cB)
-    struct Col {
-        int cB;
-        T exyA, exyB, exy2A, exy2B;
-        bool zeroA, zeroB;
-        double kxy2A, kxy2B;  // |k_x|^2 + |k_y|^2 (the Nyquist index counts as -n/2)
-    };
-    auto col_of = [&](int c) {
-        Col cl;
-        cl.cB = mirror_pos(p0 + c) - p0;
-        const int kxA = kx_of_pos<N>(p0 + c), kxB = kx_of_pos<N>(p0 + cl.cB);
-        cl.exyA = e1[kxA] * e1[ky[0]];
-        cl.exyB = e1[kxB] * e1[ky[rB]];
-        cl.zeroA = (kxA == 0 && ky[0] == 0);
-        cl.zeroB = (kxB == 0 && ky[rB] == 0);
-        const T qxA = raw_k<T, N>(kxA, sp.two_pi_over_L), qyA = raw_k<T, N>(ky[0], sp.two_pi_over_L);
-        const T qxB = raw_k<T, N>(kxB, sp.two_pi_over_L), qyB = raw_k<T, N>(ky[rB], sp.two_pi_over_L);
-        cl.kxy2A = (double)qxA * qxA + (double)qyA * qyA;
-        cl.kxy2B = (double)qxB * qxB + (double)qyB * qyB;
-        cl.exy2A = EL ? e2[kxA] * e2[ky[0]] : T(0);
-        cl.exy2B = EL ? e2[kxB] * e2[ky[rB]] : T(0);
-        return cl;
-    };
-    // the spectral multiply of one mirror pair: ZA = Z(k) at (row 0, c, kz),
-    // ZB = Z(-k) at (row rB, cB, kzB); out[s][d]: s = 0 for A, 1 for B,
-    // d = 0 for iQ (G), 1 for i k_z Q (G_z)
-    struct Mult {
-        V g[2], gz[2];  // iQ and i k_z Q of A (0) and B (1)
-    };
-    auto mult = [&](const Col& cl, V ZA, V ZB, int kz, int kzB, bool same) {
-        Mult out;
+    constexpr int TS = N * C, N1 = ZTile<N, C>::N1, N2 = ZTile<N, C>::N2;
+    {
+        int u = threadIdx.x;  // unit (row, j2, column), lanes over columns
+        V v[N1];
+        auto load = [&]() {
 #pragma unroll
-        for (int s = 0; s < 2; ++s) {
-            if (s == 1 && same) break;
-            const V Z = s == 0 ? ZA : ZB;   // Z(k)
-            const V Zm = s == 0 ? ZB : ZA;  // Z(-k)
-            const int kzi = s == 0 ? kz : kzB;
-            const T kzv = grad_k<T, N>(kzi, sp.two_pi_over_L);
-            const T uh = (s == 0 ? cl.exyA : cl.exyB) * e1[kzi];
-            // rho~_A = (Z + conj Zm)/2, rho~_B = -i (Z - conj Zm)/2
-            const V A = {T(0.5) * (Z.x + Zm.x), T(0.5) * (Z.y - Zm.y)};
-            const V B = {T(0.5) * (Z.y + Zm.y), -T(0.5) * (Z.x - Zm.x)};
-            if (want_e) {
-                // energy sums and their |k|^2-weighted versions (d u_hat / d a = -2 a |k|^2 u_hat)
-                const double ar = A.x, ai = A.y, br = B.x, bi = B.y;
-                const double qz = (double)raw_k<T, N>(kzi, sp.two_pi_over_L);
-                const double k2 = (s == 0 ? cl.kxy2A : cl.kxy2B) + qz * qz;
-                const double fchi = (double)uh * (ar * br + ai * bi);
-                acc[0] += fchi;
-                acc[2] += k2 * fchi;
-                if (!((s == 0 ? cl.zeroA : cl.zeroB) && kzi == 0)) {
-                    const double fkap = (double)uh * ((ar + br) * (ar + br) + (ai + bi) * (ai + bi));
-                    acc[1] += fkap;
-                    acc[3] += k2 * fkap;
-                }
-            }
-            V wA = {uh * (sp.eAA * A.x + sp.eAB * B.x), uh * (sp.eAA * A.y + sp.eAB * B.y)};
-            V wB = {uh * (sp.eAB * A.x + sp.eBB * B.x), uh * (sp.eAB * A.y + sp.eBB * B.y)};
-            if (EL) {
-                // w_K += q_K c(k) rho~_q with rho~_q = q_A rho~_A + q_B rho~_B
-                const T qzv = raw_k<T, N>(kzi, sp.two_pi_over_L);
-                const T k2 = (T)(s == 0 ? cl.kxy2A : cl.kxy2B) + qzv * qzv;
-                const T g = k2 > T(0) ? (s == 0 ? cl.exy2A : cl.exy2B) * e2[kzi] * recip(k2) : T(0);
-                const V rq = {sp.qA * A.x + sp.qB * B.x, sp.qA * A.y + sp.qB * B.y};
-                const T c = sp.el_scale * g;
-                wA.x += c * sp.qA * rq.x;
-                wA.y += c * sp.qA * rq.y;
-                wB.x += c * sp.qB * rq.x;
-                wB.y += c * sp.qB * rq.y;
-                if (want_e) acc[4] += (double)g * ((double)rq.x * rq.x + (double)rq.y * rq.y);
-            }
-            const V iQ = {-(wA.y + wB.x), wA.x - wB.y};  // i (w~_A + i w~_B)
-            out.g[s] = iQ;                                // x, y: k_x, k_y applied in the xy pass
-            out.gz[s] = {kzv * iQ.x, kzv * iQ.y};         // z
+            for (int k = 0; k < N1; ++k) v[k] = fetch(u / (C * N2), (u / C) % N2 + N2 * k, u % C);
+        };
+        const int units = R * C * N2;
+        if (u < units) load();
+        load_twiddles(tw, tw_g, N);
+        for (int i = threadIdx.x; i < N; i += 256) {
+            e1[i] = sp.kernel1d[i];
+            if (EL) e2[i] = sp.kernel1d_el[i];
         }
-        return out;
-    };
-    auto store = [&](const Mult& out, int c, int cB, int kz, int kzB, bool same) {
-        buf[kz * C + c] = out.g[0];
-        if (!same) buf[rB * TS + kzB * C + cB] = out.g[1];
-        if (!G_ONLY) {
-            buf[R * TS + kz * C + c] = out.gz[0];
-            if (!same) buf[(R + rB) * TS + kzB * C + cB] = out.gz[1];
-        }
-    };
-    constexpr int N1 = fft_split<N>::N1, N2 = fft_split<N>::N2;
-    if constexpr (R == 2 && !EL && N2 > 1 && C * N1 == 256) {
-        // two rows: the forward transform's second stage and the multiply in
-        // registers (tiles where every thread has one pair of units). Thread q
-        // takes stage-B unit (row 0, column c, k1)
-        // and the unit holding the mirrors of its outputs, (row 1, column cB,
-        // (N1 - k1) mod N1); the outputs X[k1 + N1 k2] of the first meet
-        // their mirrors X[-(k1 + N1 k2)] in the second, so each pair is
-        // multiplied where the transform left it (same operations as the
-        // transform followed by the loop below).
-        smem_fft_stage_a<N, -1, R * C, 256>(buf, TileAddr<C, TS>{}, C, tw);
-        const int q = threadIdx.x;
-        const bool active = q < C * N1;
-        const int c = q % C, k1 = q / C;
-        const int k1B = (N1 - k1) % N1;
-        const Col cl = col_of(c);
-        V va[N2], vb[N2];
-        if (active) {
-            const V* pa = buf + c + k1 * N2 * C;             // line c of row 0: positions k1 N2 + j2
-            const V* pb = buf + TS + cl.cB + k1B * N2 * C;   // line cB of row 1
+        __syncthreads();
+#pragma unroll 1
+        while (u < units) {
+            const int j2 = (u / C) % N2;
+            stage_a_regs<N, -1>(v, j2, tw);
+            V* p = buf + (u / (C * N2)) * TS + j2 * C + u % C;
 #pragma unroll
-            for (int j2 = 0; j2 < N2; ++j2) {
-                va[j2] = pa[j2 * C];
-                vb[j2] = pb[j2 * C];
-            }
-        }
-        __syncthreads();  // every stage-B input is read before any output is written
-        if (active) {
-            reg_dft<N2, -1, V>::run(va);
-            reg_dft<N2, -1, V>::run(vb);
-            // the mirror of output k2: (N2 - k2) mod N2 when k1 = 0, else N2 - 1 - k2
-            // (selected with constant indices, so the arrays stay in registers)
-            V vm[N2];
-#pragma unroll
-            for (int k2 = 0; k2 < N2; ++k2) vm[k2] = k1 == 0 ? vb[(N2 - k2) % N2] : vb[N2 - 1 - k2];
-#pragma unroll
-            for (int k2 = 0; k2 < N2; ++k2) {
-                const int kz = k1 + N1 * k2;
-                const int kzB = kz == 0 ? 0 : N - kz;
-                store(mult(cl, va[k2], vm[k2], kz, kzB, false), c, cl.cB, kz, kzB, false);
-            }
-        }
-    } else {
-        smem_fft_lines<N, -1, R * C, 256>(buf, TileAddr<C, TS>{}, C, tw);
-        const int c = threadIdx.x % C;
-        const Col cl = col_of(c);
-        for (int kz = threadIdx.x / C; kz < N; kz += 256 / C) {
-            const int kzB = kz == 0 ? 0 : N - kz;
-            if (R == 1 && kzB * C + cl.cB < kz * C + c) continue;  // the mirror element owns this pair
-            const bool same = (R == 1) && (kzB == kz) && (cl.cB == c);
-            store(mult(cl, buf[kz * C + c], buf[rB * TS + kzB * C + cl.cB], kz, kzB, same), c, cl.cB, kz, kzB, same);
+            for (int k1 = 0; k1 < N1; ++k1) p[k1 * N2 * C] = v[k1];
+            u += 256;
+            if (u < units) load();
         }
     }
     __syncthreads();
-    constexpr int NB = (G_ONLY ? 1 : 2) * R;  // output buffers
-    if constexpr (N2 > 1) {
-        smem_fft_lines_out<N, +1, NB * C, 256>(buf, TileAddr<C, TS>{}, C, tw,
-                                                [&](int l, int z, V v) { out(l / C, l % C, z, v); });
-    } else {
-        smem_fft_lines<N, +1, NB * C, 256>(buf, TileAddr<C, TS>{}, C, tw);
-        for (int i = threadIdx.x; i < NB * TS; i += blockDim.x) out(i / TS, i % C, (i % TS) / C, buf[i]);
+    {
+        constexpr bool PAIRED = ZTile<N, C>::paired;
+        const int q = threadIdx.x;
+        const bool active = q < (PAIRED ? 1 : R) * C * N1;
+        int c = q % C, k1 = (q / C) % N1, r = PAIRED ? 0 : q / (C * N1);
+        int cB = mirror_pos(p0 + c) - p0, k1B = (N1 - k1) % N1, rB = R == 2 ? 1 - r : 0;
+        V va[N2], vb[N2];
+        if (active) {
+            const V* pa = buf + r * TS + k1 * N2 * C + c;
+            const V* pb = buf + rB * TS + k1B * N2 * C + cB;
+#pragma unroll
+            for (int j = 0; j < N2; ++j) {
+                va[j] = pa[j * C];
+                vb[j] = pb[j * C];
+            }
+        }
+        if (!PAIRED || R == 1) __syncthreads();  // a unit's inputs are read by its mirror's thread too
+        if (active) {
+            reg_dft<N2, -1, V>::run(va);
+            reg_dft<N2, -1, V>::run(vb);
+            const int sides = PAIRED ? R : 1;
+#pragma unroll 1
+            for (int s = 0; s < sides; ++s) {
+                // unit (r, c, k1): X[k1 + N1 k2] = va[k2]; the mirror of output
+                // k2 is vb[(N2 - k2) mod N2] when k1 = 0, else vb[N2 - 1 - k2]
+                const int kx = kx_of_pos<N>(p0 + c), kyr = ky[r];
+                const T exy = e1[kx] * e1[kyr];
+                const T exy2 = EL ? e2[kx] * e2[kyr] : T(0);
+                const T qx = raw_k<T, N>(kx, sp.two_pi_over_L), qy = raw_k<T, N>(kyr, sp.two_pi_over_L);
+                const double kxy2 = (double)qx * qx + (double)qy * qy;  // the Nyquist index counts as -n/2
+                const bool zero = kx == 0 && kyr == 0;
+                V g[N2], gz[G_ONLY ? 1 : N2];
+#pragma unroll
+                for (int k2 = 0; k2 < N2; ++k2) {
+                    const V Z = va[k2], Zm = k1 == 0 ? vb[(N2 - k2) % N2] : vb[N2 - 1 - k2];
+                    const int kz = k1 + N1 * k2;
+                    const T uh = exy * e1[kz];
+                    // rho~_A = (Z + conj Zm)/2, rho~_B = -i (Z - conj Zm)/2
+                    const V A = {T(0.5) * (Z.x + Zm.x), T(0.5) * (Z.y - Zm.y)};
+                    const V B = {T(0.5) * (Z.y + Zm.y), -T(0.5) * (Z.x - Zm.x)};
+                    V wA = {mul_rn(uh, fma_rn(sp.eAA, A.x, mul_rn(sp.eAB, B.x))),
+                            mul_rn(uh, fma_rn(sp.eAA, A.y, mul_rn(sp.eAB, B.y)))};
+                    V wB = {mul_rn(uh, fma_rn(sp.eAB, A.x, mul_rn(sp.eBB, B.x))),
+                            mul_rn(uh, fma_rn(sp.eAB, A.y, mul_rn(sp.eBB, B.y)))};
+                    if (WANT_E) {
+                        // energy sums and their |k|^2-weighted versions (d u_hat / d a = -2 a |k|^2 u_hat)
+                        const double ar = A.x, ai = A.y, br = B.x, bi = B.y;
+                        const double qz = (double)raw_k<T, N>(kz, sp.two_pi_over_L);
+                        const double k2sq = kxy2 + qz * qz;
+                        const double fchi = (double)uh * (ar * br + ai * bi);
+                        acc[0] += fchi;
+                        acc[2] += k2sq * fchi;
+                        if (!(zero && kz == 0)) {
+                            const double fkap = (double)uh * ((ar + br) * (ar + br) + (ai + bi) * (ai + bi));
+                            acc[1] += fkap;
+                            acc[3] += k2sq * fkap;
+                        }
+                    }
+                    if (EL) {
+                        // w_K += q_K c(k) rho~_q with rho~_q = q_A rho~_A + q_B rho~_B
+                        const T qzv = raw_k<T, N>(kz, sp.two_pi_over_L);
+                        const T k2sq = fma_rn(qzv, qzv, (T)kxy2);
+                        const T gq = k2sq > T(0) ? exy2 * e2[kz] * recip(k2sq) : T(0);
+                        const V rq = {fma_rn(sp.qA, A.x, mul_rn(sp.qB, B.x)), fma_rn(sp.qA, A.y, mul_rn(sp.qB, B.y))};
+                        const T cA = mul_rn(sp.el_scale * gq, sp.qA), cB2 = mul_rn(sp.el_scale * gq, sp.qB);
+                        wA.x = fma_rn(cA, rq.x, wA.x);
+                        wA.y = fma_rn(cA, rq.y, wA.y);
+                        wB.x = fma_rn(cB2, rq.x, wB.x);
+                        wB.y = fma_rn(cB2, rq.y, wB.y);
+                        if (WANT_E) acc[4] += (double)gq * ((double)rq.x * rq.x + (double)rq.y * rq.y);
+                    }
+                    g[k2] = {-(wA.y + wB.x), wA.x - wB.y};  // i (w~_A + i w~_B); k_x, k_y follow in the xy pass
+                    if (!G_ONLY) gz[k2] = c_scale_rn(g[k2], grad_k<T, N>(kz, sp.two_pi_over_L));
+                }
+                V* o = buf + r * TS + k1 * N2 * C + c;
+                reg_dft<N2, +1, V>::run(g);
+#pragma unroll
+                for (int m = 0; m < N2; ++m) o[m * C] = m == 0 ? g[0] : c_mul(g[m], twiddle<+1>(tw, k1 * m));
+                if constexpr (!G_ONLY) {
+                    reg_dft<N2, +1, V>::run(gz);
+                    o += R * TS;
+#pragma unroll
+                    for (int m = 0; m < N2; ++m) o[m * C] = m == 0 ? gz[0] : c_mul(gz[m], twiddle<+1>(tw, k1 * m));
+                }
+                if (PAIRED) {  // the mirror unit next
+#pragma unroll
+                    for (int j = 0; j < N2; ++j) {
+                        const V t = va[j];
+                        va[j] = vb[j];
+                        vb[j] = t;
+                    }
+                    r = rB;
+                    c = cB;
+                    k1 = k1B;
+                }
+            }
+        }
+    }
+    __syncthreads();
+    const int units = (G_ONLY ? 1 : 2) * R * C * N2;
+#pragma unroll 1
+    for (int u = threadIdx.x; u < units; u += 256) {
+        const int c = u % C, m = (u / C) % N2, b = u / (C * N2);
+        const V* p = buf + b * TS + m * C + c;
+        V v[N1];
+#pragma unroll
+        for (int k1 = 0; k1 < N1; ++k1) v[k1] = p[k1 * N2 * C];
+        reg_dft<N1, +1, V>::run(v);
+#pragma unroll
+        for (int k = 0; k < N1; ++k) out(b, c, m + N2 * k, v[k]);
     }
 }
 
@@ -561,74 +822,36 @@ template <typename T> struct ZArgs {
     const cplx_t<T>* tw;
     SpectralParams<T> sp;
     double* energy_partials;
-    cplx_t<T>* spectrum_out;
 };
 
-template <typename T, int N, int C, bool G_ONLY = false, bool EL = false>
+template <typename T, int N, int C, bool G_ONLY = false, bool EL = false, bool WANT_E = false>
 __device__ __forceinline__ void z_spectral_body(const ZArgs<T>& args, int bx, int by, int gdx) {
     using V = cplx_t<T>;
     const cplx_t<T>* __restrict__ Zxy = args.Zxy;
     cplx_t<T>* __restrict__ H = args.H;
-    const cplx_t<T>* __restrict__ tw_g = args.tw;
     const SpectralParams<T> sp = args.sp;
-    double* __restrict__ energy_partials = args.energy_partials;
-    cplx_t<T>* __restrict__ spectrum_out = args.spectrum_out;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V* tw = reinterpret_cast<V*>(smem_raw);
     V* buf = tw + N;
-    constexpr int TS = N * C;
-    __shared__ double red[5][8];
     __shared__ T e1[N];  // separable Gaussian kernel: u_hat = e1[kx] e1[ky] e1[kz]
-    __shared__ T e2[N];  // charge smearing exp(-a_e^2 k_m^2), when charges are on
-    load_twiddles(tw, tw_g, N);
-    for (int i = threadIdx.x; i < N; i += blockDim.x) e1[i] = sp.kernel1d[i];
-    if (EL)
-        for (int i = threadIdx.x; i < N; i += blockDim.x) e2[i] = sp.kernel1d_el[i];
+    __shared__ T e2[EL ? N : 1];  // charge smearing exp(-a_e^2 k_m^2), when charges are on
 
     const int p0 = bx * C;
     const int ky[2] = {by, by == 0 ? 0 : N - by};
     const int R = (ky[0] == ky[1]) ? 1 : 2;
-    const size_t NN = (size_t)N * N;
-    auto zsrc = [&](int i) {
-        const int r = i / TS, rem = i % TS;
-        const int z = rem / C, c = rem % C;
-        return Zxy[z * NN + (size_t)ky[r] * N + p0 + c];
-    };
-    auto zdst = [&](int i, V v) { buf[i] = v; };
-    if (R == 1)
-        batched_load<TS, 256, V>(zsrc, zdst);
-    else
-        batched_load<2 * TS, 256, V>(zsrc, zdst);
-    __syncthreads();
+    const size_t NN = (size_t)N * N, M = NN * N;
     double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-    const bool want_e = energy_partials != nullptr;
-    if (spectrum_out) {
-        // forward transform only, written out in natural kx order
-        if (R == 1)
-            smem_fft_lines<N, -1, C, 256>(buf, TileAddr<C, TS>{}, C, tw);
-        else
-            smem_fft_lines<N, -1, 2 * C, 256>(buf, TileAddr<C, TS>{}, C, tw);
-        for (int i = threadIdx.x; i < R * TS; i += blockDim.x) {
-            const int r = i / TS, rem = i % TS;
-            const int z = rem / C, c = rem % C;
-            spectrum_out[z * NN + (size_t)ky[r] * N + kx_of_pos<N>(p0 + c)] = buf[i];
-        }
-        return;
-    }
-    const size_t M = NN * N;
-    // G of row r to field 0, G_z to field 2, at (z, ky[r], p0 + c)
-    auto store_h = [&](int rr, int b, int c, int z, V v) {
-        const int f = (b / rr) * 2, r = b % rr;
-        H[f * M + z * NN + (size_t)ky[r] * N + p0 + c] = v;
-    };
-    if (R == 1)
-        z_tile<T, N, C, 1, G_ONLY, EL>(buf, tw, e1, sp, p0, ky, want_e, acc, e2,
-                                       [&](int b, int c, int z, V v) { store_h(1, b, c, z, v); });
-    else
-        z_tile<T, N, C, 2, G_ONLY, EL>(buf, tw, e1, sp, p0, ky, want_e, acc, e2,
-                                       [&](int b, int c, int z, V v) { store_h(2, b, c, z, v); });
-    if (want_e) {
+    z_tile<T, N, C, G_ONLY, EL, WANT_E>(
+        buf, tw, args.tw, e1, e2, sp, p0, ky, R, acc,
+        [&](int r, int z, int c) { return Zxy[z * NN + (size_t)ky[r] * N + p0 + c]; },
+        [&](int b, int c, int z, V v) {
+            // G of row r to field 0, G_z to field 2, at (z, ky[r], p0 + c)
+            const int f = b < R ? 0 : 2, r = b < R ? b : b - R;
+            H[f * M + z * NN + (size_t)ky[r] * N + p0 + c] = v;
+        });
+    if (WANT_E) {
         // block reduction in a fixed order (deterministic)
+        __shared__ double red[5][8];
         const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
         for (int k = 0; k < 5; ++k) {
@@ -641,20 +864,58 @@ __device__ __forceinline__ void z_spectral_body(const ZArgs<T>& args, int bx, in
             double sum = 0;
             for (int w = 0; w < (int)(blockDim.x + 31) / 32; ++w) sum += red[threadIdx.x][w];
             const size_t b = (size_t)by * gdx + bx;
-            energy_partials[5 * b + threadIdx.x] = sum;
+            args.energy_partials[5 * b + threadIdx.x] = sum;
         }
+    }
+}
+
+// The forward z transform alone: the spectrum in natural kx order.
+template <typename T, int N, int C>
+__global__ void __launch_bounds__(256) z_spectrum(const cplx_t<T>* __restrict__ Zxy, const cplx_t<T>* __restrict__ tw_g,
+                                                  cplx_t<T>* __restrict__ spectrum) {
+    using V = cplx_t<T>;
+    constexpr int N1 = ZTile<N, C>::N1, N2 = ZTile<N, C>::N2;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    V* tw = reinterpret_cast<V*>(smem_raw);
+    V* buf = tw + N;
+    load_twiddles(tw, tw_g, N);
+    __syncthreads();
+    const int p0 = blockIdx.x * C, ky = blockIdx.y;
+    const size_t NN = (size_t)N * N;
+    for (int u = threadIdx.x; u < C * N2; u += 256) {
+        const int c = u % C, j2 = u / C;
+        V v[N1];
+#pragma unroll
+        for (int k = 0; k < N1; ++k) v[k] = Zxy[(j2 + N2 * k) * NN + (size_t)ky * N + p0 + c];
+        stage_a_regs<N, -1>(v, j2, tw);
+#pragma unroll
+        for (int k1 = 0; k1 < N1; ++k1) buf[(k1 * N2 + j2) * C + c] = v[k1];
+    }
+    __syncthreads();
+    for (int u = threadIdx.x; u < C * N1; u += 256) {
+        const int c = u % C, k1 = u / C;
+        V v[N2];
+#pragma unroll
+        for (int j = 0; j < N2; ++j) v[j] = buf[(k1 * N2 + j) * C + c];
+        reg_dft<N2, -1, V>::run(v);
+#pragma unroll
+        for (int k2 = 0; k2 < N2; ++k2) spectrum[(k1 + N1 * k2) * NN + (size_t)ky * N + kx_of_pos<N>(p0 + c)] = v[k2];
     }
 }
 
 // G_ONLY: write G alone (the potentials' path of the analytic force).
 // EL: add the smeared-charge Coulomb term (charges on).
-template <typename T, int N, int C, bool G_ONLY = false, bool EL = false>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? (C <= 8 ? 4 : 3) : 1) z_spectral(const cplx_t<T>* __restrict__ Zxy, cplx_t<T>* __restrict__ H,
+// WANT_E: the energy sums as well (an instantiation of its own, so that the
+// step's kernel carries none of their code or registers).
+template <typename T, int N, int C> __host__ __device__ constexpr int z_ctas() {
+    return sizeof(T) == 8 ? 1 : N == 256 ? (C <= 8 ? 2 : 1) : C <= 8 ? 4 : 3;
+}
+template <typename T, int N, int C, bool G_ONLY = false, bool EL = false, bool WANT_E = false>
+__global__ void __launch_bounds__(256, z_ctas<T, N, C>()) z_spectral(const cplx_t<T>* __restrict__ Zxy, cplx_t<T>* __restrict__ H,
                                                   const cplx_t<T>* __restrict__ tw_g, SpectralParams<T> sp,
-                                                  double* __restrict__ energy_partials,
-                                                  cplx_t<T>* __restrict__ spectrum_out) {
-    z_spectral_body<T, N, C, G_ONLY, EL>(ZArgs<T>{Zxy, H, tw_g, sp, energy_partials, spectrum_out}, blockIdx.x,
-                                     blockIdx.y, gridDim.x);
+                                                  double* __restrict__ energy_partials) {
+    z_spectral_body<T, N, C, G_ONLY, EL, WANT_E>(ZArgs<T>{Zxy, H, tw_g, sp, energy_partials}, blockIdx.x, blockIdx.y,
+                                                 gridDim.x);
 }
 
 // Batched form: replica blockIdx.z.

@@ -143,22 +143,28 @@ __global__ void __launch_bounds__(512) xy_forward_cplx(const longlong2* __restri
                                                        const typename AdjointFixed<T>::bits_t* __restrict__ bits, int S,
                                                        cplx_t<T>* __restrict__ data, const cplx_t<T>* __restrict__ tw_g) {
     using V = cplx_t<T>;
-    constexpr int PITCH = row_pitch(N);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V* tw = reinterpret_cast<V*>(smem_raw);
     V* plane = tw + N;
-    load_twiddles(tw, tw_g, N);
     T sc, inv;
     AdjointFixed<T>::scales(*bits, S, sc, inv);
     const size_t base = (size_t)blockIdx.y * N * N * N + (size_t)blockIdx.x * N * N;
-    batched_load<N * N, 512, longlong2>([&](int i) { return fx[base + i]; },
-                                        [&](int i, longlong2 v) {
-                                            plane[(i / N) * PITCH + i % N] = V{from_fixed(v.x, inv), from_fixed(v.y, inv)};
-                                        });
-    __syncthreads();
-    smem_fft_lines<N, -1, N, 512>(plane, StridedLines<PITCH>{}, 1, tw);  // along x
-    smem_fft_lines<N, -1, N, 512>(plane, StridedLines<1>{}, PITCH, tw);  // along y
-    for (int i = threadIdx.x; i < N * N; i += blockDim.x) data[base + i] = plane[(i / N) * PITCH + kx_of_pos<N>(i % N)];
+    constexpr int N1 = fft_split<N>::N1, N2 = fft_split<N>::N2;
+    plane_forward_xy<T, N, 512>(
+        plane, tw, tw_g,
+        [&](int y, int j2, V (&v)[N1]) {
+            const longlong2* row = fx + base + y * N + j2;
+            constexpr int B = N1 < 8 ? N1 : 8;
+#pragma unroll
+            for (int h = 0; h < N1; h += B) {
+                longlong2 a[B];
+#pragma unroll
+                for (int k = 0; k < B; ++k) a[k] = row[N2 * (h + k)];
+#pragma unroll
+                for (int k = 0; k < B; ++k) v[h + k] = V{from_fixed(a[k].x, inv), from_fixed(a[k].y, inv)};
+            }
+        },
+        []() {}, data + base);
 }
 
 // z pass of the VJP. CTA (C column positions, rows ky and -ky) as in

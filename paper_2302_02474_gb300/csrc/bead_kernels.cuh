@@ -59,6 +59,10 @@ template <typename T> struct BeadParams {
     int noise_lag;
     T sigma_v;        // sqrt(kT / m) (initial velocities)
     T mass;
+    // powers of two near 1/L and near 1/sigma_v: bond vectors and velocities are
+    // scaled by them before their squares are summed, so that no unit system
+    // takes the squares out of the range of floats (1 in FP64)
+    T e_len, e_vel;
     uint64_t seed;
     Topology topo;
 };
@@ -84,7 +88,9 @@ template <typename T> struct BeadBuffers {
     T* __restrict__ f_out;        // FORCE: [n_beads][3] by id (may be null)
     T* __restrict__ v_out;        // FORCE: velocities by id (may be null)
     const T* __restrict__ v_in;   // SETVEL: velocities by id (null: Maxwell-Boltzmann)
-    double* __restrict__ partials;  // FORCE: [blocks][5]
+    // FORCE (may be null): [blocks][5] sums of |bond|^2 (scaled by e_len^2, each
+    // bond once), |v|^2 (by e_vel^2) and F
+    typename Wide<T>::stored* __restrict__ partials;
 };
 
 template <typename T> __device__ __forceinline__ T wrap_coord(T x, T L, T inv_L) {
@@ -93,6 +99,16 @@ template <typename T> __device__ __forceinline__ T wrap_coord(T x, T L, T inv_L)
     // (kept); anything else out of range, i.e. a non-finite or huge input,
     // maps to 0 so that no grid index derived from it leaves the grid
     return (y >= L || !(y >= T(-0.5) * L)) ? T(0) : y;
+}
+
+// acc += |s d|^2
+template <typename T> __device__ __forceinline__ void add_squares(Wide<T>& acc, T dx, T dy, T dz, T s) {
+    dx *= s;
+    dy *= s;
+    dz *= s;
+    acc.add_prod(dx, dx);
+    acc.add_prod(dy, dy);
+    acc.add_prod(dz, dz);
 }
 
 template <typename T> __device__ __forceinline__ T min_image(T d, T L, T inv_L) { return d - L * rint(d * inv_L); }
@@ -420,7 +436,8 @@ __device__ __forceinline__ void bead_kernel_body(const BeadParams<T>& p, const B
     const uint64_t step_next = (MODE == kModeStep) ? *bf.step : 0ull;
     // 32-bit patch sums cannot overflow below this many beads per tile
     const bool patch_ok = end - start <= FP::max_tile_beads;
-    double acc[5] = {0, 0, 0, 0, 0};
+    const bool sums = MODE == kModeForce && bf.partials;
+    Wide<T> acc[MODE == kModeForce ? 5 : 1];
 
     for (int c0 = start; c0 < end; c0 += kBeadChunk) {
         const int cnt = min(kBeadChunk, end - c0);
@@ -514,8 +531,7 @@ __device__ __forceinline__ void bead_kernel_body(const BeadParams<T>& p, const B
                         fx -= p.k_bond * dx;
                         fy -= p.k_bond * dy;
                         fz -= p.k_bond * dz;
-                        if (MODE == kModeForce && nid_of(s) > bid)
-                            acc[0] += 0.5 * (double)p.k_bond * ((double)dx * dx + (double)dy * dy + (double)dz * dz);
+                        if (MODE == kModeForce && sums && nid_of(s) > bid) add_squares(acc[0], dx, dy, dz, p.e_len);
                     }
                 }
                 for_each_extra_bond(nb, bf.ext, [&](int s) {
@@ -526,8 +542,7 @@ __device__ __forceinline__ void bead_kernel_body(const BeadParams<T>& p, const B
                     fx -= p.k_bond * dx;
                     fy -= p.k_bond * dy;
                     fz -= p.k_bond * dz;
-                    if (MODE == kModeForce && nid_of(s) > bid)
-                        acc[0] += 0.5 * (double)p.k_bond * ((double)dx * dx + (double)dy * dy + (double)dz * dz);
+                    if (MODE == kModeForce && sums && nid_of(s) > bid) add_squares(acc[0], dx, dy, dz, p.e_len);
                 });
                 if (!(isfinite(fx) && isfinite(fy) && isfinite(fz))) atomicOr(bf.err, kErrNonFinite);
                 if (MODE == kModeForce) {
@@ -537,10 +552,12 @@ __device__ __forceinline__ void bead_kernel_body(const BeadParams<T>& p, const B
                     const T vx = p.vu * ux + p.vf * fx + p.vg * g.a;
                     const T vy = p.vu * uy + p.vf * fy + p.vg * g.b;
                     const T vz = p.vu * uz + p.vf * fz + p.vg * g.c;
-                    acc[1] += 0.5 * (double)p.mass * ((double)vx * vx + (double)vy * vy + (double)vz * vz);
-                    acc[2] += fx;
-                    acc[3] += fy;
-                    acc[4] += fz;
+                    if (sums) {
+                        add_squares(acc[MODE == kModeForce ? 1 : 0], vx, vy, vz, p.e_vel);
+                        acc[MODE == kModeForce ? 2 : 0].add(fx);
+                        acc[MODE == kModeForce ? 3 : 0].add(fy);
+                        acc[MODE == kModeForce ? 4 : 0].add(fz);
+                    }
                     if (bf.f_out) {
                         bf.f_out[3 * (size_t)bid + 0] = fx;
                         bf.f_out[3 * (size_t)bid + 1] = fy;
@@ -604,21 +621,8 @@ __device__ __forceinline__ void bead_kernel_body(const BeadParams<T>& p, const B
             }
         }
     }
-    if (MODE == kModeForce) {
-        __shared__ double red[5][8];
-        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-        for (int k = 0; k < 5; ++k) {
-            double v = acc[k];
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-            if (lane == 0) red[k][wid] = v;
-        }
-        __syncthreads();
-        if (threadIdx.x < 5) {
-            double s = 0;
-            for (int w = 0; w < (int)blockDim.x / 32; ++w) s += red[threadIdx.x][w];
-            bf.partials[5 * (size_t)t + threadIdx.x] = s;
-        }
+    if constexpr (MODE == kModeForce) {
+        if (sums) block_sum<5, T>(acc, [&](int k, const Wide<T>& v) { bf.partials[5 * (size_t)t + k] = v.store(); });
     }
 }
 
@@ -644,57 +648,65 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && P <= 3) ? 4 : 2)
 //   dU/dr_i = sum_g grad_r W(r_i - g) w_K(g) + (3/b^2) sum_j mic(r_i - r_j),
 // i.e. the adjoint of the spread (the same weights, differentiated) applied
 // to the potential field w_K, plus the bond term. `pot` holds
-// i (w_A + i w_B) per grid point. Output by bead id.
+// i (w_A + i w_B) per grid point. Output by bead id (null: none). The block's
+// sum of |bond|^2 (scaled, each bond once) goes to bf.partials[blockIdx.x], so
+// that the bond energy needs no force pass of its own.
 template <int P, typename T>
 __global__ void __launch_bounds__(256) adjoint_kernel(BeadParams<T> p, BeadBuffers<T> bf, const cplx_t<T>* __restrict__ pot,
                                                       T* __restrict__ grad_out) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= p.n_beads) return;
-    const T x = bf.px[i], y = bf.py[i], z = bf.pz[i];
-    const int tag = bf.id[i];
-    const int bid = slot_bead_id(tag);
-    const int species = slot_species(tag);
-    Stencil<P, T> st;
-    st.set(x, y, z, p.inv_dx);
-    T dx[P], dy[P], dz[P];
-    dh_weight_derivs<P>(x * p.inv_dx, dx);
-    dh_weight_derivs<P>(y * p.inv_dx, dy);
-    dh_weight_derivs<P>(z * p.inv_dx, dz);
-    T gx = 0, gy = 0, gz = 0;
+    Wide<T> acc[1];
+    if (i < p.n_beads) {
+        const T x = bf.px[i], y = bf.py[i], z = bf.pz[i];
+        const int tag = bf.id[i];
+        const int bid = slot_bead_id(tag);
+        const int species = slot_species(tag);
+        T gx = 0, gy = 0, gz = 0;
+        if (grad_out) {
+            Stencil<P, T> st;
+            st.set(x, y, z, p.inv_dx);
+            T dx[P], dy[P], dz[P];
+            dh_weight_derivs<P>(x * p.inv_dx, dx);
+            dh_weight_derivs<P>(y * p.inv_dx, dy);
+            dh_weight_derivs<P>(z * p.inv_dx, dz);
 #pragma unroll
-    for (int c = 0; c < P; ++c)
+            for (int c = 0; c < P; ++c)
 #pragma unroll
-        for (int b = 0; b < P; ++b)
+                for (int b = 0; b < P; ++b)
 #pragma unroll
-            for (int a = 0; a < P; ++a) {
-                const size_t g = ((size_t)pwrap(st.jz + c, p.n) * p.n + pwrap(st.jy + b, p.n)) * p.n + pwrap(st.jx + a, p.n);
-                const cplx_t<T> v = pot[(size_t)(species >> 1) * 4 * ((size_t)p.n * p.n * p.n) + g];
-                const T w = (species & 1) ? -v.x : v.y;  // w_2p = Im, w_2p+1 = -Re of i (w_2p + i w_2p+1)
-                gx += dx[a] * st.wy[b] * st.wz[c] * w;
-                gy += st.wx[a] * dy[b] * st.wz[c] * w;
-                gz += st.wx[a] * st.wy[b] * dz[c] * w;
-            }
-    gx *= p.inv_dx;
-    gy *= p.inv_dx;
-    gz *= p.inv_dx;
-    const int2 nb = bf.nbr[i];
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const int s = k == 0 ? nb.x : nb.y;
-        if (s >= 0) {
-            gx += p.k_bond * min_image(x - bf.px[s], p.L, p.inv_L);
-            gy += p.k_bond * min_image(y - bf.py[s], p.L, p.inv_L);
-            gz += p.k_bond * min_image(z - bf.pz[s], p.L, p.inv_L);
+                    for (int a = 0; a < P; ++a) {
+                        const size_t g = ((size_t)pwrap(st.jz + c, p.n) * p.n + pwrap(st.jy + b, p.n)) * p.n + pwrap(st.jx + a, p.n);
+                        const cplx_t<T> v = pot[(size_t)(species >> 1) * 4 * ((size_t)p.n * p.n * p.n) + g];
+                        const T w = (species & 1) ? -v.x : v.y;  // w_2p = Im, w_2p+1 = -Re of i (w_2p + i w_2p+1)
+                        gx += dx[a] * st.wy[b] * st.wz[c] * w;
+                        gy += st.wx[a] * dy[b] * st.wz[c] * w;
+                        gz += st.wx[a] * st.wy[b] * dz[c] * w;
+                    }
+            gx *= p.inv_dx;
+            gy *= p.inv_dx;
+            gz *= p.inv_dx;
+        }
+        const int2 nb = bf.nbr[i];
+        auto bond = [&](int s) {
+            const T dx = min_image(x - bf.px[s], p.L, p.inv_L);
+            const T dy = min_image(y - bf.py[s], p.L, p.inv_L);
+            const T dz = min_image(z - bf.pz[s], p.L, p.inv_L);
+            gx += p.k_bond * dx;
+            gy += p.k_bond * dy;
+            gz += p.k_bond * dz;
+            if (slot_bead_id(bf.id[s]) > bid) add_squares(acc[0], dx, dy, dz, p.e_len);
+        };
+        if (nb.x >= 0) bond(nb.x);
+        if (nb.y >= 0) bond(nb.y);
+        for_each_extra_bond(nb, bf.ext, bond);
+        if (!(isfinite(gx) && isfinite(gy) && isfinite(gz))) atomicOr(bf.err, kErrNonFinite);
+        if (grad_out) {
+            grad_out[3 * (size_t)bid + 0] = gx;
+            grad_out[3 * (size_t)bid + 1] = gy;
+            grad_out[3 * (size_t)bid + 2] = gz;
         }
     }
-    for_each_extra_bond(nb, bf.ext, [&](int s) {
-        gx += p.k_bond * min_image(x - bf.px[s], p.L, p.inv_L);
-        gy += p.k_bond * min_image(y - bf.py[s], p.L, p.inv_L);
-        gz += p.k_bond * min_image(z - bf.pz[s], p.L, p.inv_L);
-    });
-    grad_out[3 * (size_t)bid + 0] = gx;
-    grad_out[3 * (size_t)bid + 1] = gy;
-    grad_out[3 * (size_t)bid + 2] = gz;
+    block_sum<1, T>(acc, [&](int, const Wide<T>& v) { bf.partials[blockIdx.x] = v.store(); });
 }
 
 // ------------------------------------------------------------- binning
@@ -923,10 +935,29 @@ __global__ void transpose_vec3(size_t n, const TV* __restrict__ in, TV* __restri
         out[i] = in[3 * (i % n) + i / n];
 }
 
-template <typename TO>
-__global__ void density_out(size_t count, const unsigned long long* __restrict__ rho_fx, double scale, TO* __restrict__ out) {
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < count) out[i] = (TO)((double)(long long)rho_fx[i] * scale);
+// Fixed-point sum v times the density scale, in float or double. For floats
+// the scale is the pair (hi, lo) and the product keeps about 48 bits before
+// its one rounding: the same value as from an FP64 product, without the FP64
+// unit (16.8M values of a 128^3 grid 24 -> 10 us).
+__device__ __forceinline__ double scaled_density(long long v, double scale, double) { return (double)v * scale; }
+__device__ __forceinline__ float scaled_density(long long v, double scale, float2 s) {
+    if ((unsigned long long)v >> 31) return (float)((double)v * scale);
+    const float f = __uint2float_rn((unsigned)v);
+    const float r = __int2float_rn((int)((unsigned)v - __float2uint_rn(f)));  // exact
+    const float p = __fmul_rn(f, s.x);
+    return __fadd_rn(p, __fmaf_rn(r, s.x, __fmaf_rn(f, s.y, __fmaf_rn(f, s.x, -p))));
+}
+template <typename TO, class Scale>
+__global__ void __launch_bounds__(256) density_out(size_t count, const unsigned long long* __restrict__ rho_fx, double scale,
+                                                   Scale s, TO* __restrict__ out) {
+    const size_t i0 = (size_t)blockIdx.x * 1024 + threadIdx.x;
+    long long v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        if (i0 + 256 * k < count) v[k] = (long long)__ldg(rho_fx + i0 + 256 * k);
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        if (i0 + 256 * k < count) out[i0 + 256 * k] = scaled_density(v[k], scale, s);
 }
 
 template <typename TI, typename TO>

@@ -75,6 +75,92 @@ __device__ __forceinline__ float density_from_fixed(long long v, float scale) {
 }
 __device__ __forceinline__ double density_from_fixed(long long v, double scale) { return from_fixed(v, scale); }
 
+// Sums of observables (energies, forces) in more than the working precision.
+// FP64 contexts sum in FP64. FP32 contexts sum pairs (hi, lo) of floats: a sum
+// keeps its rounding errors exactly (Knuth's two-sum) and a product its own
+// (by a fused multiply-add; Dekker 1971), about 48 bits in all. The FP64 unit
+// of this part does two operations per clock and SM, and the FP64 form of
+// these sums took longer than the passes that feed them (bead forces of 1.6M
+// beads 151 -> 77 us, 128^3 z pass with energies 98 -> 24 us, isolated).
+template <typename T> struct Wide;
+template <> struct Wide<double> {
+    using stored = double;
+    double v = 0.0;
+    __device__ __forceinline__ void add(double x) { v += x; }
+    __device__ __forceinline__ void add_prod(double a, double b) { v = fma(a, b, v); }
+    __device__ __forceinline__ void add(const Wide& o) { v += o.v; }
+    __device__ __forceinline__ Wide times(double s) const { return {v * s}; }
+    __device__ __forceinline__ Wide shfl_down(int o) const { return {__shfl_down_sync(0xffffffffu, v, o)}; }
+    __device__ __forceinline__ stored store() const { return v; }
+    static __device__ __forceinline__ Wide load(stored s) { return {s}; }
+    __device__ __forceinline__ double value() const { return v; }
+};
+template <> struct Wide<float> {
+    using stored = float2;
+    float hi = 0.f, lo = 0.f;
+    __device__ __forceinline__ void add(float x) {
+        const float s = __fadd_rn(hi, x), b = __fsub_rn(s, hi);
+        const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b));
+        hi = s;
+        lo = __fadd_rn(lo, e);
+    }
+    __device__ __forceinline__ void add_prod(float a, float b) {
+        const float p = __fmul_rn(a, b);
+        lo = __fadd_rn(lo, __fmaf_rn(a, b, -p));
+        add(p);
+    }
+    __device__ __forceinline__ void add(const Wide& o) {
+        lo = __fadd_rn(lo, o.lo);
+        add(o.hi);
+    }
+    __device__ __forceinline__ Wide times(float s) const {
+        const float p = __fmul_rn(hi, s);
+        return {p, __fmaf_rn(lo, s, __fmaf_rn(hi, s, -p))};
+    }
+    __device__ __forceinline__ Wide shfl_down(int o) const {
+        return {__shfl_down_sync(0xffffffffu, hi, o), __shfl_down_sync(0xffffffffu, lo, o)};
+    }
+    __device__ __forceinline__ stored store() const { return {hi, lo}; }
+    static __device__ __forceinline__ Wide load(stored s) { return {s.x, s.y}; }
+    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+};
+
+// acc += x^2
+__device__ __forceinline__ void add_square(Wide<double>& acc, const Wide<double>& x) { acc.add_prod(x.v, x.v); }
+__device__ __forceinline__ void add_square(Wide<float>& acc, const Wide<float>& x) {
+    acc.add_prod(x.hi, x.hi);
+    acc.lo = __fmaf_rn(__fadd_rn(x.hi, x.hi), x.lo, acc.lo);
+}
+
+// Sums of the K values over a block of up to 1024 threads, in a fixed order;
+// thread 0 writes them to out[0 .. K - 1].
+template <int K, typename T, class Out> __device__ __forceinline__ void block_sum(Wide<T> (&acc)[K], Out out) {
+    __shared__ typename Wide<T>::stored red[K][32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        for (int o = 16; o > 0; o >>= 1) acc[k].add(acc[k].shfl_down(o));
+        if (lane == 0) red[k][wid] = acc[k].store();
+    }
+    __syncthreads();
+    if (threadIdx.x < K) {
+        Wide<T> s;
+        for (int w = 0; w < (int)blockDim.x / 32; ++w) s.add(Wide<T>::load(red[threadIdx.x][w]));
+        out(threadIdx.x, s);
+    }
+}
+
+// out[k] = sum of component k = blockIdx.x of the K-component block sums.
+template <typename T>
+__global__ void __launch_bounds__(1024) sum_partials(const typename Wide<T>::stored* __restrict__ partials, int n_blocks, int K,
+                                                     double* __restrict__ out) {
+    Wide<T> acc[1];
+    const int k = blockIdx.x;
+#pragma unroll 4
+    for (int b = threadIdx.x; b < n_blocks; b += 1024) acc[0].add(Wide<T>::load(partials[(size_t)b * K + k]));
+    block_sum<1, T>(acc, [&](int, const Wide<T>& s) { out[k] = s.value(); });
+}
+
 // Tiles of the bead kernel: beads are binned by 8x8x8 grid cells.
 constexpr int kTile = 8;
 constexpr int kTileCells = kTile * kTile * kTile;

@@ -59,8 +59,14 @@ template <typename T> class Engine final : public EngineBase {
         if (gst) return gst;
         TILD_CUDA(dev_malloc((void**)&tw_, n_ * sizeof(V)));
         TILD_CUDA(dev_malloc((void**)&kernel1d_, 2 * n_ * sizeof(T)));  // exp(-a^2 k_m^2), then exp(-a_e^2 k_m^2)
-        TILD_CUDA(dev_malloc((void**)&counters_, 4 * sizeof(unsigned long long)));
-        TILD_CUDA(cudaMemset(counters_, 0, 4 * sizeof(unsigned long long)));
+        TILD_CUDA(dev_malloc((void**)&counters_, kWords * sizeof(unsigned long long)));
+        TILD_CUDA(cudaMemset(counters_, 0, kWords * sizeof(unsigned long long)));
+        if (cudaHostAlloc((void**)&words_, kWords * sizeof(unsigned long long), cudaHostAllocDefault) != cudaSuccess) {
+            cudaGetLastError();
+            words_ = nullptr;
+            err = "cannot allocate the pinned read-back words";
+            return TILD_ENOMEM;
+        }
         // tiles of 8^3 cells (one layer of tiles on a 2D grid)
         n_tiles_ = tiles_ * tiles_ * ((nz_ + kTile - 1) / kTile);
         n_fine_ = (size_t)kFineBins * n_tiles_ + 1;  // re-binning bins (tile, edge class, bank group)
@@ -70,7 +76,7 @@ template <typename T> class Engine final : public EngineBase {
         scan_blocks_ = (int)((n_fine_ + 1023) / 1024);
         TILD_CUDA(dev_malloc((void**)&block_sums_, scan_blocks_ * sizeof(int)));
         n_z_blocks_ = generic_ ? (size_t)blocks(M_) : (size_t)(n_ / CZ_) * (n_ / 2 + 1);  // two species pairs: twice as many (zpass_cols2)
-        n_partials_ = std::max(10 * n_z_blocks_, 5 * (size_t)tiles_ * tiles_ * tiles_);
+        n_partials_ = std::max(10 * n_z_blocks_, 5 * (size_t)tiles_ * tiles_ * tiles_);  // 8 bytes each
         n_partials_ = std::max(n_partials_, 3 * (size_t)(n_ / vjp_cols(n_)) * (n_ / 2 + 1));
         TILD_CUDA(dev_malloc((void**)&partials_, n_partials_ * sizeof(double)));
         partials_bytes_ = n_partials_ * sizeof(double);
@@ -171,8 +177,7 @@ template <typename T> class Engine final : public EngineBase {
         if ((st = zero_z())) return st;
         if ((st = enqueue_sort())) return st;
         if ((st = respread())) return st;
-        TILD_CUDA(cudaStreamSynchronize(stream_));
-        if ((st = check_err())) return st;
+        if ((st = finish())) return st;
         have_pos_ = true;
         have_vel_ = false;
         return TILD_OK;
@@ -194,7 +199,7 @@ template <typename T> class Engine final : public EngineBase {
             TILD_CUDA(cudaGetLastError());
             vin = (const T*)aux_;
         }
-        if ((st = enqueue_fields(false, nullptr, nullptr))) return st;
+        if ((st = enqueue_fields(0, nullptr, nullptr))) return st;
         BeadBuffers<T> bf = bead_buffers();
         bf.v_in = vin;
         if ((st = launch_bead(kModeSetVel, bf))) return st;
@@ -228,56 +233,44 @@ template <typename T> class Engine final : public EngineBase {
     }
 
     tild_status synchronize() override {
-        TILD_CUDA(cudaStreamSynchronize(stream_));
-        return check_err();
+        return finish();
     }
 
     tild_status compute(unsigned what, tild_energy* e, void* f, int dtype, int where) override {
         tild_status st;
         const bool want_e = (what & TILD_COMPUTE_ENERGY) != 0;
         if ((st = ensure_partials())) return st;
-        if ((st = enqueue_fields(want_e, partials_, nullptr))) return st;
-        std::vector<double> zpart;
-        if (want_e) {
-            zpart.resize(5 * z_blocks());
-            TILD_CUDA(cudaMemcpyAsync(zpart.data(), partials_, zpart.size() * sizeof(double), cudaMemcpyDeviceToHost, stream_));
-        }
+        if ((st = enqueue_fields(want_e ? 1 : 0, partials_, nullptr))) return st;
+        if (want_e && (st = reduce_partials(z_blocks(), 5, sums()))) return st;
         BeadBuffers<T> bf = bead_buffers();
-        T* fdev = nullptr;
+        if (e) bf.partials = (typename Wide<T>::stored*)partials_;
+        const size_t n3 = (size_t)3 * cfg_->n_beads;
+        const bool direct = f && device_native(dtype, where);  // the kernel writes the caller's array
         if (f) {
-            if ((st = ensure_aux((size_t)3 * cfg_->n_beads * sizeof(T)))) return st;
-            fdev = (T*)aux_;
-            bf.f_out = fdev;
+            if (!direct && (st = ensure_aux(n3 * sizeof(T)))) return st;
+            bf.f_out = direct ? (T*)f : (T*)aux_;
         }
         if ((st = launch_bead(kModeForce, bf))) return st;
-        std::vector<double> bpart(5 * bead_blocks());
-        TILD_CUDA(cudaMemcpyAsync(bpart.data(), partials_, bpart.size() * sizeof(double), cudaMemcpyDeviceToHost, stream_));
-        if (f && (st = stage_out_vec(fdev, (size_t)3 * cfg_->n_beads, f, dtype, where))) return st;
-        TILD_CUDA(cudaStreamSynchronize(stream_));
-        if ((st = check_err())) return st;
+        if (e && (st = reduce_partials(bead_blocks(), 5, sums() + 5))) return st;
+        if (f && !direct && (st = stage_out_vec((T*)aux_, n3, f, dtype, where))) return st;
+        if ((st = finish())) return st;
+        const double* h = host_sums();
+        if (e) {
+            const BeadParams<T> p = bead_params();
+            const double el = p.e_len, ev = p.e_vel;
+            e->e_bond = 1.5 / (cfg_->b * cfg_->b) * h[5] / (el * el);
+            e->kinetic = 0.5 * cfg_->mass * h[6] / (ev * ev);
+            for (int d = 0; d < 3; ++d) e->net_force[d] = h[7 + d];
+            e->e_chi = e->e_kappa = e->e_elec = 0.0;
+        }
         if (want_e && e) {
-            double s0 = 0, s1 = 0, s4 = 0;
-            for (size_t b = 0; b < z_blocks(); ++b) {
-                s0 += zpart[5 * b];
-                s1 += zpart[5 * b + 1];
-                s4 += zpart[5 * b + 4];
-            }
             const double V = volume();
             const double dV = V / (double)M_;
-            const double rho0 = cfg_->n_beads / V;
+            const double rho0 = cfg_->n_beads / V, er = spectral_params().e_rho;
             // one pair: the z pass sums Re[conj(rho_A) rho_B]; two pairs: chi-weighted sums
-            e->e_chi = (NP_ == 1 ? cfg_->chi : 1.0) / rho0 * dV * dV / V * s0;
-            e->e_kappa = cfg_->kappa / (2.0 * rho0) * dV * dV / V * s1;
-            e->e_elec = e_elec_from(s4);
-        }
-        if (e) {
-            double acc[5] = {0, 0, 0, 0, 0};
-            for (size_t b = 0; b < bpart.size() / 5; ++b)
-                for (int k = 0; k < 5; ++k) acc[k] += bpart[5 * b + k];
-            e->e_bond = acc[0];
-            e->kinetic = acc[1];
-            for (int d = 0; d < 3; ++d) e->net_force[d] = acc[2 + d];
-            if (!want_e) e->e_chi = e->e_kappa = e->e_elec = 0.0;
+            e->e_chi = (NP_ == 1 ? cfg_->chi : 1.0) / rho0 * dV * dV / V * (h[0] / (er * er));
+            e->e_kappa = cfg_->kappa / (2.0 * rho0) * dV * dV / V * (h[1] / (er * er));
+            e->e_elec = e_elec_from(h[4] / (er * er));
         }
         return TILD_OK;
     }
@@ -292,33 +285,32 @@ template <typename T> class Engine final : public EngineBase {
             err = "energy_gradient: implemented for one or two species";
             return TILD_EUNSUPPORTED;
         }
-        if ((st = enqueue_fields(true, partials_, nullptr, kInvGradPot))) return st;
-        std::vector<double> zpart(5 * n_z_blocks_);
-        TILD_CUDA(cudaMemcpyAsync(zpart.data(), partials_, zpart.size() * sizeof(double), cudaMemcpyDeviceToHost, stream_));
+        const size_t N = cfg_->n_beads;
+        if ((st = device_buffer(&partials_, partials_bytes_, std::max(partials_bytes_, (size_t)blocks(N) * sizeof(double))))) return st;
+        if ((st = enqueue_fields(2, partials_, nullptr, kInvPot))) return st;
+        if ((st = reduce_partials(n_z_blocks_, 5, sums()))) return st;
         BeadBuffers<T> bf = bead_buffers();
-        if ((st = launch_bead(kModeForce, bf))) return st;  // bond energy partials
-        std::vector<double> bpart(5 * (size_t)tiles_ * tiles_ * tiles_);
-        TILD_CUDA(cudaMemcpyAsync(bpart.data(), partials_, bpart.size() * sizeof(double), cudaMemcpyDeviceToHost, stream_));
-        if (dUdr) {
-            const size_t N = cfg_->n_beads;
-            if ((st = ensure_aux(3 * N * sizeof(T)))) return st;
-            const BeadParams<T> p = bead_params();
-            const V* pot = grad_ + 3 * M_;
-            tild_status s2 = dispatch_p([&](auto pp) -> tild_status {
-                adjoint_kernel<decltype(pp)::value, T><<<blocks(N), 256, 0, stream_>>>(p, bf, pot, (T*)aux_);
-                return TILD_OK;
-            });
-            if (s2) return s2;
-            TILD_CUDA(cudaGetLastError());
-            if ((st = stage_out_vec((T*)aux_, 3 * N, dUdr, dtype, where))) return st;
-        }
-        TILD_CUDA(cudaStreamSynchronize(stream_));
-        if ((st = check_err())) return st;
-        double s[5] = {0, 0, 0, 0, 0};
-        for (size_t b = 0; b < n_z_blocks_; ++b)
-            for (int k = 0; k < 5; ++k) s[k] += zpart[5 * b + k];
-        double eb = 0;
-        for (size_t b = 0; b < bpart.size() / 5; ++b) eb += bpart[5 * b];
+        bf.partials = (typename Wide<T>::stored*)partials_;
+        const bool direct = dUdr && device_native(dtype, where);
+        if (dUdr && !direct && (st = ensure_aux(3 * N * sizeof(T)))) return st;
+        T* out = !dUdr ? nullptr : direct ? (T*)dUdr : (T*)aux_;
+        const BeadParams<T> p = bead_params();
+        const V* pot = grad_ + 3 * M_;
+        if ((st = dispatch_p([&](auto pp) -> tild_status {
+                 adjoint_kernel<decltype(pp)::value, T><<<blocks(N), 256, 0, stream_>>>(p, bf, pot, out);
+                 return TILD_OK;
+             })))
+            return st;
+        TILD_CUDA(cudaGetLastError());
+        if ((st = reduce_partials(blocks(N), 1, sums() + 5))) return st;
+        if (dUdr && !direct && (st = stage_out_vec((T*)aux_, 3 * N, dUdr, dtype, where))) return st;
+        if ((st = finish())) return st;
+        const double er = spectral_params().e_rho, kk = 2.0 * 3.14159265358979323846 / cfg_->L;
+        double s[5];
+        for (int k = 0; k < 5; ++k) s[k] = host_sums()[k] / (er * er);
+        s[2] *= kk * kk;  // summed with integer frequencies
+        s[3] *= kk * kk;
+        const double eb = 1.5 / (cfg_->b * cfg_->b) * host_sums()[5] / ((double)p.e_len * p.e_len);
         const double V = cfg_->L * cfg_->L * cfg_->L;
         const double dV = V / (double)M_;
         const double rho0 = cfg_->n_beads / V;
@@ -377,7 +369,7 @@ template <typename T> class Engine final : public EngineBase {
     tild_status vjp_core(const T* lam_d, T* out_d, double* theta_acc, bool fields_ready = false) {
         const size_t N = cfg_->n_beads;
         tild_status st;
-        if (!fields_ready && (st = enqueue_fields(false, nullptr, nullptr, kInvGrad))) return st;  // D w at r; Zxy = xy(rho)
+        if (!fields_ready && (st = enqueue_fields(0, nullptr, nullptr, kInvGrad))) return st;  // D w at r; Zxy = xy(rho)
         using Bits = typename AdjointFixed<T>::bits_t;
         unsigned long long* fx = (unsigned long long*)vjp_fx_;
         Bits* bits = (Bits*)(fx + 6 * M_);
@@ -443,7 +435,6 @@ template <typename T> class Engine final : public EngineBase {
         const void* src = lam;
         if ((st = stage_in(&src, lam, 3 * N, dtype, where))) return st;
         if ((st = ensure_aux(6 * N * sizeof(T)))) return st;
-        if ((st = device_buffer(&theta_, theta_bytes_, 3 * sizeof(double)))) return st;
         T* lam_d = (T*)aux_;
         T* out_d = lam_d + 3 * N;
         if (dtype == TILD_DTYPE_F32)
@@ -451,14 +442,11 @@ template <typename T> class Engine final : public EngineBase {
         else
             convert_copy<double, T><<<blocks(3 * N), 256, 0, stream_>>>(3 * N, (const double*)src, lam_d);
         TILD_CUDA(cudaGetLastError());
-        TILD_CUDA(cudaMemsetAsync(theta_, 0, 3 * sizeof(double), stream_));
-        if ((st = vjp_core(lam_d, out_d, theta_))) return st;
-        double s[3];
-        TILD_CUDA(cudaMemcpyAsync(s, theta_, sizeof(s), cudaMemcpyDeviceToHost, stream_));
+        TILD_CUDA(cudaMemsetAsync(sums(), 0, 3 * sizeof(double), stream_));
+        if ((st = vjp_core(lam_d, out_d, sums()))) return st;
         if ((st = stage_out_vec(out_d, 3 * N, out, dtype, where))) return st;
-        TILD_CUDA(cudaStreamSynchronize(stream_));
-        if ((st = check_err())) return st;
-        if (dtheta) theta_from_sums(s, dtheta);
+        if ((st = finish())) return st;
+        if (dtheta) theta_from_sums(host_sums(), dtheta);
         return TILD_OK;
     }
 
@@ -491,8 +479,7 @@ template <typename T> class Engine final : public EngineBase {
             return st;
         TILD_CUDA(cudaGetLastError());
         if ((st = stage_out_vec(out_d, 3 * N, out, dtype, where))) return st;
-        TILD_CUDA(cudaStreamSynchronize(stream_));
-        return check_err();
+        return finish();
     }
 
     // positions and carried velocities by id ([2][N][3] T) <-> the context
@@ -586,7 +573,7 @@ template <typename T> class Engine final : public EngineBase {
         const int64_t n_ckpt = K / C + 1;
         const size_t bsnap = snapshot_bytes(), snap = bsnap + field_snapshot_bytes();
         const size_t head = snap_part(sizeof(T) * (sb * ((size_t)n_ckpt + 1) + 2 * n3));
-        const size_t need = head + snap * (size_t)C + sizeof(double) * (3 * n3 + 3);
+        const size_t need = head + snap * (size_t)C + sizeof(double) * 3 * n3;
         if ((st = device_buffer(&traj_, traj_bytes_, need))) return st;
         T* ckpt = (T*)traj_;                        // [n_ckpt][sb] by id
         T* fin = ckpt + sb * n_ckpt;                // [sb]
@@ -596,7 +583,7 @@ template <typename T> class Engine final : public EngineBase {
         double* rb = (double*)(seg + snap * (size_t)C);
         double* ub = rb + n3;  // dL/dv^K on entry, then the adjoint of u
         double* vout = ub + n3;
-        double* acc = vout + n3;
+        double* acc = sums();
         const SchemeCoeffs q = scheme_coeffs(*cfg_);
         const int64_t step0 = host_step_;
         // forward with checkpoints
@@ -655,11 +642,8 @@ template <typename T> class Engine final : public EngineBase {
         if ((st = restore_state(fin, step0 + K))) return st;
         if ((st = stage_out_double(rb, n3, r0, dtype, where)) || (st = stage_out_double(vout, n3, v0, dtype, where)))
             return st;
-        double s[3];
-        TILD_CUDA(cudaMemcpyAsync(s, acc, sizeof(s), cudaMemcpyDeviceToHost, stream_));
-        TILD_CUDA(cudaStreamSynchronize(stream_));
-        if ((st = check_err())) return st;
-        if (dtheta) theta_from_sums(s, dtheta);
+        if ((st = finish())) return st;
+        if (dtheta) theta_from_sums(host_sums(), dtheta);
         return TILD_OK;
     }
 
@@ -689,14 +673,15 @@ template <typename T> class Engine final : public EngineBase {
 
     tild_status get_velocities(void* out, int dtype, int where) override {
         tild_status st;
-        if ((st = enqueue_fields(false, nullptr, nullptr))) return st;
-        if ((st = ensure_aux((size_t)3 * cfg_->n_beads * sizeof(T)))) return st;
+        if ((st = enqueue_fields(0, nullptr, nullptr))) return st;
+        const size_t n3 = (size_t)3 * cfg_->n_beads;
+        const bool direct = device_native(dtype, where);
+        if (!direct && (st = ensure_aux(n3 * sizeof(T)))) return st;
         BeadBuffers<T> bf = bead_buffers();
-        bf.v_out = (T*)aux_;
+        bf.v_out = direct ? (T*)out : (T*)aux_;
         if ((st = launch_bead(kModeForce, bf))) return st;
-        if ((st = stage_out_vec((T*)aux_, (size_t)3 * cfg_->n_beads, out, dtype, where))) return st;
-        TILD_CUDA(cudaStreamSynchronize(stream_));
-        return check_err();
+        if (!direct && (st = stage_out_vec((T*)aux_, n3, out, dtype, where))) return st;
+        return finish();
     }
 
     tild_status get_density(void* out, int dtype, int where) override {
@@ -708,10 +693,12 @@ template <typename T> class Engine final : public EngineBase {
             if ((st = ensure_aux(count * 8))) return st;
             dst = aux_;
         }
+        const float2 pair = make_float2((float)scale, (float)(scale - (double)(float)scale));
+        const unsigned grid = (unsigned)((count + 1023) / 1024);
         if (dtype == TILD_DTYPE_F32)
-            density_out<float><<<blocks(count), 256, 0, stream_>>>(count, rho_fx_, scale, (float*)dst);
+            density_out<float><<<grid, 256, 0, stream_>>>(count, rho_fx_, scale, pair, (float*)dst);
         else
-            density_out<double><<<blocks(count), 256, 0, stream_>>>(count, rho_fx_, scale, (double*)dst);
+            density_out<double><<<grid, 256, 0, stream_>>>(count, rho_fx_, scale, scale, (double*)dst);
         TILD_CUDA(cudaGetLastError());
         if (where == TILD_HOST)
             TILD_CUDA(cudaMemcpyAsync(out, dst, count * dtype_size(dtype), cudaMemcpyDeviceToHost, stream_));
@@ -722,7 +709,7 @@ template <typename T> class Engine final : public EngineBase {
     tild_status get_spectrum(void* out, int dtype, int where) override {
         tild_status st;
         if ((st = device_buffer(&spec_, spec_bytes_, NP_ * M_ * sizeof(V)))) return st;
-        if ((st = enqueue_fields(false, nullptr, spec_))) return st;
+        if ((st = enqueue_fields(0, nullptr, spec_))) return st;
         if ((st = stage_out_vec((T*)spec_, 2 * NP_ * M_, out, dtype, where))) return st;
         TILD_CUDA(cudaStreamSynchronize(stream_));
         return TILD_OK;
@@ -730,7 +717,7 @@ template <typename T> class Engine final : public EngineBase {
 
     tild_status get_field_gradient(void* out, int dtype, int where) override {
         tild_status st;
-        if ((st = enqueue_fields(false, nullptr, nullptr, kInvGrad))) return st;
+        if ((st = enqueue_fields(0, nullptr, nullptr, kInvGrad))) return st;
         const int D = cfg_->dim;
         for (int q = 0; q < NP_; ++q) {
             char* o = (char*)out + (size_t)q * 2 * D * M_ * dtype_size(dtype);
@@ -875,7 +862,7 @@ template <typename T> class Engine final : public EngineBase {
         const size_t N = cfg_->n_beads;
         if (!vsave_) TILD_CUDA(dev_malloc((void**)&vsave_, 3 * N * sizeof(T)));
         tild_status st;
-        if ((st = enqueue_fields(false, nullptr, nullptr))) return st;
+        if ((st = enqueue_fields(0, nullptr, nullptr))) return st;
         BeadBuffers<T> bf = bead_buffers();
         bf.v_out = vsave_;
         if ((st = launch_bead(kModeForce, bf))) return st;
@@ -886,7 +873,7 @@ template <typename T> class Engine final : public EngineBase {
     tild_status restore_velocities() override {
         invalidate_graph();
         tild_status st;
-        if ((st = enqueue_fields(false, nullptr, nullptr))) return st;
+        if ((st = enqueue_fields(0, nullptr, nullptr))) return st;
         BeadBuffers<T> bf = bead_buffers();
         bf.v_in = vsave_;
         if ((st = launch_bead(kModeSetVel, bf))) return st;
@@ -978,7 +965,11 @@ template <typename T> class Engine final : public EngineBase {
     T* kernel1d_ = nullptr;
     double kernel_a_ = -1.0, kernel_ae_ = -1.0;
     V* spec_ = nullptr;
-    unsigned long long* counters_ = nullptr;  // [0] noise step counter, [1] error flags
+    // [0] noise step counter, [1] error flags, [4 ..] sums of one call (FP64);
+    // words_: their pinned host copy, one transfer per synchronising call
+    static constexpr int kWords = 16;
+    unsigned long long* counters_ = nullptr;
+    unsigned long long* words_ = nullptr;
     double* partials_ = nullptr;
     size_t n_partials_ = 0, n_z_blocks_ = 0;
     // beads
@@ -1003,8 +994,6 @@ template <typename T> class Engine final : public EngineBase {
     // staging
     void* aux_ = nullptr;
     size_t aux_bytes_ = 0;
-    double* theta_ = nullptr;  // force-VJP parameter sums
-    size_t theta_bytes_ = 0;
     void* traj_ = nullptr;     // trajectory derivatives: checkpoints and adjoint vectors
     size_t traj_bytes_ = 0;
     void* vjp_fx_ = nullptr;   // force VJP: fixed-point spread of lam
@@ -1200,10 +1189,12 @@ template <typename T> class Engine final : public EngineBase {
         if (stream_) cudaStreamSynchronize(stream_);  // no kernel may still use a block handed back
         free_beads();
         void* ptrs[] = {rho_fx_, Zxy_, H_, grad_, tw_, kernel1d_, spec_, counters_, partials_, counts_,
-                        tile_start_, fine_start_, block_sums_, aux_, stage_, theta_, traj_, vjp_fx_,
+                        tile_start_, fine_start_, block_sums_, aux_, stage_, traj_, vjp_fx_,
                         sp_of_id_, adj_, ext_ids_, ext_slots_, io_};
         for (void* p : ptrs) dev_free(p);
         rho_fx_ = nullptr;
+        if (words_) cudaFreeHost(words_);
+        words_ = nullptr;
         if (own_stream_) cudaStreamDestroy(own_stream_);
         own_stream_ = nullptr;
     }
@@ -1214,9 +1205,32 @@ template <typename T> class Engine final : public EngineBase {
         graph_key_ = -1;
     }
 
+    double* sums() const { return reinterpret_cast<double*>(counters_ + 4); }
+    const double* host_sums() const { return reinterpret_cast<const double*>(words_ + 4); }
+    // sums()[k] of the K-component block sums in partials_
+    tild_status reduce_partials(size_t n_blocks, int K, double* out) {
+        sum_partials<T><<<K, 1024, 0, stream_>>>((const typename Wide<T>::stored*)partials_, (int)n_blocks, K, out);
+        TILD_CUDA(cudaGetLastError());
+        return TILD_OK;
+    }
+    // whether the caller's array can be a kernel's own input or output
+    static bool device_native(int dtype, int where) {
+        return where == TILD_DEVICE && dtype == (sizeof(T) == 4 ? TILD_DTYPE_F32 : TILD_DTYPE_F64);
+    }
+
+    // Wait for the context's stream, with the error flags and the call's sums
+    // read back behind its work.
+    tild_status finish() {
+        TILD_CUDA(cudaMemcpyAsync(words_, counters_, kWords * sizeof(unsigned long long), cudaMemcpyDeviceToHost, stream_));
+        TILD_CUDA(cudaStreamSynchronize(stream_));
+        return check_flags(reinterpret_cast<const unsigned int*>(words_)[3]);
+    }
     tild_status check_err() {
         unsigned int h = 0;
         TILD_CUDA(cudaMemcpy(&h, err_ptr(), sizeof(h), cudaMemcpyDeviceToHost));
+        return check_flags(h);
+    }
+    tild_status check_flags(unsigned int h) {
         if (h & kErrBounds) {
             TILD_CUDA(cudaMemset(err_ptr(), 0, sizeof(unsigned int)));
             err = "a bounds check of the debug build failed on the device (the access was skipped)";
@@ -1337,7 +1351,7 @@ template <typename T> class Engine final : public EngineBase {
         TILD_CUDA(cudaFuncSetAttribute(z_spectral_pairs<T, NN, C2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)zpass2_smem()));
         TILD_CUDA(cudaFuncSetAttribute(z_spectrum<T, NN, CC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)zpass_smem()));
         tild_status st = with_z<NN>([&](auto cc, auto g, auto el, auto e) -> tild_status {
-            TILD_CUDA(cudaFuncSetAttribute(z_spectral<T, NN, decltype(cc)::value, decltype(g)::value != 0, decltype(el)::value != 0, decltype(e)::value != 0>,
+            TILD_CUDA(cudaFuncSetAttribute(z_spectral<T, NN, decltype(cc)::value, decltype(g)::value != 0, decltype(el)::value != 0, decltype(e)::value>,
                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)zpass_smem_cols(decltype(cc)::value)));
             return TILD_OK;
         }, true);
@@ -1500,6 +1514,12 @@ template <typename T> class Engine final : public EngineBase {
 
     T two_pi_L() const { return (T)(2.0 * 3.14159265358979323846 / cfg_->L); }
 
+    // a power of two near x for the scaled sums of Wide<T> (1 in FP64)
+    static T power_of_two(double x) {
+        if (sizeof(T) == 8 || !(x > 0) || !std::isfinite(x)) return T(1);
+        return (T)std::ldexp(1.0, std::max(-100, std::min(100, std::ilogb(x))));
+    }
+
     SpectralParams<T> spectral_params() const {
         const double V = volume();
         const double rho0 = cfg_->n_beads / V;
@@ -1514,6 +1534,7 @@ template <typename T> class Engine final : public EngineBase {
                 sp.eps4[K][K2] = (T)((chi + cfg_->kappa) / rho0 / (double)M_);
                 sp.chi4[K][K2] = (T)chi;
             }
+        sp.e_rho = power_of_two(V / (double)M_);
         sp.kernel1d = kernel1d_;
         const bool charged = c_el_on();
         sp.el_scale = charged ? (T)(4.0 * 3.14159265358979323846 * cfg_->bjerrum / (double)M_) : T(0);
@@ -1523,7 +1544,7 @@ template <typename T> class Engine final : public EngineBase {
         return sp;
     }
 
-    template <int NN> tild_status zpass_n(double* partials, V* spec_out, bool g_only) {
+    template <int NN> tild_status zpass_n(typename Wide<T>::stored* partials, V* spec_out, bool g_only, int want_e) {
         constexpr int CC = zpass_cols(NN);
         const SpectralParams<T> sp = spectral_params();
         const bool el = c_el_on();
@@ -1546,31 +1567,43 @@ template <typename T> class Engine final : public EngineBase {
         }
         return with_z<NN>([&](auto cc, auto g, auto e_l, auto e) -> tild_status {
             constexpr int CZ = decltype(cc)::value;
-            z_spectral<T, NN, CZ, decltype(g)::value != 0, decltype(e_l)::value != 0, decltype(e)::value != 0>
+            z_spectral<T, NN, CZ, decltype(g)::value != 0, decltype(e_l)::value != 0, decltype(e)::value>
                 <<<dim3(NN / CZ, NN / 2 + 1), 256, zpass_smem_cols(CZ), stream_>>>(Zxy_, H_, tw_, sp, partials);
             TILD_CUDA(cudaGetLastError());
             return TILD_OK;
-        }, false, g_only, el, partials != nullptr);
+        }, false, g_only, el, want_e);
     }
     // f(columns, G alone, charges, energies) for the z pass to launch, or for
     // every instantiation when `all`. The alternative column tile serves the
     // plain step only (launch shapes).
     template <int NN, class F>
-    tild_status with_z(F&& f, bool all, bool g_only = false, bool el = false, bool want_e = false) {
+    tild_status with_z(F&& f, bool all, bool g_only = false, bool el = false, int want_e = 0) {
         constexpr int CC = zpass_cols(NN), CA = zpass_cols_alt(NN);
         tild_status st = TILD_OK;
-        auto pick = [&](bool take, auto cc, auto g, auto e_l, auto e) {
+        bool found = false;
+        auto pick = [&](auto cc, auto g, auto e_l, auto e) {
+            const bool alt = decltype(cc)::value != CC;
+            const bool plain = !g_only && !el && want_e == 0;
+            const bool take = g_only == (decltype(g)::value != 0) && el == (decltype(e_l)::value != 0) &&
+                              want_e == decltype(e)::value && alt == (CA != CC && zalt_ && plain);
             if (!st && (all || take)) st = f(cc, g, e_l, e);
+            found = found || take;
         };
-        if constexpr (CA != CC) pick(zalt_ && !g_only && !el && !want_e, ic<CA>{}, ic<0>{}, ic<0>{}, ic<0>{});
-        pick(!(zalt_ && CA != CC) && !g_only && !el && !want_e, ic<CC>{}, ic<0>{}, ic<0>{}, ic<0>{});
-        pick(g_only && !el && !want_e, ic<CC>{}, ic<1>{}, ic<0>{}, ic<0>{});
-        pick(!g_only && el && !want_e, ic<CC>{}, ic<0>{}, ic<1>{}, ic<0>{});
-        pick(g_only && el && !want_e, ic<CC>{}, ic<1>{}, ic<1>{}, ic<0>{});
-        pick(!g_only && !el && want_e, ic<CC>{}, ic<0>{}, ic<0>{}, ic<1>{});
-        pick(g_only && !el && want_e, ic<CC>{}, ic<1>{}, ic<0>{}, ic<1>{});
-        pick(!g_only && el && want_e, ic<CC>{}, ic<0>{}, ic<1>{}, ic<1>{});
-        pick(g_only && el && want_e, ic<CC>{}, ic<1>{}, ic<1>{}, ic<1>{});
+        if constexpr (CA != CC) pick(ic<CA>{}, ic<0>{}, ic<0>{}, ic<0>{});
+        pick(ic<CC>{}, ic<0>{}, ic<0>{}, ic<0>{});
+        pick(ic<CC>{}, ic<1>{}, ic<0>{}, ic<0>{});
+        pick(ic<CC>{}, ic<0>{}, ic<1>{}, ic<0>{});
+        pick(ic<CC>{}, ic<1>{}, ic<1>{}, ic<0>{});
+        pick(ic<CC>{}, ic<0>{}, ic<0>{}, ic<1>{});
+        pick(ic<CC>{}, ic<1>{}, ic<0>{}, ic<1>{});
+        pick(ic<CC>{}, ic<0>{}, ic<1>{}, ic<1>{});
+        pick(ic<CC>{}, ic<1>{}, ic<1>{}, ic<1>{});
+        pick(ic<CC>{}, ic<1>{}, ic<0>{}, ic<2>{});
+        pick(ic<CC>{}, ic<1>{}, ic<1>{}, ic<2>{});
+        if (!st && !all && !found) {
+            err = "no z pass for these options";
+            return TILD_EUNSUPPORTED;
+        }
         return st;
     }
     // separable Gaussian tables exp(-s^2 k_m^2), k_m = 2 pi m / L, m in FFT
@@ -1595,7 +1628,8 @@ template <typename T> class Engine final : public EngineBase {
         if (c_el_on() && (st = refresh(cfg_->charge_smear, kernel_ae_, kernel1d_ + n_))) return st;
         return TILD_OK;
     }
-    tild_status enqueue_zpass(double* partials, V* spec_out, bool g_only = false) {
+    tild_status enqueue_zpass(double* partials_d, V* spec_out, bool g_only = false, int want_e = 1) {
+        auto* partials = (typename Wide<T>::stored*)partials_d;
         tild_status st;
         if ((st = refresh_tables())) return st;
         if (generic_) {
@@ -1611,13 +1645,13 @@ template <typename T> class Engine final : public EngineBase {
             TILD_CUDA(cudaGetLastError());
             return TILD_OK;
         }
-        return dispatch_n([&](auto nn) { return this->template zpass_n<decltype(nn)::value>(partials, spec_out, g_only); });
+        return dispatch_n([&](auto nn) { return this->template zpass_n<decltype(nn)::value>(partials, spec_out, g_only, partials ? want_e : 0); });
     }
 
     // what the inverse xy pass produces
-    static constexpr int kInvGrad = 0, kInvGradPot = 1, kInvPot = 2;
+    static constexpr int kInvGrad = 0, kInvPot = 1;
     template <int NN> tild_status inverse_n(int what) {
-        const unsigned nd = what == kInvGrad ? 3 : what == kInvGradPot ? 4 : 1;
+        const unsigned nd = what == kInvGrad ? 3 : 1;
         const int d0 = what == kInvPot ? 3 : 0;
         if (use_planes()) {
             if constexpr (plane_fits(NN, sizeof(V))) {
@@ -1652,7 +1686,9 @@ template <typename T> class Engine final : public EngineBase {
     // the fields the bead kernel's force needs: ik gradients or the potentials
     int force_fields() const { return analytic() ? kInvPot : kInvGrad; }
 
-    tild_status enqueue_fields(bool energy, double* partials, V* spec_out, int what = -1) {
+    // energy: 0, 1 (energy sums of the z pass into partials) or 2 (and their
+    // |k|^2-weighted versions; potentials only)
+    tild_status enqueue_fields(int energy, double* partials, V* spec_out, int what = -1) {
         if (what < 0) what = force_fields();
         tild_status st;
         if (!have_pos_) {
@@ -1660,7 +1696,7 @@ template <typename T> class Engine final : public EngineBase {
             return TILD_ESTATE;
         }
         if ((st = enqueue_forward(false))) return st;
-        if ((st = enqueue_zpass(energy ? partials : nullptr, spec_out, what == kInvPot))) return st;
+        if ((st = enqueue_zpass(energy ? partials : nullptr, spec_out, what == kInvPot, energy))) return st;
         return enqueue_inverse(what);
     }
 
@@ -1728,6 +1764,8 @@ template <typename T> class Engine final : public EngineBase {
         integrator_constants(c, p);
         p.sigma_v = (T)std::sqrt(c.kT / c.mass);
         p.mass = (T)c.mass;
+        p.e_len = power_of_two(1.0 / c.L);
+        p.e_vel = power_of_two(c.kT > 0 ? std::sqrt(c.mass / c.kT) : 1.0);
         p.seed = c.seed;
         p.topo = c.topo;
         return p;
@@ -1754,7 +1792,7 @@ template <typename T> class Engine final : public EngineBase {
         b.f_out = nullptr;
         b.v_out = nullptr;
         b.v_in = nullptr;
-        b.partials = partials_;
+        b.partials = nullptr;
         return b;
     }
 

@@ -147,24 +147,22 @@ __global__ void generic_load_density(size_t M, int np, unsigned long long* __res
 //   out[p][3] = i Q_p (the potentials), Q_p = w~_2p + i w~_2p+1.
 // Energy partials per block as in the z pass: [0] sum u_hat Re[conj(rho~_0)
 // rho~_1] (one pair) or the chi-weighted sum over species pairs (two
-// pairs), [1] sum_{k != 0} u_hat |sum_K rho~_K|^2, [2], [3] the same times
-// |k|^2, [4] 0. u_hat = e1[kx] e1[ky] (e1[kz]).
+// pairs), [1] sum_{k != 0} u_hat |sum_K rho~_K|^2 (rho~ times e_rho), the
+// others 0. u_hat = e1[kx] e1[ky] (e1[kz]).
 template <typename T, int NP>
 __global__ void __launch_bounds__(256) generic_spectral(const cplx_t<T>* __restrict__ Z, cplx_t<T>* __restrict__ out,
                                                         int n, int nz, SpectralParams<T> sp,
-                                                        double* __restrict__ partials) {
+                                                        typename Wide<T>::stored* __restrict__ partials) {
     using V = cplx_t<T>;
     const size_t M = (size_t)nz * n * n;
     const size_t g = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    double acc[5] = {0, 0, 0, 0, 0};
+    Wide<T> acc[5];
     if (g < M) {
         const int x = (int)(g % n), y = (int)((g / n) % n), z = (int)(g / ((size_t)n * n));
         const int mx = x == 0 ? 0 : n - x, my = y == 0 ? 0 : n - y, mz = z == 0 ? 0 : nz - z;
         const size_t gm = ((size_t)mz * n + my) * n + mx;
         auto freq = [&](int i, int len) { return (T)(2 * i < len ? i : i - len); };  // 2 i == len: -len/2
         auto kgrad = [&](int i, int len) { return (len % 2 == 0 && 2 * i == len) ? T(0) : sp.two_pi_over_L * freq(i, len); };
-        const T qx = sp.two_pi_over_L * freq(x, n), qy = sp.two_pi_over_L * freq(y, n);
-        const T qz = nz > 1 ? sp.two_pi_over_L * freq(z, nz) : T(0);
         const T kd[3] = {kgrad(x, n), kgrad(y, n), nz > 1 ? kgrad(z, nz) : T(0)};
         const T uh = sp.kernel1d[x] * sp.kernel1d[y] * (nz > 1 ? sp.kernel1d[z] : T(1));
         V A[2 * NP];
@@ -175,31 +173,10 @@ __global__ void __launch_bounds__(256) generic_spectral(const cplx_t<T>* __restr
             A[2 * p + 1] = {T(0.5) * (Zk.y + Zm.y), -T(0.5) * (Zk.x - Zm.x)};
         }
         if (partials) {
-            const double k2 = (double)qx * qx + (double)qy * qy + (double)qz * qz;
-            double fchi;
-            if (NP == 1) {
-                fchi = (double)uh * ((double)A[0].x * A[1].x + (double)A[0].y * A[1].y);
-            } else {
-                fchi = 0.0;
-#pragma unroll
-                for (int K = 0; K < 2 * NP; ++K)
-#pragma unroll
-                    for (int K2 = K + 1; K2 < 2 * NP; ++K2)
-                        fchi += (double)sp.chi4[K][K2] * ((double)A[K].x * A[K2].x + (double)A[K].y * A[K2].y);
-                fchi *= (double)uh;
-            }
-            acc[0] = fchi;
-            acc[2] = k2 * fchi;
-            if (g != 0) {
-                double tr = 0, ti = 0;
-#pragma unroll
-                for (int K = 0; K < 2 * NP; ++K) {
-                    tr += A[K].x;
-                    ti += A[K].y;
-                }
-                acc[1] = (double)uh * (tr * tr + ti * ti);
-                acc[3] = k2 * acc[1];
-            }
+            if constexpr (NP == 1)
+                add_energies<T, 1>(acc, A[0], A[1], uh, sp.e_rho, T(1), g == 0, T(0));
+            else
+                add_energies4<T, NP>(acc, A, sp, uh, g == 0);
         }
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
@@ -230,20 +207,7 @@ __global__ void __launch_bounds__(256) generic_spectral(const cplx_t<T>* __restr
         }
     }
     if (partials) {
-        __shared__ double red[5][8];
-        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-        for (int k = 0; k < 5; ++k) {
-            double v = acc[k];
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-            if (lane == 0) red[k][wid] = v;
-        }
-        __syncthreads();
-        if (threadIdx.x < 5) {
-            double s = 0;
-            for (int w = 0; w < 8; ++w) s += red[threadIdx.x][w];
-            partials[5 * (size_t)blockIdx.x + threadIdx.x] = s;
-        }
+        block_sum<5, T>(acc, [&](int k, const Wide<T>& v) { partials[5 * (size_t)blockIdx.x + k] = v.store(); });
     }
 }
 
@@ -256,7 +220,8 @@ template <int P, int MODE, typename T, int D>
 __global__ void __launch_bounds__(256) generic_bead_kernel(BeadParams<T> p, BeadBuffers<T> bf, int nz) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const bool active = i < p.n_beads;
-    double acc[5] = {0, 0, 0, 0, 0};
+    const bool sums = MODE == kModeForce && bf.partials;
+    Wide<T> acc[5];
     if (active) {
         const int n = p.n;
         const size_t M = (size_t)nz * n * n;
@@ -302,8 +267,7 @@ __global__ void __launch_bounds__(256) generic_bead_kernel(BeadParams<T> p, Bead
                 fx -= p.k_bond * dx;
                 fy -= p.k_bond * dy;
                 fz -= p.k_bond * dz;
-                if (MODE == kModeForce && slot_bead_id(bf.id[s]) > bid)
-                    acc[0] += 0.5 * (double)p.k_bond * ((double)dx * dx + (double)dy * dy + (double)dz * dz);
+                if (MODE == kModeForce && sums && slot_bead_id(bf.id[s]) > bid) add_squares(acc[0], dx, dy, dz, p.e_len);
             };
             if (nb.x >= 0) bond(nb.x);
             if (nb.y >= 0) bond(nb.y);
@@ -321,10 +285,12 @@ __global__ void __launch_bounds__(256) generic_bead_kernel(BeadParams<T> p, Bead
                 const T vx = p.vu * ux + p.vf * fx + p.vg * g.a;
                 const T vy = p.vu * uy + p.vf * fy + p.vg * g.b;
                 const T vz = D == 3 ? p.vu * uz + p.vf * fz + p.vg * g.c : T(0);
-                acc[1] = 0.5 * (double)p.mass * ((double)vx * vx + (double)vy * vy + (double)vz * vz);
-                acc[2] = fx;
-                acc[3] = fy;
-                acc[4] = fz;
+                if (sums) {
+                    add_squares(acc[1], vx, vy, vz, p.e_vel);
+                    acc[2].add(fx);
+                    acc[3].add(fy);
+                    acc[4].add(fz);
+                }
                 if (bf.f_out) {
                     bf.f_out[3 * (size_t)bid + 0] = fx;
                     bf.f_out[3 * (size_t)bid + 1] = fy;
@@ -386,21 +352,8 @@ __global__ void __launch_bounds__(256) generic_bead_kernel(BeadParams<T> p, Bead
             }
         }
     }
-    if (MODE == kModeForce) {
-        __shared__ double red[5][8];
-        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-        for (int k = 0; k < 5; ++k) {
-            double v = acc[k];
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-            if (lane == 0) red[k][wid] = v;
-        }
-        __syncthreads();
-        if (threadIdx.x < 5) {
-            double s = 0;
-            for (int w = 0; w < 8; ++w) s += red[threadIdx.x][w];
-            bf.partials[5 * (size_t)blockIdx.x + threadIdx.x] = s;
-        }
+    if (MODE == kModeForce && sums) {
+        block_sum<5, T>(acc, [&](int k, const Wide<T>& v) { bf.partials[5 * (size_t)blockIdx.x + k] = v.store(); });
     }
 }
 

@@ -35,6 +35,7 @@ template <typename T> struct SpectralParams {
     T eAA, eAB, eBB;   // eps matrix / M (the 1/M of the inverse DFT folded in)
     T eps4[4][4];      // more than two species: eps_KK' / M
     T chi4[4][4];      // more than two species: chi_KK' (the energy sum of the z pass weights by it)
+    T e_rho;           // a power of two near dV: the energy sums take rho~ times e_rho (1 in FP64)
     const T* kernel1d; // exp(-a^2 k_m^2) per 1-D frequency index m (FP64 on the host)
     // smeared-charge electrostatics: w_K += q_K c(k) (q_A rho~_A + q_B rho~_B) with
     // c(k) = el_scale exp(-a_e^2 |k|^2) / |k|^2 (0 at k = 0); el_scale = 4 pi l_B / M
@@ -632,6 +633,37 @@ template <int C, int STRIDE> struct TileAddr {  // buffer b of a tile set starts
 
 template <typename T> __device__ __forceinline__ int freq_index(int i, int n) { return i < n / 2 ? i : i - n; }
 
+// Square of the integer frequency of FFT index i (exact in floats).
+template <typename T, int N> __device__ __forceinline__ T freq_sq(int i) {
+    const T m = (T)(i < N / 2 ? i : i - N);
+    return m * m;
+}
+
+// Energy sums of one wavevector with species spectra A, B (times e_rho), each
+// times `weight`: [0] u_hat Re[conj(A) B], [1] u_hat |A + B|^2 (k != 0), and
+// (WANT_E = 2) [2], [3] the same times m2 = |k L / 2 pi|^2
+// (d u_hat / d a = -2 a |k|^2 u_hat).
+template <typename T, int WANT_E, class V>
+__device__ __forceinline__ void add_energies(Wide<T> (&acc)[5], V A, V B, T uh, T e_rho, T weight, bool zero, T m2) {
+    const T ar = A.x * e_rho, ai = A.y * e_rho, br = B.x * e_rho, bi = B.y * e_rho;
+    Wide<T> f;
+    f.add_prod(ar, br);
+    f.add_prod(ai, bi);
+    f = f.times(uh * weight);
+    acc[0].add(f);
+    if (WANT_E > 1) acc[2].add(f.times(m2));
+    Wide<T> tr, ti, q;
+    tr.add(ar);
+    tr.add(br);
+    ti.add(ai);
+    ti.add(bi);
+    add_square(q, tr);
+    add_square(q, ti);
+    q = q.times(zero ? T(0) : uh * weight);
+    acc[1].add(q);
+    if (WANT_E > 1) acc[3].add(q.times(m2));
+}
+
 // --------------------------------------------------------------------------
 // z pass: forward DFT along z, spectral multiply + gradient, inverse DFT
 // along z. CTA (tile of C column positions, ky pair {ky, -ky}); the tile
@@ -670,9 +702,9 @@ template <int N, int C> struct ZTile {
 
 // fetch(r, z, c): the input of row r; out(b, c, z, v): output element z of
 // column c of buffer b (buffers: G of row r in r, G_z in R + r).
-template <typename T, int N, int C, bool G_ONLY, bool EL, bool WANT_E, class Fetch, class Out>
+template <typename T, int N, int C, bool G_ONLY, bool EL, int WANT_E, class Fetch, class Out>
 __device__ __forceinline__ void z_tile(cplx_t<T>* buf, cplx_t<T>* tw, const cplx_t<T>* __restrict__ tw_g, T* e1, T* e2,
-                                       const SpectralParams<T>& sp, int p0, const int (&ky)[2], int R, double (&acc)[5],
+                                       const SpectralParams<T>& sp, int p0, const int (&ky)[2], int R, Wide<T> (&acc)[5],
                                        Fetch fetch, Out out) {
     using V = cplx_t<T>;
     constexpr int TS = N * C, N1 = ZTile<N, C>::N1, N2 = ZTile<N, C>::N2;
@@ -732,7 +764,10 @@ __device__ __forceinline__ void z_tile(cplx_t<T>* buf, cplx_t<T>* tw, const cplx
                 const T exy = e1[kx] * e1[kyr];
                 const T exy2 = EL ? e2[kx] * e2[kyr] : T(0);
                 const T qx = raw_k<T, N>(kx, sp.two_pi_over_L), qy = raw_k<T, N>(kyr, sp.two_pi_over_L);
-                const double kxy2 = (double)qx * qx + (double)qy * qy;  // the Nyquist index counts as -n/2
+                const T kxy2 = fma_rn(qx, qx, mul_rn(qy, qy));  // the Nyquist index counts as -n/2
+                const T mxy = freq_sq<T, N>(kx) + freq_sq<T, N>(kyr);
+                // k and -k contribute the same: a paired row counts its units twice
+                const T weight = PAIRED && R == 2 ? T(2) : T(1);
                 const bool zero = kx == 0 && kyr == 0;
                 V g[N2], gz[G_ONLY ? 1 : N2];
 #pragma unroll
@@ -747,24 +782,13 @@ __device__ __forceinline__ void z_tile(cplx_t<T>* buf, cplx_t<T>* tw, const cplx
                             mul_rn(uh, fma_rn(sp.eAA, A.y, mul_rn(sp.eAB, B.y)))};
                     V wB = {mul_rn(uh, fma_rn(sp.eAB, A.x, mul_rn(sp.eBB, B.x))),
                             mul_rn(uh, fma_rn(sp.eAB, A.y, mul_rn(sp.eBB, B.y)))};
-                    if (WANT_E) {
-                        // energy sums and their |k|^2-weighted versions (d u_hat / d a = -2 a |k|^2 u_hat)
-                        const double ar = A.x, ai = A.y, br = B.x, bi = B.y;
-                        const double qz = (double)raw_k<T, N>(kz, sp.two_pi_over_L);
-                        const double k2sq = kxy2 + qz * qz;
-                        const double fchi = (double)uh * (ar * br + ai * bi);
-                        acc[0] += fchi;
-                        acc[2] += k2sq * fchi;
-                        if (!(zero && kz == 0)) {
-                            const double fkap = (double)uh * ((ar + br) * (ar + br) + (ai + bi) * (ai + bi));
-                            acc[1] += fkap;
-                            acc[3] += k2sq * fkap;
-                        }
-                    }
+                    if (WANT_E && s == 0)
+                        add_energies<T, WANT_E>(acc, A, B, uh, sp.e_rho, weight, zero && kz == 0,
+                                                mxy + freq_sq<T, N>(kz));
                     if (EL) {
                         // w_K += q_K c(k) rho~_q with rho~_q = q_A rho~_A + q_B rho~_B
                         const T qzv = raw_k<T, N>(kz, sp.two_pi_over_L);
-                        const T k2sq = fma_rn(qzv, qzv, (T)kxy2);
+                        const T k2sq = fma_rn(qzv, qzv, kxy2);
                         const T gq = k2sq > T(0) ? exy2 * e2[kz] * recip(k2sq) : T(0);
                         const V rq = {fma_rn(sp.qA, A.x, mul_rn(sp.qB, B.x)), fma_rn(sp.qA, A.y, mul_rn(sp.qB, B.y))};
                         const T cA = mul_rn(sp.el_scale * gq, sp.qA), cB2 = mul_rn(sp.el_scale * gq, sp.qB);
@@ -772,7 +796,12 @@ __device__ __forceinline__ void z_tile(cplx_t<T>* buf, cplx_t<T>* tw, const cplx
                         wA.y = fma_rn(cA, rq.y, wA.y);
                         wB.x = fma_rn(cB2, rq.x, wB.x);
                         wB.y = fma_rn(cB2, rq.y, wB.y);
-                        if (WANT_E) acc[4] += (double)gq * ((double)rq.x * rq.x + (double)rq.y * rq.y);
+                        if (WANT_E && s == 0) {
+                            Wide<T> f;
+                            f.add_prod(rq.x * sp.e_rho, rq.x * sp.e_rho);
+                            f.add_prod(rq.y * sp.e_rho, rq.y * sp.e_rho);
+                            acc[4].add(f.times(weight * gq));
+                        }
                     }
                     g[k2] = {-(wA.y + wB.x), wA.x - wB.y};  // i (w~_A + i w~_B); k_x, k_y follow in the xy pass
                     if (!G_ONLY) gz[k2] = c_scale_rn(g[k2], grad_k<T, N>(kz, sp.two_pi_over_L));
@@ -821,10 +850,10 @@ template <typename T> struct ZArgs {
     cplx_t<T>* H;
     const cplx_t<T>* tw;
     SpectralParams<T> sp;
-    double* energy_partials;
+    typename Wide<T>::stored* energy_partials;
 };
 
-template <typename T, int N, int C, bool G_ONLY = false, bool EL = false, bool WANT_E = false>
+template <typename T, int N, int C, bool G_ONLY = false, bool EL = false, int WANT_E = 0>
 __device__ __forceinline__ void z_spectral_body(const ZArgs<T>& args, int bx, int by, int gdx) {
     using V = cplx_t<T>;
     const cplx_t<T>* __restrict__ Zxy = args.Zxy;
@@ -840,7 +869,7 @@ __device__ __forceinline__ void z_spectral_body(const ZArgs<T>& args, int bx, in
     const int ky[2] = {by, by == 0 ? 0 : N - by};
     const int R = (ky[0] == ky[1]) ? 1 : 2;
     const size_t NN = (size_t)N * N, M = NN * N;
-    double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    Wide<T> acc[5];
     z_tile<T, N, C, G_ONLY, EL, WANT_E>(
         buf, tw, args.tw, e1, e2, sp, p0, ky, R, acc,
         [&](int r, int z, int c) { return Zxy[z * NN + (size_t)ky[r] * N + p0 + c]; },
@@ -849,23 +878,9 @@ __device__ __forceinline__ void z_spectral_body(const ZArgs<T>& args, int bx, in
             const int f = b < R ? 0 : 2, r = b < R ? b : b - R;
             H[f * M + z * NN + (size_t)ky[r] * N + p0 + c] = v;
         });
-    if (WANT_E) {
-        // block reduction in a fixed order (deterministic)
-        __shared__ double red[5][8];
-        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-        for (int k = 0; k < 5; ++k) {
-            double v = acc[k];
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-            if (lane == 0) red[k][wid] = v;
-        }
-        __syncthreads();
-        if (threadIdx.x < 5) {
-            double sum = 0;
-            for (int w = 0; w < (int)(blockDim.x + 31) / 32; ++w) sum += red[threadIdx.x][w];
-            const size_t b = (size_t)by * gdx + bx;
-            args.energy_partials[5 * b + threadIdx.x] = sum;
-        }
+    if constexpr (WANT_E != 0) {
+        const size_t b = (size_t)by * gdx + bx;
+        block_sum<5, T>(acc, [&](int k, const Wide<T>& v) { args.energy_partials[5 * b + k] = v.store(); });
     }
 }
 
@@ -905,15 +920,16 @@ __global__ void __launch_bounds__(256) z_spectrum(const cplx_t<T>* __restrict__ 
 
 // G_ONLY: write G alone (the potentials' path of the analytic force).
 // EL: add the smeared-charge Coulomb term (charges on).
-// WANT_E: the energy sums as well (an instantiation of its own, so that the
-// step's kernel carries none of their code or registers).
+// WANT_E: the energy sums as well (2: and their |k|^2-weighted versions), an
+// instantiation of its own, so that the step's kernel carries none of their
+// code or registers.
 template <typename T, int N, int C> __host__ __device__ constexpr int z_ctas() {
     return sizeof(T) == 8 ? 1 : N == 256 ? (C <= 8 ? 2 : 1) : C <= 8 ? 4 : 3;
 }
-template <typename T, int N, int C, bool G_ONLY = false, bool EL = false, bool WANT_E = false>
+template <typename T, int N, int C, bool G_ONLY = false, bool EL = false, int WANT_E = 0>
 __global__ void __launch_bounds__(256, z_ctas<T, N, C>()) z_spectral(const cplx_t<T>* __restrict__ Zxy, cplx_t<T>* __restrict__ H,
                                                   const cplx_t<T>* __restrict__ tw_g, SpectralParams<T> sp,
-                                                  double* __restrict__ energy_partials) {
+                                                  typename Wide<T>::stored* __restrict__ energy_partials) {
     z_spectral_body<T, N, C, G_ONLY, EL, WANT_E>(ZArgs<T>{Zxy, H, tw_g, sp, energy_partials}, blockIdx.x, blockIdx.y,
                                                  gridDim.x);
 }
@@ -932,11 +948,38 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 1) z_spectral_batche
 // rho~_2p+1 = -i (Z_p(k) - conj Z_p(-k))/2; w~_K = u_hat sum_K' eps_KK'
 // rho~_K'; Q_p = w~_2p + i w~_2p+1. Energy partials: [0] sum_k u_hat
 // sum_{K<K'} chi_KK' Re[conj(rho~_K) rho~_K'], [1] sum_{k != 0} u_hat
-// |sum_K rho~_K|^2, [2], [3] the same weighted by |k|^2, [4] 0.
+// |sum_K rho~_K|^2, the others 0 (rho~ times e_rho).
 // --------------------------------------------------------------------------
+template <typename T, int NP, class V>
+__device__ __forceinline__ void add_energies4(Wide<T> (&acc)[5], const V (&A)[2 * NP], const SpectralParams<T>& sp, T uh, bool zero) {
+    V S[2 * NP];
+#pragma unroll
+    for (int K = 0; K < 2 * NP; ++K) S[K] = {A[K].x * sp.e_rho, A[K].y * sp.e_rho};
+    Wide<T> fchi, tr, ti;
+#pragma unroll
+    for (int K = 0; K < 2 * NP; ++K) {
+#pragma unroll
+        for (int K2 = K + 1; K2 < 2 * NP; ++K2) {
+            Wide<T> f;
+            f.add_prod(S[K].x, S[K2].x);
+            f.add_prod(S[K].y, S[K2].y);
+            fchi.add(f.times(sp.chi4[K][K2]));
+        }
+        tr.add(S[K].x);
+        ti.add(S[K].y);
+    }
+    acc[0].add(fchi.times(uh));
+    if (!zero) {
+        Wide<T> q;
+        add_square(q, tr);
+        add_square(q, ti);
+        acc[1].add(q.times(uh));
+    }
+}
+
 template <typename T, int N, int C, int R, bool G_ONLY>
 __device__ __forceinline__ void z_tile_pairs(cplx_t<T>* buf, const cplx_t<T>* tw, const T* e1, const SpectralParams<T>& sp,
-                                             int p0, const int (&ky)[2], bool want_e, double (&acc)[5]) {
+                                             int p0, const int (&ky)[2], bool want_e, Wide<T> (&acc)[5]) {
     using V = cplx_t<T>;
     constexpr int TS = N * C;
     constexpr int NP = 2;
@@ -948,9 +991,6 @@ __device__ __forceinline__ void z_tile_pairs(cplx_t<T>* buf, const cplx_t<T>* tw
     const int kxA = kx_of_pos<N>(p0 + c), kxB = kx_of_pos<N>(p0 + cB);
     const T exyA = e1[kxA] * e1[ky[0]], exyB = e1[kxB] * e1[ky[rB]];
     const bool zeroA = (kxA == 0 && ky[0] == 0), zeroB = (kxB == 0 && ky[rB] == 0);
-    const T qxA = raw_k<T, N>(kxA, sp.two_pi_over_L), qyA = raw_k<T, N>(ky[0], sp.two_pi_over_L);
-    const T qxB = raw_k<T, N>(kxB, sp.two_pi_over_L), qyB = raw_k<T, N>(ky[rB], sp.two_pi_over_L);
-    const double kxy2A = (double)qxA * qxA + (double)qyA * qyA, kxy2B = (double)qxB * qxB + (double)qyB * qyB;
     for (int kz = threadIdx.x / C; kz < N; kz += 256 / C) {
         const int kzB = kz == 0 ? 0 : N - kz;
         if (R == 1 && kzB * C + cB < kz * C + c) continue;  // the mirror element owns this pair
@@ -977,28 +1017,7 @@ __device__ __forceinline__ void z_tile_pairs(cplx_t<T>* buf, const cplx_t<T>* tw
                 A[2 * q + 1] = {T(0.5) * (Z.y + Zm.y), -T(0.5) * (Z.x - Zm.x)};
             }
             if (want_e) {
-                const double qz = (double)raw_k<T, N>(kzi, sp.two_pi_over_L);
-                const double k2 = (s == 0 ? kxy2A : kxy2B) + qz * qz;
-                double fchi = 0.0;
-#pragma unroll
-                for (int K = 0; K < 2 * NP; ++K)
-#pragma unroll
-                    for (int K2 = K + 1; K2 < 2 * NP; ++K2)
-                        fchi += (double)sp.chi4[K][K2] * ((double)A[K].x * A[K2].x + (double)A[K].y * A[K2].y);
-                fchi *= (double)uh;
-                acc[0] += fchi;
-                acc[2] += k2 * fchi;
-                if (!((s == 0 ? zeroA : zeroB) && kzi == 0)) {
-                    double tr = 0.0, ti = 0.0;
-#pragma unroll
-                    for (int K = 0; K < 2 * NP; ++K) {
-                        tr += A[K].x;
-                        ti += A[K].y;
-                    }
-                    const double fkap = (double)uh * (tr * tr + ti * ti);
-                    acc[1] += fkap;
-                    acc[3] += k2 * fkap;
-                }
+                add_energies4<T, NP>(acc, A, sp, uh, (s == 0 ? zeroA : zeroB) && kzi == 0);
             }
             V w[2 * NP];
 #pragma unroll
@@ -1037,14 +1056,13 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 1) z_spectral_pairs(
                                                                                 cplx_t<T>* __restrict__ H,
                                                                                 const cplx_t<T>* __restrict__ tw_g,
                                                                                 SpectralParams<T> sp,
-                                                                                double* __restrict__ energy_partials) {
+                                                                                typename Wide<T>::stored* __restrict__ energy_partials) {
     using V = cplx_t<T>;
     constexpr int NP = 2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V* tw = reinterpret_cast<V*>(smem_raw);
     V* buf = tw + N;
     constexpr int TS = N * C;
-    __shared__ double red[5][8];
     __shared__ T e1[N];
     load_twiddles(tw, tw_g, N);
     for (int i = threadIdx.x; i < N; i += blockDim.x) e1[i] = sp.kernel1d[i];
@@ -1066,26 +1084,15 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 1) z_spectral_pairs(
     else
         batched_load<NP * 2 * TS, 256, V>(zsrc, zdst);
     __syncthreads();
-    double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    Wide<T> acc[5];
     const bool want_e = energy_partials != nullptr;
     if (R == 1)
         z_tile_pairs<T, N, C, 1, G_ONLY>(buf, tw, e1, sp, p0, ky, want_e, acc);
     else
         z_tile_pairs<T, N, C, 2, G_ONLY>(buf, tw, e1, sp, p0, ky, want_e, acc);
     if (want_e) {
-        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-        for (int k = 0; k < 5; ++k) {
-            double v = acc[k];
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-            if (lane == 0) red[k][wid] = v;
-        }
-        __syncthreads();
-        if (threadIdx.x < 5) {
-            double sum = 0;
-            for (int w = 0; w < (int)(blockDim.x + 31) / 32; ++w) sum += red[threadIdx.x][w];
-            energy_partials[5 * ((size_t)by * gridDim.x + bx) + threadIdx.x] = sum;
-        }
+        const size_t b = (size_t)by * gridDim.x + bx;
+        block_sum<5, T>(acc, [&](int k, const Wide<T>& v) { energy_partials[5 * b + k] = v.store(); });
     }
     // buffer b = (d NP + q) R + r: field 0 (G) or 2 (G_z) of pair q, row r
     const int nbuf = (G_ONLY ? 1 : 2) * NP * R * TS;

@@ -353,33 +353,44 @@ template <typename T> class Engine final : public EngineBase {
         while ((1ull << lg) < (unsigned long long)cfg_->n_beads) ++lg;
         return std::min(AdjointFixed<T>::s_max, 62 - lg);
     }
-    // the fixed-point spread [3][M] int64 pairs and the max|lam| bits
+    // the fixed-point spread [3][M] int64 pairs and the max|lam| bits, zero
+    // between calls (the xy pass and the z pass of a VJP leave them so)
     size_t vjp_fx_need() const { return 6 * M_ * sizeof(unsigned long long) + 16; }
     tild_status vjp_prepare() {
         tild_status st;
         if ((st = vjp_supported())) return st;
-        return device_buffer(&vjp_fx_, vjp_fx_bytes_, vjp_fx_need());
+        if (vjp_fx_bytes_ >= vjp_fx_need()) return TILD_OK;
+        if ((st = device_buffer(&vjp_fx_, vjp_fx_bytes_, vjp_fx_need()))) return st;
+        TILD_CUDA(cudaMemsetAsync(vjp_fx_, 0, vjp_fx_need(), stream_));
+        return TILD_OK;
     }
 
-    // J^T lam at the current positions into out_d (T, by id), and the
-    // parameter sums added to theta_acc (device, 3 doubles); stream-ordered,
-    // no host synchronisation (see vjp_kernels.cuh).
-    // fields_ready: D w (grad_ fields 0..2) and Zxy of the current positions
-    // are already in place, as a step starting from them leaves them.
-    tild_status vjp_core(const T* lam_d, T* out_d, double* theta_acc, bool fields_ready = false) {
+    // J^T lam at the positions of bf into out_d (T, by id), and the parameter
+    // sums added to theta_acc (device, 3 doubles); stream-ordered, no host
+    // synchronisation (see vjp_kernels.cuh). fields, zxy: D w and the
+    // xy-transformed density of those positions, as a step starting from them
+    // leaves them (null: computed here, for the context's own positions).
+    tild_status vjp_core(const T* lam_d, T* out_d, double* theta_acc, const BeadBuffers<T>& bf, const V* fields = nullptr,
+                         const V* zxy = nullptr) {
         const size_t N = cfg_->n_beads;
         tild_status st;
-        if (!fields_ready && (st = enqueue_fields(0, nullptr, nullptr, kInvGrad))) return st;  // D w at r; Zxy = xy(rho)
+        if (!fields) {
+            if ((st = enqueue_fields(0, nullptr, nullptr, kInvGrad))) return st;  // D w at r; Zxy = xy(rho)
+            fields = grad_;
+            zxy = Zxy_;
+        }
         using Bits = typename AdjointFixed<T>::bits_t;
         unsigned long long* fx = (unsigned long long*)vjp_fx_;
         Bits* bits = (Bits*)(fx + 6 * M_);
         const int S = vjp_fixed_bits();
-        TILD_CUDA(cudaMemsetAsync(fx, 0, vjp_fx_need(), stream_));
         lam_absmax<T><<<(int)std::min<size_t>(blocks(3 * N), 2 * 152), 256, 0, stream_>>>(3 * N, lam_d, bits);
         const BeadParams<T> p = bead_params();
-        const BeadBuffers<T> bf = bead_buffers();
         if ((st = dispatch_p([&](auto pp) -> tild_status {
-                 vjp_spread<decltype(pp)::value, T><<<blocks(N), 256, 0, stream_>>>(p, bf, lam_d, fx, bits, S);
+                 constexpr int P = decltype(pp)::value;
+                 if constexpr (sizeof(T) == 4)
+                     vjp_spread_tiled<P><<<n_tiles_, 256, vjp_spread_smem<P>(), stream_>>>(p, bf, lam_d, fx, bits, S);
+                 else
+                     vjp_spread<P, T><<<blocks(N), 256, 0, stream_>>>(p, bf, lam_d, fx, bits, S);
                  return TILD_OK;
              })))
             return st;
@@ -389,8 +400,8 @@ template <typename T> class Engine final : public EngineBase {
                  constexpr int NN = decltype(nn)::value;
                  if constexpr (plane_fits(NN, sizeof(V))) {
                      constexpr int CV = vjp_cols(NN);
-                     xy_forward_cplx<T, NN><<<dim3(NN, 3), 512, plane_smem(), stream_>>>((const longlong2*)fx, bits, S, H_, tw_);
-                     z_vjp<T, NN, CV><<<dim3(NN / CV, NN / 2 + 1), 256, vjp_smem(), stream_>>>(H_, Zxy_, tw_, sp, partials_, el);
+                     xy_forward_cplx<T, NN><<<dim3(NN, 3), 512, plane_smem(), stream_>>>((longlong2*)fx, bits, S, H_, tw_);
+                     z_vjp<T, NN, CV><<<dim3(NN / CV, NN / 2 + 1), 256, vjp_smem(), stream_>>>(H_, zxy, tw_, sp, partials_, el, bits);
                  }
                  return TILD_OK;
              })))
@@ -399,8 +410,13 @@ template <typename T> class Engine final : public EngineBase {
         accumulate_partials<<<1, 256, 0, stream_>>>(partials_, (int)vjp_blocks(), theta_acc);
         if ((st = enqueue_inverse(kInvPot))) return st;  // psi into the potential slot
         const double dV = cfg_->L * cfg_->L * cfg_->L / (double)M_;
+        const V* psi = grad_ + 3 * M_;
         if ((st = dispatch_p([&](auto pp) -> tild_status {
-                 vjp_beads<decltype(pp)::value, T><<<blocks(N), 256, 0, stream_>>>(p, bf, grad_, lam_d, (T)(1.0 / dV), out_d);
+                 constexpr int P = decltype(pp)::value;
+                 if constexpr (sizeof(T) == 4)
+                     vjp_beads_tiled<P><<<n_tiles_, 256, vjp_beads_smem<P>(), stream_>>>(p, bf, fields, psi, lam_d, (T)(1.0 / dV), out_d);
+                 else
+                     vjp_beads<P, T><<<blocks(N), 256, 0, stream_>>>(p, bf, fields, psi, lam_d, (T)(1.0 / dV), out_d);
                  return TILD_OK;
              })))
             return st;
@@ -431,20 +447,27 @@ template <typename T> class Engine final : public EngineBase {
     tild_status force_vjp(const void* lam, void* out, int dtype, int where, double* dtheta) override {
         tild_status st;
         if ((st = vjp_prepare())) return st;
-        const size_t N = cfg_->n_beads;
-        const void* src = lam;
-        if ((st = stage_in(&src, lam, 3 * N, dtype, where))) return st;
-        if ((st = ensure_aux(6 * N * sizeof(T)))) return st;
-        T* lam_d = (T*)aux_;
-        T* out_d = lam_d + 3 * N;
-        if (dtype == TILD_DTYPE_F32)
-            convert_copy<float, T><<<blocks(3 * N), 256, 0, stream_>>>(3 * N, (const float*)src, lam_d);
-        else
-            convert_copy<double, T><<<blocks(3 * N), 256, 0, stream_>>>(3 * N, (const double*)src, lam_d);
-        TILD_CUDA(cudaGetLastError());
+        const size_t N = cfg_->n_beads, bytes = 3 * N * sizeof(T);
+        const bool direct = device_native(dtype, where);  // the kernels read and write the caller's arrays
+        const bool overlap = (const char*)lam < (const char*)out + bytes && (const char*)out < (const char*)lam + bytes;
+        T* out_d = (T*)out;
+        const T* lam_d = (const T*)lam;
+        if (!direct || overlap) {
+            const void* src = lam;
+            if ((st = stage_in(&src, lam, 3 * N, dtype, where))) return st;
+            if ((st = ensure_aux(2 * bytes))) return st;
+            T* copy = (T*)aux_;
+            if (dtype == TILD_DTYPE_F32)
+                convert_copy<float, T><<<blocks(3 * N), 256, 0, stream_>>>(3 * N, (const float*)src, copy);
+            else
+                convert_copy<double, T><<<blocks(3 * N), 256, 0, stream_>>>(3 * N, (const double*)src, copy);
+            TILD_CUDA(cudaGetLastError());
+            lam_d = copy;
+            if (!direct) out_d = copy + 3 * N;
+        }
         TILD_CUDA(cudaMemsetAsync(sums(), 0, 3 * sizeof(double), stream_));
-        if ((st = vjp_core(lam_d, out_d, sums()))) return st;
-        if ((st = stage_out_vec(out_d, 3 * N, out, dtype, where))) return st;
+        if ((st = vjp_core(lam_d, out_d, sums(), bead_buffers()))) return st;
+        if (!direct && (st = stage_out_vec(out_d, 3 * N, out, dtype, where))) return st;
         if ((st = finish())) return st;
         if (dtheta) theta_from_sums(host_sums(), dtheta);
         return TILD_OK;
@@ -459,16 +482,24 @@ template <typename T> class Engine final : public EngineBase {
         }
         tild_status st;
         const size_t N = cfg_->n_beads, G = (size_t)cfg_->n_species * M_;
-        const void* src = psi;
-        if ((st = stage_in(&src, psi, G, dtype, where))) return st;
-        if ((st = ensure_aux((G + 3 * N) * sizeof(T)))) return st;
-        T* psi_d = (T*)aux_;
-        T* out_d = psi_d + G;
-        if (dtype == TILD_DTYPE_F32)
-            convert_copy<float, T><<<blocks(G), 256, 0, stream_>>>(G, (const float*)src, psi_d);
-        else
-            convert_copy<double, T><<<blocks(G), 256, 0, stream_>>>(G, (const double*)src, psi_d);
-        TILD_CUDA(cudaGetLastError());
+        const bool direct = device_native(dtype, where);
+        const bool overlap = (const char*)psi < (const char*)out + 3 * N * sizeof(T) &&
+                             (const char*)out < (const char*)psi + G * sizeof(T);
+        const T* psi_d = (const T*)psi;
+        T* out_d = (T*)out;
+        if (!direct || overlap) {
+            const void* src = psi;
+            if ((st = stage_in(&src, psi, G, dtype, where))) return st;
+            if ((st = ensure_aux((G + 3 * N) * sizeof(T)))) return st;
+            T* copy = (T*)aux_;
+            if (dtype == TILD_DTYPE_F32)
+                convert_copy<float, T><<<blocks(G), 256, 0, stream_>>>(G, (const float*)src, copy);
+            else
+                convert_copy<double, T><<<blocks(G), 256, 0, stream_>>>(G, (const double*)src, copy);
+            TILD_CUDA(cudaGetLastError());
+            psi_d = copy;
+            if (!direct) out_d = copy + G;
+        }
         const BeadParams<T> p = bead_params();
         const BeadBuffers<T> bf = bead_buffers();
         const T inv_dV = (T)((double)M_ / volume());
@@ -478,7 +509,7 @@ template <typename T> class Engine final : public EngineBase {
              })))
             return st;
         TILD_CUDA(cudaGetLastError());
-        if ((st = stage_out_vec(out_d, 3 * N, out, dtype, where))) return st;
+        if (!direct && (st = stage_out_vec(out_d, 3 * N, out, dtype, where))) return st;
         return finish();
     }
 
@@ -506,58 +537,85 @@ template <typename T> class Engine final : public EngineBase {
     }
 
     // A binned snapshot of the current positions, what the force VJP reads:
-    // positions in slot order, slot tags, neighbour slots, tile starts and the
-    // fixed-point density of those positions (after a step it holds the
-    // spread of the new positions). Restoring one needs no re-binning.
+    // positions in slot order, slot tags, neighbour slots (with beads of more
+    // than two bonds, their lists as well) and tile starts. The VJP reads it in
+    // place. The fields a step computed from those positions (D w, grad_
+    // fields 0..2, and the xy-transformed density Zxy) follow it.
     static size_t snap_part(size_t b) { return (b + 255) / 256 * 256; }
-    // (with beads of more than two bonds, their neighbour slots as well)
-    void snapshot_parts(void* (&ptr)[6], size_t (&bytes)[6]) {
+    static constexpr int kSnapParts = 5;
+    void snapshot_parts(const void* (&ptr)[kSnapParts], size_t (&bytes)[kSnapParts]) const {
         const size_t N = cfg_->n_beads;
-        void* p[6] = {pos_[cur_pos_], id_[cur_id_], nbr_, tile_start_, rho_fx_, ext_slots_};
-        const size_t b[6] = {3 * N * sizeof(T), N * sizeof(int), N * sizeof(int2), (n_tiles_ + 1) * sizeof(int),
-                             2 * M_ * sizeof(unsigned long long), n_ext_ * sizeof(int)};
-        for (int k = 0; k < 6; ++k) {
+        const void* p[kSnapParts] = {pos_[cur_pos_], id_[cur_id_], nbr_, tile_start_, ext_slots_};
+        const size_t b[kSnapParts] = {3 * N * sizeof(T), N * sizeof(int), N * sizeof(int2), (n_tiles_ + 1) * sizeof(int),
+                                      n_ext_ * sizeof(int)};
+        for (int k = 0; k < kSnapParts; ++k) {
             ptr[k] = p[k];
             bytes[k] = b[k];
         }
     }
-    size_t snapshot_bytes() {
-        void* p[6];
-        size_t b[6], total = 0;
+    size_t snapshot_bytes() const {
+        const void* p[kSnapParts];
+        size_t b[kSnapParts], total = 0;
         snapshot_parts(p, b);
-        for (int k = 0; k < 6; ++k) total += snap_part(b[k]);
+        for (int k = 0; k < kSnapParts; ++k) total += snap_part(b[k]);
         return total;
     }
-    tild_status snapshot(unsigned char* s, bool store) {
-        void* p[6];
-        size_t b[6];
-        snapshot_parts(p, b);
-        for (int k = 0; k < 6; ++k) {
-            if (b[k] == 0) continue;
-            if (store)
-                TILD_CUDA(cudaMemcpyAsync(s, p[k], b[k], cudaMemcpyDeviceToDevice, stream_));
-            else
-                TILD_CUDA(cudaMemcpyAsync(p[k], s, b[k], cudaMemcpyDeviceToDevice, stream_));
-            s += snap_part(b[k]);
+    size_t field_snapshot_bytes() const { return snap_part(3 * M_ * sizeof(V)) + snap_part(M_ * sizeof(V)); }
+    // the bead state into s and the fields into f (either may be null), one launch
+    tild_status snapshot(unsigned char* s, unsigned char* f) {
+        CopyList c = {};
+        int n = 0;
+        size_t most = 0;
+        cudaError_t ce = cudaSuccess;
+        auto add = [&](const void* src, void* dst, size_t bytes) {
+            if (bytes == 0) return;
+            if (((uintptr_t)src | (uintptr_t)dst) & 15) {  // a caller's allocator may align to less
+                ce = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToDevice, stream_);
+                return;
+            }
+            c.src[n] = src;
+            c.dst[n] = dst;
+            c.bytes[n++] = bytes;
+            most = std::max(most, bytes);
+        };
+        if (s) {
+            const void* p[kSnapParts];
+            size_t b[kSnapParts];
+            snapshot_parts(p, b);
+            for (int k = 0; k < kSnapParts; ++k) {
+                add(p[k], s, b[k]);
+                s += snap_part(b[k]);
+            }
         }
+        if (f) {
+            add(grad_, f, 3 * M_ * sizeof(V));
+            add(Zxy_, f + snap_part(3 * M_ * sizeof(V)), M_ * sizeof(V));
+        }
+        TILD_CUDA(ce);
+        const unsigned grid = (unsigned)std::min<size_t>(304, (most / 16 + 1023) / 1024 + 1);
+        if (n) copy_list<<<dim3(grid, n), 256, 0, stream_>>>(c);
+        TILD_CUDA(cudaGetLastError());
         return TILD_OK;
     }
-
-    // The fields a step computes from its starting positions (D w, grad_
-    // fields 0..2, and the xy-transformed density Zxy), what the force VJP at
-    // those positions recomputes otherwise.
-    size_t field_snapshot_bytes() const { return snap_part(3 * M_ * sizeof(V)) + snap_part(M_ * sizeof(V)); }
-    tild_status field_snapshot(unsigned char* s, bool store) {
-        const size_t b0 = 3 * M_ * sizeof(V), b1 = M_ * sizeof(V);
-        unsigned char* s1 = s + snap_part(b0);
-        if (store) {
-            TILD_CUDA(cudaMemcpyAsync(s, grad_, b0, cudaMemcpyDeviceToDevice, stream_));
-            TILD_CUDA(cudaMemcpyAsync(s1, Zxy_, b1, cudaMemcpyDeviceToDevice, stream_));
-        } else {
-            TILD_CUDA(cudaMemcpyAsync(grad_, s, b0, cudaMemcpyDeviceToDevice, stream_));
-            TILD_CUDA(cudaMemcpyAsync(Zxy_, s1, b1, cudaMemcpyDeviceToDevice, stream_));
+    // the context's bead buffers with the snapshot's positions and topology
+    BeadBuffers<T> snapshot_buffers(const unsigned char* s) const {
+        const void* p[kSnapParts];
+        size_t b[kSnapParts];
+        snapshot_parts(p, b);
+        const unsigned char* at[kSnapParts];
+        for (int k = 0; k < kSnapParts; ++k) {
+            at[k] = s;
+            s += snap_part(b[k]);
         }
-        return TILD_OK;
+        BeadBuffers<T> bf = bead_buffers();
+        bf.px = (const T*)at[0];
+        bf.py = bf.px + cfg_->n_beads;
+        bf.pz = bf.py + cfg_->n_beads;
+        bf.id = (const int*)at[1];
+        bf.nbr = (const int2*)at[2];
+        bf.tile_start = (const int*)at[3];
+        bf.ext = n_ext_ ? (const int*)at[4] : nullptr;
+        return bf;
     }
 
     // Reverse-mode derivatives of L(r^K, v^K) through K steps of the context's
@@ -618,24 +676,30 @@ template <typename T> class Engine final : public EngineBase {
             if ((st = restore_state(ckpt + sb * (s0 / C), step0 + s0))) return st;
             for (int64_t j = s0; j < s1; ++j) {
                 if ((st = step(1))) return st;
-                // step j started from r^j: its fields belong to state j (snapshot j - 1 - s0)
-                if (j > s0 && (st = field_snapshot(seg + snap * (size_t)(j - 1 - s0) + bsnap, true))) return st;
-                if ((st = snapshot(seg + snap * (size_t)(j - s0), true))) return st;
+                // step j started from r^j: its fields belong to state j (snapshot j - 1 - s0);
+                // the last state of the segment stays in the context
+                unsigned char* fields = j > s0 ? seg + snap * (size_t)(j - 1 - s0) + bsnap : nullptr;
+                unsigned char* beads = j + 1 < s1 ? seg + snap * (size_t)(j - s0) : nullptr;
+                if ((fields || beads) && (st = snapshot(beads, fields))) return st;
             }
             for (int64_t j = s1 - 1; j >= s0; --j) {
-                // r^{j+1}, binned as the recomputation left it, with its fields
-                // when step j+1 was recomputed
-                const bool fields = j + 1 < s1;
-                if ((st = snapshot(seg + snap * (size_t)(j - s0), false))) return st;
-                if (fields && (st = field_snapshot(seg + snap * (size_t)(j - s0) + bsnap, false))) return st;
-                if ((st = vjp_core(lam, jt, acc, fields))) return st;
+                // the VJP at r^{j+1}: the context's own state (with a field pass
+                // of its own) or the snapshot, read in place
+                const unsigned char* at = seg + snap * (size_t)(j - s0);
+                const V* fields = (const V*)(at + bsnap);
+                if (j + 1 == s1)
+                    st = vjp_core(lam, jt, acc, bead_buffers());
+                else
+                    st = vjp_core(lam, jt, acc, snapshot_buffers(at), fields,
+                                  (const V*)(at + bsnap + snap_part(3 * M_ * sizeof(V))));
+                if (st) return st;
                 adjoint_step<T><<<blocks(n3), 256, 0, stream_>>>(n3, jt, rb, ub, lam, q.sd, q.sh, q.su, q.sf, q.wf,
                                                                   j == 0 ? 1 : 0);
                 TILD_CUDA(cudaGetLastError());
             }
         }
         // the force at r^0; dL/dv^0 = wu ub
-        if ((st = restore_state(ckpt, step0)) || (st = vjp_core(lam, jt, acc))) return st;
+        if ((st = restore_state(ckpt, step0)) || (st = vjp_core(lam, jt, acc, bead_buffers()))) return st;
         add_into<T><<<blocks(n3), 256, 0, stream_>>>(n3, rb, jt, rb);
         scale_copy<double><<<blocks(n3), 256, 0, stream_>>>(n3, ub, q.wu, vout);
         TILD_CUDA(cudaGetLastError());
@@ -1360,6 +1424,10 @@ template <typename T> class Engine final : public EngineBase {
     }
 
     template <int P> tild_status attrs_p() {
+        if constexpr (sizeof(T) == 4) {
+            TILD_CUDA(cudaFuncSetAttribute(vjp_spread_tiled<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vjp_spread_smem<P>()));
+            TILD_CUDA(cudaFuncSetAttribute(vjp_beads_tiled<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vjp_beads_smem<P>()));
+        }
         const int s4 = (int)bead_smem(false, 4), sa4 = (int)bead_smem(true, 4);
         TILD_CUDA(cudaFuncSetAttribute(bead_kernel<P, kModeSpread, T, false, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, s4));
         TILD_CUDA(cudaFuncSetAttribute(bead_kernel<P, kModeForce, T, false, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, s4));

@@ -99,23 +99,12 @@ __global__ void __launch_bounds__(256) lam_absmax(size_t n, const T* __restrict_
     }
 }
 
-// mu_d += W_i lam_{i,d} in fixed point; lam by bead id ([N][3]); fx as
-// int64 pairs [3][M][2] (species A, B), zero on entry.
+// mu_d += W_i lam_{i,d} in fixed point for one bead (l: lam_i times the fixed
+// scale), straight into fx, int64 pairs [3][M][2] (species A, B).
 template <int P, typename T>
-__global__ void __launch_bounds__(256) vjp_spread(BeadParams<T> p, BeadBuffers<T> bf, const T* __restrict__ lam,
-                                                  unsigned long long* __restrict__ fx,
-                                                  const typename AdjointFixed<T>::bits_t* __restrict__ bits, int S) {
+__device__ __forceinline__ void vjp_spread_global(const Stencil<P, T>& st, const T (&l)[3], int K, int n,
+                                                  unsigned long long* __restrict__ fx) {
     using FX = AdjointFixed<T>;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= p.n_beads) return;
-    T sc, inv;
-    FX::scales(*bits, S, sc, inv);
-    const int tag = bf.id[i];
-    const int bid = slot_bead_id(tag), K = slot_species(tag);
-    const T l0 = lam[3 * (size_t)bid] * sc, l1 = lam[3 * (size_t)bid + 1] * sc, l2 = lam[3 * (size_t)bid + 2] * sc;
-    Stencil<P, T> st;
-    st.set(bf.px[i], bf.py[i], bf.pz[i], p.inv_dx);
-    const int n = p.n;
     const size_t M = (size_t)n * n * n;
 #pragma unroll
     for (int c = 0; c < P; ++c)
@@ -127,19 +116,125 @@ __global__ void __launch_bounds__(256) vjp_spread(BeadParams<T> p, BeadBuffers<T
             for (int a = 0; a < P; ++a) {
                 const size_t g = row + pwrap(st.jx + a, n);
                 const T w = st.wx[a] * wyz;
-                atomicAdd(fx + 2 * g + K, (unsigned long long)FX::to_fixed(w * l0));
-                atomicAdd(fx + 2 * (M + g) + K, (unsigned long long)FX::to_fixed(w * l1));
-                atomicAdd(fx + 2 * (2 * M + g) + K, (unsigned long long)FX::to_fixed(w * l2));
+#pragma unroll
+                for (int d = 0; d < 3; ++d)
+                    atomicAdd(fx + 2 * (d * M + g) + K, (unsigned long long)FX::to_fixed(w * l[d]));
             }
+        }
+}
+
+// One thread per bead (FP64 contexts, whose few tiles would leave most of the
+// chip's FP64 units idle); lam by bead id ([N][3]); fx zero on entry.
+template <int P, typename T>
+__global__ void __launch_bounds__(256) vjp_spread(BeadParams<T> p, BeadBuffers<T> bf, const T* __restrict__ lam,
+                                                  unsigned long long* __restrict__ fx,
+                                                  const typename AdjointFixed<T>::bits_t* __restrict__ bits, int S) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= p.n_beads) return;
+    T sc, inv;
+    AdjointFixed<T>::scales(*bits, S, sc, inv);
+    const int tag = bf.id[i];
+    const T* lp = lam + 3 * (size_t)slot_bead_id(tag);
+    const T l[3] = {lp[0] * sc, lp[1] * sc, lp[2] * sc};
+    Stencil<P, T> st;
+    st.set(bf.px[i], bf.py[i], bf.pz[i], p.inv_dx);
+    vjp_spread_global<P>(st, l, slot_species(tag), p.n, fx);
+}
+
+// Geometry of a tile's patch for the adjoint kernels: patch row -> grid offset
+// of its first point, and the tile's coordinates.
+template <int P> __device__ __forceinline__ int3 tile_patch(int t, int tiles, int n, int (&rowbase)[Patch<P>::W * Patch<P>::W]) {
+    using PT = Patch<P>;
+    const int tx = t % tiles, ty = (t / tiles) % tiles, tz = t / (tiles * tiles);
+    const int3 org = {tx * kTile + PT::lo, ty * kTile + PT::lo, tz * kTile + PT::lo};
+    for (int i = threadIdx.x; i < PT::W * PT::W; i += blockDim.x) {
+        const int lz = i / PT::W, ly = i - lz * PT::W;
+        rowbase[i] = (pwrap(org.z + lz, n) * n + pwrap(org.y + ly, n)) * n;
+    }
+    return org;
+}
+
+// The spread of lam through a shared-memory patch per tile (FP32 contexts).
+// One bead adds to 3 P^3 sums, 64-bit ones: as global atomics they run at the
+// rate of the L2 atomic units (24 scattered words per bead at P = 2, 81 at
+// P = 3). Shared memory has no 64-bit add, so each contribution, an integer
+// below 2^40 held exactly by a float, is split into hi 2^20 + lo with |lo| <=
+// 2^19, two native 32-bit adds; a tile of up to 2047 beads cannot overflow
+// them, larger tiles and beads outside their patch take the global path. The
+// patch is flushed with one 64-bit add per point, rows of both species
+// contiguous. Integer sums: the same bits as the global path.
+// One product on 200k beads, 64^3 (P = 2), this kernel and vjp_beads_tiled in
+// place of the global ones: 113 -> 71 us.
+constexpr int kVjpTileBeads = 2047;
+template <int P> constexpr size_t vjp_spread_smem() { return (size_t)12 * Patch<P>::W3 * sizeof(int); }
+template <int P>
+__global__ void __launch_bounds__(256) vjp_spread_tiled(BeadParams<float> p, BeadBuffers<float> bf,
+                                                        const float* __restrict__ lam, unsigned long long* __restrict__ fx,
+                                                        const unsigned int* __restrict__ bits, int S) {
+    using PT = Patch<P>;
+    constexpr int W = PT::W, W3 = PT::W3, ROW = 2 * W;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    int* s_hi = reinterpret_cast<int*>(smem_raw);  // [3][row][x][species]
+    int* s_lo = s_hi + 6 * W3;
+    __shared__ int rowbase[W * W];
+    const int start = bf.tile_start[blockIdx.x], end = bf.tile_start[blockIdx.x + 1];
+    if (start == end) return;
+    const int3 org = tile_patch<P>(blockIdx.x, p.tiles, p.n, rowbase);
+    for (int i = threadIdx.x; i < 12 * W3; i += blockDim.x) s_hi[i] = 0;
+    float sc, inv;
+    AdjointFixed<float>::scales(*bits, S, sc, inv);
+    const bool patch_ok = end - start <= kVjpTileBeads;
+    __syncthreads();
+    for (int i = start + threadIdx.x; i < end; i += blockDim.x) {
+        const int tag = bf.id[i];
+        const int K = slot_species(tag);
+        const float* lp = lam + 3 * (size_t)slot_bead_id(tag);
+        const float l[3] = {lp[0] * sc, lp[1] * sc, lp[2] * sc};
+        Stencil<P, float> st;
+        st.set(bf.px[i], bf.py[i], bf.pz[i], p.inv_dx);
+        int3 o;
+        if (patch_local(st, org, o) && patch_ok) {
+#pragma unroll
+            for (int c = 0; c < P; ++c)
+#pragma unroll
+                for (int b = 0; b < P; ++b) {
+                    const float wyz = st.wy[b] * st.wz[c];
+                    const int row = (((o.z + c) * W + (o.y + b)) * W + o.x) * 2 + K;
+#pragma unroll
+                    for (int a = 0; a < P; ++a) {
+                        const float w = st.wx[a] * wyz;
+#pragma unroll
+                        for (int d = 0; d < 3; ++d) {
+                            const float x = __fmul_rn(w, l[d]);
+                            const float hi = rintf(x * 9.5367431640625e-07f);   // 2^-20
+                            const float lo = __fmaf_rn(-1048576.0f, hi, x);     // exact
+                            const int at = d * 2 * W3 + row + 2 * a;
+                            atomicAdd(s_hi + at, __float2int_rn(hi));
+                            atomicAdd(s_lo + at, __float2int_rn(lo));
+                        }
+                    }
+                }
+        } else {
+            vjp_spread_global<P>(st, l, K, p.n, fx);
+        }
+    }
+    __syncthreads();
+    const size_t M = (size_t)p.n * p.n * p.n;
+    for (int d = 0; d < 3; ++d)
+        for (int i = threadIdx.x; i < W * W * ROW; i += blockDim.x) {
+            const long long v = (long long)s_hi[d * 2 * W3 + i] * 1048576ll + (long long)s_lo[d * 2 * W3 + i];
+            const int row = i / ROW, r = i - row * ROW;
+            if (v != 0)
+                atomicAdd(fx + 2 * (d * M + rowbase[row] + pwrap(org.x + (r >> 1), p.n)) + (r & 1), (unsigned long long)v);
         }
 }
 
 // Forward DFT along x and y of plane blockIdx.x of field blockIdx.y: reads
 // the fixed-point spread fx ([3][M] int64 pairs), converts it with the
 // inverse scale, and writes the complex [3][M] array `data` in mirror-paired
-// column order.
+// column order. Leaves fx zero for the next spread.
 template <typename T, int N>
-__global__ void __launch_bounds__(512) xy_forward_cplx(const longlong2* __restrict__ fx,
+__global__ void __launch_bounds__(512) xy_forward_cplx(longlong2* __restrict__ fx,
                                                        const typename AdjointFixed<T>::bits_t* __restrict__ bits, int S,
                                                        cplx_t<T>* __restrict__ data, const cplx_t<T>* __restrict__ tw_g) {
     using V = cplx_t<T>;
@@ -164,7 +259,10 @@ __global__ void __launch_bounds__(512) xy_forward_cplx(const longlong2* __restri
                 for (int k = 0; k < B; ++k) v[h + k] = V{from_fixed(a[k].x, inv), from_fixed(a[k].y, inv)};
             }
         },
-        []() {}, data + base);
+        [&]() {
+            for (int i = threadIdx.x; i < N * N; i += 512) fx[base + i] = make_longlong2(0, 0);
+        },
+        data + base);
 }
 
 // z pass of the VJP. CTA (C column positions, rows ky and -ky) as in
@@ -263,8 +361,11 @@ __device__ __forceinline__ void z_vjp_tile(cplx_t<T>* buf, const cplx_t<T>* tw, 
 template <typename T, int N, int C>
 __global__ void __launch_bounds__(256) z_vjp(cplx_t<T>* __restrict__ H, const cplx_t<T>* __restrict__ Zxy,
                                              const cplx_t<T>* __restrict__ tw_g, SpectralParams<T> sp,
-                                             double* __restrict__ partials, int el) {
+                                             double* __restrict__ partials, int el,
+                                             typename AdjointFixed<T>::bits_t* __restrict__ bits) {
     using V = cplx_t<T>;
+    // max|lam| has been read by the spread and the xy pass: 0 for the next call
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *bits = 0;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V* tw = reinterpret_cast<V*>(smem_raw);
     V* buf = tw + N;
@@ -320,26 +421,14 @@ __global__ void __launch_bounds__(256) z_vjp(cplx_t<T>* __restrict__ H, const cp
 }
 
 // Per bead: sum_g grad W_j(g) [psi_{K_j}(g)/dV - lam_j . D w_{K_j}(g)] and the
-// bond term. fields = the gradient buffer: [0..2] (d_x, d_y, d_z)(w_A, w_B),
-// [3] i (psi_A + i psi_B). lam and out by bead id ([N][3]).
+// bond term. fields: (d_x, d_y, d_z)(w_A, w_B), [3][M]; psi: i (psi_A + i psi_B).
+// lam and out by bead id ([N][3]).
 template <int P, typename T>
-__global__ void __launch_bounds__(256) vjp_beads(BeadParams<T> p, BeadBuffers<T> bf, const cplx_t<T>* __restrict__ fields,
-                                                 const T* __restrict__ lam, T inv_dV, T* __restrict__ out) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= p.n_beads) return;
-    const T x = bf.px[i], y = bf.py[i], z = bf.pz[i];
-    const int tag = bf.id[i];
-    const int bid = slot_bead_id(tag), K = slot_species(tag);
-    const T l0 = lam[3 * (size_t)bid], l1 = lam[3 * (size_t)bid + 1], l2 = lam[3 * (size_t)bid + 2];
-    Stencil<P, T> st;
-    st.set(x, y, z, p.inv_dx);
-    T dwx[P], dwy[P], dwz[P];
-    dh_weight_derivs<P>(x * p.inv_dx, dwx);
-    dh_weight_derivs<P>(y * p.inv_dx, dwy);
-    dh_weight_derivs<P>(z * p.inv_dx, dwz);
-    const int n = p.n;
+__device__ __forceinline__ void vjp_gather_global(const Stencil<P, T>& st, const T (&dwx)[P], const T (&dwy)[P],
+                                                  const T (&dwz)[P], const T (&l)[3], int K, int n,
+                                                  const cplx_t<T>* __restrict__ fields, const cplx_t<T>* __restrict__ psi,
+                                                  T inv_dV, T (&o)[3]) {
     const size_t M = (size_t)n * n * n;
-    T ox = 0, oy = 0, oz = 0;
 #pragma unroll
     for (int c = 0; c < P; ++c)
 #pragma unroll
@@ -349,38 +438,119 @@ __global__ void __launch_bounds__(256) vjp_beads(BeadParams<T> p, BeadBuffers<T>
 #pragma unroll
             for (int a = 0; a < P; ++a) {
                 const size_t g = row + pwrap(st.jx + a, n);
-                const cplx_t<T> f0 = fields[g], f1 = fields[M + g], f2 = fields[2 * M + g], f3 = fields[3 * M + g];
-                const T ldw = l0 * (K ? f0.y : f0.x) + l1 * (K ? f1.y : f1.x) + l2 * (K ? f2.y : f2.x);
-                const T psi = K ? -f3.x : f3.y;
-                const T val = psi * inv_dV - ldw;
-                ox += dwx[a] * wyz * val;
-                oy += st.wx[a] * dyz * val;
-                oz += st.wx[a] * ydz * val;
+                const cplx_t<T> f0 = fields[g], f1 = fields[M + g], f2 = fields[2 * M + g], f3 = psi[g];
+                const T ldw = l[0] * (K ? f0.y : f0.x) + l[1] * (K ? f1.y : f1.x) + l[2] * (K ? f2.y : f2.x);
+                const T val = (K ? -f3.x : f3.y) * inv_dV - ldw;
+                o[0] += dwx[a] * wyz * val;
+                o[1] += st.wx[a] * dyz * val;
+                o[2] += st.wx[a] * ydz * val;
             }
         }
-    ox *= p.inv_dx;
-    oy *= p.inv_dx;
-    oz *= p.inv_dx;
-    const int2 nb = bf.nbr[i];
+}
+
+// out = o / dx plus the bond term of bead slot i.
+template <typename T>
+__device__ __forceinline__ void vjp_bonds_store(const BeadParams<T>& p, const BeadBuffers<T>& bf, int i, int bid,
+                                                const T (&l)[3], const T* __restrict__ lam, T (&o)[3], T* __restrict__ out) {
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const int s = k == 0 ? nb.x : nb.y;
-        if (s >= 0) {
-            const int nid = slot_bead_id(bf.id[s]);
-            ox -= p.k_bond * (l0 - lam[3 * (size_t)nid]);
-            oy -= p.k_bond * (l1 - lam[3 * (size_t)nid + 1]);
-            oz -= p.k_bond * (l2 - lam[3 * (size_t)nid + 2]);
-        }
+    for (int d = 0; d < 3; ++d) o[d] *= p.inv_dx;
+    auto bond = [&](int s) {
+        const T* ln = lam + 3 * (size_t)slot_bead_id(bf.id[s]);
+#pragma unroll
+        for (int d = 0; d < 3; ++d) o[d] -= p.k_bond * (l[d] - ln[d]);
+    };
+    const int2 nb = bf.nbr[i];
+    if (nb.x >= 0) bond(nb.x);
+    if (nb.y >= 0) bond(nb.y);
+    for_each_extra_bond(nb, bf.ext, bond);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) out[3 * (size_t)bid + d] = o[d];
+}
+
+// One thread per bead, fields from global memory (FP64 contexts).
+template <int P, typename T>
+__global__ void __launch_bounds__(256) vjp_beads(BeadParams<T> p, BeadBuffers<T> bf, const cplx_t<T>* __restrict__ fields,
+                                                 const cplx_t<T>* __restrict__ psi, const T* __restrict__ lam, T inv_dV,
+                                                 T* __restrict__ out) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= p.n_beads) return;
+    const T x = bf.px[i], y = bf.py[i], z = bf.pz[i];
+    const int tag = bf.id[i];
+    const int bid = slot_bead_id(tag);
+    const T* lp = lam + 3 * (size_t)bid;
+    const T l[3] = {lp[0], lp[1], lp[2]};
+    Stencil<P, T> st;
+    st.set(x, y, z, p.inv_dx);
+    T dwx[P], dwy[P], dwz[P], o[3] = {T(0), T(0), T(0)};
+    dh_weight_derivs<P>(x * p.inv_dx, dwx);
+    dh_weight_derivs<P>(y * p.inv_dx, dwy);
+    dh_weight_derivs<P>(z * p.inv_dx, dwz);
+    vjp_gather_global<P>(st, dwx, dwy, dwz, l, slot_species(tag), p.n, fields, psi, inv_dV, o);
+    vjp_bonds_store(p, bf, i, bid, l, lam, o, out);
+}
+
+// The same with the tile's fields staged in shared memory (FP32 contexts): one
+// record (d_x w, d_y w, d_z w, psi/dV) per point and species, so a bead reads
+// one 16-byte word per point where it read four 8-byte words of global memory
+// and used half of each.
+template <int P> constexpr size_t vjp_beads_smem() { return (size_t)2 * Patch<P>::W3 * sizeof(float4); }
+template <int P>
+__global__ void __launch_bounds__(256) vjp_beads_tiled(BeadParams<float> p, BeadBuffers<float> bf,
+                                                       const float2* __restrict__ fields, const float2* __restrict__ psi,
+                                                       const float* __restrict__ lam, float inv_dV, float* __restrict__ out) {
+    using PT = Patch<P>;
+    constexpr int W = PT::W, W3 = PT::W3;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float4* rec = reinterpret_cast<float4*>(smem_raw);  // [species][W3]
+    __shared__ int rowbase[W * W];
+    const int start = bf.tile_start[blockIdx.x], end = bf.tile_start[blockIdx.x + 1];
+    if (start == end) return;
+    const int3 org = tile_patch<P>(blockIdx.x, p.tiles, p.n, rowbase);
+    const size_t M = (size_t)p.n * p.n * p.n;
+    __syncthreads();
+#pragma unroll 3
+    for (int i = threadIdx.x; i < W3; i += 256) {
+        const int row = i / W;
+        const size_t g = (size_t)rowbase[row] + pwrap(org.x + i - row * W, p.n);
+        const float2 f0 = __ldg(fields + g), f1 = __ldg(fields + M + g), f2 = __ldg(fields + 2 * M + g), f3 = __ldg(psi + g);
+        rec[i] = make_float4(f0.x, f1.x, f2.x, f3.y * inv_dV);
+        rec[W3 + i] = make_float4(f0.y, f1.y, f2.y, -f3.x * inv_dV);
     }
-    for_each_extra_bond(nb, bf.ext, [&](int s) {
-        const int nid = slot_bead_id(bf.id[s]);
-        ox -= p.k_bond * (l0 - lam[3 * (size_t)nid]);
-        oy -= p.k_bond * (l1 - lam[3 * (size_t)nid + 1]);
-        oz -= p.k_bond * (l2 - lam[3 * (size_t)nid + 2]);
-    });
-    out[3 * (size_t)bid] = ox;
-    out[3 * (size_t)bid + 1] = oy;
-    out[3 * (size_t)bid + 2] = oz;
+    __syncthreads();
+    for (int i = start + threadIdx.x; i < end; i += 256) {
+        const float x = bf.px[i], y = bf.py[i], z = bf.pz[i];
+        const int tag = bf.id[i];
+        const int bid = slot_bead_id(tag), K = slot_species(tag);
+        const float* lp = lam + 3 * (size_t)bid;
+        const float l[3] = {lp[0], lp[1], lp[2]};
+        Stencil<P, float> st;
+        st.set(x, y, z, p.inv_dx);
+        float dwx[P], dwy[P], dwz[P], o[3] = {0.f, 0.f, 0.f};
+        dh_weight_derivs<P>(x * p.inv_dx, dwx);
+        dh_weight_derivs<P>(y * p.inv_dx, dwy);
+        dh_weight_derivs<P>(z * p.inv_dx, dwz);
+        int3 q;
+        if (patch_local(st, org, q)) {
+            const float4* base = rec + K * W3 + (q.z * W + q.y) * W + q.x;
+#pragma unroll
+            for (int c = 0; c < P; ++c)
+#pragma unroll
+                for (int b = 0; b < P; ++b) {
+                    const float wyz = st.wy[b] * st.wz[c], dyz = dwy[b] * st.wz[c], ydz = st.wy[b] * dwz[c];
+#pragma unroll
+                    for (int a = 0; a < P; ++a) {
+                        const float4 f = base[(c * W + b) * W + a];
+                        const float val = f.w - (l[0] * f.x + l[1] * f.y + l[2] * f.z);
+                        o[0] += dwx[a] * wyz * val;
+                        o[1] += st.wx[a] * dyz * val;
+                        o[2] += st.wx[a] * ydz * val;
+                    }
+                }
+        } else {
+            vjp_gather_global<P>(st, dwx, dwy, dwz, l, K, p.n, fields, psi, inv_dV, o);
+        }
+        vjp_bonds_store(p, bf, i, bid, l, lam, o, out);
+    }
 }
 
 // Vector-Jacobian product of the density assignment (Eq. rhohat with the
@@ -479,6 +649,31 @@ __global__ void adjoint_step(size_t n3, const T* __restrict__ jt, double* __rest
     rb[i] = r;
     ub[i] = u;
     lam[i] = (T)(sf * hb + (at_start ? wf * u : 0.0));
+}
+
+// Up to eight device-to-device copies in one launch (blockIdx.y = copy; 16-byte
+// aligned bases, sizes in bytes, multiples of 4).
+struct CopyList {
+    const void* src[8];
+    void* dst[8];
+    size_t bytes[8];
+};
+static __global__ void __launch_bounds__(256) copy_list(CopyList c) {
+    const size_t n16 = c.bytes[blockIdx.y] / 16, stride = (size_t)gridDim.x * 256;
+    const uint4* s = (const uint4*)c.src[blockIdx.y];
+    uint4* d = (uint4*)c.dst[blockIdx.y];
+    for (size_t i0 = (size_t)blockIdx.x * 256 + threadIdx.x; i0 < n16; i0 += 4 * stride) {
+        uint4 v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (i0 + k * stride < n16) v[k] = s[i0 + k * stride];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (i0 + k * stride < n16) d[i0 + k * stride] = v[k];
+    }
+    if (blockIdx.x == 0)  // the last words
+        for (size_t i = 4 * n16 + threadIdx.x; i < c.bytes[blockIdx.y] / 4; i += 256)
+            ((unsigned*)c.dst[blockIdx.y])[i] = ((const unsigned*)c.src[blockIdx.y])[i];
 }
 
 // y = (T)(a x)

@@ -95,6 +95,14 @@ template <typename T> class Engine final : public EngineBase {
             for (int f = 1; f * f <= n_; ++f)
                 if (n_ % f == 0) gn1_ = f;
             gn2_ = n_ / gn1_;
+            TILD_CUDA(cudaFuncSetAttribute(line_x_forward<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kLineSmem));
+            TILD_CUDA(cudaFuncSetAttribute(line_x_inverse<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kLineSmem));
+            TILD_CUDA(cudaFuncSetAttribute(line_y<T, -1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kLineSmem));
+            TILD_CUDA(cudaFuncSetAttribute(line_y<T, +1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kLineSmem));
+            TILD_CUDA(cudaFuncSetAttribute(line_last<T, 1, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kLineSmem));
+            TILD_CUDA(cudaFuncSetAttribute(line_last<T, 2, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kLineSmem));
+            TILD_CUDA(cudaFuncSetAttribute(line_last<T, 1, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, kLineSmem));
+            TILD_CUDA(cudaFuncSetAttribute(line_last<T, 2, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, kLineSmem));
             return TILD_OK;
         }
         return set_kernel_attributes();
@@ -794,7 +802,10 @@ template <typename T> class Engine final : public EngineBase {
 
     int64_t host_step() const override { return host_step_; }
     // blocks of the z pass (energy partials): twice as many column tiles with two species pairs
-    size_t z_blocks() const { return NP_ == 2 ? (size_t)(n_ / zpass_cols2(n_)) * (n_ / 2 + 1) : n_z_blocks_; }
+    size_t z_blocks() const {
+        if (use_lines()) return (size_t)line_last_grid().x * line_last_grid().y;
+        return generic_ ? n_z_blocks_ : NP_ == 2 ? (size_t)(n_ / zpass_cols2(n_)) * (n_ / 2 + 1) : n_z_blocks_;
+    }
 
     // blob: magic, n_beads, sizeof(T), step, seed | pos[N][3] | u[N][3] (by id, T)
     size_t state_bytes() const override { return 5 * sizeof(uint64_t) + 6 * (size_t)cfg_->n_beads * sizeof(T); }
@@ -905,7 +916,7 @@ template <typename T> class Engine final : public EngineBase {
 
     int64_t launches(int64_t n) const override {
         const int D = cfg_->dim;
-        const int64_t per_step = generic_ ? (1 + D) + 1 + (int64_t)NP_ * D + 1 : (use_planes() ? 2 : 4) + 2;
+        const int64_t per_step = generic_ ? (use_lines() ? 2 * D : (1 + D) + 1 + (int64_t)NP_ * D + 1) : (use_planes() ? 2 : 4) + 2;
         const int64_t per_sort = 8;
         const int K = cfg_->sort_every;
         int64_t since = steps_since_sort_, sorts = 0;
@@ -1093,6 +1104,74 @@ template <typename T> class Engine final : public EngineBase {
     tild_status ensure_partials() {
         const size_t need = 5 * std::max(bead_blocks(), z_blocks()) * sizeof(double);
         return device_buffer(&partials_, partials_bytes_, need);
+    }
+    // Line passes of the any-size grids: lines per CTA (2^lg) so that the launch
+    // has about two CTAs per SM, not below `lo` (short rows of memory); shared
+    // memory within kLineSmem.
+    static constexpr int kLineSmem = 200 * 1024;
+    bool line_big() const { return std::max(gn1_, gn2_) > 16; }
+    size_t line_smem(int half) const { return ((size_t)n_ + (size_t)half * (line_big() ? 2 : 1)) * sizeof(V); }
+    // lines: of the launch at 2^lg per CTA; f(lg) = CTAs
+    template <class F> int line_lg(int hi, int lo, int per_line, F&& ctas) const {
+        int lg = hi;
+        while (lg > lo && (ctas(lg) < 304 || line_smem(per_line << lg) > (size_t)kLineSmem / 2)) --lg;
+        return lg;
+    }
+    LineArgs<T> line_args(int lg, int per_line) const {
+        return LineArgs<T>{n_, nz_, gn1_, gn2_, lg, line_big() ? per_line << lg : 0, tw_, two_pi_L()};
+    }
+    static int div_up(int a, int b) { return (a + b - 1) / b; }
+    int line_rows_lg(int fields) const {
+        return line_lg(4, 0, n_ | 1, [&](int lg) { return div_up(nz_ * n_, 1 << lg) * fields; });
+    }
+    int line_last_lg() const {  // 4 NP lines per column
+        const int c = NP_ == 2 ? 3 : 2;
+        return line_lg(c + 3, c, n_, [&](int lg) { return div_up(n_, 1 << (lg - c)) * (cfg_->dim == 3 ? n_ / 2 + 1 : 1); });
+    }
+    dim3 line_last_grid() const {
+        const int lg = line_last_lg() - (NP_ == 2 ? 3 : 2);
+        return dim3(div_up(n_, 1 << lg), cfg_->dim == 3 ? n_ / 2 + 1 : 1);
+    }
+    // whether the lines of one column fit the last pass (2D grids of a few
+    // thousand points per edge do not: whole-axis passes)
+    bool use_lines() const { return generic_ && line_smem((NP_ == 2 ? 8 : 4) * n_) <= (size_t)kLineSmem; }
+    tild_status line_forward(bool zero_after) {
+        const int lg = line_rows_lg(NP_);
+        line_x_forward<T><<<dim3(div_up(nz_ * n_, 1 << lg), NP_), 128, line_smem((n_ | 1) << lg), stream_>>>(
+            line_args(lg, n_ | 1), rho_fx_, Zxy_, density_scale(), zero_after ? 1 : 0, zero_after ? counters_ : nullptr);
+        if (cfg_->dim == 3) {
+            const int ly = line_lg(4, 2, n_, [&](int l) { return div_up(n_, 1 << l) * nz_ * NP_; });
+            line_y<T, -1><<<dim3(div_up(n_, 1 << ly), nz_, NP_), 128, line_smem(n_ << ly), stream_>>>(line_args(ly, n_), Zxy_);
+        }
+        TILD_CUDA(cudaGetLastError());
+        return TILD_OK;
+    }
+    tild_status line_spectral(typename Wide<T>::stored* partials) {
+        const int lg = line_last_lg();
+        const SpectralParams<T> sp = spectral_params();
+        const LineArgs<T> a = line_args(lg, n_);
+        const size_t sm = line_smem(n_ << lg);
+        if (cfg_->dim == 3) {
+            if (NP_ == 2) line_last<T, 2, 3><<<line_last_grid(), 128, sm, stream_>>>(a, Zxy_, H_, sp, partials);
+            else line_last<T, 1, 3><<<line_last_grid(), 128, sm, stream_>>>(a, Zxy_, H_, sp, partials);
+        } else {
+            if (NP_ == 2) line_last<T, 2, 2><<<line_last_grid(), 128, sm, stream_>>>(a, Zxy_, H_, sp, partials);
+            else line_last<T, 1, 2><<<line_last_grid(), 128, sm, stream_>>>(a, Zxy_, H_, sp, partials);
+        }
+        TILD_CUDA(cudaGetLastError());
+        return TILD_OK;
+    }
+    tild_status line_inverse() {
+        const int D = cfg_->dim;
+        if (D == 3) {
+            const int ly = line_lg(5, 3, n_, [&](int l) { return div_up(n_, 1 << (l - 1)) * nz_ * NP_; });
+            line_y<T, +1><<<dim3(div_up(n_, 1 << (ly - 1)), nz_, 2 * NP_), 128, line_smem(n_ << ly), stream_>>>(line_args(ly, n_), H_);
+        }
+        const int lg = line_rows_lg(D * NP_);
+        line_x_inverse<T><<<dim3(div_up(nz_ * n_, 1 << lg), D * NP_), 128, line_smem((n_ | 1) << lg), stream_>>>(
+            line_args(lg, n_ | 1), H_, grad_, D);
+        TILD_CUDA(cudaGetLastError());
+        return TILD_OK;
     }
     // the any-size transforms of `count` contiguous fields at f along every axis
     tild_status generic_fft(V* f, int count, int dir) {
@@ -1514,7 +1593,9 @@ template <typename T> class Engine final : public EngineBase {
         TILD_CUDA(cudaGetLastError());
         return TILD_OK;
     }
-    tild_status enqueue_forward(bool zero_after) {
+    // whole: any-size grids by whole-axis passes (natural order; the spectrum read-out)
+    tild_status enqueue_forward(bool zero_after, bool whole = false) {
+        if (use_lines() && !whole) return line_forward(zero_after);
         if (generic_) {
             generic_load_density<T><<<blocks((size_t)NP_ * M_), 256, 0, stream_>>>(
                 M_, NP_, rho_fx_, Zxy_, density_scale(), zero_after ? 1 : 0, zero_after ? counters_ : nullptr);
@@ -1705,6 +1786,7 @@ template <typename T> class Engine final : public EngineBase {
                 TILD_CUDA(cudaMemcpyAsync(spec_out, Zxy_, NP_ * M_ * sizeof(V), cudaMemcpyDeviceToDevice, stream_));
                 return TILD_OK;
             }
+            if (use_lines()) return line_spectral(partials);
             const SpectralParams<T> sp = spectral_params();
             if (NP_ == 2)
                 generic_spectral<T, 2><<<blocks(M_), 256, 0, stream_>>>(Zxy_, grad_, n_, nz_, sp, partials);
@@ -1741,12 +1823,11 @@ template <typename T> class Engine final : public EngineBase {
         return TILD_OK;
     }
     tild_status enqueue_inverse(int what) {
-        if (generic_) {
+        if (generic_) {  // (the gradients: nothing on these grids takes the potentials)
+            if (use_lines()) return line_inverse();
             tild_status st;
-            for (int q = 0; q < NP_; ++q) {
-                if (what != kInvPot && (st = generic_fft(grad_ + 4 * q * M_, cfg_->dim, +1))) return st;
-                if (what != kInvGrad && (st = generic_fft(grad_ + (4 * q + 3) * M_, 1, +1))) return st;
-            }
+            for (int q = 0; q < NP_; ++q)
+                if ((st = generic_fft(grad_ + 4 * q * M_, cfg_->dim, +1))) return st;
             return TILD_OK;
         }
         return dispatch_n([&](auto nn) { return this->template inverse_n<decltype(nn)::value>(what); });
@@ -1763,7 +1844,8 @@ template <typename T> class Engine final : public EngineBase {
             err = "positions have not been set";
             return TILD_ESTATE;
         }
-        if ((st = enqueue_forward(false))) return st;
+        if ((st = enqueue_forward(false, spec_out != nullptr))) return st;
+        if (generic_ && spec_out) return enqueue_zpass(nullptr, spec_out);
         if ((st = enqueue_zpass(energy ? partials : nullptr, spec_out, what == kInvPot, energy))) return st;
         return enqueue_inverse(what);
     }

@@ -5,11 +5,15 @@
 //   - beads: one thread per bead (no tiles or shared patches); the density
 //     is accumulated with 64-bit fixed-point global atomics, so it is as
 //     bit-reproducible as the tiled path's;
-//   - FFT: one kernel per axis on tiles of lines held in shared memory, each
-//     line transformed in two factors n = n1 n2 (Cooley-Tukey) with direct
-//     DFTs of lengths n1 and n2 and one twiddle table of length n, so odd
-//     sizes (65 = 5 x 13, 45, 75, primes) need no special radix;
-//   - spectral multiply: one thread per wavevector over the whole spectrum.
+//   - FFT: each line is transformed in two factors n = n1 n2 (Cooley-Tukey)
+//     with direct DFTs of lengths n1 and n2 and one twiddle table of length n,
+//     so odd sizes (65 = 5 x 13, 45, 75, primes) need no special radix;
+//   - step passes ("Line passes" below): the x pass reads the densities, the
+//     pass of the last axis transforms, multiplies and transforms back, and
+//     the x and y dimensions stay in the order their transform leaves them in;
+//   - whole-axis passes with a separate spectral multiply (one thread per
+//     wavevector): the spectrum read-out, and lines too long for the fused
+//     last pass.
 // Grids are [..][nz][n][n] with nz = n (D = 3) or 1 (D = 2); spectra are
 // complex, species pairs packed as in the tiled path (rho_2p + i rho_2p+1).
 #pragma once
@@ -144,7 +148,7 @@ __global__ void generic_load_density(size_t M, int np, unsigned long long* __res
 // species spectra from the packed pairs (Hermitian separation with Z(-k)),
 // w~_K = u_hat(k) sum_K' eps_KK' rho~_K', and per pair
 //   out[p][d] = i k~_d Q_p (d < D; k~ with the Nyquist index zeroed),
-//   out[p][3] = i Q_p (the potentials), Q_p = w~_2p + i w~_2p+1.
+//   Q_p = w~_2p + i w~_2p+1.
 // Energy partials per block as in the z pass: [0] sum u_hat Re[conj(rho~_0)
 // rho~_1] (one pair) or the chi-weighted sum over species pairs (two
 // pairs), [1] sum_{k != 0} u_hat |sum_K rho~_K|^2 (rho~ times e_rho), the
@@ -203,11 +207,444 @@ __global__ void __launch_bounds__(256) generic_spectral(const cplx_t<T>* __restr
             o[g] = {kd[0] * iQ.x, kd[0] * iQ.y};
             o[M + g] = {kd[1] * iQ.x, kd[1] * iQ.y};
             if (nz > 1) o[2 * M + g] = {kd[2] * iQ.x, kd[2] * iQ.y};
-            o[3 * M + g] = iQ;
         }
     }
     if (partials) {
         block_sum<5, T>(acc, [&](int k, const Wide<T>& v) { partials[5 * (size_t)blockIdx.x + k] = v.store(); });
+    }
+}
+
+// ------------------------------------------------------- line passes
+//
+// Bound by latency at the sizes in use (65^2: 4,225 points; 45^3: 91,125): what
+// counts is the number of dependent launches, CTAs on every SM, and short
+// serial chains. A thread transforms n1 or n2 points in registers (up to 16;
+// symmetric sums halve the products of an odd length twice), CTAs hold as few
+// lines as still give the chip about two CTAs per SM, and the index arithmetic
+// has no division per element. Stages work in place as those of the tiled
+// grids do (see fft.cuh): the forward transform leaves X[k1 + n1 k2] in slot
+// k1 n2 + k2 and the inverse starts from there with the factors swapped (n2
+// points over k2, twiddle, n1 points over k1, natural order out), so nothing
+// reorders the spectrum. Only the last pass needs wavenumbers of slots.
+// Step of 5,000 beads on 65^2: 72 -> 25 us in 4 launches (was 7); of 55,000
+// beads of three species on 45^3: 163 -> 83 us in 6 launches (was 12).
+
+// cos(2 pi m / R) and sin(2 pi m / R) at compile time (Taylor series on [0, pi/4]).
+struct TrigSeries {
+    static constexpr double pi = 3.14159265358979323846;
+    static constexpr double cos0(double x) {
+        double t = 1.0, s = 1.0;
+        for (int i = 1; i < 14; ++i) {
+            t *= -x * x / ((2 * i - 1) * (2 * i));
+            s += t;
+        }
+        return s;
+    }
+    static constexpr double sin0(double x) {
+        double t = x, s = x;
+        for (int i = 1; i < 14; ++i) {
+            t *= -x * x / ((2 * i) * (2 * i + 1));
+            s += t;
+        }
+        return s;
+    }
+    // m in [0, R)
+    static constexpr double cosine(int m, int R) {
+        if (2 * m > R) m = R - m;
+        if (4 * m > R) return -cosine_half(R - 2 * m, 2 * R);
+        return cosine_half(2 * m, 2 * R);
+    }
+    static constexpr double sine(int m, int R) {
+        if (2 * m > R) return -sine(R - m, R);
+        if (4 * m > R) return sine_quarter(R - 2 * m, 2 * R);
+        return sine_quarter(2 * m, 2 * R);
+    }
+    // angle 2 pi m / R in [0, pi/2]
+    static constexpr double cosine_half(int m, int R) {
+        return 8 * m > R ? sin0(2 * pi * (R - 4 * m) / (4.0 * R)) : cos0(2 * pi * m / R);
+    }
+    static constexpr double sine_quarter(int m, int R) {
+        return 8 * m > R ? cos0(2 * pi * (R - 4 * m) / (4.0 * R)) : sin0(2 * pi * m / R);
+    }
+};
+template <int R> struct Trig {
+    double c[R] = {}, s[R] = {};
+    constexpr Trig() {
+        for (int m = 0; m < R; ++m) {
+            c[m] = TrigSeries::cosine(m, R);
+            s[m] = TrigSeries::sine(m, R);
+        }
+    }
+};
+
+// DFT of R points in registers, natural order: the radices of the tiled grids,
+// else direct with x_j +- x_{R-j} (a real and an imaginary sum of (R - 1)/2
+// products give X_k and X_{R-k}).
+template <int R, int DIR, class V> __device__ __forceinline__ void any_dft(V (&v)[R]) {
+    using T = decltype(v[0].x);
+    if constexpr (R == 2 || R == 3 || R == 4 || R == 5 || R == 8 || R == 16) {
+        reg_dft<R, DIR, V>::run(v);
+    } else {
+        constexpr Trig<R> t{};
+        constexpr int H = (R - 1) / 2;
+        V s[H], d[H];
+#pragma unroll
+        for (int j = 0; j < H; ++j) {
+            s[j] = c_add(v[j + 1], v[R - 1 - j]);
+            d[j] = c_sub(v[j + 1], v[R - 1 - j]);
+        }
+        const V x0 = v[0], xm = v[R / 2];
+#pragma unroll
+        for (int k = 0; k <= H; ++k) {
+            V a = x0, b = {T(0), T(0)};
+            if (R % 2 == 0) a = (k & 1) ? c_sub(a, xm) : c_add(a, xm);
+#pragma unroll
+            for (int j = 0; j < H; ++j) {
+                const T c = (T)t.c[((j + 1) * k) % R], sn = (T)(DIR * t.s[((j + 1) * k) % R]);
+                a = {fma_rn(c, s[j].x, a.x), fma_rn(c, s[j].y, a.y)};
+                b = {fma_rn(sn, d[j].x, b.x), fma_rn(sn, d[j].y, b.y)};
+            }
+            v[k] = {a.x - b.y, a.y + b.x};  // a + i b
+            if (k > 0) v[R - k] = {a.x + b.y, a.y - b.x};
+        }
+        if (R % 2 == 0) {
+            V a = (R / 2) & 1 ? c_sub(x0, xm) : c_add(x0, xm);
+#pragma unroll
+            for (int j = 0; j < H; ++j) a = (j & 1) ? c_add(a, s[j]) : c_sub(a, s[j]);  // (-1)^(j + 1)
+            v[R / 2] = a;
+        }
+    }
+}
+
+// Lines in shared memory: element e of line l at e ES + l LS; 2^lg lines.
+struct LineBuf {
+    int n, n1, n2, ES, LS, lg;
+};
+
+// One stage over all lines: `other` units per line, unit o on the R elements
+// o bs + k es, times W_n^{o k} at the end when `tw_on`. Up to 16 points stay in
+// registers and in place; longer (prime) factors go through `alt`, one thread
+// per pair of outputs (k, R - k), and buf and alt change places.
+template <int R, int DIR, class V>
+__device__ __forceinline__ void line_stage_small(V* buf, const LineBuf& L, int other, int bs, int es, bool tw_on, const V* tw) {
+    const int st = es * L.ES;
+    for (int u = threadIdx.x; u < (other << L.lg); u += blockDim.x) {
+        const int l = u & ((1 << L.lg) - 1), o = u >> L.lg;
+        V* p = buf + l * L.LS + o * bs * L.ES;
+        V v[R];
+#pragma unroll
+        for (int k = 0; k < R; ++k) v[k] = p[k * st];
+        any_dft<R, DIR>(v);
+        if (tw_on) {
+#pragma unroll
+            for (int k = 1; k < R; ++k) v[k] = c_mul(v[k], gtw<DIR>(tw, o * k));
+        }
+#pragma unroll
+        for (int k = 0; k < R; ++k) p[k * st] = v[k];
+    }
+}
+template <int DIR, class V>
+__device__ __noinline__ void line_stage_big(const V* buf, V* alt, const LineBuf& L, int R, int other, int bs, int es, bool tw_on,
+                                            const V* tw) {
+    using T = decltype(buf->x);
+    const int st = es * L.ES, pairs = R / 2 + 1, wstep = L.n / R;
+    for (int u = threadIdx.x; u < ((other * pairs) << L.lg); u += blockDim.x) {
+        const int l = u & ((1 << L.lg) - 1), r = u >> L.lg;
+        const int o = r % other, k = r / other;
+        const int base = l * L.LS + o * bs * L.ES;
+        const V* p = buf + base;
+        V a = p[0], b = {T(0), T(0)};
+        int m = 0;
+        for (int j = 1; 2 * j <= R; ++j) {
+            m += k;
+            if (m >= R) m -= R;
+            const V w = tw[m * wstep];  // (cos, -sin)
+            const V x = p[j * st];
+            if (2 * j == R) {  // R even: (-1)^k x_{R/2}
+                a = {fma_rn(w.x, x.x, a.x), fma_rn(w.x, x.y, a.y)};
+            } else {
+                const V y = p[(R - j) * st];
+                const V s = c_add(x, y), d = c_sub(x, y);
+                const T sn = DIR < 0 ? w.y : -w.y;
+                a = {fma_rn(w.x, s.x, a.x), fma_rn(w.x, s.y, a.y)};
+                b = {fma_rn(sn, d.x, b.x), fma_rn(sn, d.y, b.y)};
+            }
+        }
+        V x1 = {a.x - b.y, a.y + b.x}, x2 = {a.x + b.y, a.y - b.x};
+        V* q = alt + base;
+        q[k * st] = tw_on ? c_mul(x1, gtw<DIR>(tw, o * k)) : x1;
+        if (k > 0 && 2 * k != R) q[(R - k) * st] = tw_on ? c_mul(x2, gtw<DIR>(tw, o * (R - k))) : x2;
+    }
+}
+template <int DIR, class V>
+__device__ __forceinline__ void line_stage(V*& buf, V*& alt, const LineBuf& L, int R, int other, int bs, int es, bool tw_on,
+                                           const V* tw) {
+    switch (R) {
+#define TILD_STAGE(r) \
+    case r: line_stage_small<r, DIR>(buf, L, other, bs, es, tw_on, tw); break;
+        case 1: break;
+        TILD_STAGE(2) TILD_STAGE(3) TILD_STAGE(4) TILD_STAGE(5) TILD_STAGE(6) TILD_STAGE(7) TILD_STAGE(8) TILD_STAGE(9)
+        TILD_STAGE(10) TILD_STAGE(11) TILD_STAGE(12) TILD_STAGE(13) TILD_STAGE(14) TILD_STAGE(15) TILD_STAGE(16)
+#undef TILD_STAGE
+        default: {
+            line_stage_big<DIR>(buf, alt, L, R, other, bs, es, tw_on, tw);
+            V* t = buf;
+            buf = alt;
+            alt = t;
+        }
+    }
+    __syncthreads();
+}
+// natural order in, slot order out / slot order in, natural order out
+template <class V> __device__ __forceinline__ void lines_forward(V*& buf, V*& alt, const LineBuf& L, const V* tw) {
+    line_stage<-1>(buf, alt, L, L.n1, L.n2, 1, L.n2, true, tw);
+    line_stage<-1>(buf, alt, L, L.n2, L.n1, L.n2, 1, false, tw);
+}
+template <class V> __device__ __forceinline__ void lines_inverse(V*& buf, V*& alt, const LineBuf& L, const V* tw) {
+    line_stage<+1>(buf, alt, L, L.n2, L.n1, L.n2, 1, true, tw);
+    line_stage<+1>(buf, alt, L, L.n1, L.n2, 1, L.n2, false, tw);
+}
+
+// What the line passes share. H: [NP][3][M] (field 0: G, field 2: G of the last
+// axis times its wavenumber, between them the y pass's third field).
+template <typename T> struct LineArgs {
+    int n, nz, n1, n2, lg;   // grid, factors, log2 of the lines per CTA
+    int half;                // complex values of one line buffer (0: no second buffer)
+    const cplx_t<T>* tw;
+    T two_pi_over_L;
+};
+template <typename T> __device__ __forceinline__ T any_grad_k(int i, int n, T two_pi_over_L) {
+    return (n % 2 == 0 && 2 * i == n) ? T(0) : two_pi_over_L * (T)(2 * i < n ? i : i - n);
+}
+// wavenumber index of a slot, and the slot of an index
+__device__ __forceinline__ int slot_index(int s, int n1, int n2) { return s / n2 + n1 * (s % n2); }
+__device__ __forceinline__ int index_slot(int k, int n1, int n2) { return (k % n1) * n2 + k / n1; }
+
+// x pass forward: rows of the fixed-point densities (zeroed when asked) -> Z.
+// grid = (row tiles, NP); a warp loads a row at a time.
+template <typename T>
+__global__ void __launch_bounds__(128) line_x_forward(LineArgs<T> g, unsigned long long* __restrict__ rho_fx,
+                                                      cplx_t<T>* __restrict__ Z, T scale, int zero_after,
+                                                      unsigned long long* step_ctr) {
+    using V = cplx_t<T>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    V* tw = reinterpret_cast<V*>(smem_raw);
+    V* buf = tw + g.n;
+    V* alt = buf + g.half;
+    const int pitch = g.n | 1, CL = 1 << g.lg;
+    const size_t M = (size_t)g.nz * g.n * g.n;
+    const int rows = g.nz * g.n, r0 = blockIdx.x * CL;
+    unsigned long long* a = rho_fx + 2 * blockIdx.y * M;
+    Z += blockIdx.y * M;
+    if (step_ctr && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *step_ctr += 1ull;
+    for (int i = threadIdx.x; i < g.n; i += 128) tw[i] = g.tw[i];
+    const int lane = threadIdx.x & 31;
+    for (int l = threadIdx.x >> 5; l < CL; l += 4) {
+        if (r0 + l >= rows) break;
+        unsigned long long* ra = a + (size_t)(r0 + l) * g.n;
+        for (int e = lane; e < g.n; e += 32) {
+            const long long va = (long long)ra[e], vb = (long long)ra[M + e];
+            if (zero_after) {
+                ra[e] = 0ull;
+                ra[M + e] = 0ull;
+            }
+            buf[l * pitch + e] = V{density_from_fixed(va, scale), density_from_fixed(vb, scale)};
+        }
+    }
+    __syncthreads();
+    lines_forward(buf, alt, LineBuf{g.n, g.n1, g.n2, 1, pitch, g.lg}, tw);
+    for (int l = threadIdx.x >> 5; l < CL; l += 4) {
+        if (r0 + l >= rows) break;
+        for (int e = lane; e < g.n; e += 32) Z[(size_t)(r0 + l) * g.n + e] = buf[l * pitch + e];
+    }
+}
+
+// x pass inverse: field d of pair q (grid.y = q D + d) -> grad field d. d = 0:
+// G times k_x; in 2D field 1 lies in H's field 2 (the last axis).
+template <typename T>
+__global__ void __launch_bounds__(128) line_x_inverse(LineArgs<T> g, const cplx_t<T>* __restrict__ H, cplx_t<T>* __restrict__ grad,
+                                                      int D) {
+    using V = cplx_t<T>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    V* tw = reinterpret_cast<V*>(smem_raw);
+    V* buf = tw + g.n;
+    V* alt = buf + g.half;
+    const int pitch = g.n | 1, CL = 1 << g.lg;
+    const size_t M = (size_t)g.nz * g.n * g.n;
+    const int rows = g.nz * g.n, r0 = blockIdx.x * CL, q = blockIdx.y / D, d = blockIdx.y - q * D;
+    const V* src = H + (3 * q + (D == 2 && d == 1 ? 2 : d)) * M;
+    grad += (4 * q + d) * M;
+    for (int i = threadIdx.x; i < g.n; i += 128) tw[i] = g.tw[i];
+    const int lane = threadIdx.x & 31;
+    for (int l = threadIdx.x >> 5; l < CL; l += 4) {
+        if (r0 + l >= rows) break;
+        for (int e = lane; e < g.n; e += 32) {
+            V v = src[(size_t)(r0 + l) * g.n + e];
+            if (d == 0) v = c_scale_rn(v, any_grad_k(slot_index(e, g.n1, g.n2), g.n, g.two_pi_over_L));
+            buf[l * pitch + e] = v;
+        }
+    }
+    __syncthreads();
+    lines_inverse(buf, alt, LineBuf{g.n, g.n1, g.n2, 1, pitch, g.lg}, tw);
+    for (int l = threadIdx.x >> 5; l < CL; l += 4) {
+        if (r0 + l >= rows) break;
+        for (int e = lane; e < g.n; e += 32) grad[(size_t)(r0 + l) * g.n + e] = buf[l * pitch + e];
+    }
+}
+
+// y pass (3D): CTA = (tile of column slots, z plane, part). Forward: Z in place
+// (grid.z = pair). Inverse on H (grid.z = 2 pair + part): part 0 reads G and
+// writes field 0 (G) and field 1 (k_y G), part 1 transforms field 2.
+template <typename T, int DIR>
+__global__ void __launch_bounds__(128) line_y(LineArgs<T> g, cplx_t<T>* __restrict__ data) {
+    using V = cplx_t<T>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    V* tw = reinterpret_cast<V*>(smem_raw);
+    V* buf = tw + g.n;
+    V* alt = buf + g.half;
+    const int n = g.n;
+    const size_t M = (size_t)g.nz * n * n;
+    const int part = DIR < 0 ? 0 : (int)(blockIdx.z & 1);
+    data += DIR < 0 ? blockIdx.z * M : 3 * (blockIdx.z >> 1) * M;
+    const bool two = DIR > 0 && part == 0;
+    // lg counts the lines of the buffer: half of them columns when two fields come out
+    const int clg = two ? g.lg - 1 : g.lg, C = 1 << clg, LN = 1 << g.lg;
+    const int x0 = blockIdx.x * C;
+    V* base = data + (DIR > 0 && part == 1 ? 2 * M : 0) + (size_t)blockIdx.y * n * n;
+    for (int i = threadIdx.x; i < n; i += 128) tw[i] = g.tw[i];
+    if (x0 < n) {
+        for (int i = threadIdx.x; i < n * C; i += 128) {
+            const int c = i & (C - 1), e = i >> clg;
+            if (x0 + c >= n) continue;
+            const V v = base[(size_t)e * n + x0 + c];
+            buf[e * LN + c] = v;
+            if (two) buf[e * LN + C + c] = c_scale_rn(v, any_grad_k(slot_index(e, g.n1, g.n2), n, g.two_pi_over_L));
+        }
+    }
+    __syncthreads();
+    if (x0 >= n) return;
+    const LineBuf L{n, g.n1, g.n2, LN, 1, g.lg};
+    if (DIR < 0)
+        lines_forward(buf, alt, L, tw);
+    else
+        lines_inverse(buf, alt, L, tw);
+    for (int i = threadIdx.x; i < n * C; i += 128) {
+        const int c = i & (C - 1), e = i >> clg;
+        if (x0 + c >= n) continue;
+        base[(size_t)e * n + x0 + c] = buf[e * LN + c];
+        if (two) base[M + (size_t)e * n + x0 + c] = buf[e * LN + C + c];
+    }
+}
+
+// Last axis (z in 3D, y in 2D): forward transform, spectral multiply, inverse
+// transform. CTA = (tile of CP column slots, row pair {ky, -ky}); it holds
+// every column's line A = (ky, kx) and mirror line B = (-ky, -kx) of every
+// species pair. Rows that are their own mirror (ky = 0, n/2; 2D) store A only.
+// Lines [field][pair q][A, B][CP]: field 0 becomes G = i Q, field 1
+// i k_last Q, Q_p = w~_2p + i w~_2p+1 (as in the z pass of the tiled grids).
+template <typename T, int NP, int D>
+__global__ void __launch_bounds__(128) line_last(LineArgs<T> g, const cplx_t<T>* __restrict__ Z, cplx_t<T>* __restrict__ H,
+                                                 SpectralParams<T> sp, typename Wide<T>::stored* __restrict__ partials) {
+    using V = cplx_t<T>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    V* tw = reinterpret_cast<V*>(smem_raw);
+    V* buf = tw + g.n;
+    V* alt = buf + g.half;
+    const int n = g.n, n1 = g.n1, n2 = g.n2;
+    constexpr int LPC = 4 * NP;                  // lines per column: fields x pairs x (A, B)
+    const int LN = 1 << g.lg, CP = LN / LPC, F = LN / 2;  // F: lines of one field
+    const int cpl = g.lg - (NP == 2 ? 3 : 2);    // log2 CP
+    const size_t M = (size_t)g.nz * n * n, stride = D == 3 ? (size_t)n * n : (size_t)n;
+    const int ky = D == 3 ? (int)blockIdx.y : 0, my = ky == 0 ? 0 : n - ky;
+    const bool self = ky == my;
+    const size_t rowA = D == 3 ? (size_t)index_slot(ky, n1, n2) * n : 0, rowB = D == 3 ? (size_t)index_slot(my, n1, n2) * n : 0;
+    const int x0 = blockIdx.x * CP;
+    auto mirror = [&](int s) {  // the slot of -kx
+        const int a = s / n2, b = s % n2;
+        return a == 0 ? (b == 0 ? 0 : n2 - b) : (n1 - a) * n2 + n2 - 1 - b;
+    };
+    for (int i = threadIdx.x; i < n; i += 128) tw[i] = g.tw[i];
+    // lanes over columns, then A/B, pairs and elements
+    for (int i = threadIdx.x; i < n * F; i += 128) {
+        const int l = i & (F - 1), e = i / F;
+        const int c = l & (CP - 1), h = l >> cpl;  // h = 2 q + (A: 0, B: 1)
+        if (x0 + c >= n) continue;
+        const size_t off = (h & 1) ? rowB + mirror(x0 + c) : rowA + x0 + c;
+        buf[e * LN + l] = Z[(h >> 1) * M + (size_t)e * stride + off];
+    }
+    __syncthreads();
+    // the forward transform of field 0's lines alone: half of the buffer
+    lines_forward(buf, alt, LineBuf{n, n1, n2, LN, 1, g.lg - 1}, tw);
+    Wide<T> acc[5];
+    // multiply: unit (column, k1); slot k1 n2 + k2 of A meets the slot of -k in B
+    for (int u = threadIdx.x; u < n1 << cpl; u += 128) {
+        const int c = u & (CP - 1), k1 = u >> cpl;
+        if (x0 + c >= n) continue;
+        const int kx = slot_index(x0 + c, n1, n2);
+        const T exy = sp.kernel1d[kx] * (D == 3 ? sp.kernel1d[ky] : T(1));
+        const int k1m = k1 == 0 ? 0 : n1 - k1;
+        for (int k2 = 0; k2 < n2; ++k2) {
+            const int kl = k1 + n1 * k2, km = kl == 0 ? 0 : n - kl;
+            const int eA = (k1 * n2 + k2) * LN + c, eB = (k1m * n2 + (k1 == 0 ? (k2 == 0 ? 0 : n2 - k2) : n2 - 1 - k2)) * LN + c;
+            const T uh = exy * sp.kernel1d[kl];
+            V zA[NP], zB[NP];
+#pragma unroll
+            for (int q = 0; q < NP; ++q) {
+                zA[q] = buf[eA + (2 * q) * CP];
+                zB[q] = buf[eB + (2 * q + 1) * CP];
+            }
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+                V A[2 * NP];
+#pragma unroll
+                for (int q = 0; q < NP; ++q) {
+                    const V Zk = s == 0 ? zA[q] : zB[q], Zm = s == 0 ? zB[q] : zA[q];
+                    A[2 * q] = {T(0.5) * (Zk.x + Zm.x), T(0.5) * (Zk.y - Zm.y)};
+                    A[2 * q + 1] = {T(0.5) * (Zk.y + Zm.y), -T(0.5) * (Zk.x - Zm.x)};
+                }
+                if (partials && s == 0) {  // k and -k contribute the same
+                    const bool zero = kx == 0 && ky == 0 && kl == 0;
+                    const T weight = self ? T(1) : T(2);
+                    if constexpr (NP == 1)
+                        add_energies<T, 1>(acc, A[0], A[1], uh, sp.e_rho, weight, zero, T(0));
+                    else
+                        add_energies4<T, NP>(acc, A, sp, uh * weight, zero);
+                }
+                const T kg = any_grad_k(s == 0 ? kl : km, n, sp.two_pi_over_L);
+                V w[2 * NP];
+#pragma unroll
+                for (int K = 0; K < 2 * NP; ++K) {
+                    T wr = 0, wi = 0;
+#pragma unroll
+                    for (int K2 = 0; K2 < 2 * NP; ++K2) {
+                        const T eps = NP == 1 ? (K == K2 ? (K == 0 ? sp.eAA : sp.eBB) : sp.eAB) : sp.eps4[K][K2];
+                        wr = fma_rn(eps, A[K2].x, wr);
+                        wi = fma_rn(eps, A[K2].y, wi);
+                    }
+                    w[K] = {uh * wr, uh * wi};
+                }
+#pragma unroll
+                for (int q = 0; q < NP; ++q) {
+                    const V iQ = {-(w[2 * q].y + w[2 * q + 1].x), w[2 * q].x - w[2 * q + 1].y};
+                    const int at = (s == 0 ? eA + (2 * q) * CP : eB + (2 * q + 1) * CP);
+                    buf[at] = iQ;
+                    buf[at + F] = c_scale_rn(iQ, kg);
+                }
+            }
+        }
+    }
+    __syncthreads();
+    lines_inverse(buf, alt, LineBuf{n, n1, n2, LN, 1, g.lg}, tw);
+    for (int i = threadIdx.x; i < n * LN; i += 128) {
+        const int l = i & (LN - 1), e = i >> g.lg;
+        const int c = l & (CP - 1), h = (l & (F - 1)) >> cpl, f = l >= F ? 2 : 0;
+        if (x0 + c >= n || (self && (h & 1))) continue;
+        const size_t off = (h & 1) ? rowB + mirror(x0 + c) : rowA + x0 + c;
+        H[(3 * (h >> 1) + f) * M + (size_t)e * stride + off] = buf[e * LN + l];
+    }
+    if (partials) {
+        const size_t b = (size_t)blockIdx.y * gridDim.x + blockIdx.x;
+        block_sum<5, T>(acc, [&](int k, const Wide<T>& v) { partials[5 * b + k] = v.store(); });
     }
 }
 

@@ -163,8 +163,8 @@ template <int P> __device__ __forceinline__ int3 tile_patch(int t, int tiles, in
 // them, larger tiles and beads outside their patch take the global path. The
 // patch is flushed with one 64-bit add per point, rows of both species
 // contiguous. Integer sums: the same bits as the global path.
-// One product on 200k beads, 64^3 (P = 2), this kernel and vjp_beads_tiled in
-// place of the global ones: 113 -> 71 us.
+// 200k beads, 64^3: 28.1 -> 16.1 us (P = 2); vjp_beads_tiled in place of the
+// per-bead gather 20.6 -> 14.3 us.
 constexpr int kVjpTileBeads = 2047;
 template <int P> constexpr size_t vjp_spread_smem() { return (size_t)12 * Patch<P>::W3 * sizeof(int); }
 template <int P>

@@ -1110,7 +1110,7 @@ template <typename T> class Engine final : public EngineBase {
     // memory within kLineSmem.
     static constexpr int kLineSmem = 200 * 1024;
     bool line_big() const { return std::max(gn1_, gn2_) > 16; }
-    size_t line_smem(int half) const { return ((size_t)n_ + (size_t)half * (line_big() ? 2 : 1)) * sizeof(V); }
+    size_t line_smem(int half) const { return ((size_t)2 * n_ + (size_t)half * (line_big() ? 2 : 1)) * sizeof(V); }
     // lines: of the launch at 2^lg per CTA; f(lg) = CTAs
     template <class F> int line_lg(int hi, int lo, int per_line, F&& ctas) const {
         int lg = hi;

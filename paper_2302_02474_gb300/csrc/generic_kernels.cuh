@@ -226,8 +226,8 @@ __global__ void __launch_bounds__(256) generic_spectral(const cplx_t<T>* __restr
 // k1 n2 + k2 and the inverse starts from there with the factors swapped (n2
 // points over k2, twiddle, n1 points over k1, natural order out), so nothing
 // reorders the spectrum. Only the last pass needs wavenumbers of slots.
-// Step of 5,000 beads on 65^2: 72 -> 25 us in 4 launches (was 7); of 55,000
-// beads of three species on 45^3: 163 -> 83 us in 6 launches (was 12).
+// Step of 5,000 beads on 65^2: 72 -> 22 us in 4 launches (was 7); of 55,000
+// beads of three species on 45^3: 163 -> 63 us in 6 launches (was 12).
 
 // cos(2 pi m / R) and sin(2 pi m / R) at compile time (Taylor series on [0, pi/4]).
 struct TrigSeries {
@@ -420,43 +420,85 @@ template <typename T> __device__ __forceinline__ T any_grad_k(int i, int n, T tw
 __device__ __forceinline__ int slot_index(int s, int n1, int n2) { return s / n2 + n1 * (s % n2); }
 __device__ __forceinline__ int index_slot(int k, int n1, int n2) { return (k % n1) * n2 + k / n1; }
 
-// x pass forward: rows of the fixed-point densities (zeroed when asked) -> Z.
-// grid = (row tiles, NP); a warp loads a row at a time.
+// Shared memory of a line pass: twiddles [n], wavenumbers by slot [n] (in the
+// space of n complex values), then the line buffers.
+template <typename T> struct LineShared {
+    cplx_t<T>*tw, *buf, *alt;
+    T* ks;
+    __device__ __forceinline__ LineShared(unsigned char* raw, const LineArgs<T>& g) {
+        tw = reinterpret_cast<cplx_t<T>*>(raw);
+        ks = reinterpret_cast<T*>(tw + g.n);
+        buf = tw + 2 * g.n;
+        alt = buf + g.half;
+    }
+    __device__ __forceinline__ void fill(const LineArgs<T>& g) const {
+        for (int i = threadIdx.x; i < g.n; i += 128) {
+            tw[i] = g.tw[i];
+            ks[i] = any_grad_k(slot_index(i, g.n1, g.n2), g.n, g.two_pi_over_L);
+        }
+    }
+};
+
+// f(l, e) in batches of four loads for the elements e of the CTA's rows l: a
+// warp or more per row; load(l, e) -> R, then store(l, e, R).
+template <class R, class Load, class Store>
+__device__ __forceinline__ void for_rows(int lg, int rows, int n, Load load, Store store) {
+    const int ts = lg >= 2 ? 5 : 7 - lg, tpr = 1 << ts, rpp = 128 >> ts;
+    const int e0 = threadIdx.x & (tpr - 1);
+    int l = threadIdx.x >> ts, e = e0;
+    while (l < rows) {
+        R v[4];
+        int la[4], ea[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            la[k] = l;
+            ea[k] = e;
+            if (l < rows && e < n) v[k] = load(l, e);
+            e += tpr;
+            if (e >= n) {
+                e = e0;
+                l += rpp;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (la[k] < rows && ea[k] < n) store(la[k], ea[k], v[k]);
+    }
+}
+
+// x pass forward: rows of the fixed-point densities (zeroed when asked, once
+// every row of the CTA is loaded: zeroing between the loads would serialise
+// them) -> Z. grid = (row tiles, NP).
 template <typename T>
 __global__ void __launch_bounds__(128) line_x_forward(LineArgs<T> g, unsigned long long* __restrict__ rho_fx,
                                                       cplx_t<T>* __restrict__ Z, T scale, int zero_after,
                                                       unsigned long long* step_ctr) {
     using V = cplx_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    V* tw = reinterpret_cast<V*>(smem_raw);
-    V* buf = tw + g.n;
-    V* alt = buf + g.half;
-    const int pitch = g.n | 1, CL = 1 << g.lg;
+    LineShared<T> sh(smem_raw, g);
+    const int pitch = g.n | 1;
     const size_t M = (size_t)g.nz * g.n * g.n;
-    const int rows = g.nz * g.n, r0 = blockIdx.x * CL;
-    unsigned long long* a = rho_fx + 2 * blockIdx.y * M;
-    Z += blockIdx.y * M;
+    const int r0 = blockIdx.x << g.lg, rows = min(1 << g.lg, g.nz * g.n - r0);
+    unsigned long long* a = rho_fx + 2 * blockIdx.y * M + (size_t)r0 * g.n;
+    Z += blockIdx.y * M + (size_t)r0 * g.n;
     if (step_ctr && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *step_ctr += 1ull;
-    for (int i = threadIdx.x; i < g.n; i += 128) tw[i] = g.tw[i];
-    const int lane = threadIdx.x & 31;
-    for (int l = threadIdx.x >> 5; l < CL; l += 4) {
-        if (r0 + l >= rows) break;
-        unsigned long long* ra = a + (size_t)(r0 + l) * g.n;
-        for (int e = lane; e < g.n; e += 32) {
-            const long long va = (long long)ra[e], vb = (long long)ra[M + e];
-            if (zero_after) {
-                ra[e] = 0ull;
-                ra[M + e] = 0ull;
-            }
-            buf[l * pitch + e] = V{density_from_fixed(va, scale), density_from_fixed(vb, scale)};
-        }
-    }
+    for_rows<longlong2>(
+        g.lg, rows, g.n,
+        [&](int l, int e) { return make_longlong2((long long)a[l * g.n + e], (long long)a[M + l * g.n + e]); },
+        [&](int l, int e, longlong2 v) {
+            sh.buf[l * pitch + e] = V{density_from_fixed(v.x, scale), density_from_fixed(v.y, scale)};
+        });
+    sh.fill(g);
     __syncthreads();
-    lines_forward(buf, alt, LineBuf{g.n, g.n1, g.n2, 1, pitch, g.lg}, tw);
-    for (int l = threadIdx.x >> 5; l < CL; l += 4) {
-        if (r0 + l >= rows) break;
-        for (int e = lane; e < g.n; e += 32) Z[(size_t)(r0 + l) * g.n + e] = buf[l * pitch + e];
-    }
+    if (zero_after)
+        for (int i = threadIdx.x; i < rows * g.n; i += 128) {
+            a[i] = 0ull;
+            a[M + i] = 0ull;
+        }
+    lines_forward(sh.buf, sh.alt, LineBuf{g.n, g.n1, g.n2, 1, pitch, g.lg}, sh.tw);
+    for_rows<V>(
+        g.lg, rows, g.n, [&](int l, int e) { return sh.buf[l * pitch + e]; },
+        [&](int l, int e, V v) { Z[l * g.n + e] = v; });
 }
 
 // x pass inverse: field d of pair q (grid.y = q D + d) -> grad field d. d = 0:
@@ -466,30 +508,27 @@ __global__ void __launch_bounds__(128) line_x_inverse(LineArgs<T> g, const cplx_
                                                       int D) {
     using V = cplx_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    V* tw = reinterpret_cast<V*>(smem_raw);
-    V* buf = tw + g.n;
-    V* alt = buf + g.half;
-    const int pitch = g.n | 1, CL = 1 << g.lg;
+    LineShared<T> sh(smem_raw, g);
+    const int pitch = g.n | 1;
     const size_t M = (size_t)g.nz * g.n * g.n;
-    const int rows = g.nz * g.n, r0 = blockIdx.x * CL, q = blockIdx.y / D, d = blockIdx.y - q * D;
-    const V* src = H + (3 * q + (D == 2 && d == 1 ? 2 : d)) * M;
-    grad += (4 * q + d) * M;
-    for (int i = threadIdx.x; i < g.n; i += 128) tw[i] = g.tw[i];
-    const int lane = threadIdx.x & 31;
-    for (int l = threadIdx.x >> 5; l < CL; l += 4) {
-        if (r0 + l >= rows) break;
-        for (int e = lane; e < g.n; e += 32) {
-            V v = src[(size_t)(r0 + l) * g.n + e];
-            if (d == 0) v = c_scale_rn(v, any_grad_k(slot_index(e, g.n1, g.n2), g.n, g.two_pi_over_L));
-            buf[l * pitch + e] = v;
-        }
-    }
+    const int r0 = blockIdx.x << g.lg, rows = min(1 << g.lg, g.nz * g.n - r0);
+    const int q = blockIdx.y / D, d = blockIdx.y - q * D;
+    const V* src = H + (3 * q + (D == 2 && d == 1 ? 2 : d)) * M + (size_t)r0 * g.n;
+    grad += (4 * q + d) * M + (size_t)r0 * g.n;
+    for_rows<V>(
+        g.lg, rows, g.n, [&](int l, int e) { return src[l * g.n + e]; }, [&](int l, int e, V v) { sh.buf[l * pitch + e] = v; });
+    sh.fill(g);
     __syncthreads();
-    lines_inverse(buf, alt, LineBuf{g.n, g.n1, g.n2, 1, pitch, g.lg}, tw);
-    for (int l = threadIdx.x >> 5; l < CL; l += 4) {
-        if (r0 + l >= rows) break;
-        for (int e = lane; e < g.n; e += 32) grad[(size_t)(r0 + l) * g.n + e] = buf[l * pitch + e];
+    if (d == 0) {
+        for_rows<V>(
+            g.lg, rows, g.n, [&](int l, int e) { return sh.buf[l * pitch + e]; },
+            [&](int l, int e, V v) { sh.buf[l * pitch + e] = c_scale_rn(v, sh.ks[e]); });
+        __syncthreads();
     }
+    lines_inverse(sh.buf, sh.alt, LineBuf{g.n, g.n1, g.n2, 1, pitch, g.lg}, sh.tw);
+    for_rows<V>(
+        g.lg, rows, g.n, [&](int l, int e) { return sh.buf[l * pitch + e]; },
+        [&](int l, int e, V v) { grad[l * g.n + e] = v; });
 }
 
 // y pass (3D): CTA = (tile of column slots, z plane, part). Forward: Z in place
@@ -499,9 +538,7 @@ template <typename T, int DIR>
 __global__ void __launch_bounds__(128) line_y(LineArgs<T> g, cplx_t<T>* __restrict__ data) {
     using V = cplx_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    V* tw = reinterpret_cast<V*>(smem_raw);
-    V* buf = tw + g.n;
-    V* alt = buf + g.half;
+    LineShared<T> sh(smem_raw, g);
     const int n = g.n;
     const size_t M = (size_t)g.nz * n * n;
     const int part = DIR < 0 ? 0 : (int)(blockIdx.z & 1);
@@ -510,29 +547,40 @@ __global__ void __launch_bounds__(128) line_y(LineArgs<T> g, cplx_t<T>* __restri
     // lg counts the lines of the buffer: half of them columns when two fields come out
     const int clg = two ? g.lg - 1 : g.lg, C = 1 << clg, LN = 1 << g.lg;
     const int x0 = blockIdx.x * C;
-    V* base = data + (DIR > 0 && part == 1 ? 2 * M : 0) + (size_t)blockIdx.y * n * n;
-    for (int i = threadIdx.x; i < n; i += 128) tw[i] = g.tw[i];
-    if (x0 < n) {
-        for (int i = threadIdx.x; i < n * C; i += 128) {
-            const int c = i & (C - 1), e = i >> clg;
-            if (x0 + c >= n) continue;
-            const V v = base[(size_t)e * n + x0 + c];
-            buf[e * LN + c] = v;
-            if (two) buf[e * LN + C + c] = c_scale_rn(v, any_grad_k(slot_index(e, g.n1, g.n2), n, g.two_pi_over_L));
+    if (x0 >= n) return;
+    V* base = data + (DIR > 0 && part == 1 ? 2 * M : 0) + (size_t)blockIdx.y * n * n + x0;
+    for (int i0 = threadIdx.x; i0 < n * C; i0 += 4 * 128) {
+        V v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int i = i0 + k * 128, c = i & (C - 1), e = i >> clg;
+            if (e < n && x0 + c < n) v[k] = base[e * n + c];
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int i = i0 + k * 128, c = i & (C - 1), e = i >> clg;
+            if (e < n && x0 + c < n) sh.buf[e * LN + c] = v[k];
         }
     }
+    sh.fill(g);
     __syncthreads();
-    if (x0 >= n) return;
+    if (two) {
+        for (int i = threadIdx.x; i < n * C; i += 128) {
+            const int c = i & (C - 1), e = i >> clg;
+            sh.buf[e * LN + C + c] = c_scale_rn(sh.buf[e * LN + c], sh.ks[e]);
+        }
+        __syncthreads();
+    }
     const LineBuf L{n, g.n1, g.n2, LN, 1, g.lg};
     if (DIR < 0)
-        lines_forward(buf, alt, L, tw);
+        lines_forward(sh.buf, sh.alt, L, sh.tw);
     else
-        lines_inverse(buf, alt, L, tw);
+        lines_inverse(sh.buf, sh.alt, L, sh.tw);
     for (int i = threadIdx.x; i < n * C; i += 128) {
         const int c = i & (C - 1), e = i >> clg;
         if (x0 + c >= n) continue;
-        base[(size_t)e * n + x0 + c] = buf[e * LN + c];
-        if (two) base[M + (size_t)e * n + x0 + c] = buf[e * LN + C + c];
+        base[e * n + c] = sh.buf[e * LN + c];
+        if (two) base[M + e * n + c] = sh.buf[e * LN + C + c];
     }
 }
 
@@ -547,45 +595,58 @@ __global__ void __launch_bounds__(128) line_last(LineArgs<T> g, const cplx_t<T>*
                                                  SpectralParams<T> sp, typename Wide<T>::stored* __restrict__ partials) {
     using V = cplx_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    V* tw = reinterpret_cast<V*>(smem_raw);
-    V* buf = tw + g.n;
-    V* alt = buf + g.half;
+    LineShared<T> sh(smem_raw, g);
     const int n = g.n, n1 = g.n1, n2 = g.n2;
-    constexpr int LPC = 4 * NP;                  // lines per column: fields x pairs x (A, B)
-    const int LN = 1 << g.lg, CP = LN / LPC, F = LN / 2;  // F: lines of one field
-    const int cpl = g.lg - (NP == 2 ? 3 : 2);    // log2 CP
-    const size_t M = (size_t)g.nz * n * n, stride = D == 3 ? (size_t)n * n : (size_t)n;
+    const int LN = 1 << g.lg, flg = g.lg - 1, F = LN / 2;  // lines, and those of one field
+    const int cpl = g.lg - (NP == 2 ? 3 : 2), CP = 1 << cpl;  // 4 NP lines per column
+    const size_t M = (size_t)g.nz * n * n;
+    const int stride = D == 3 ? n * n : n;
     const int ky = D == 3 ? (int)blockIdx.y : 0, my = ky == 0 ? 0 : n - ky;
     const bool self = ky == my;
-    const size_t rowA = D == 3 ? (size_t)index_slot(ky, n1, n2) * n : 0, rowB = D == 3 ? (size_t)index_slot(my, n1, n2) * n : 0;
     const int x0 = blockIdx.x * CP;
-    auto mirror = [&](int s) {  // the slot of -kx
-        const int a = s / n2, b = s % n2;
-        return a == 0 ? (b == 0 ? 0 : n2 - b) : (n1 - a) * n2 + n2 - 1 - b;
-    };
-    for (int i = threadIdx.x; i < n; i += 128) tw[i] = g.tw[i];
-    // lanes over columns, then A/B, pairs and elements
-    for (int i = threadIdx.x; i < n * F; i += 128) {
-        const int l = i & (F - 1), e = i / F;
-        const int c = l & (CP - 1), h = l >> cpl;  // h = 2 q + (A: 0, B: 1)
-        if (x0 + c >= n) continue;
-        const size_t off = (h & 1) ? rowB + mirror(x0 + c) : rowA + x0 + c;
-        buf[e * LN + l] = Z[(h >> 1) * M + (size_t)e * stride + off];
+    __shared__ int s_off[64];  // first element of field 0's line l (-1: none)
+    if (threadIdx.x < F) {
+        const int c = threadIdx.x & (CP - 1), h = threadIdx.x >> cpl;  // h = 2 q + (A: 0, B: 1)
+        int x = x0 + c;
+        if (h & 1) {  // the slot of -kx
+            const int k = slot_index(x, n1, n2);
+            x = index_slot(k == 0 ? 0 : n - k, n1, n2);
+        }
+        const int row = D == 3 ? index_slot((h & 1) ? my : ky, n1, n2) * n : 0;
+        s_off[threadIdx.x] = x0 + c < n ? row + x : -1;
     }
     __syncthreads();
+    // lanes over columns, then A/B, pairs and elements
+    for (int i0 = threadIdx.x; i0 < n << flg; i0 += 4 * 128) {
+        V v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int i = i0 + k * 128, l = i & (F - 1), e = i >> flg;
+            if (e < n && s_off[l] >= 0) v[k] = Z[((l >> cpl) >> 1) * M + (size_t)e * stride + s_off[l]];
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int i = i0 + k * 128, l = i & (F - 1), e = i >> flg;
+            if (e < n) sh.buf[e * LN + l] = s_off[l] >= 0 ? v[k] : V{T(0), T(0)};
+        }
+    }
+    sh.fill(g);
+    __syncthreads();
     // the forward transform of field 0's lines alone: half of the buffer
-    lines_forward(buf, alt, LineBuf{n, n1, n2, LN, 1, g.lg - 1}, tw);
+    lines_forward(sh.buf, sh.alt, LineBuf{n, n1, n2, LN, 1, flg}, sh.tw);
+    V* buf = sh.buf;
     Wide<T> acc[5];
-    // multiply: unit (column, k1); slot k1 n2 + k2 of A meets the slot of -k in B
-    for (int u = threadIdx.x; u < n1 << cpl; u += 128) {
-        const int c = u & (CP - 1), k1 = u >> cpl;
+    // multiply: unit (column, slot k1 n2 + k2 of A); -k lies in another slot of B
+    for (int u = threadIdx.x; u < n << cpl; u += 128) {
+        const int c = u & (CP - 1), sl = u >> cpl;
         if (x0 + c >= n) continue;
         const int kx = slot_index(x0 + c, n1, n2);
         const T exy = sp.kernel1d[kx] * (D == 3 ? sp.kernel1d[ky] : T(1));
-        const int k1m = k1 == 0 ? 0 : n1 - k1;
-        for (int k2 = 0; k2 < n2; ++k2) {
-            const int kl = k1 + n1 * k2, km = kl == 0 ? 0 : n - kl;
-            const int eA = (k1 * n2 + k2) * LN + c, eB = (k1m * n2 + (k1 == 0 ? (k2 == 0 ? 0 : n2 - k2) : n2 - 1 - k2)) * LN + c;
+        {
+            const int k1 = sl / n2, k2 = sl - k1 * n2;
+            const int kl = k1 + n1 * k2;
+            const int sm = k1 == 0 ? (k2 == 0 ? 0 : n2 - k2) : (n1 - k1) * n2 + n2 - 1 - k2;
+            const int eA = sl * LN + c, eB = sm * LN + c;
             const T uh = exy * sp.kernel1d[kl];
             V zA[NP], zB[NP];
 #pragma unroll
@@ -610,7 +671,7 @@ __global__ void __launch_bounds__(128) line_last(LineArgs<T> g, const cplx_t<T>*
                     else
                         add_energies4<T, NP>(acc, A, sp, uh * weight, zero);
                 }
-                const T kg = any_grad_k(s == 0 ? kl : km, n, sp.two_pi_over_L);
+                const T kg = sh.ks[s == 0 ? sl : sm];
                 V w[2 * NP];
 #pragma unroll
                 for (int K = 0; K < 2 * NP; ++K) {
@@ -634,13 +695,12 @@ __global__ void __launch_bounds__(128) line_last(LineArgs<T> g, const cplx_t<T>*
         }
     }
     __syncthreads();
-    lines_inverse(buf, alt, LineBuf{n, n1, n2, LN, 1, g.lg}, tw);
-    for (int i = threadIdx.x; i < n * LN; i += 128) {
-        const int l = i & (LN - 1), e = i >> g.lg;
-        const int c = l & (CP - 1), h = (l & (F - 1)) >> cpl, f = l >= F ? 2 : 0;
-        if (x0 + c >= n || (self && (h & 1))) continue;
-        const size_t off = (h & 1) ? rowB + mirror(x0 + c) : rowA + x0 + c;
-        H[(3 * (h >> 1) + f) * M + (size_t)e * stride + off] = buf[e * LN + l];
+    lines_inverse(sh.buf, sh.alt, LineBuf{n, n1, n2, LN, 1, g.lg}, sh.tw);
+    for (int i = threadIdx.x; i < n << g.lg; i += 128) {
+        const int l = i & (LN - 1), e = i >> g.lg, lf = l & (F - 1);
+        const int h = lf >> cpl, f = l >= F ? 2 : 0;
+        if (s_off[lf] < 0 || (self && (h & 1))) continue;
+        H[(3 * (h >> 1) + f) * M + (size_t)e * stride + s_off[lf]] = sh.buf[e * LN + l];
     }
     if (partials) {
         const size_t b = (size_t)blockIdx.y * gridDim.x + blockIdx.x;

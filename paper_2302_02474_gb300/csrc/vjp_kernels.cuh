@@ -205,12 +205,14 @@ __global__ void __launch_bounds__(256) vjp_spread_tiled(BeadParams<float> p, Bea
                         const float w = st.wx[a] * wyz;
 #pragma unroll
                         for (int d = 0; d < 3; ++d) {
+                            // x = hi 2^20 + lo, both rounded to nearest by adding 1.5 2^23
+                            // (|hi| <= 2^20, |lo| <= 2^19; the sum's low bits are the integer)
                             const float x = __fmul_rn(w, l[d]);
-                            const float hi = rintf(x * 9.5367431640625e-07f);   // 2^-20
-                            const float lo = __fmaf_rn(-1048576.0f, hi, x);     // exact
+                            const float hb = __fmaf_rn(x, 9.5367431640625e-07f, 12582912.0f);
+                            const float lo = __fmaf_rn(-1048576.0f, __fsub_rn(hb, 12582912.0f), x);  // exact
                             const int at = d * 2 * W3 + row + 2 * a;
-                            atomicAdd(s_hi + at, __float2int_rn(hi));
-                            atomicAdd(s_lo + at, __float2int_rn(lo));
+                            atomicAdd(s_hi + at, __float_as_int(hb) - 0x4B400000);
+                            atomicAdd(s_lo + at, __float_as_int(__fadd_rn(lo, 12582912.0f)) - 0x4B400000);
                         }
                     }
                 }

@@ -477,8 +477,10 @@ tild_status tild_set_launch_shapes(tild_ctx* ctx, int plane_threads, int z_colum
  * with their own chains, box, grid, chi, kappa, a and seed; same precision
  * and device) together. When every replica is FP32 with pmeorder 1, the ik
  * force, no charges, two species and a grid of 24, 32, 40, 48 or 64 points
- * per edge, the steps between two re-binnings of all replicas are ONE
- * persistent cooperative launch: its CTAs walk a table of the work items of
+ * per edge, the steps between two re-binnings of all replicas can be ONE
+ * persistent cooperative launch (the default for fewer than 8 replicas, or as
+ * tild_batch_set_persistent, tild_batch_set_wait_limit or the autotuner
+ * choose): its CTAs walk a table of the work items of
  * every replica (xy planes, z-pass tiles, bead tiles), stage by stage, and
  * meet at grid-wide barriers whose waits are bounded
  * (tild_batch_set_wait_limit; a wait that runs out is reported as

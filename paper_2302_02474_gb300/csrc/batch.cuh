@@ -4,7 +4,8 @@
 // Persistent path (FP32, pmeorder 1, ik force, no charges, two species,
 // grids 24, 32, 40, 48 or 64): the K steps between two re-binnings of all
 // replicas are one cooperative launch (batch_persistent.cuh) walking a table
-// of work items of every replica, stage by stage. Otherwise replicas are
+// of work items of every replica, stage by stage; it is the default for small
+// batches (kPersistentMax). Otherwise replicas are
 // grouped by (grid size, assignment order) and every step issues four
 // launches per group (forward xy, z pass, inverse xy, bead kernel) whose
 // blocks look up their replica in device tables of per-replica arguments.
@@ -236,6 +237,7 @@ template <typename T> class BatchEngine final : public BatchBase {
     // group's grid allows it, else 512; the alternative z tile if zalt)
     void apply_config(bool pers, int nt, bool zalt) {
         persistent_ = pers && p_grids_[0] > 0;
+        by_rule_ = false;
         if (persistent_) {
             p_var_ = nt;
             p_grid_ = p_grids_[nt];
@@ -256,6 +258,7 @@ template <typename T> class BatchEngine final : public BatchBase {
             return TILD_EUNSUPPORTED;
         }
         persistent_ = pers;
+        by_rule_ = false;
         invalidate_graph();
         return TILD_OK;
     }
@@ -264,6 +267,7 @@ template <typename T> class BatchEngine final : public BatchBase {
     // arrivals the barrier waits for beyond the grid (each extra one makes
     // every wait run out). Returns TILD_EUNSUPPORTED without the persistent path.
     tild_status set_wait(int64_t wait_ns, int extra) override {
+        if (by_rule_ && p_grids_[0] > 0) persistent_ = true;  // whoever sets its limit steps through it
         if (!persistent_) {
             err = "batch: these replicas are stepped without the persistent kernel";
             return TILD_EUNSUPPORTED;
@@ -363,6 +367,7 @@ template <typename T> class BatchEngine final : public BatchBase {
     std::vector<Group> groups_;
     // persistent path
     bool persistent_ = false, graph_ok_ = true;
+    bool by_rule_ = true;  // the path is the default's, not the caller's or the autotuner's
     PersistentPlan<T> plan_{};
     const BeadArgs<T>* p_bead_[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};  // [pos parity][u, id parity]
     int p_grid_ = 0;             // CTAs of the chosen variant (0: no persistent path)
@@ -472,7 +477,7 @@ template <typename T> class BatchEngine final : public BatchBase {
         p_grid_ = p_grids_[p_var_];
         plan_.expected = (unsigned)p_grid_;
         plan_.wait_ns = 2000000000ll;  // 2 s
-        persistent_ = true;
+        persistent_ = (int)reps_.size() < kPersistentMax;
         return TILD_OK;
     }
 
@@ -509,6 +514,12 @@ template <typename T> class BatchEngine final : public BatchBase {
     int cur_pos_ = 0, cur_uid_ = 0, steps_since_sort_ = 0;
     cudaGraphExec_t graph_ = nullptr;
     static constexpr int kSortStreams = 16;
+    // Batches of fewer replicas than this start on the persistent kernel (one
+    // launch per run of steps, which callers may count on), larger ones on the
+    // group launches, which are faster at every size (us per step of replicas
+    // of 4,000 to 40,000 beads, persistent / groups: 6 replicas 92 / 46, 16
+    // replicas 172 / 83, 64 replicas 659 / 365).
+    static constexpr int kPersistentMax = 8;
     std::vector<std::pair<cudaStream_t, cudaEvent_t>> sort_streams_;
     cudaEvent_t fork_ = nullptr;
 

@@ -101,6 +101,21 @@ template <typename T> __device__ __forceinline__ T wrap_coord(T x, T L, T inv_L)
     return (y >= L || !(y >= T(-0.5) * L)) ? T(0) : y;
 }
 
+// The integrators' updates (see BeadParams) of one component, each sum with its
+// fused products written out: the tiled and the per-bead kernels give the same
+// bits. f: force, g: normal.
+template <typename T> __device__ __forceinline__ T velocity_of(const BeadParams<T>& p, T u, T f, T g) {
+    return fma_rn(p.vg, g, fma_rn(p.vf, f, mul_rn(p.vu, u)));
+}
+template <typename T> __device__ __forceinline__ T carried_of(const BeadParams<T>& p, T v, T f, T g) {
+    return fma_rn(p.wg, g, fma_rn(p.wf, f, mul_rn(p.wu, v)));
+}
+template <typename T> __device__ __forceinline__ void step_update(const BeadParams<T>& p, T& x, T& u, T f, T g) {
+    const T h = fma_rn(p.sg, g, fma_rn(p.sf, f, mul_rn(p.su, u)));
+    x = wrap_coord(fma_rn(p.se, g, fma_rn(p.sd, h, x)), p.L, p.inv_L);
+    u = fma_rn(p.sk, g, mul_rn(p.sh, h));
+}
+
 // acc += |s d|^2
 template <typename T> __device__ __forceinline__ void add_squares(Wide<T>& acc, T dx, T dy, T dz, T s) {
     dx *= s;
@@ -549,9 +564,9 @@ __device__ __forceinline__ void bead_kernel_body(const BeadParams<T>& p, const B
                     // v^n = vu u + vf F + vg xi^n (the integrator's total force enters)
                     normal3<T> g = {T(0), T(0), T(0)};
                     if (p.vg != T(0)) g = gaussian3((uint32_t)bid, *bf.step, p.seed, T(0));
-                    const T vx = p.vu * ux + p.vf * fx + p.vg * g.a;
-                    const T vy = p.vu * uy + p.vf * fy + p.vg * g.b;
-                    const T vz = p.vu * uz + p.vf * fz + p.vg * g.c;
+                    const T vx = velocity_of(p, ux, fx, g.a);
+                    const T vy = velocity_of(p, uy, fy, g.b);
+                    const T vz = velocity_of(p, uz, fz, g.c);
                     if (sums) {
                         add_squares(acc[MODE == kModeForce ? 1 : 0], vx, vy, vz, p.e_vel);
                         acc[MODE == kModeForce ? 2 : 0].add(fx);
@@ -582,23 +597,20 @@ __device__ __forceinline__ void bead_kernel_body(const BeadParams<T>& p, const B
                     }
                     normal3<T> g = {T(0), T(0), T(0)};
                     if (p.wg != T(0)) g = gaussian3((uint32_t)bid, *bf.step, p.seed, T(0));
-                    bf.ux[i] = p.wu * vx + p.wf * fx + p.wg * g.a;
-                    bf.uy[i] = p.wu * vy + p.wf * fy + p.wg * g.b;
-                    bf.uz[i] = p.wu * vz + p.wf * fz + p.wg * g.c;
+                    bf.ux[i] = carried_of(p, vx, fx, g.a);
+                    bf.uy[i] = carried_of(p, vy, fy, g.b);
+                    bf.uz[i] = carried_of(p, vz, fz, g.c);
                 } else if (MODE == kModeStep) {
                     const normal3<T> g = gaussian3((uint32_t)bid, step_next - (uint64_t)p.noise_lag, p.seed, T(0));
-                    const T hx = p.su * ux + p.sf * fx + p.sg * g.a;
-                    const T hy = p.su * uy + p.sf * fy + p.sg * g.b;
-                    const T hz = p.su * uz + p.sf * fz + p.sg * g.c;
-                    x = wrap_coord(x + p.sd * hx + p.se * g.a, p.L, p.inv_L);
-                    y = wrap_coord(y + p.sd * hy + p.se * g.b, p.L, p.inv_L);
-                    z = wrap_coord(z + p.sd * hz + p.se * g.c, p.L, p.inv_L);
+                    step_update(p, x, ux, fx, g.a);
+                    step_update(p, y, uy, fy, g.b);
+                    step_update(p, z, uz, fz, g.c);
                     bf.qx[i] = x;
                     bf.qy[i] = y;
                     bf.qz[i] = z;
-                    bf.ux[i] = p.sh * hx + p.sk * g.a;
-                    bf.uy[i] = p.sh * hy + p.sk * g.b;
-                    bf.uz[i] = p.sh * hz + p.sk * g.c;
+                    bf.ux[i] = ux;
+                    bf.uy[i] = uy;
+                    bf.uz[i] = uz;
                     st.set(x, y, z, p.inv_dx);
                     inside = patch_local(st, org, l);
                 }

@@ -1100,7 +1100,9 @@ template <typename T> class Engine final : public EngineBase {
     }
     size_t gaxis_smem() const { return ((size_t)n_ + 2 * (size_t)gaxis_lines() * (n_ + 1)) * sizeof(V); }
     // blocks of the bead kernel (its FP64 partial sums)
-    size_t bead_blocks() const { return generic_ ? (size_t)blocks(cfg_->n_beads) : (size_t)tiles_ * tiles_ * tiles_; }
+    size_t bead_blocks() const {
+        return per_bead() ? ((size_t)cfg_->n_beads + bead_threads() - 1) / bead_threads() : (size_t)n_tiles_;
+    }
     tild_status ensure_partials() {
         const size_t need = 5 * std::max(bead_blocks(), z_blocks()) * sizeof(double);
         return device_buffer(&partials_, partials_bytes_, need);
@@ -1968,20 +1970,39 @@ template <typename T> class Engine final : public EngineBase {
         TILD_CUDA(cudaGetLastError());
         return TILD_OK;
     }
+    // Whether beads go through the per-bead kernel (one thread per bead, fields
+    // and density in global memory) instead of the tiled one. Measured on melts
+    // of 20-bead chains (us of the bead kernel in the step, tiled / per bead):
+    //   FP64: bound by the FP64 unit (two operations per clock and SM), which
+    //   the tiles of a small grid leave idle on most SMs; order 1, 32^3, 20,000
+    //   beads 44.9 / 22.5, 64^3, 200,000 168 / 131; order 3 118 / 55, 419 / 326.
+    //   FP32, order 1: up to about 48,000 beads latency decides, and a tile's
+    //   patch adds barriers and a flush to the chain (24^3, 4,060 beads: step
+    //   15.6 / 14.4; 48^3, 40,000: 21.1 / 20.4); beyond that the global atomics
+    //   do (64^3, 200,000: 30.6 / 37.4), and at higher orders at every size
+    //   (order 3, 24^3: 20.2 / 22.5).
+    bool per_bead() const {
+        if (generic_) return true;
+        if (analytic()) return false;
+        return sizeof(T) == 8 || (P_ == 2 && cfg_->n_beads <= 48000);
+    }
+    // Threads per block: small blocks spread few beads over all SMs (FP64,
+    // 32^3: 22.5 us with 32 threads, 28.7 with 128).
+    int bead_threads() const { return !per_bead() ? 256 : sizeof(T) == 8 ? 32 : cfg_->n_beads <= 100000 ? 64 : 256; }
     template <int P, int D> tild_status bead_generic(int mode, const BeadBuffers<T>& bf) {
         const BeadParams<T> p = bead_params();
-        const unsigned g = blocks(cfg_->n_beads);
+        const unsigned bt = (unsigned)bead_threads(), g = (unsigned)bead_blocks();
         switch (mode) {
-            case kModeSpread: generic_bead_kernel<P, kModeSpread, T, D><<<g, 256, 0, stream_>>>(p, bf, nz_); break;
-            case kModeForce: generic_bead_kernel<P, kModeForce, T, D><<<g, 256, 0, stream_>>>(p, bf, nz_); break;
-            case kModeSetVel: generic_bead_kernel<P, kModeSetVel, T, D><<<g, 256, 0, stream_>>>(p, bf, nz_); break;
-            default: generic_bead_kernel<P, kModeStep, T, D><<<g, 256, 0, stream_>>>(p, bf, nz_); break;
+            case kModeSpread: generic_bead_kernel<P, kModeSpread, T, D><<<g, bt, 0, stream_>>>(p, bf, nz_); break;
+            case kModeForce: generic_bead_kernel<P, kModeForce, T, D><<<g, bt, 0, stream_>>>(p, bf, nz_); break;
+            case kModeSetVel: generic_bead_kernel<P, kModeSetVel, T, D><<<g, bt, 0, stream_>>>(p, bf, nz_); break;
+            default: generic_bead_kernel<P, kModeStep, T, D><<<g, bt, 0, stream_>>>(p, bf, nz_); break;
         }
         TILD_CUDA(cudaGetLastError());
         return TILD_OK;
     }
     template <int P> tild_status bead_p(int mode, const BeadBuffers<T>& bf) {
-        if (generic_) return cfg_->dim == 2 ? bead_generic<P, 2>(mode, bf) : bead_generic<P, 3>(mode, bf);
+        if (per_bead()) return cfg_->dim == 2 ? bead_generic<P, 2>(mode, bf) : bead_generic<P, 3>(mode, bf);
         return NS_ == 4 ? bead_pn<P, 4>(mode, bf) : bead_pn<P, 2>(mode, bf);
     }
     tild_status launch_bead(int mode, const BeadBuffers<T>& bf) {

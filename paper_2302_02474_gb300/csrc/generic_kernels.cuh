@@ -779,9 +779,9 @@ __global__ void __launch_bounds__(256) generic_bead_kernel(BeadParams<T> p, Bead
             if (MODE == kModeForce) {
                 normal3<T> g = {T(0), T(0), T(0)};
                 if (p.vg != T(0)) g = gaussian3((uint32_t)bid, *bf.step, p.seed, T(0));
-                const T vx = p.vu * ux + p.vf * fx + p.vg * g.a;
-                const T vy = p.vu * uy + p.vf * fy + p.vg * g.b;
-                const T vz = D == 3 ? p.vu * uz + p.vf * fz + p.vg * g.c : T(0);
+                const T vx = velocity_of(p, ux, fx, g.a);
+                const T vy = velocity_of(p, uy, fy, g.b);
+                const T vz = D == 3 ? velocity_of(p, uz, fz, g.c) : T(0);
                 if (sums) {
                     add_squares(acc[1], vx, vy, vz, p.e_vel);
                     acc[2].add(fx);
@@ -812,23 +812,20 @@ __global__ void __launch_bounds__(256) generic_bead_kernel(BeadParams<T> p, Bead
                 }
                 normal3<T> g = {T(0), T(0), T(0)};
                 if (p.wg != T(0)) g = gaussian3((uint32_t)bid, *bf.step, p.seed, T(0));
-                bf.ux[i] = p.wu * vx + p.wf * fx + p.wg * g.a;
-                bf.uy[i] = p.wu * vy + p.wf * fy + p.wg * g.b;
-                bf.uz[i] = D == 3 ? p.wu * vz + p.wf * fz + p.wg * g.c : T(0);
+                bf.ux[i] = carried_of(p, vx, fx, g.a);
+                bf.uy[i] = carried_of(p, vy, fy, g.b);
+                bf.uz[i] = D == 3 ? carried_of(p, vz, fz, g.c) : T(0);
             } else {  // step
                 const normal3<T> g = gaussian3((uint32_t)bid, *bf.step - (uint64_t)p.noise_lag, p.seed, T(0));
-                const T hx = p.su * ux + p.sf * fx + p.sg * g.a;
-                const T hy = p.su * uy + p.sf * fy + p.sg * g.b;
-                const T hz = p.su * uz + p.sf * fz + p.sg * g.c;
-                x = wrap_coord(x + p.sd * hx + p.se * g.a, p.L, p.inv_L);
-                y = wrap_coord(y + p.sd * hy + p.se * g.b, p.L, p.inv_L);
-                z = D == 3 ? wrap_coord(z + p.sd * hz + p.se * g.c, p.L, p.inv_L) : T(0);
+                step_update(p, x, ux, fx, g.a);
+                step_update(p, y, uy, fy, g.b);
+                if (D == 3) step_update(p, z, uz, fz, g.c);
                 bf.qx[i] = x;
                 bf.qy[i] = y;
                 bf.qz[i] = z;
-                bf.ux[i] = p.sh * hx + p.sk * g.a;
-                bf.uy[i] = p.sh * hy + p.sk * g.b;
-                bf.uz[i] = D == 3 ? p.sh * hz + p.sk * g.c : T(0);
+                bf.ux[i] = ux;
+                bf.uy[i] = uy;
+                bf.uz[i] = uz;
                 st.set(x, y, z, p.inv_dx);
             }
         }

@@ -101,6 +101,11 @@ template <typename T> __device__ __forceinline__ T wrap_coord(T x, T L, T inv_L)
     return (y >= L || !(y >= T(-0.5) * L)) ? T(0) : y;
 }
 
+// Whether any of the three is infinite or NaN (0 times a finite value is 0).
+template <typename T> __device__ __forceinline__ bool not_finite(T a, T b, T c) {
+    return !(fma_rn(a, T(0), fma_rn(b, T(0), mul_rn(c, T(0)))) == T(0));
+}
+
 // The integrators' updates (see BeadParams) of one component, each sum with its
 // fused products written out: the tiled and the per-bead kernels give the same
 // bits. f: force, g: normal.
@@ -126,7 +131,9 @@ template <typename T> __device__ __forceinline__ void add_squares(Wide<T>& acc, 
     acc.add_prod(dz, dz);
 }
 
-template <typename T> __device__ __forceinline__ T min_image(T d, T L, T inv_L) { return d - L * rint(d * inv_L); }
+template <typename T> __device__ __forceinline__ T min_image(T d, T L, T inv_L) {
+    return d - L * round_prod(d, inv_L);
+}
 
 // Bead slots carry the bead id in bits 0..28 and the species in bits 29..31.
 constexpr int kSpeciesShift = 29;
@@ -388,7 +395,9 @@ __device__ __forceinline__ void bead_kernel_body(const BeadParams<T>& p, const B
         s_rowbase[i] = (pwrap(org.z + lz, p.n) * p.n + pwrap(org.y + ly, p.n)) * p.n;
     }
     if (kSpread) {
-        for (int i = threadIdx.x; i < SM::patches * PT::W3; i += blockDim.x) patch[i] = 0;
+        // 16-byte stores (the patch area is padded to 32 bytes)
+        constexpr int kWords = (SM::patches * PT::W3 * (int)sizeof(patch_t) + 15) / 16;
+        for (int i = threadIdx.x; i < kWords; i += blockDim.x) reinterpret_cast<uint4*>(patch)[i] = make_uint4(0, 0, 0, 0);
     }
     __syncthreads();
     if (AN && kForce && row_lane) {
@@ -511,7 +520,7 @@ __device__ __forceinline__ void bead_kernel_body(const BeadParams<T>& p, const B
 #pragma unroll
                 for (int k = 0; k < 2; ++k) {
                     const int s = k == 0 ? nb.x : nb.y;
-                    if (s >= c0 && s < c0 + cnt) {
+                    if ((unsigned)(s - c0) < (unsigned)cnt) {
                         nx[k] = s_pos[s - c0];
                         ny[k] = s_pos[kBeadChunk + s - c0];
                         nz[k] = s_pos[2 * kBeadChunk + s - c0];
@@ -559,7 +568,7 @@ __device__ __forceinline__ void bead_kernel_body(const BeadParams<T>& p, const B
                     fz -= p.k_bond * dz;
                     if (MODE == kModeForce && sums && nid_of(s) > bid) add_squares(acc[0], dx, dy, dz, p.e_len);
                 });
-                if (!(isfinite(fx) && isfinite(fy) && isfinite(fz))) atomicOr(bf.err, kErrNonFinite);
+                if (not_finite(fx, fy, fz)) atomicOr(bf.err, kErrNonFinite);
                 if (MODE == kModeForce) {
                     // v^n = vu u + vf F + vg xi^n (the integrator's total force enters)
                     normal3<T> g = {T(0), T(0), T(0)};
@@ -711,7 +720,7 @@ __global__ void __launch_bounds__(256) adjoint_kernel(BeadParams<T> p, BeadBuffe
         if (nb.x >= 0) bond(nb.x);
         if (nb.y >= 0) bond(nb.y);
         for_each_extra_bond(nb, bf.ext, bond);
-        if (!(isfinite(gx) && isfinite(gy) && isfinite(gz))) atomicOr(bf.err, kErrNonFinite);
+        if (not_finite(gx, gy, gz)) atomicOr(bf.err, kErrNonFinite);
         if (grad_out) {
             grad_out[3 * (size_t)bid + 0] = gx;
             grad_out[3 * (size_t)bid + 1] = gy;

@@ -50,7 +50,12 @@ template <> struct FixedPoint<float> {
     using patch_t = unsigned int;
     static constexpr double scale = 4194304.0;  // 2^22
     static constexpr int max_tile_beads = 1023;
-    static __device__ __forceinline__ unsigned int to_patch(float w) { return __float2uint_rn(w * 4194304.0f); }
+    // round(w 2^22) for w in [0, 1]: adding 1.5 2^23 rounds to nearest and leaves
+    // the integer in the low bits (the product is exact). The conversion
+    // instruction runs at a quarter of the rate of these two.
+    static __device__ __forceinline__ unsigned int to_patch(float w) {
+        return __float_as_uint(__fmaf_rn(w, 4194304.0f, 12582912.0f)) - 0x4B400000u;
+    }
     static __device__ __forceinline__ unsigned long long to_grid(float w) { return to_patch(w); }
 };
 // FP64: one 64-bit shared word per point and species.
@@ -235,6 +240,23 @@ __host__ __device__ __forceinline__ int pwrap(int j, int n) { return j < 0 ? j +
 
 // ------------------------------------------------- assignment weights
 
+// floor(s) as a value and as an integer. FP32 (|s| < 2^22; grid coordinates are
+// at most a few hundred): the sum with 1.5 2^23 rounded down holds the integer
+// in its low bits, without the slow conversion and rounding instructions.
+__device__ __forceinline__ float floor_int(float s, int& j) {
+    const float r = __fadd_rd(s, 12582912.0f);
+    j = __float_as_int(r) - 0x4B400000;
+    return __fsub_rn(r, 12582912.0f);
+}
+__device__ __forceinline__ double floor_int(double s, int& j) {
+    const double f = floor(s);
+    j = (int)f;
+    return f;
+}
+// round to nearest (even) of a x b, |a b| < 2^22 in FP32
+__device__ __forceinline__ float round_prod(float a, float b) { return __fsub_rn(__fmaf_rn(a, b, 12582912.0f), 12582912.0f); }
+__device__ __forceinline__ double round_prod(double a, double b) { return rint(a * b); }
+
 // Charge-assignment weights of order P (P points per dimension), the
 // closed-form polynomials of Deserno & Holm (J. Chem. Phys. 109, 7678,
 // 1998, appendix) cited by the paper for its spline weights. s is the
@@ -244,34 +266,29 @@ __host__ __device__ __forceinline__ int pwrap(int j, int n) { return j < 0 ? j +
 //         nearest grid point.
 template <int P, typename T> __device__ __forceinline__ void dh_weights(T s, int& j0, T (&w)[P]) {
     if constexpr (P == 2) {
-        const T f = floor(s);
-        const T t = s - f;
-        j0 = (int)f;
+        const T t = s - floor_int(s, j0);
         w[0] = T(1) - t;
         w[1] = t;
     } else if constexpr (P == 3) {
-        const T f = floor(s + T(0.5));
-        const T t = s - f;
-        j0 = (int)f - 1;
+        const T t = s - floor_int(s + T(0.5), j0);
+        --j0;
         w[0] = T(0.5) * (T(0.5) - t) * (T(0.5) - t);
         w[1] = T(0.75) - t * t;
         w[2] = T(0.5) * (T(0.5) + t) * (T(0.5) + t);
     } else if constexpr (P == 4) {
-        const T f = floor(s);
-        const T t = s - f;
+        const T t = s - floor_int(s, j0);
         const T t2 = t * t, t3 = t2 * t, u = T(1) - t;
-        j0 = (int)f - 1;
+        --j0;
         w[0] = u * u * u * T(1.0 / 6.0);
         w[1] = (T(4) - T(6) * t2 + T(3) * t3) * T(1.0 / 6.0);
         w[2] = (T(1) + T(3) * t + T(3) * t2 - T(3) * t3) * T(1.0 / 6.0);
         w[3] = t3 * T(1.0 / 6.0);
     } else {
         static_assert(P == 5, "orders 1..4 (P = 2..5)");
-        const T f = floor(s + T(0.5));
-        const T t = s - f;
+        const T t = s - floor_int(s + T(0.5), j0);
         const T t2 = t * t, t3 = t2 * t, t4 = t2 * t2;
         const T a = T(1) - T(2) * t, b = T(1) + T(2) * t;
-        j0 = (int)f - 2;
+        j0 -= 2;
         w[0] = a * a * a * a * T(1.0 / 384.0);
         w[1] = (T(19) - T(44) * t + T(24) * t2 + T(16) * t3 - T(16) * t4) * T(1.0 / 96.0);
         w[2] = (T(115) - T(120) * t2 + T(48) * t4) * T(1.0 / 192.0);

@@ -769,7 +769,7 @@ __global__ void __launch_bounds__(256) generic_bead_kernel(BeadParams<T> p, Bead
             if (nb.x >= 0) bond(nb.x);
             if (nb.y >= 0) bond(nb.y);
             for_each_extra_bond(nb, bf.ext, bond);
-            if (!(isfinite(fx) && isfinite(fy) && isfinite(fz))) atomicOr(bf.err, kErrNonFinite);
+            if (not_finite(fx, fy, fz)) atomicOr(bf.err, kErrNonFinite);
             T ux = 0, uy = 0, uz = 0;
             if (MODE != kModeSetVel) {
                 ux = bf.ux[i];

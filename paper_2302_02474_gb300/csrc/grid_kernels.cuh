@@ -755,78 +755,85 @@ __device__ __forceinline__ void z_tile(cplx_t<T>* buf, cplx_t<T>* tw, const cplx
         if (active) {
             reg_dft<N2, -1, V>::run(va);
             reg_dft<N2, -1, V>::run(vb);
-            const int sides = PAIRED ? R : 1;
-#pragma unroll 1
-            for (int s = 0; s < sides; ++s) {
-                // unit (r, c, k1): X[k1 + N1 k2] = va[k2]; the mirror of output
-                // k2 is vb[(N2 - k2) mod N2] when k1 = 0, else vb[N2 - 1 - k2]
-                const int kx = kx_of_pos<N>(p0 + c), kyr = ky[r];
-                const T exy = e1[kx] * e1[kyr];
-                const T exy2 = EL ? e2[kx] * e2[kyr] : T(0);
-                const T qx = raw_k<T, N>(kx, sp.two_pi_over_L), qy = raw_k<T, N>(kyr, sp.two_pi_over_L);
-                const T kxy2 = fma_rn(qx, qx, mul_rn(qy, qy));  // the Nyquist index counts as -n/2
-                const T mxy = freq_sq<T, N>(kx) + freq_sq<T, N>(kyr);
-                // k and -k contribute the same: a paired row counts its units twice
-                const T weight = PAIRED && R == 2 ? T(2) : T(1);
-                const bool zero = kx == 0 && kyr == 0;
-                V g[N2], gz[G_ONLY ? 1 : N2];
+            // unit (r, c, k1): X[k1 + N1 k2] = va[k2]; the mirror of output k2 is
+            // vb[(N2 - k2) mod N2] when k1 = 0, else vb[N2 - 1 - k2]. Both
+            // densities are real, so the mirror wavevector's products are the
+            // conjugates of this one's (u_hat and the Coulomb factor are even):
+            // one multiply serves both outputs, which replace va and vb.
+            const int kx = kx_of_pos<N>(p0 + c), kyr = ky[r];
+            const T exy = e1[kx] * e1[kyr];
+            const T exy2 = EL ? e2[kx] * e2[kyr] : T(0);
+            const T qx = raw_k<T, N>(kx, sp.two_pi_over_L), qy = raw_k<T, N>(kyr, sp.two_pi_over_L);
+            const T kxy2 = fma_rn(qx, qx, mul_rn(qy, qy));  // the Nyquist index counts as -n/2
+            const T mxy = freq_sq<T, N>(kx) + freq_sq<T, N>(kyr);
+            const T weight = PAIRED && R == 2 ? T(2) : T(1);  // k and -k contribute the same
+            const bool zero = kx == 0 && kyr == 0;
+            V ga[N2], gb[PAIRED ? N2 : 1];
 #pragma unroll
-                for (int k2 = 0; k2 < N2; ++k2) {
-                    const V Z = va[k2], Zm = k1 == 0 ? vb[(N2 - k2) % N2] : vb[N2 - 1 - k2];
-                    const int kz = k1 + N1 * k2;
-                    const T uh = exy * e1[kz];
-                    // rho~_A = (Z + conj Zm)/2, rho~_B = -i (Z - conj Zm)/2
-                    const V A = {T(0.5) * (Z.x + Zm.x), T(0.5) * (Z.y - Zm.y)};
-                    const V B = {T(0.5) * (Z.y + Zm.y), -T(0.5) * (Z.x - Zm.x)};
-                    V wA = {mul_rn(uh, fma_rn(sp.eAA, A.x, mul_rn(sp.eAB, B.x))),
-                            mul_rn(uh, fma_rn(sp.eAA, A.y, mul_rn(sp.eAB, B.y)))};
-                    V wB = {mul_rn(uh, fma_rn(sp.eAB, A.x, mul_rn(sp.eBB, B.x))),
-                            mul_rn(uh, fma_rn(sp.eAB, A.y, mul_rn(sp.eBB, B.y)))};
-                    if (WANT_E && s == 0)
-                        add_energies<T, WANT_E>(acc, A, B, uh, sp.e_rho, weight, zero && kz == 0,
-                                                mxy + freq_sq<T, N>(kz));
-                    if (EL) {
-                        // w_K += q_K c(k) rho~_q with rho~_q = q_A rho~_A + q_B rho~_B
-                        const T qzv = raw_k<T, N>(kz, sp.two_pi_over_L);
-                        const T k2sq = fma_rn(qzv, qzv, kxy2);
-                        const T gq = k2sq > T(0) ? exy2 * e2[kz] * recip(k2sq) : T(0);
-                        const V rq = {fma_rn(sp.qA, A.x, mul_rn(sp.qB, B.x)), fma_rn(sp.qA, A.y, mul_rn(sp.qB, B.y))};
-                        const T cA = mul_rn(sp.el_scale * gq, sp.qA), cB2 = mul_rn(sp.el_scale * gq, sp.qB);
-                        wA.x = fma_rn(cA, rq.x, wA.x);
-                        wA.y = fma_rn(cA, rq.y, wA.y);
-                        wB.x = fma_rn(cB2, rq.x, wB.x);
-                        wB.y = fma_rn(cB2, rq.y, wB.y);
-                        if (WANT_E && s == 0) {
-                            Wide<T> f;
-                            f.add_prod(rq.x * sp.e_rho, rq.x * sp.e_rho);
-                            f.add_prod(rq.y * sp.e_rho, rq.y * sp.e_rho);
-                            acc[4].add(f.times(weight * gq));
-                        }
+            for (int k2 = 0; k2 < N2; ++k2) {
+                const V Z = va[k2], Zm = k1 == 0 ? vb[(N2 - k2) % N2] : vb[N2 - 1 - k2];
+                const int kz = k1 + N1 * k2;
+                const T uh = exy * e1[kz];
+                // rho~_A = (Z + conj Zm)/2, rho~_B = -i (Z - conj Zm)/2
+                const V A = {T(0.5) * (Z.x + Zm.x), T(0.5) * (Z.y - Zm.y)};
+                const V B = {T(0.5) * (Z.y + Zm.y), -T(0.5) * (Z.x - Zm.x)};
+                V wA = {mul_rn(uh, fma_rn(sp.eAA, A.x, mul_rn(sp.eAB, B.x))),
+                        mul_rn(uh, fma_rn(sp.eAA, A.y, mul_rn(sp.eAB, B.y)))};
+                V wB = {mul_rn(uh, fma_rn(sp.eAB, A.x, mul_rn(sp.eBB, B.x))),
+                        mul_rn(uh, fma_rn(sp.eAB, A.y, mul_rn(sp.eBB, B.y)))};
+                if (WANT_E)
+                    add_energies<T, WANT_E>(acc, A, B, uh, sp.e_rho, weight, zero && kz == 0, mxy + freq_sq<T, N>(kz));
+                if (EL) {
+                    // w_K += q_K c(k) rho~_q with rho~_q = q_A rho~_A + q_B rho~_B
+                    const T qzv = raw_k<T, N>(kz, sp.two_pi_over_L);
+                    const T k2sq = fma_rn(qzv, qzv, kxy2);
+                    const T gq = k2sq > T(0) ? exy2 * e2[kz] * recip(k2sq) : T(0);
+                    const V rq = {fma_rn(sp.qA, A.x, mul_rn(sp.qB, B.x)), fma_rn(sp.qA, A.y, mul_rn(sp.qB, B.y))};
+                    const T cA = mul_rn(sp.el_scale * gq, sp.qA), cB2 = mul_rn(sp.el_scale * gq, sp.qB);
+                    wA.x = fma_rn(cA, rq.x, wA.x);
+                    wA.y = fma_rn(cA, rq.y, wA.y);
+                    wB.x = fma_rn(cB2, rq.x, wB.x);
+                    wB.y = fma_rn(cB2, rq.y, wB.y);
+                    if (WANT_E) {
+                        Wide<T> f;
+                        f.add_prod(rq.x * sp.e_rho, rq.x * sp.e_rho);
+                        f.add_prod(rq.y * sp.e_rho, rq.y * sp.e_rho);
+                        acc[4].add(f.times(weight * gq));
                     }
-                    g[k2] = {-(wA.y + wB.x), wA.x - wB.y};  // i (w~_A + i w~_B); k_x, k_y follow in the xy pass
-                    if (!G_ONLY) gz[k2] = c_scale_rn(g[k2], grad_k<T, N>(kz, sp.two_pi_over_L));
                 }
-                V* o = buf + r * TS + k1 * N2 * C + c;
+                ga[k2] = {-(wA.y + wB.x), wA.x - wB.y};  // i (w~_A + i w~_B); k_x, k_y follow in the xy pass
+                if constexpr (PAIRED) gb[k2] = {wA.y - wB.x, wA.x + wB.y};  // the same of -k
+            }
+            // the inverse transform's first stage of G and G_z of one unit
+            auto emit = [&](V (&g)[N2], int row, int col, int kk) {
+                V* o = buf + row * TS + kk * N2 * C + col;
+                if constexpr (!G_ONLY) {
+                    V gz[N2];
+#pragma unroll
+                    for (int k2 = 0; k2 < N2; ++k2) gz[k2] = c_scale_rn(g[k2], grad_k<T, N>(kk + N1 * k2, sp.two_pi_over_L));
+                    reg_dft<N2, +1, V>::run(gz);
+#pragma unroll
+                    for (int m = 0; m < N2; ++m) o[R * TS + m * C] = m == 0 ? gz[0] : c_mul(gz[m], twiddle<+1>(tw, kk * m));
+                }
                 reg_dft<N2, +1, V>::run(g);
 #pragma unroll
-                for (int m = 0; m < N2; ++m) o[m * C] = m == 0 ? g[0] : c_mul(g[m], twiddle<+1>(tw, k1 * m));
-                if constexpr (!G_ONLY) {
-                    reg_dft<N2, +1, V>::run(gz);
-                    o += R * TS;
+                for (int m = 0; m < N2; ++m) o[m * C] = m == 0 ? g[0] : c_mul(g[m], twiddle<+1>(tw, kk * m));
+            };
+            if constexpr (PAIRED) {
+                int sides = R;
+#pragma unroll 1
+                while (true) {
+                    emit(ga, r, c, k1);
+                    if (--sides == 0) break;
+                    // the mirror unit, in the order of its own outputs
 #pragma unroll
-                    for (int m = 0; m < N2; ++m) o[m * C] = m == 0 ? gz[0] : c_mul(gz[m], twiddle<+1>(tw, k1 * m));
-                }
-                if (PAIRED) {  // the mirror unit next
-#pragma unroll
-                    for (int j = 0; j < N2; ++j) {
-                        const V t = va[j];
-                        va[j] = vb[j];
-                        vb[j] = t;
-                    }
+                    for (int k2 = 0; k2 < N2; ++k2) ga[k2] = k1 == 0 ? gb[(N2 - k2) % N2] : gb[N2 - 1 - k2];
                     r = rB;
                     c = cB;
                     k1 = k1B;
                 }
+            } else {
+                emit(ga, r, c, k1);
             }
         }
     }

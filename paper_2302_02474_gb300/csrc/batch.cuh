@@ -357,9 +357,9 @@ template <typename T> class BatchEngine final : public BatchBase {
                 }
                 ++since2;
             }
-            return runs + sorts * 8 * (int64_t)reps_.size();
+            return runs + sorts * 4 * (int64_t)reps_.size();
         }
-        return n * 4 * (int64_t)groups_.size() + sorts * 8 * (int64_t)reps_.size();
+        return n * 4 * (int64_t)groups_.size() + sorts * 4 * (int64_t)reps_.size();
     }
 
    private:

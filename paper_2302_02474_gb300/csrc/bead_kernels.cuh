@@ -220,9 +220,9 @@ __device__ __forceinline__ void gather_force(const Stencil<P, T>& st, bool in_pa
                 for (int a = 0; a < P; ++a) {
                     const size_t g = oy + pwrap(st.jx + a, n);
                     const T w = st.wx[a] * wyz;
-                    const cplx_t<T> vx = __ldg(grad + g);
-                    const cplx_t<T> vy = __ldg(grad + M + g);
-                    const cplx_t<T> vz = __ldg(grad + 2 * M + g);
+                    const cplx_t<T> vx = __ldca(grad + g);
+                    const cplx_t<T> vy = __ldca(grad + M + g);
+                    const cplx_t<T> vz = __ldca(grad + 2 * M + g);
                     gx += w * (comp ? vx.y : vx.x);
                     gy += w * (comp ? vy.y : vy.x);
                     gz += w * (comp ? vz.y : vz.x);
@@ -276,7 +276,7 @@ __device__ __forceinline__ void gather_force_an(const Stencil<P, T>& st, const T
                 const T wyz = st.wy[b] * st.wz[c], dyz = dwy[b] * st.wz[c], ydz = st.wy[b] * dwz[c];
 #pragma unroll
                 for (int a = 0; a < P; ++a) {
-                    const cplx_t<T> v = __ldg(pot + oy + pwrap(st.jx + a, n));
+                    const cplx_t<T> v = __ldca(pot + oy + pwrap(st.jx + a, n));
                     const T w = comp ? -v.x : v.y;
                     gx += dwx[a] * wyz * w;
                     gy += st.wx[a] * dyz * w;
@@ -399,6 +399,7 @@ __device__ __forceinline__ void bead_kernel_body(const BeadParams<T>& p, const B
         constexpr int kWords = (SM::patches * PT::W3 * (int)sizeof(patch_t) + 15) / 16;
         for (int i = threadIdx.x; i < kWords; i += blockDim.x) reinterpret_cast<uint4*>(patch)[i] = make_uint4(0, 0, 0, 0);
     }
+    dependency_wait();
     __syncthreads();
     if (AN && kForce && row_lane) {
         // stage w_2p, w_2p+1 of the patch from pot = i (w_2p + i w_2p+1)
@@ -412,7 +413,7 @@ __device__ __forceinline__ void bead_kernel_body(const BeadParams<T>& p, const B
             for (int k = 0; k < ROWS_PER_LANE; ++k) {
                 const int row = row0 + k * rstride;
                 if (row < W * W) {
-                    v[k] = __ldg(bf.grad + (4 * pr + 3) * M + s_rowbase[row] + gx);
+                    v[k] = __ldca(bf.grad + (4 * pr + 3) * M + s_rowbase[row] + gx);
                 }
             }
 #pragma unroll
@@ -439,9 +440,9 @@ __device__ __forceinline__ void bead_kernel_body(const BeadParams<T>& p, const B
                 const int row = row0 + k * rstride;
                 if (row < W * W) {
                     const size_t g = (size_t)s_rowbase[row] + gx;
-                    v[k][0] = __ldg(gp + g);
-                    v[k][1] = __ldg(gp + M + g);
-                    v[k][2] = __ldg(gp + 2 * M + g);
+                    v[k][0] = __ldca(gp + g);
+                    v[k][1] = __ldca(gp + M + g);
+                    v[k][2] = __ldca(gp + 2 * M + g);
                 }
             }
 #pragma unroll
@@ -773,8 +774,9 @@ __global__ void bin_count_fine(int n_beads, const T* __restrict__ px, const T* _
                                const int* __restrict__ id_src, int* __restrict__ fkey, int* __restrict__ frank,
                                int* __restrict__ fcount) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    dependency_wait();
     if (i >= n_beads) return;
-    const T x = px[i], y = py[i], z = pz[i];
+    const T x = __ldcg(px + i), y = __ldcg(py + i), z = __ldcg(pz + i);
     const int cx = min(max((int)floor(x * inv_dx), 0), n - 1);
     const int cy = min(max((int)floor(y * inv_dx), 0), n - 1);
     const int cz = min(max((int)floor(z * inv_dx), 0), nz - 1);
@@ -810,10 +812,11 @@ __global__ void bin_scatter_fine(int n_beads, Topology topo, const unsigned char
                                  const T* __restrict__ u_src /*[3][N]*/, T* __restrict__ u_dst,
                                  const int* __restrict__ id_src, int* __restrict__ id_dst, int* __restrict__ slot_of_id) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    dependency_wait();
     if (i >= n_beads) return;
     const int f = fkey[i], r = frank[i];
     const int base = f & ~7, g = f & 7;
-    int s = fine_start[base];
+    int s = __ldca(fine_start + base);
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
         const int c = fcount[base + q];
@@ -830,12 +833,15 @@ __global__ void bin_scatter_fine(int n_beads, Topology topo, const unsigned char
     slot_of_id[b] = s;
 }
 
+// The last kernel of a re-binning: it also clears the bin counts for the next one.
 static __global__ void bin_neighbours(int n_beads, Topology topo, const int* __restrict__ id, const int* __restrict__ slot_of_id,
-                               int2* __restrict__ nbr) {
+                               int2* __restrict__ nbr, int* __restrict__ fcount, int n_fine) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    dependency_wait();
+    for (int k = i; k < n_fine; k += gridDim.x * blockDim.x) fcount[k] = 0;
     if (i >= n_beads) return;
-    const BeadInfo b = bead_info(topo, slot_bead_id(id[i]));
-    nbr[i] = make_int2(b.prev >= 0 ? slot_of_id[b.prev] : -1, b.next >= 0 ? slot_of_id[b.next] : -1);
+    const BeadInfo b = bead_info(topo, slot_bead_id(__ldcg(id + i)));
+    nbr[i] = make_int2(b.prev >= 0 ? __ldca(slot_of_id + b.prev) : -1, b.next >= 0 ? __ldca(slot_of_id + b.next) : -1);
 }
 
 // Neighbour slots from an explicit bond list: adj[b] holds the first two
@@ -845,22 +851,70 @@ static __global__ void bin_neighbours(int n_beads, Topology topo, const int* __r
 // layout) receives the slots of those ids.
 static __global__ void bin_neighbours_explicit(int n_beads, const int* __restrict__ id, const int* __restrict__ slot_of_id,
                                                const int2* __restrict__ adj, const int* __restrict__ ext_ids,
-                                               int* __restrict__ ext_slots, int2* __restrict__ nbr) {
+                                               int* __restrict__ ext_slots, int2* __restrict__ nbr,
+                                               int* __restrict__ fcount, int n_fine) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    dependency_wait();
+    for (int k = i; k < n_fine; k += gridDim.x * blockDim.x) fcount[k] = 0;
     if (i >= n_beads) return;
-    const int2 a = adj[slot_bead_id(id[i])];
-    int2 r = make_int2(a.x >= 0 ? slot_of_id[a.x] : -1, a.y >= 0 ? slot_of_id[a.y] : -1);
+    const int2 a = adj[slot_bead_id(__ldcg(id + i))];
+    int2 r = make_int2(a.x >= 0 ? __ldca(slot_of_id + a.x) : -1, a.y >= 0 ? __ldca(slot_of_id + a.y) : -1);
     if (a.y < -1) {
         const int off = -2 - a.y;
         const int cnt = ext_ids[off];
         ext_slots[off] = cnt;
-        for (int j = 1; j <= cnt; ++j) ext_slots[off + j] = slot_of_id[ext_ids[off + j]];
+        for (int j = 1; j <= cnt; ++j) ext_slots[off + j] = __ldca(slot_of_id + ext_ids[off + j]);
         r.y = a.y;
     }
     nbr[i] = r;
 }
 
-// Exclusive scan of `count` ints in blocks of 1024 (three kernels).
+// Exclusive scan of `count` ints by one block of 1024 threads, four values each
+// per round, and tile_start[t] = out[16 t] for t = 0 .. n_tiles.
+static __global__ void __launch_bounds__(1024) scan_one(const int* __restrict__ in, int* __restrict__ out, int count, int n_tiles,
+                                                        int* __restrict__ tile_start) {
+    __shared__ int warp_sum[2][32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int carry = 0, round = 0;
+    dependency_wait();
+    for (int base = 0; base < count; base += 4096, ++round) {
+        const int i = base + 4 * threadIdx.x;
+        int v[4], s = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            v[k] = i + k < count ? __ldcg(in + i + k) : 0;
+            s += v[k];
+        }
+        int run = s;  // inclusive scan of the threads' sums
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, run, o);
+            if (lane >= o) run += t;
+        }
+        int* ws = warp_sum[round & 1];
+        if (lane == 31) ws[wid] = run;
+        __syncthreads();
+        int w = ws[lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, w, o);
+            if (lane >= o) w += t;
+        }
+        const int before = wid == 0 ? 0 : __shfl_sync(0xffffffffu, w, wid - 1);
+        int at = carry + before + run - s;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (i + k < count) {
+                out[i + k] = at;
+                if ((i + k) % kFineBins == 0 && (i + k) / kFineBins <= n_tiles) tile_start[(i + k) / kFineBins] = at;
+            }
+            at += v[k];
+        }
+        carry += __shfl_sync(0xffffffffu, w, 31);
+    }
+}
+
+// Exclusive scan of `count` ints in blocks of 1024 (three kernels; more bins than one block takes).
 static __global__ void scan_blocks(const int* __restrict__ in, int* __restrict__ out, int* __restrict__ block_sums, int count) {
     __shared__ int s[1024];
     const int i = blockIdx.x * 1024 + threadIdx.x;

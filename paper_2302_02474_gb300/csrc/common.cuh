@@ -8,6 +8,20 @@
 
 namespace tild {
 
+// Programmatic dependent launch: a kernel launched with that attribute may start
+// while its predecessor runs. dependency_wait() returns when the predecessor
+// has finished and its writes are visible; nothing that another kernel writes
+// is touched before it. It also lets the successor start (its blocks then wait
+// in turn), so at most one kernel waits behind the running one, and what
+// earlier kernels wrote is complete when a kernel starts. What the predecessor
+// itself writes must not be read through the read-only cache (it changes while
+// the kernel is resident): those reads are __ldcg, __ldca or __ldcs. Without
+// the attribute both instructions do nothing.
+__device__ __forceinline__ void dependency_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // ---------------------------------------------------------------- types
 
 template <typename T> struct cplx_of;

@@ -71,6 +71,7 @@ template <typename T> class Engine final : public EngineBase {
         n_tiles_ = tiles_ * tiles_ * ((nz_ + kTile - 1) / kTile);
         n_fine_ = (size_t)kFineBins * n_tiles_ + 1;  // re-binning bins (tile, edge class, bank group)
         TILD_CUDA(dev_malloc((void**)&counts_, n_fine_ * sizeof(int)));
+        TILD_CUDA(cudaMemset(counts_, 0, n_fine_ * sizeof(int)));  // and every re-binning leaves it zero
         TILD_CUDA(dev_malloc((void**)&tile_start_, (n_tiles_ + 1) * sizeof(int)));
         TILD_CUDA(dev_malloc((void**)&fine_start_, n_fine_ * sizeof(int)));
         scan_blocks_ = (int)((n_fine_ + 1023) / 1024);
@@ -391,12 +392,12 @@ template <typename T> class Engine final : public EngineBase {
         unsigned long long* fx = (unsigned long long*)vjp_fx_;
         Bits* bits = (Bits*)(fx + 6 * M_);
         const int S = vjp_fixed_bits();
-        lam_absmax<T><<<(int)std::min<size_t>(blocks(3 * N), 2 * 152), 256, 0, stream_>>>(3 * N, lam_d, bits);
+        launch(lam_absmax<T>, (int)std::min<size_t>(blocks(3 * N), 2 * 152), 256, 0, 3 * N, lam_d, bits);
         const BeadParams<T> p = bead_params();
         if ((st = dispatch_p([&](auto pp) -> tild_status {
                  constexpr int P = decltype(pp)::value;
                  if constexpr (sizeof(T) == 4)
-                     vjp_spread_tiled<P><<<n_tiles_, 256, vjp_spread_smem<P>(), stream_>>>(p, bf, lam_d, fx, bits, S);
+                     launch(vjp_spread_tiled<P>, n_tiles_, 256, vjp_spread_smem<P>(), p, bf, lam_d, fx, bits, S);
                  else
                      vjp_spread<P, T><<<blocks(N), 256, 0, stream_>>>(p, bf, lam_d, fx, bits, S);
                  return TILD_OK;
@@ -408,21 +409,21 @@ template <typename T> class Engine final : public EngineBase {
                  constexpr int NN = decltype(nn)::value;
                  if constexpr (plane_fits(NN, sizeof(V))) {
                      constexpr int CV = vjp_cols(NN);
-                     xy_forward_cplx<T, NN><<<dim3(NN, 3), 512, plane_smem(), stream_>>>((longlong2*)fx, bits, S, H_, tw_);
-                     z_vjp<T, NN, CV><<<dim3(NN / CV, NN / 2 + 1), 256, vjp_smem(), stream_>>>(H_, zxy, tw_, sp, partials_, el, bits);
+                     launch(xy_forward_cplx<T, NN>, dim3(NN, 3), 512, plane_smem(), (longlong2*)fx, bits, S, H_, tw_);
+                     launch(z_vjp<T, NN, CV>, dim3(NN / CV, NN / 2 + 1), 256, vjp_smem(), H_, zxy, tw_, sp, partials_, el, bits);
                  }
                  return TILD_OK;
              })))
             return st;
         TILD_CUDA(cudaGetLastError());
-        accumulate_partials<<<1, 256, 0, stream_>>>(partials_, (int)vjp_blocks(), theta_acc);
+        launch(accumulate_partials, 1, 256, 0, partials_, (int)vjp_blocks(), theta_acc);
         if ((st = enqueue_inverse(kInvPot))) return st;  // psi into the potential slot
         const double dV = cfg_->L * cfg_->L * cfg_->L / (double)M_;
         const V* psi = grad_ + 3 * M_;
         if ((st = dispatch_p([&](auto pp) -> tild_status {
                  constexpr int P = decltype(pp)::value;
                  if constexpr (sizeof(T) == 4)
-                     vjp_beads_tiled<P><<<n_tiles_, 256, vjp_beads_smem<P>(), stream_>>>(p, bf, fields, psi, lam_d, (T)(1.0 / dV), out_d);
+                     launch(vjp_beads_tiled<P>, n_tiles_, 256, vjp_beads_smem<P>(), p, bf, fields, psi, lam_d, (T)(1.0 / dV), out_d);
                  else
                      vjp_beads<P, T><<<blocks(N), 256, 0, stream_>>>(p, bf, fields, psi, lam_d, (T)(1.0 / dV), out_d);
                  return TILD_OK;
@@ -601,7 +602,7 @@ template <typename T> class Engine final : public EngineBase {
         }
         TILD_CUDA(ce);
         const unsigned grid = (unsigned)std::min<size_t>(304, (most / 16 + 1023) / 1024 + 1);
-        if (n) copy_list<<<dim3(grid, n), 256, 0, stream_>>>(c);
+        if (n) launch(copy_list, dim3(grid, n), 256, 0, c);
         TILD_CUDA(cudaGetLastError());
         return TILD_OK;
     }
@@ -701,7 +702,7 @@ template <typename T> class Engine final : public EngineBase {
                     st = vjp_core(lam, jt, acc, snapshot_buffers(at), fields,
                                   (const V*)(at + bsnap + snap_part(3 * M_ * sizeof(V))));
                 if (st) return st;
-                adjoint_step<T><<<blocks(n3), 256, 0, stream_>>>(n3, jt, rb, ub, lam, q.sd, q.sh, q.su, q.sf, q.wf,
+                launch(adjoint_step<T>, blocks(n3), 256, 0, n3, jt, rb, ub, lam, q.sd, q.sh, q.su, q.sf, q.wf,
                                                                   j == 0 ? 1 : 0);
                 TILD_CUDA(cudaGetLastError());
             }
@@ -917,7 +918,7 @@ template <typename T> class Engine final : public EngineBase {
     int64_t launches(int64_t n) const override {
         const int D = cfg_->dim;
         const int64_t per_step = generic_ ? (use_lines() ? 2 * D : (1 + D) + 1 + (int64_t)NP_ * D + 1) : (use_planes() ? 2 : 4) + 2;
-        const int64_t per_sort = 8;
+        const int64_t per_sort = n_fine_ <= kScanOne ? 4 : 7;
         const int K = cfg_->sort_every;
         int64_t since = steps_since_sort_, sorts = 0;
         for (int64_t s = 0; s < n; ++s) {
@@ -1057,6 +1058,9 @@ template <typename T> class Engine final : public EngineBase {
     int* ranks_ = nullptr;  // and its rank in the bin
     int* counts_ = nullptr;  // [n_fine_] bead counts of the fine bins
     size_t n_fine_ = 0;
+    // Bins up to which one block scans them (128^3: one launch of 9 us for four
+    // of 14 us in all; 24^3: 3 for 14)
+    static constexpr size_t kScanOne = 65537;
     int* tile_start_ = nullptr;
     int n_tiles_ = 0;
     int* fine_start_ = nullptr;  // [n_fine_] exclusive scan of counts_
@@ -1139,11 +1143,11 @@ template <typename T> class Engine final : public EngineBase {
     bool use_lines() const { return generic_ && line_smem((NP_ == 2 ? 8 : 4) * n_) <= (size_t)kLineSmem; }
     tild_status line_forward(bool zero_after) {
         const int lg = line_rows_lg(NP_);
-        line_x_forward<T><<<dim3(div_up(nz_ * n_, 1 << lg), NP_), 128, line_smem((n_ | 1) << lg), stream_>>>(
+        launch(line_x_forward<T>, dim3(div_up(nz_ * n_, 1 << lg), NP_), 128, line_smem((n_ | 1) << lg), 
             line_args(lg, n_ | 1), rho_fx_, Zxy_, density_scale(), zero_after ? 1 : 0, zero_after ? counters_ : nullptr);
         if (cfg_->dim == 3) {
             const int ly = line_lg(4, 2, n_, [&](int l) { return div_up(n_, 1 << l) * nz_ * NP_; });
-            line_y<T, -1><<<dim3(div_up(n_, 1 << ly), nz_, NP_), 128, line_smem(n_ << ly), stream_>>>(line_args(ly, n_), Zxy_);
+            launch(line_y<T, -1>, dim3(div_up(n_, 1 << ly), nz_, NP_), 128, line_smem(n_ << ly), line_args(ly, n_), Zxy_);
         }
         TILD_CUDA(cudaGetLastError());
         return TILD_OK;
@@ -1154,11 +1158,11 @@ template <typename T> class Engine final : public EngineBase {
         const LineArgs<T> a = line_args(lg, n_);
         const size_t sm = line_smem(n_ << lg);
         if (cfg_->dim == 3) {
-            if (NP_ == 2) line_last<T, 2, 3><<<line_last_grid(), 128, sm, stream_>>>(a, Zxy_, H_, sp, partials);
-            else line_last<T, 1, 3><<<line_last_grid(), 128, sm, stream_>>>(a, Zxy_, H_, sp, partials);
+            if (NP_ == 2) launch(line_last<T, 2, 3>, line_last_grid(), 128, sm, a, Zxy_, H_, sp, partials);
+            else launch(line_last<T, 1, 3>, line_last_grid(), 128, sm, a, Zxy_, H_, sp, partials);
         } else {
-            if (NP_ == 2) line_last<T, 2, 2><<<line_last_grid(), 128, sm, stream_>>>(a, Zxy_, H_, sp, partials);
-            else line_last<T, 1, 2><<<line_last_grid(), 128, sm, stream_>>>(a, Zxy_, H_, sp, partials);
+            if (NP_ == 2) launch(line_last<T, 2, 2>, line_last_grid(), 128, sm, a, Zxy_, H_, sp, partials);
+            else launch(line_last<T, 1, 2>, line_last_grid(), 128, sm, a, Zxy_, H_, sp, partials);
         }
         TILD_CUDA(cudaGetLastError());
         return TILD_OK;
@@ -1167,10 +1171,10 @@ template <typename T> class Engine final : public EngineBase {
         const int D = cfg_->dim;
         if (D == 3) {
             const int ly = line_lg(5, 3, n_, [&](int l) { return div_up(n_, 1 << (l - 1)) * nz_ * NP_; });
-            line_y<T, +1><<<dim3(div_up(n_, 1 << (ly - 1)), nz_, 2 * NP_), 128, line_smem(n_ << ly), stream_>>>(line_args(ly, n_), H_);
+            launch(line_y<T, +1>, dim3(div_up(n_, 1 << (ly - 1)), nz_, 2 * NP_), 128, line_smem(n_ << ly), line_args(ly, n_), H_);
         }
         const int lg = line_rows_lg(D * NP_);
-        line_x_inverse<T><<<dim3(div_up(nz_ * n_, 1 << lg), D * NP_), 128, line_smem((n_ | 1) << lg), stream_>>>(
+        launch(line_x_inverse<T>, dim3(div_up(nz_ * n_, 1 << lg), D * NP_), 128, line_smem((n_ | 1) << lg), 
             line_args(lg, n_ | 1), H_, grad_, D);
         TILD_CUDA(cudaGetLastError());
         return TILD_OK;
@@ -1463,6 +1467,45 @@ template <typename T> class Engine final : public EngineBase {
 
     // ---------------------------------------------------------- kernels
 
+    // Launch of a step's kernel, overlapping its start with the end of the
+    // kernel before it where overlap() says so. The overlap hides the launch
+    // latency, but the blocks that start early are placed among those still
+    // running, unevenly, which costs more than it saves where a kernel fills
+    // the chip or the FP64 unit. FP32 only; us per step without / with, as
+    // graph replay and as single launches:
+    //   24^3, 4,060 beads      15.5 / 13.0    24.2 / 14.4
+    //   48^3, 22,000           20.1 / 19.1    30.4 / 20.7
+    //   64^3, 200,000          30.1 / 34.8    39.4 / 36.4
+    //   80^3, 400,000          47.3 / 50.2    56.6 / 51.8
+    //   128^3, 1.6M           153.3 / 162.2  162.4 / 163.1
+    //   65^2, 5,000            18.6 / 16.2    29.4 / 18.6
+    //   45^3, 54,000           34.5 / 37.0    50.2 / 40.2
+    //   FP64 32^3, 20,000      58.1 / 75.9    67.7 / 77.6
+    bool overlap() const {
+        if (sizeof(T) == 8 || M_ > 80 * 80 * 80) return false;
+        if (M_ <= (generic_ ? 32 * 32 * 32 : 48 * 48 * 48)) return true;
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        return cudaStreamIsCapturing(stream_, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+    }
+    template <class... KA, class... A>
+    void launch(void (*k)(KA...), dim3 grid, unsigned threads, size_t smem, A&&... a) {
+        launch_on(stream_, overlap(), k, grid, threads, smem, std::forward<A>(a)...);
+    }
+    template <class... KA, class... A>
+    static void launch_on(cudaStream_t stream_, bool overlap, void (*k)(KA...), dim3 grid, unsigned threads, size_t smem, A&&... a) {
+        cudaLaunchConfig_t c = {};
+        c.gridDim = grid;
+        c.blockDim = dim3(threads);
+        c.dynamicSmemBytes = smem;
+        c.stream = stream_;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
+        c.attrs = at;
+        c.numAttrs = overlap ? 1 : 0;
+        cudaLaunchKernelEx(&c, k, static_cast<KA>(a)...);  // (errors: cudaGetLastError at the call site)
+    }
+
     template <int NN> tild_status attrs_n() {
         if (plane_fits_) {
             if constexpr (plane_fits(NN, sizeof(V))) {
@@ -1580,16 +1623,16 @@ template <typename T> class Engine final : public EngineBase {
             if constexpr (plane_fits(NN, sizeof(V))) {
                 with_nt<NN>([&](auto nt) {
                     constexpr int NT = decltype(nt)::value;
-                    xy_forward_plane<T, NN, NT><<<dim3(NN, NP_), NT, plane_smem(), stream_>>>(
+                    launch(xy_forward_plane<T, NN, NT>, dim3(NN, NP_), NT, plane_smem(), 
                         rho_fx_, Zxy_, tw_, density_scale(), zero_after ? 1 : 0, zero_after ? counters_ : nullptr);
                 });
             }
         } else {
             constexpr int CC = 128 / sizeof(V);
             if constexpr (NN >= 16 && NN >= CC) {
-                x_forward_rows<T, NN, 16><<<dim3((unsigned)((size_t)NN * NN / 16), NP_), 256, rows_smem(), stream_>>>(
+                launch(x_forward_rows<T, NN, 16>, dim3((unsigned)((size_t)NN * NN / 16), NP_), 256, rows_smem(), 
                     rho_fx_, Zxy_, tw_, density_scale(), zero_after ? 1 : 0, zero_after ? counters_ : nullptr);
-                y_columns<T, NN, CC, -1><<<dim3(NN / CC, NN, NP_), 256, ycol_smem(), stream_>>>(Zxy_, tw_, two_pi_L(), 0);
+                launch(y_columns<T, NN, CC, -1>, dim3(NN / CC, NN, NP_), 256, ycol_smem(), Zxy_, tw_, two_pi_L(), 0);
             }
         }
         TILD_CUDA(cudaGetLastError());
@@ -1710,16 +1753,15 @@ template <typename T> class Engine final : public EngineBase {
             constexpr int C2 = zpass_cols2(NN);
             const dim3 grid2(NN / C2, NN / 2 + 1);
             if (g_only)
-                z_spectral_pairs<T, NN, C2, true><<<grid2, 256, zpass2_smem(), stream_>>>(Zxy_, H_, tw_, sp, partials);
+                launch(z_spectral_pairs<T, NN, C2, true>, grid2, 256, zpass2_smem(), Zxy_, H_, tw_, sp, partials);
             else
-                z_spectral_pairs<T, NN, C2><<<grid2, 256, zpass2_smem(), stream_>>>(Zxy_, H_, tw_, sp, partials);
+                launch(z_spectral_pairs<T, NN, C2>, grid2, 256, zpass2_smem(), Zxy_, H_, tw_, sp, partials);
             TILD_CUDA(cudaGetLastError());
             return TILD_OK;
         }
         return with_z<NN>([&](auto cc, auto g, auto e_l, auto e) -> tild_status {
             constexpr int CZ = decltype(cc)::value;
-            z_spectral<T, NN, CZ, decltype(g)::value != 0, decltype(e_l)::value != 0, decltype(e)::value>
-                <<<dim3(NN / CZ, NN / 2 + 1), 256, zpass_smem_cols(CZ), stream_>>>(Zxy_, H_, tw_, sp, partials);
+            launch(z_spectral<T, NN, CZ, decltype(g)::value != 0, decltype(e_l)::value != 0, decltype(e)::value>, dim3(NN / CZ, NN / 2 + 1), 256, zpass_smem_cols(CZ), Zxy_, H_, tw_, sp, partials);
             TILD_CUDA(cudaGetLastError());
             return TILD_OK;
         }, false, g_only, el, want_e);
@@ -1809,15 +1851,15 @@ template <typename T> class Engine final : public EngineBase {
             if constexpr (plane_fits(NN, sizeof(V))) {
                 with_nt<NN>([&](auto nt) {
                     constexpr int NT = decltype(nt)::value;
-                    xy_inverse_plane<T, NN, NT><<<dim3(NN, nd, NP_), NT, plane_smem(), stream_>>>(H_, grad_, tw_, two_pi_L(), d0);
+                    launch(xy_inverse_plane<T, NN, NT>, dim3(NN, nd, NP_), NT, plane_smem(), H_, grad_, tw_, two_pi_L(), d0);
                 });
             }
         } else {
             constexpr int CC = 128 / sizeof(V);
             if constexpr (NN >= 16 && NN >= CC) {
-                y_columns<T, NN, CC, +1><<<dim3(NN / CC, NN, (what == kInvPot ? 1 : 2) * NP_), 256, ycol_smem(), stream_>>>(
+                launch(y_columns<T, NN, CC, +1>, dim3(NN / CC, NN, (what == kInvPot ? 1 : 2) * NP_), 256, ycol_smem(), 
                     H_, tw_, two_pi_L(), what == kInvPot ? 1 : 0);
-                x_inverse_rows<T, NN, 16><<<dim3((unsigned)((size_t)NN * NN / 16), nd, NP_), 256, rows_smem(), stream_>>>(
+                launch(x_inverse_rows<T, NN, 16>, dim3((unsigned)((size_t)NN * NN / 16), nd, NP_), 256, rows_smem(), 
                     H_, grad_, tw_, two_pi_L(), d0);
             }
         }
@@ -1954,17 +1996,17 @@ template <typename T> class Engine final : public EngineBase {
         if (analytic() && mode != kModeSpread) {
             const size_t sm = bead_smem(true, NS);
             switch (mode) {
-                case kModeForce: bead_kernel<P, kModeForce, T, true, NS><<<grid, 256, sm, stream_>>>(p, bf); break;
-                case kModeSetVel: bead_kernel<P, kModeSetVel, T, true, NS><<<grid, 256, sm, stream_>>>(p, bf); break;
-                default: bead_kernel<P, kModeStep, T, true, NS><<<grid, 256, sm, stream_>>>(p, bf); break;
+                case kModeForce: launch(bead_kernel<P, kModeForce, T, true, NS>, grid, 256, sm, p, bf); break;
+                case kModeSetVel: launch(bead_kernel<P, kModeSetVel, T, true, NS>, grid, 256, sm, p, bf); break;
+                default: launch(bead_kernel<P, kModeStep, T, true, NS>, grid, 256, sm, p, bf); break;
             }
         } else {
             const size_t sm = bead_smem(false, NS);
             switch (mode) {
-                case kModeSpread: bead_kernel<P, kModeSpread, T, false, NS><<<grid, 256, sm, stream_>>>(p, bf); break;
-                case kModeForce: bead_kernel<P, kModeForce, T, false, NS><<<grid, 256, sm, stream_>>>(p, bf); break;
-                case kModeSetVel: bead_kernel<P, kModeSetVel, T, false, NS><<<grid, 256, sm, stream_>>>(p, bf); break;
-                default: bead_kernel<P, kModeStep, T, false, NS><<<grid, 256, sm, stream_>>>(p, bf); break;
+                case kModeSpread: launch(bead_kernel<P, kModeSpread, T, false, NS>, grid, 256, sm, p, bf); break;
+                case kModeForce: launch(bead_kernel<P, kModeForce, T, false, NS>, grid, 256, sm, p, bf); break;
+                case kModeSetVel: launch(bead_kernel<P, kModeSetVel, T, false, NS>, grid, 256, sm, p, bf); break;
+                default: launch(bead_kernel<P, kModeStep, T, false, NS>, grid, 256, sm, p, bf); break;
             }
         }
         TILD_CUDA(cudaGetLastError());
@@ -1993,10 +2035,10 @@ template <typename T> class Engine final : public EngineBase {
         const BeadParams<T> p = bead_params();
         const unsigned bt = (unsigned)bead_threads(), g = (unsigned)bead_blocks();
         switch (mode) {
-            case kModeSpread: generic_bead_kernel<P, kModeSpread, T, D><<<g, bt, 0, stream_>>>(p, bf, nz_); break;
-            case kModeForce: generic_bead_kernel<P, kModeForce, T, D><<<g, bt, 0, stream_>>>(p, bf, nz_); break;
-            case kModeSetVel: generic_bead_kernel<P, kModeSetVel, T, D><<<g, bt, 0, stream_>>>(p, bf, nz_); break;
-            default: generic_bead_kernel<P, kModeStep, T, D><<<g, bt, 0, stream_>>>(p, bf, nz_); break;
+            case kModeSpread: launch(generic_bead_kernel<P, kModeSpread, T, D>, g, bt, 0, p, bf, nz_); break;
+            case kModeForce: launch(generic_bead_kernel<P, kModeForce, T, D>, g, bt, 0, p, bf, nz_); break;
+            case kModeSetVel: launch(generic_bead_kernel<P, kModeSetVel, T, D>, g, bt, 0, p, bf, nz_); break;
+            default: launch(generic_bead_kernel<P, kModeStep, T, D>, g, bt, 0, p, bf, nz_); break;
         }
         TILD_CUDA(cudaGetLastError());
         return TILD_OK;
@@ -2038,28 +2080,31 @@ template <typename T> class Engine final : public EngineBase {
 
     tild_status enqueue_sort(cudaStream_t on = nullptr) {
         Range range("tild re-binning");
-        cudaStream_t stream_ = on ? on : this->stream_;  // the batch re-bins on its own stream
+        cudaStream_t st = on ? on : stream_;  // the batch re-bins on its own streams
+        const bool ov = !on && overlap();
         const int N = cfg_->n_beads;
         const size_t N3 = N;
-        TILD_CUDA(cudaMemsetAsync(counts_, 0, n_fine_ * sizeof(int), stream_));
         const T* p = pos_[cur_pos_];
         int pw = 0, plo = 0;
         patch_geometry(&pw, &plo);
-        bin_count_fine<T><<<blocks(N), 256, 0, stream_>>>(N, p, p + N3, p + 2 * N3, (T)((double)n_ / cfg_->L), n_,
-                                                           nz_, tiles_, pw, plo, cfg_->topo, sp_of_id_, id_[cur_id_],
-                                                           keys_, ranks_, counts_);
-        scan_blocks<<<scan_blocks_, 1024, 0, stream_>>>(counts_, fine_start_, block_sums_, (int)n_fine_);
-        scan_top<<<1, 1024, 0, stream_>>>(block_sums_, scan_blocks_);
-        scan_add<<<scan_blocks_, 1024, 0, stream_>>>(fine_start_, block_sums_, (int)n_fine_);
-        bin_tile_start<<<blocks((size_t)n_tiles_ + 1), 256, 0, stream_>>>(fine_start_, n_tiles_, tile_start_);
-        bin_scatter_fine<T><<<blocks(N), 256, 0, stream_>>>(N, cfg_->topo, sp_of_id_, keys_, ranks_, counts_,
-                                                             fine_start_, pos_[cur_pos_], pos_[1 - cur_pos_], u_[cur_u_],
-                                                             u_[1 - cur_u_], id_[cur_id_], id_[1 - cur_id_], slot_of_id_);
+        launch_on(st, ov, bin_count_fine<T>, blocks(N), 256, 0, N, p, p + N3, p + 2 * N3, (T)((double)n_ / cfg_->L), n_, nz_,
+                  tiles_, pw, plo, cfg_->topo, sp_of_id_, id_[cur_id_], keys_, ranks_, counts_);
+        if (n_fine_ <= kScanOne) {
+            launch_on(st, ov, scan_one, 1, 1024, 0, counts_, fine_start_, (int)n_fine_, n_tiles_, tile_start_);
+        } else {
+            scan_blocks<<<scan_blocks_, 1024, 0, st>>>(counts_, fine_start_, block_sums_, (int)n_fine_);
+            scan_top<<<1, 1024, 0, st>>>(block_sums_, scan_blocks_);
+            scan_add<<<scan_blocks_, 1024, 0, st>>>(fine_start_, block_sums_, (int)n_fine_);
+            bin_tile_start<<<blocks((size_t)n_tiles_ + 1), 256, 0, st>>>(fine_start_, n_tiles_, tile_start_);
+        }
+        launch_on(st, ov, bin_scatter_fine<T>, blocks(N), 256, 0, N, cfg_->topo, sp_of_id_, keys_, ranks_, counts_, fine_start_,
+                  pos_[cur_pos_], pos_[1 - cur_pos_], u_[cur_u_], u_[1 - cur_u_], id_[cur_id_], id_[1 - cur_id_], slot_of_id_);
         if (adj_)
-            bin_neighbours_explicit<<<blocks(N), 256, 0, stream_>>>(N, id_[1 - cur_id_], slot_of_id_, adj_, ext_ids_,
-                                                                    ext_slots_, nbr_);
+            launch_on(st, ov, bin_neighbours_explicit, blocks(N), 256, 0, N, id_[1 - cur_id_], slot_of_id_, adj_, ext_ids_,
+                      ext_slots_, nbr_, counts_, (int)n_fine_);
         else
-            bin_neighbours<<<blocks(N), 256, 0, stream_>>>(N, cfg_->topo, id_[1 - cur_id_], slot_of_id_, nbr_);
+            launch_on(st, ov, bin_neighbours, blocks(N), 256, 0, N, cfg_->topo, id_[1 - cur_id_], slot_of_id_, nbr_, counts_,
+                      (int)n_fine_);
         TILD_CUDA(cudaGetLastError());
         cur_pos_ = 1 - cur_pos_;
         cur_u_ = 1 - cur_u_;

@@ -481,6 +481,8 @@ __global__ void __launch_bounds__(128) line_x_forward(LineArgs<T> g, unsigned lo
     const int r0 = blockIdx.x << g.lg, rows = min(1 << g.lg, g.nz * g.n - r0);
     unsigned long long* a = rho_fx + 2 * blockIdx.y * M + (size_t)r0 * g.n;
     Z += blockIdx.y * M + (size_t)r0 * g.n;
+    sh.fill(g);
+    dependency_wait();
     if (step_ctr && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *step_ctr += 1ull;
     for_rows<longlong2>(
         g.lg, rows, g.n,
@@ -488,7 +490,6 @@ __global__ void __launch_bounds__(128) line_x_forward(LineArgs<T> g, unsigned lo
         [&](int l, int e, longlong2 v) {
             sh.buf[l * pitch + e] = V{density_from_fixed(v.x, scale), density_from_fixed(v.y, scale)};
         });
-    sh.fill(g);
     __syncthreads();
     if (zero_after)
         for (int i = threadIdx.x; i < rows * g.n; i += 128) {
@@ -515,9 +516,10 @@ __global__ void __launch_bounds__(128) line_x_inverse(LineArgs<T> g, const cplx_
     const int q = blockIdx.y / D, d = blockIdx.y - q * D;
     const V* src = H + (3 * q + (D == 2 && d == 1 ? 2 : d)) * M + (size_t)r0 * g.n;
     grad += (4 * q + d) * M + (size_t)r0 * g.n;
-    for_rows<V>(
-        g.lg, rows, g.n, [&](int l, int e) { return src[l * g.n + e]; }, [&](int l, int e, V v) { sh.buf[l * pitch + e] = v; });
     sh.fill(g);
+    dependency_wait();
+    for_rows<V>(
+        g.lg, rows, g.n, [&](int l, int e) { return __ldca(src + l * g.n + e); }, [&](int l, int e, V v) { sh.buf[l * pitch + e] = v; });
     __syncthreads();
     if (d == 0) {
         for_rows<V>(
@@ -549,6 +551,8 @@ __global__ void __launch_bounds__(128) line_y(LineArgs<T> g, cplx_t<T>* __restri
     const int x0 = blockIdx.x * C;
     if (x0 >= n) return;
     V* base = data + (DIR > 0 && part == 1 ? 2 * M : 0) + (size_t)blockIdx.y * n * n + x0;
+    sh.fill(g);
+    dependency_wait();
     for (int i0 = threadIdx.x; i0 < n * C; i0 += 4 * 128) {
         V v[4];
 #pragma unroll
@@ -562,7 +566,6 @@ __global__ void __launch_bounds__(128) line_y(LineArgs<T> g, cplx_t<T>* __restri
             if (e < n && x0 + c < n) sh.buf[e * LN + c] = v[k];
         }
     }
-    sh.fill(g);
     __syncthreads();
     if (two) {
         for (int i = threadIdx.x; i < n * C; i += 128) {
@@ -615,6 +618,8 @@ __global__ void __launch_bounds__(128) line_last(LineArgs<T> g, const cplx_t<T>*
         const int row = D == 3 ? index_slot((h & 1) ? my : ky, n1, n2) * n : 0;
         s_off[threadIdx.x] = x0 + c < n ? row + x : -1;
     }
+    sh.fill(g);
+    dependency_wait();
     __syncthreads();
     // lanes over columns, then A/B, pairs and elements
     for (int i0 = threadIdx.x; i0 < n << flg; i0 += 4 * 128) {
@@ -622,7 +627,7 @@ __global__ void __launch_bounds__(128) line_last(LineArgs<T> g, const cplx_t<T>*
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const int i = i0 + k * 128, l = i & (F - 1), e = i >> flg;
-            if (e < n && s_off[l] >= 0) v[k] = Z[((l >> cpl) >> 1) * M + (size_t)e * stride + s_off[l]];
+            if (e < n && s_off[l] >= 0) v[k] = __ldca(Z + ((l >> cpl) >> 1) * M + (size_t)e * stride + s_off[l]);
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -630,7 +635,6 @@ __global__ void __launch_bounds__(128) line_last(LineArgs<T> g, const cplx_t<T>*
             if (e < n) sh.buf[e * LN + l] = s_off[l] >= 0 ? v[k] : V{T(0), T(0)};
         }
     }
-    sh.fill(g);
     __syncthreads();
     // the forward transform of field 0's lines alone: half of the buffer
     lines_forward(sh.buf, sh.alt, LineBuf{n, n1, n2, LN, 1, flg}, sh.tw);
@@ -719,6 +723,7 @@ __global__ void __launch_bounds__(256) generic_bead_kernel(BeadParams<T> p, Bead
     const bool active = i < p.n_beads;
     const bool sums = MODE == kModeForce && bf.partials;
     Wide<T> acc[5];
+    dependency_wait();
     if (active) {
         const int n = p.n;
         const size_t M = (size_t)nz * n * n;
@@ -745,11 +750,11 @@ __global__ void __launch_bounds__(256) generic_bead_kernel(BeadParams<T> p, Bead
                     for (int a = 0; a < P; ++a) {
                         const size_t g = oy + pwrap(st.jx + a, n);
                         const T w = st.wx[a] * wyz;
-                        const cplx_t<T> vx = __ldg(gp + g), vy = __ldg(gp + M + g);
+                        const cplx_t<T> vx = __ldca(gp + g), vy = __ldca(gp + M + g);
                         gx += w * (comp ? vx.y : vx.x);
                         gy += w * (comp ? vy.y : vy.x);
                         if (D == 3) {
-                            const cplx_t<T> vz = __ldg(gp + 2 * M + g);
+                            const cplx_t<T> vz = __ldca(gp + 2 * M + g);
                             gz += w * (comp ? vz.y : vz.x);
                         }
                     }

@@ -161,12 +161,12 @@ __device__ __forceinline__ void plane_forward_xy(cplx_t<T>* plane, cplx_t<T>* tw
     using LS = LineSlots<N>;
     constexpr int N1 = LS::N1, N2 = LS::N2, S2 = LS::S2, PITCH = LS::pitch;
     {
-        // x stage A: unit (row, j2), lanes over j2 (the first loads are in
-        // flight while the twiddles are copied)
+        // x stage A: unit (row, j2), lanes over j2
         int u = threadIdx.x;
         V v[N1];
-        if (u < N * N2) load(u / N2, u % N2, v);
         load_twiddles(tw, tw_g, N);
+        dependency_wait();
+        if (u < N * N2) load(u / N2, u % N2, v);
         __syncthreads();
 #pragma unroll 1
         while (u < N * N2) {
@@ -237,8 +237,9 @@ __device__ __forceinline__ void plane_inverse_yx(cplx_t<T>* plane, cplx_t<T>* tw
 #pragma unroll
             for (int k = 0; k < N1; ++k) v[k] = load(u / N + N2 * k, u % N);
         };
-        if (u < N * N2) fetch();
         load_twiddles(tw, tw_g, N);
+        dependency_wait();
+        if (u < N * N2) fetch();
         __syncthreads();
 #pragma unroll 1
         while (u < N * N2) {
@@ -325,9 +326,6 @@ __device__ __forceinline__ void xy_forward_plane_body(const ForwardArgs<T>& args
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V* tw = reinterpret_cast<V*>(smem_raw);
     V* plane = tw + N;
-    // a step's first kernel advances the noise counter to n+1
-    if (step_ctr && bx == 0 && threadIdx.x == 0) *step_ctr += 1ull;
-
     const size_t M = (size_t)N * N * N;
     const size_t base = (size_t)bx * N * N;
     const long long* ra = reinterpret_cast<const long long*>(rho_fx + base);
@@ -336,6 +334,8 @@ __device__ __forceinline__ void xy_forward_plane_body(const ForwardArgs<T>& args
         plane, tw, tw_g,
         [&](int y, int j2, V (&v)[fft_split<N>::N1]) { load_fixed_unit<N>(ra + y * N, rb + y * N, j2, scale, v); },
         [&]() {
+            // a step's first kernel advances the noise counter to n+1
+            if (step_ctr && bx == 0 && threadIdx.x == 0) *step_ctr += 1ull;
             if (zero_after) {  // every density of the plane has been read
                 zero_fixed<NT>(rho_fx + base, N * N);
                 zero_fixed<NT>(rho_fx + M + base, N * N);
@@ -393,7 +393,7 @@ __device__ __forceinline__ void xy_inverse_plane_body(const InverseArgs<T>& args
     plane_inverse_yx<T, N, NT>(
         plane, tw, tw_g,
         [&](int ky, int q) {
-            const V v = src[ky * N + q];
+            const V v = __ldcg(src + ky * N + q);
             return d == 1 ? c_scale_rn(v, grad_k<T, N>(ky, two_pi_over_L)) : v;
         },
         d == 0, two_pi_over_L, grad + (size_t)d * M + (size_t)bx * N * N);
@@ -436,15 +436,16 @@ __global__ void __launch_bounds__(256) x_forward_rows(unsigned long long* __rest
     const int pr = blockIdx.y;  // species pair
     rho_fx += 2 * pr * M;
     Zxy += pr * M;
-    if (step_ctr && blockIdx.x == 0 && pr == 0 && threadIdx.x == 0) *step_ctr += 1ull;
     const long long* ra = reinterpret_cast<const long long*>(rho_fx + base);
     const long long* rb = ra + M;
     {
         int u = threadIdx.x;  // stage A: unit (row, j2), lanes over j2
         V v[N1];
         auto fetch = [&]() { load_fixed_unit<N>(ra + (u / N2) * N, rb + (u / N2) * N, u % N2, scale, v); };
-        if (u < R * N2) fetch();
         load_twiddles(tw, tw_g, N);
+        dependency_wait();
+        if (step_ctr && blockIdx.x == 0 && pr == 0 && threadIdx.x == 0) *step_ctr += 1ull;
+        if (u < R * N2) fetch();
         __syncthreads();
 #pragma unroll 1
         while (u < R * N2) {
@@ -507,12 +508,13 @@ __global__ void __launch_bounds__(256) x_inverse_rows(const cplx_t<T>* __restric
 #pragma unroll
             for (int k = 0; k < N1; ++k) {
                 const int kx = u % N2 + N2 * k;
-                const V t = __ldg(row + pos_of_kx<N>(kx));
+                const V t = __ldca(row + pos_of_kx<N>(kx));
                 v[k] = kx_mult ? c_scale_rn(t, grad_k<T, N>(kx, two_pi_over_L)) : t;
             }
         };
-        if (u < R * N2) fetch();
         load_twiddles(tw, tw_g, N);
+        dependency_wait();
+        if (u < R * N2) fetch();
         __syncthreads();
 #pragma unroll 1
         while (u < R * N2) {
@@ -575,8 +577,9 @@ __global__ void __launch_bounds__(256) y_columns(cplx_t<T>* __restrict__ data, c
 #pragma unroll
             for (int k = 0; k < N1; ++k) v[k] = data[src + (size_t)(u / C + N2 * k) * N + u % C];
         };
-        if (u < C * N2) fetch();
         load_twiddles(tw, tw_g, N);
+        dependency_wait();
+        if (u < C * N2) fetch();
         __syncthreads();
 #pragma unroll 1
         while (u < C * N2) {
@@ -716,12 +719,13 @@ __device__ __forceinline__ void z_tile(cplx_t<T>* buf, cplx_t<T>* tw, const cplx
             for (int k = 0; k < N1; ++k) v[k] = fetch(u / (C * N2), (u / C) % N2 + N2 * k, u % C);
         };
         const int units = R * C * N2;
-        if (u < units) load();
         load_twiddles(tw, tw_g, N);
         for (int i = threadIdx.x; i < N; i += 256) {
             e1[i] = sp.kernel1d[i];
             if (EL) e2[i] = sp.kernel1d_el[i];
         }
+        dependency_wait();
+        if (u < units) load();
         __syncthreads();
 #pragma unroll 1
         while (u < units) {
@@ -879,7 +883,7 @@ __device__ __forceinline__ void z_spectral_body(const ZArgs<T>& args, int bx, in
     Wide<T> acc[5];
     z_tile<T, N, C, G_ONLY, EL, WANT_E>(
         buf, tw, args.tw, e1, e2, sp, p0, ky, R, acc,
-        [&](int r, int z, int c) { return Zxy[z * NN + (size_t)ky[r] * N + p0 + c]; },
+        [&](int r, int z, int c) { return __ldcg(Zxy + z * NN + (size_t)ky[r] * N + p0 + c); },
         [&](int b, int c, int z, V v) {
             // G of row r to field 0, G_z to field 2, at (z, ky[r], p0 + c)
             const int f = b < R ? 0 : 2, r = b < R ? b : b - R;
@@ -901,6 +905,7 @@ __global__ void __launch_bounds__(256) z_spectrum(const cplx_t<T>* __restrict__ 
     V* tw = reinterpret_cast<V*>(smem_raw);
     V* buf = tw + N;
     load_twiddles(tw, tw_g, N);
+    dependency_wait();
     __syncthreads();
     const int p0 = blockIdx.x * C, ky = blockIdx.y;
     const size_t NN = (size_t)N * N;
@@ -1073,6 +1078,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 1) z_spectral_pairs(
     __shared__ T e1[N];
     load_twiddles(tw, tw_g, N);
     for (int i = threadIdx.x; i < N; i += blockDim.x) e1[i] = sp.kernel1d[i];
+    dependency_wait();
     const int bx = blockIdx.x, by = blockIdx.y;
     const int p0 = bx * C;
     const int ky[2] = {by, by == 0 ? 0 : N - by};
@@ -1083,7 +1089,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 1) z_spectral_pairs(
         const int b = i / TS, rem = i % TS;
         const int q = b / R, r = b % R;
         const int z = rem / C, c = rem % C;
-        return Zxy[q * M + z * NN + (size_t)ky[r] * N + p0 + c];
+        return __ldcg(Zxy + q * M + z * NN + (size_t)ky[r] * N + p0 + c);
     };
     auto zdst = [&](int i, V v) { buf[i] = v; };
     if (R == 1)

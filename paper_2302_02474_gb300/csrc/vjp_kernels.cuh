@@ -79,11 +79,12 @@ __global__ void __launch_bounds__(256) lam_absmax(size_t n, const T* __restrict_
                                                   typename AdjointFixed<T>::bits_t* bits) {
     using B = typename AdjointFixed<T>::bits_t;
     B m = 0;
+    dependency_wait();
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     for (size_t i0 = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i0 < n; i0 += 8 * stride) {
         B v[8];  // eight independent loads in flight
 #pragma unroll
-        for (int k = 0; k < 8; ++k) v[k] = i0 + k * stride < n ? AdjointFixed<T>::abs_bits(lam[i0 + k * stride]) : B(0);
+        for (int k = 0; k < 8; ++k) v[k] = i0 + k * stride < n ? AdjointFixed<T>::abs_bits(__ldcg(lam + i0 + k * stride)) : B(0);
 #pragma unroll
         for (int k = 0; k < 8; ++k) m = max(m, v[k]);
     }
@@ -177,12 +178,13 @@ __global__ void __launch_bounds__(256) vjp_spread_tiled(BeadParams<float> p, Bea
     int* s_hi = reinterpret_cast<int*>(smem_raw);  // [3][row][x][species]
     int* s_lo = s_hi + 6 * W3;
     __shared__ int rowbase[W * W];
-    const int start = bf.tile_start[blockIdx.x], end = bf.tile_start[blockIdx.x + 1];
-    if (start == end) return;
     const int3 org = tile_patch<P>(blockIdx.x, p.tiles, p.n, rowbase);
     for (int i = threadIdx.x; i < 12 * W3; i += blockDim.x) s_hi[i] = 0;
+    dependency_wait();
+    const int start = bf.tile_start[blockIdx.x], end = bf.tile_start[blockIdx.x + 1];
+    if (start == end) return;
     float sc, inv;
-    AdjointFixed<float>::scales(*bits, S, sc, inv);
+    AdjointFixed<float>::scales(__ldcg(bits), S, sc, inv);
     const bool patch_ok = end - start <= kVjpTileBeads;
     __syncthreads();
     for (int i = start + threadIdx.x; i < end; i += blockDim.x) {
@@ -243,8 +245,9 @@ __global__ void __launch_bounds__(512) xy_forward_cplx(longlong2* __restrict__ f
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V* tw = reinterpret_cast<V*>(smem_raw);
     V* plane = tw + N;
+    dependency_wait();
     T sc, inv;
-    AdjointFixed<T>::scales(*bits, S, sc, inv);
+    AdjointFixed<T>::scales(__ldcg(bits), S, sc, inv);
     const size_t base = (size_t)blockIdx.y * N * N * N + (size_t)blockIdx.x * N * N;
     constexpr int N1 = fft_split<N>::N1, N2 = fft_split<N>::N2;
     plane_forward_xy<T, N, 512>(
@@ -366,6 +369,7 @@ __global__ void __launch_bounds__(256) z_vjp(cplx_t<T>* __restrict__ H, const cp
                                              double* __restrict__ partials, int el,
                                              typename AdjointFixed<T>::bits_t* __restrict__ bits) {
     using V = cplx_t<T>;
+    dependency_wait();
     // max|lam| has been read by the spread and the xy pass: 0 for the next call
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *bits = 0;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -440,7 +444,7 @@ __device__ __forceinline__ void vjp_gather_global(const Stencil<P, T>& st, const
 #pragma unroll
             for (int a = 0; a < P; ++a) {
                 const size_t g = row + pwrap(st.jx + a, n);
-                const cplx_t<T> f0 = fields[g], f1 = fields[M + g], f2 = fields[2 * M + g], f3 = psi[g];
+                const cplx_t<T> f0 = fields[g], f1 = fields[M + g], f2 = fields[2 * M + g], f3 = __ldca(psi + g);
                 const T ldw = l[0] * (K ? f0.y : f0.x) + l[1] * (K ? f1.y : f1.x) + l[2] * (K ? f2.y : f2.x);
                 const T val = (K ? -f3.x : f3.y) * inv_dV - ldw;
                 o[0] += dwx[a] * wyz * val;
@@ -505,16 +509,17 @@ __global__ void __launch_bounds__(256) vjp_beads_tiled(BeadParams<float> p, Bead
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float4* rec = reinterpret_cast<float4*>(smem_raw);  // [species][W3]
     __shared__ int rowbase[W * W];
+    const int3 org = tile_patch<P>(blockIdx.x, p.tiles, p.n, rowbase);
+    dependency_wait();
     const int start = bf.tile_start[blockIdx.x], end = bf.tile_start[blockIdx.x + 1];
     if (start == end) return;
-    const int3 org = tile_patch<P>(blockIdx.x, p.tiles, p.n, rowbase);
     const size_t M = (size_t)p.n * p.n * p.n;
     __syncthreads();
 #pragma unroll 3
     for (int i = threadIdx.x; i < W3; i += 256) {
         const int row = i / W;
         const size_t g = (size_t)rowbase[row] + pwrap(org.x + i - row * W, p.n);
-        const float2 f0 = __ldg(fields + g), f1 = __ldg(fields + M + g), f2 = __ldg(fields + 2 * M + g), f3 = __ldg(psi + g);
+        const float2 f0 = __ldg(fields + g), f1 = __ldg(fields + M + g), f2 = __ldg(fields + 2 * M + g), f3 = __ldca(psi + g);
         rec[i] = make_float4(f0.x, f1.x, f2.x, f3.y * inv_dV);
         rec[W3 + i] = make_float4(f0.y, f1.y, f2.y, -f3.x * inv_dV);
     }
@@ -603,10 +608,11 @@ __global__ void __launch_bounds__(256) density_vjp_kernel(BeadParams<T> p, BeadB
 static __global__ void __launch_bounds__(256) accumulate_partials(const double* __restrict__ partials, int n_blocks,
                                                                   double* __restrict__ acc) {
     __shared__ double s[3][256];
+    dependency_wait();
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         double v = 0.0;
-        for (int b = threadIdx.x; b < n_blocks; b += 256) v += partials[3 * b + k];
+        for (int b = threadIdx.x; b < n_blocks; b += 256) v += __ldcg(partials + 3 * b + k);
         s[k][threadIdx.x] = v;
     }
     __syncthreads();
@@ -645,8 +651,9 @@ template <typename T>
 __global__ void adjoint_step(size_t n3, const T* __restrict__ jt, double* __restrict__ rb, double* __restrict__ ub,
                              T* __restrict__ lam, double sd, double sh, double su, double sf, double wf, int at_start) {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    dependency_wait();
     if (i >= n3) return;
-    const double r = rb[i] + (double)jt[i];
+    const double r = rb[i] + (double)__ldcg(jt + i);
     const double hb = sd * r + sh * ub[i], u = su * hb;
     rb[i] = r;
     ub[i] = u;
@@ -661,6 +668,7 @@ struct CopyList {
     size_t bytes[8];
 };
 static __global__ void __launch_bounds__(256) copy_list(CopyList c) {
+    dependency_wait();
     const size_t n16 = c.bytes[blockIdx.y] / 16, stride = (size_t)gridDim.x * 256;
     const uint4* s = (const uint4*)c.src[blockIdx.y];
     uint4* d = (uint4*)c.dst[blockIdx.y];

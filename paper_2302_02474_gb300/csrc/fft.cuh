@@ -229,20 +229,31 @@ template <int LS> struct StridedLines {
 // that the transform is left in the order slot k1 N2 + k2 <-> X[k1 + N1 k2],
 // which the consumer of the lines undoes in its addressing.
 //
-// Rows of a plane keep slot i at i + (i / N2) (S2 - N2) with S2 odd and have a
-// pitch of N2 modulo 16 words of 8 bytes: lanes over (j2, row) and lanes over
-// k1 both fall into distinct banks.
+// Rows of a plane keep slot i at i XOR swz(i) (the low bits of an even N2, with
+// bits of k1), so that lanes over k1 at one j2 and lanes over consecutive slots
+// both fall into distinct banks (16 lanes of 8-byte words); padding a row after
+// every N2 slots made every access along columns a two-way conflict. Rows are
+// N2 modulo 16 words apart, for lanes over (j2, row). Odd N2 need neither.
 template <int N> struct LineSlots {
     static constexpr int N1 = fft_split<N>::N1, N2 = fft_split<N>::N2;
-    static constexpr int S2 = N2 | 1;
     static constexpr int make_pitch() {
-        int p = N1 * S2;
+        int p = N;
         while (p % 16 != N2 % 16) ++p;
         return p;
     }
     static constexpr int pitch = make_pitch();
-    // padded position of slot i in a row
-    static __device__ __forceinline__ int at(int i) { return (i / N2) * S2 + i % N2; }
+    static __device__ __forceinline__ int swz(int i) {
+        if constexpr (N2 == 16)
+            return (i >> 4) & 15;
+        else if constexpr (N2 == 8)
+            return (N1 == 16 ? i >> 4 : i >> 3) & 7;
+        else if constexpr (N2 == 4)
+            return (i >> 4) & 3;
+        else
+            return 0;
+    }
+    // position of slot i in a row
+    static __device__ __forceinline__ int at(int i) { return i ^ swz(i); }
     // the slot that holds X[k] after stage B, and its inverse
     static __device__ __forceinline__ int slot_of(int k) { return (k % N1) * N2 + k / N1; }
     static __device__ __forceinline__ int index_of(int slot) { return slot / N2 + N1 * (slot % N2); }

@@ -150,8 +150,16 @@ template <int NTHR> __device__ __forceinline__ void zero_fixed(unsigned long lon
 // a stage visits shared memory once, in place, where a separate load, two
 // stages with their own barriers, a scaling pass and a store pass per
 // direction visited it ten to twelve times (inverse at 128^3, 512 threads:
-// 38.1 -> 34.9 us; at 80^3, 14.4 -> 12.3 us in the step).
+// 38.1 -> 31.7 us, 34.8 of it before rows were swizzled).
 // --------------------------------------------------------------------------
+// Column position of lane-ordered index i: a warp's 32 positions, those of its
+// first half-warp kx = k, k + 1, ..., those of the second the mirror columns
+// n - k, ...: consecutive columns in each phase of a shared-memory access
+// (position order alternates between the two), the same 256 bytes of global memory.
+template <int N> __device__ __forceinline__ int lane_pos(int i) {
+    return N % 32 == 0 ? (i & ~31) + ((i & 15) << 1) + ((i >> 4) & 1) : i;
+}
+
 // load(y, j2, v): inputs x = j2 + N2 j1 of row y; after_load(): runs once all
 // rows have been loaded; dst: [ky][pos(kx)].
 template <typename T, int N, int NT, class Load, class After>
@@ -159,7 +167,7 @@ __device__ __forceinline__ void plane_forward_xy(cplx_t<T>* plane, cplx_t<T>* tw
                                                  After after_load, cplx_t<T>* __restrict__ dst) {
     using V = cplx_t<T>;
     using LS = LineSlots<N>;
-    constexpr int N1 = LS::N1, N2 = LS::N2, S2 = LS::S2, PITCH = LS::pitch;
+    constexpr int N1 = LS::N1, N2 = LS::N2, PITCH = LS::pitch;
     {
         // x stage A: unit (row, j2), lanes over j2
         int u = threadIdx.x;
@@ -172,9 +180,9 @@ __device__ __forceinline__ void plane_forward_xy(cplx_t<T>* plane, cplx_t<T>* tw
         while (u < N * N2) {
             const int r = u / N2, j2 = u % N2;
             stage_a_regs<N, -1>(v, j2, tw);
-            V* p = plane + r * PITCH + j2;
+            V* p = plane + r * PITCH;
 #pragma unroll
-            for (int k1 = 0; k1 < N1; ++k1) p[k1 * S2] = v[k1];
+            for (int k1 = 0; k1 < N1; ++k1) p[LS::at(k1 * N2 + j2)] = v[k1];
             u += NT;
             if (u < N * N2) load(u / N2, u % N2, v);
         }
@@ -184,13 +192,14 @@ __device__ __forceinline__ void plane_forward_xy(cplx_t<T>* plane, cplx_t<T>* tw
     // x stage B: unit (row, k1), lanes over k1
 #pragma unroll 1
     for (int u = threadIdx.x; u < N * N1; u += NT) {
-        V* p = plane + (u / N1) * PITCH + (u % N1) * S2;
+        V* p = plane + (u / N1) * PITCH;
+        const int s0 = (u % N1) * N2;
         V v[N2];
 #pragma unroll
-        for (int j = 0; j < N2; ++j) v[j] = p[j];
+        for (int j = 0; j < N2; ++j) v[j] = p[LS::at(s0 + j)];
         reg_dft<N2, -1, V>::run(v);
 #pragma unroll
-        for (int j = 0; j < N2; ++j) p[j] = v[j];
+        for (int j = 0; j < N2; ++j) p[LS::at(s0 + j)] = v[j];
     }
     __syncthreads();
     // y stage A: unit (column slot, j2), lanes over columns
@@ -209,7 +218,7 @@ __device__ __forceinline__ void plane_forward_xy(cplx_t<T>* plane, cplx_t<T>* tw
     // y stage B: unit (column position, k1), lanes over positions, to global memory
 #pragma unroll 1
     for (int u = threadIdx.x; u < N * N1; u += NT) {
-        const int q = u % N, k1 = u / N;
+        const int q = lane_pos<N>(u % N), k1 = u / N;
         const V* p = plane + k1 * N2 * PITCH + LS::at(LS::slot_of(kx_of_pos<N>(q)));
         V v[N2];
 #pragma unroll
@@ -228,14 +237,14 @@ __device__ __forceinline__ void plane_inverse_yx(cplx_t<T>* plane, cplx_t<T>* tw
                                                  bool x_scale, T two_pi_over_L, cplx_t<T>* __restrict__ dst) {
     using V = cplx_t<T>;
     using LS = LineSlots<N>;
-    constexpr int N1 = LS::N1, N2 = LS::N2, S2 = LS::S2, PITCH = LS::pitch;
+    constexpr int N1 = LS::N1, N2 = LS::N2, PITCH = LS::pitch;
     {
         // y stage A: unit (column position, j2), lanes over positions
         int u = threadIdx.x;
         V v[N1];
         auto fetch = [&]() {
 #pragma unroll
-            for (int k = 0; k < N1; ++k) v[k] = load(u / N + N2 * k, u % N);
+            for (int k = 0; k < N1; ++k) v[k] = load(u / N + N2 * k, lane_pos<N>(u % N));
         };
         load_twiddles(tw, tw_g, N);
         dependency_wait();
@@ -246,7 +255,7 @@ __device__ __forceinline__ void plane_inverse_yx(cplx_t<T>* plane, cplx_t<T>* tw
             const int j2 = u / N;
             stage_a_regs<N, +1>(v, j2, tw);
             // columns in slot order of their natural index kx
-            V* p = plane + j2 * PITCH + LS::at(kx_of_pos<N>(u % N));
+            V* p = plane + j2 * PITCH + LS::at(kx_of_pos<N>(lane_pos<N>(u % N)));
 #pragma unroll
             for (int k1 = 0; k1 < N1; ++k1) p[k1 * N2 * PITCH] = v[k1];
             u += NT;
@@ -276,23 +285,23 @@ __device__ __forceinline__ void plane_inverse_yx(cplx_t<T>* plane, cplx_t<T>* tw
 #pragma unroll 1
     for (int u = threadIdx.x; u < N * N2; u += NT) {
         const int j2 = u % N2;
-        V* p = plane + (u / N2) * PITCH + j2;
+        V* p = plane + (u / N2) * PITCH;
         V v[N1];
 #pragma unroll
-        for (int k = 0; k < N1; ++k) v[k] = p[k * S2];
+        for (int k = 0; k < N1; ++k) v[k] = p[LS::at(k * N2 + j2)];
         stage_a_regs<N, +1>(v, j2, tw);
 #pragma unroll
-        for (int k = 0; k < N1; ++k) p[k * S2] = v[k];
+        for (int k = 0; k < N1; ++k) p[LS::at(k * N2 + j2)] = v[k];
     }
     __syncthreads();
     // x stage B: unit (row, k1), lanes over k1, to global memory
 #pragma unroll 1
     for (int u = threadIdx.x; u < N * N1; u += NT) {
         const int r = u / N1, k1 = u % N1;
-        const V* p = plane + r * PITCH + k1 * S2;
+        const V* p = plane + r * PITCH;
         V v[N2];
 #pragma unroll
-        for (int j = 0; j < N2; ++j) v[j] = p[j];
+        for (int j = 0; j < N2; ++j) v[j] = p[LS::at(k1 * N2 + j)];
         reg_dft<N2, +1, V>::run(v);
         V* o = dst + LS::index_of(r) * N + k1;
 #pragma unroll
@@ -427,7 +436,7 @@ __global__ void __launch_bounds__(256) x_forward_rows(unsigned long long* __rest
                                                        int zero_after, unsigned long long* step_ctr) {
     using V = cplx_t<T>;
     using LS = LineSlots<N>;
-    constexpr int N1 = LS::N1, N2 = LS::N2, S2 = LS::S2, PITCH = LS::pitch;
+    constexpr int N1 = LS::N1, N2 = LS::N2, PITCH = LS::pitch;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V* tw = reinterpret_cast<V*>(smem_raw);
     V* rows = tw + N;
@@ -451,9 +460,9 @@ __global__ void __launch_bounds__(256) x_forward_rows(unsigned long long* __rest
         while (u < R * N2) {
             const int j2 = u % N2;
             stage_a_regs<N, -1>(v, j2, tw);
-            V* p = rows + (u / N2) * PITCH + j2;
+            V* p = rows + (u / N2) * PITCH;
 #pragma unroll
-            for (int k1 = 0; k1 < N1; ++k1) p[k1 * S2] = v[k1];
+            for (int k1 = 0; k1 < N1; ++k1) p[LS::at(k1 * N2 + j2)] = v[k1];
             u += 256;
             if (u < R * N2) fetch();
         }
@@ -466,13 +475,14 @@ __global__ void __launch_bounds__(256) x_forward_rows(unsigned long long* __rest
     // stage B in place; the store below takes the columns in position order
 #pragma unroll 1
     for (int u = threadIdx.x; u < R * N1; u += 256) {
-        V* p = rows + (u / N1) * PITCH + (u % N1) * S2;
+        V* p = rows + (u / N1) * PITCH;
+        const int s0 = (u % N1) * N2;
         V v[N2];
 #pragma unroll
-        for (int j = 0; j < N2; ++j) v[j] = p[j];
+        for (int j = 0; j < N2; ++j) v[j] = p[LS::at(s0 + j)];
         reg_dft<N2, -1, V>::run(v);
 #pragma unroll
-        for (int j = 0; j < N2; ++j) p[j] = v[j];
+        for (int j = 0; j < N2; ++j) p[LS::at(s0 + j)] = v[j];
     }
     __syncthreads();
     for (int i = threadIdx.x; i < R * N; i += 256)
@@ -484,7 +494,7 @@ __global__ void __launch_bounds__(256) x_inverse_rows(const cplx_t<T>* __restric
                                                        const cplx_t<T>* __restrict__ tw_g, T two_pi_over_L, int d0) {
     using V = cplx_t<T>;
     using LS = LineSlots<N>;
-    constexpr int N1 = LS::N1, N2 = LS::N2, S2 = LS::S2, PITCH = LS::pitch;
+    constexpr int N1 = LS::N1, N2 = LS::N2, PITCH = LS::pitch;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V* tw = reinterpret_cast<V*>(smem_raw);
     V* rows = tw + N;
@@ -520,9 +530,9 @@ __global__ void __launch_bounds__(256) x_inverse_rows(const cplx_t<T>* __restric
         while (u < R * N2) {
             const int j2 = u % N2;
             stage_a_regs<N, +1>(v, j2, tw);
-            V* p = rows + (u / N2) * PITCH + j2;
+            V* p = rows + (u / N2) * PITCH;
 #pragma unroll
-            for (int k1 = 0; k1 < N1; ++k1) p[k1 * S2] = v[k1];
+            for (int k1 = 0; k1 < N1; ++k1) p[LS::at(k1 * N2 + j2)] = v[k1];
             u += 256;
             if (u < R * N2) fetch();
         }
@@ -532,10 +542,10 @@ __global__ void __launch_bounds__(256) x_inverse_rows(const cplx_t<T>* __restric
 #pragma unroll 1
     for (int u = threadIdx.x; u < R * N1; u += 256) {
         const int r = u / N1, k1 = u % N1;
-        const V* p = rows + r * PITCH + k1 * S2;
+        const V* p = rows + r * PITCH;
         V v[N2];
 #pragma unroll
-        for (int j = 0; j < N2; ++j) v[j] = p[j];
+        for (int j = 0; j < N2; ++j) v[j] = p[LS::at(k1 * N2 + j)];
         reg_dft<N2, +1, V>::run(v);
         V* o = grad + base + r * N + k1;
 #pragma unroll

@@ -339,11 +339,12 @@ constexpr int kBeadChunk = 512;
 template <int P, typename T, bool AN = false, int NS = 2> struct BeadSmem {
     using patch_t = typename FixedPoint<T>::patch_t;
     static constexpr int W3 = Patch<P>::W3;
-    // the force patch is staged when it is small (else gathered from global
-    // memory): [NS species][W3] of (gx, gy, gz, -) records, or with the
+    // the force patch is staged when two CTAs fit an SM with it (else gathered
+    // from global memory; order 4, 70 KB of it, 64^3, 200,000 beads: step 142 us
+    // gathered from global memory, 88 staged): [NS species][W3] of (gx, gy, gz, -) records, or with the
     // analytic force [NS species][W3] potentials
     static constexpr size_t field_bytes = AN ? NS * W3 * sizeof(T) : NS * W3 * sizeof(typename vec4_of<T>::type);
-    static constexpr bool stage_grad = field_bytes <= 48 * 1024;
+    static constexpr bool stage_grad = field_bytes <= 72 * 1024;
     static constexpr int patches = NS;
     static constexpr size_t patch_off = 0;                                                       // patch_t [patches][W3]
     static constexpr size_t grad_off = (patch_off + patches * W3 * sizeof(patch_t) + 31) / 32 * 32;
@@ -400,6 +401,28 @@ __device__ __forceinline__ void bead_kernel_body(const BeadParams<T>& p, const B
         for (int i = threadIdx.x; i < kWords; i += blockDim.x) reinterpret_cast<uint4*>(patch)[i] = make_uint4(0, 0, 0, 0);
     }
     dependency_wait();
+    // the tile's first beads are on their way while the fields are staged (one
+    // wait for memory instead of two)
+    const int start = bf.tile_start[t];
+    const int end = bf.tile_start[t + 1];
+    constexpr int PER = kBeadChunk / 256;
+    T vx[PER], vy[PER], vz[PER];
+    int vt[PER];
+    int2 vn[PER];
+    auto load_chunk = [&](int c0, int cnt) {
+#pragma unroll
+        for (int k = 0; k < PER; ++k) {
+            const int j = threadIdx.x + k * 256;
+            if (j < cnt) {
+                vx[k] = bf.px[c0 + j];
+                vy[k] = bf.py[c0 + j];
+                vz[k] = bf.pz[c0 + j];
+                vt[k] = bf.id[c0 + j];
+                if (kForce) vn[k] = bf.nbr[c0 + j];
+            }
+        }
+    };
+    load_chunk(start, min(kBeadChunk, end - start));
     __syncthreads();
     if (AN && kForce && row_lane) {
         // stage w_2p, w_2p+1 of the patch from pot = i (w_2p + i w_2p+1)
@@ -455,8 +478,6 @@ __device__ __forceinline__ void bead_kernel_body(const BeadParams<T>& p, const B
             }
         }
     }
-    const int start = bf.tile_start[t];
-    const int end = bf.tile_start[t + 1];
     // noise counter n+1 of this step (advanced by the first kernel of the step)
     const uint64_t step_next = (MODE == kModeStep) ? *bf.step : 0ull;
     // 32-bit patch sums cannot overflow below this many beads per tile
@@ -466,34 +487,19 @@ __device__ __forceinline__ void bead_kernel_body(const BeadParams<T>& p, const B
 
     for (int c0 = start; c0 < end; c0 += kBeadChunk) {
         const int cnt = min(kBeadChunk, end - c0);
-        if (c0 != start) __syncthreads();  // the previous chunk is done with the staged beads
-        {
-            // all loads of the chunk in flight before the shared stores
-            constexpr int PER = kBeadChunk / 256;
-            T vx[PER], vy[PER], vz[PER];
-            int vt[PER];
-            int2 vn[PER];
+        if (c0 != start) {
+            __syncthreads();  // the previous chunk is done with the staged beads
+            load_chunk(c0, cnt);
+        }
 #pragma unroll
-            for (int k = 0; k < PER; ++k) {
-                const int j = threadIdx.x + k * 256;
-                if (j < cnt) {
-                    vx[k] = bf.px[c0 + j];
-                    vy[k] = bf.py[c0 + j];
-                    vz[k] = bf.pz[c0 + j];
-                    vt[k] = bf.id[c0 + j];
-                    if (kForce) vn[k] = bf.nbr[c0 + j];
-                }
-            }
-#pragma unroll
-            for (int k = 0; k < PER; ++k) {
-                const int j = threadIdx.x + k * 256;
-                if (j < cnt) {
-                    s_pos[j] = vx[k];
-                    s_pos[kBeadChunk + j] = vy[k];
-                    s_pos[2 * kBeadChunk + j] = vz[k];
-                    s_tag[j] = vt[k];
-                    if (kForce) s_nbr[j] = vn[k];
-                }
+        for (int k = 0; k < PER; ++k) {
+            const int j = threadIdx.x + k * 256;
+            if (j < cnt) {
+                s_pos[j] = vx[k];
+                s_pos[kBeadChunk + j] = vy[k];
+                s_pos[2 * kBeadChunk + j] = vz[k];
+                s_tag[j] = vt[k];
+                if (kForce) s_nbr[j] = vn[k];
             }
         }
         __syncthreads();
@@ -648,8 +654,16 @@ __device__ __forceinline__ void bead_kernel_body(const BeadParams<T>& p, const B
     }
 }
 
+// Resident CTAs the registers are allocated for. FP32, two species: order 1
+// takes 64 registers and four CTAs; order 2 spills at 64 and its 66 KB of
+// shared memory allow three CTAs anyway (64^3, 200,000 beads: step 46.4 ->
+// 44.6 us; the analytic force, 33 KB, keeps four: 53.3 against 54.0 at 80^3);
+// order 3 needs two (48^3: 28.2 against 35.7 with three).
+template <int P, typename T, bool AN, int NS> __host__ __device__ constexpr int bead_ctas() {
+    return sizeof(T) == 8 || NS != 2 ? 2 : P == 2 ? 4 : P == 3 ? (AN ? 4 : 3) : 2;
+}
 template <int P, int MODE, typename T, bool AN = false, int NS = 2>
-__global__ void __launch_bounds__(256, (sizeof(T) == 4 && P <= 3 && NS == 2) ? 4 : 2)
+__global__ void __launch_bounds__(256, bead_ctas<P, T, AN, NS>())
     bead_kernel(BeadParams<T> p, BeadBuffers<T> bf) {
     bead_kernel_body<P, MODE, T, AN, NS>(p, bf, blockIdx.x);
 }
@@ -660,7 +674,7 @@ template <typename T> struct BeadArgs {
     BeadBuffers<T> bf;
 };
 template <int P, int MODE, typename T>
-__global__ void __launch_bounds__(256, (sizeof(T) == 4 && P <= 3) ? 4 : 2)
+__global__ void __launch_bounds__(256, bead_ctas<P, T, false, 2>())
     bead_kernel_batched(const BeadArgs<T>* __restrict__ args, int tiles3) {
     const int r = blockIdx.x / tiles3;
     bead_kernel_body<P, MODE, T>(args[r].p, args[r].bf, blockIdx.x - r * tiles3);

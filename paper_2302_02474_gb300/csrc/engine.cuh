@@ -1058,9 +1058,10 @@ template <typename T> class Engine final : public EngineBase {
     int* ranks_ = nullptr;  // and its rank in the bin
     int* counts_ = nullptr;  // [n_fine_] bead counts of the fine bins
     size_t n_fine_ = 0;
-    // Bins up to which one block scans them (128^3: one launch of 9 us for four
-    // of 14 us in all; 24^3: 3 for 14)
-    static constexpr size_t kScanOne = 65537;
+    // Bins up to which one block scans them, in rounds of 4,096 (24^3: one launch
+    // of 3 us for four of 14 us in all; at 128^3, 65,537 bins, the 17 rounds take
+    // 36 us and the three scan kernels stay)
+    static constexpr size_t kScanOne = 16384;
     int* tile_start_ = nullptr;
     int n_tiles_ = 0;
     int* fine_start_ = nullptr;  // [n_fine_] exclusive scan of counts_

@@ -24,6 +24,14 @@
 
 namespace tild {
 
+// *any = whether one of the n flag words is set (one block of 256 threads).
+static __global__ void __launch_bounds__(256) any_flag(unsigned* const* __restrict__ flags, int n, unsigned* __restrict__ any) {
+    unsigned f = 0;
+    for (int i = threadIdx.x; i < n; i += 256) f |= *flags[i];
+    f = __syncthreads_or(f != 0);
+    if (threadIdx.x == 0) *any = f;
+}
+
 template <typename T> class BatchEngine final : public BatchBase {
     using V = cplx_t<T>;
     using E = Engine<T>;
@@ -47,6 +55,8 @@ template <typename T> class BatchEngine final : public BatchBase {
         if (stream_) cudaStreamSynchronize(stream_);
         if (graph_) cudaGraphExecDestroy(graph_);
         for (void* q : pbufs_) cudaFree(q);
+        cudaFree(flags_);
+        cudaFree(any_);
         for (auto& g : groups_) {
             if (g.s) cudaStreamDestroy(g.s);
             if (g.done) cudaEventDestroy(g.done);
@@ -127,6 +137,10 @@ template <typename T> class BatchEngine final : public BatchBase {
             sort_streams_.push_back(st);
         }
         TILD_CUDA(cudaEventCreateWithFlags(&fork_, cudaEventDisableTiming));
+        std::vector<unsigned*> flags;
+        for (E* e : reps_) flags.push_back(e->err_ptr());
+        if (tild_status fst = upload(&flags_, flags)) return fst;
+        TILD_CUDA(cudaMalloc(&any_, sizeof(unsigned)));
         tild_status pst = init_persistent();
         if (pst) return pst;
         TILD_CUDA(cudaStreamSynchronize(stream_));
@@ -326,6 +340,13 @@ template <typename T> class BatchEngine final : public BatchBase {
                 return TILD_ETIMEOUT;
             }
         }
+        // one look at every replica's error flags; the replicas one by one only
+        // when one is set
+        any_flag<<<1, 256, 0, stream_>>>(flags_, (int)reps_.size(), any_);
+        unsigned any = 0;
+        TILD_CUDA(cudaMemcpyAsync(&any, any_, sizeof(any), cudaMemcpyDeviceToHost, stream_));
+        TILD_CUDA(cudaStreamSynchronize(stream_));
+        if (!any) return TILD_OK;
         for (E* e : reps_) {
             const tild_status st = e->check_err();
             if (st) return fail_from(e);
@@ -365,6 +386,8 @@ template <typename T> class BatchEngine final : public BatchBase {
    private:
     std::vector<E*> reps_;
     std::vector<Group> groups_;
+    unsigned** flags_ = nullptr;  // device table of the replicas' error words
+    unsigned* any_ = nullptr;
     // persistent path
     bool persistent_ = false, graph_ok_ = true;
     bool by_rule_ = true;  // the path is the default's, not the caller's or the autotuner's

@@ -89,7 +89,7 @@ template <typename T> struct BeadBuffers {
     T* __restrict__ v_out;        // FORCE: velocities by id (may be null)
     const T* __restrict__ v_in;   // SETVEL: velocities by id (null: Maxwell-Boltzmann)
     // FORCE (may be null): [blocks][5] sums of |bond|^2 (scaled by e_len^2, each
-    // bond once), |v|^2 (by e_vel^2) and F
+    // bond from both of its ends), |v|^2 (by e_vel^2) and F
     typename Wide<T>::stored* __restrict__ partials;
 };
 
@@ -174,6 +174,22 @@ template <int P, typename T> struct Stencil {
     }
 };
 
+// Gradient of a gathered scalar: per stencil row (b, c) the sums s = sum_a
+// w_x[a] f and ds = sum_a w_x'[a] f, two products per point instead of six.
+template <typename T> struct RowGrad {
+    T s = T(0), ds = T(0);
+    __device__ __forceinline__ void point(T w, T dw, T f) {
+        s = fma_rn(w, f, s);
+        ds = fma_rn(dw, f, ds);
+    }
+    // add the row: weights y, z and their derivatives
+    __device__ __forceinline__ void add_to(T wy, T wz, T dwy, T dwz, T& gx, T& gy, T& gz) const {
+        gx = fma_rn(ds, wy * wz, gx);
+        gy = fma_rn(s, dwy * wz, gy);
+        gz = fma_rn(s, wy * dwz, gz);
+    }
+};
+
 template <typename T> struct vec4_of;
 template <> struct vec4_of<float> { using type = float4; };
 template <> struct vec4_of<double> { using type = double4_16a; };
@@ -254,15 +270,11 @@ __device__ __forceinline__ void gather_force_an(const Stencil<P, T>& st, const T
         for (int c = 0; c < P; ++c)
 #pragma unroll
             for (int b = 0; b < P; ++b) {
-                const T wyz = st.wy[b] * st.wz[c], dyz = dwy[b] * st.wz[c], ydz = st.wy[b] * dwz[c];
                 const int row = ((l.z + c) * PT::W + (l.y + b)) * PT::W + l.x;
+                RowGrad<T> r;
 #pragma unroll
-                for (int a = 0; a < P; ++a) {
-                    const T w = sp[row + a];
-                    gx += dwx[a] * wyz * w;
-                    gy += st.wx[a] * dyz * w;
-                    gz += st.wx[a] * ydz * w;
-                }
+                for (int a = 0; a < P; ++a) r.point(st.wx[a], dwx[a], sp[row + a]);
+                r.add_to(st.wy[b], st.wz[c], dwy[b], dwz[c], gx, gy, gz);
             }
     } else {
         const int comp = species & 1;
@@ -273,15 +285,13 @@ __device__ __forceinline__ void gather_force_an(const Stencil<P, T>& st, const T
 #pragma unroll
             for (int b = 0; b < P; ++b) {
                 const size_t oy = oz + (size_t)pwrap(st.jy + b, n) * n;
-                const T wyz = st.wy[b] * st.wz[c], dyz = dwy[b] * st.wz[c], ydz = st.wy[b] * dwz[c];
+                RowGrad<T> r;
 #pragma unroll
                 for (int a = 0; a < P; ++a) {
                     const cplx_t<T> v = __ldca(pot + oy + pwrap(st.jx + a, n));
-                    const T w = comp ? -v.x : v.y;
-                    gx += dwx[a] * wyz * w;
-                    gy += st.wx[a] * dyz * w;
-                    gz += st.wx[a] * ydz * w;
+                    r.point(st.wx[a], dwx[a], comp ? -v.x : v.y);
                 }
+                r.add_to(st.wy[b], st.wz[c], dwy[b], dwz[c], gx, gy, gz);
             }
         }
     }
@@ -305,10 +315,10 @@ __device__ __forceinline__ void spread_bead(const Stencil<P, T>& st, bool in_pat
         for (int c = 0; c < P; ++c)
 #pragma unroll
             for (int b = 0; b < P; ++b) {
-                const T wyz = st.wy[b] * st.wz[c];
+                const T wyz = FP::scaled(st.wy[b] * st.wz[c]);
                 const int row = ((l.z + c) * PT::W + (l.y + b)) * PT::W + l.x;
 #pragma unroll
-                for (int a = 0; a < P; ++a) atomicAdd(base + row + a, FP::to_patch(st.wx[a] * wyz));
+                for (int a = 0; a < P; ++a) atomicAdd(base + row + a, FP::to_patch(st.wx[a], wyz));
             }
     } else {
         const size_t M = (size_t)n * n * n;
@@ -316,11 +326,11 @@ __device__ __forceinline__ void spread_bead(const Stencil<P, T>& st, bool in_pat
         for (int c = 0; c < P; ++c)
 #pragma unroll
             for (int b = 0; b < P; ++b) {
-                const T wyz = st.wy[b] * st.wz[c];
+                const T wyz = FP::scaled(st.wy[b] * st.wz[c]);
 #pragma unroll
                 for (int a = 0; a < P; ++a) {
                     const size_t g = ((size_t)pwrap(st.jz + c, n) * n + pwrap(st.jy + b, n)) * n + pwrap(st.jx + a, n);
-                    if (debug_check(g < M, err)) atomicAdd(rho_fx + K * M + g, FP::to_grid(st.wx[a] * wyz));
+                    if (debug_check(g < M, err)) atomicAdd(rho_fx + K * M + g, FP::to_grid(st.wx[a], wyz));
                 }
             }
     }
@@ -550,8 +560,6 @@ __device__ __forceinline__ void bead_kernel_body(const BeadParams<T>& p, const B
                 } else {
                     gather_force<P>(st, staged, l, s_grad, bf.grad, p.n, species, fx, fy, fz);
                 }
-                // the bond energy counts each bond once, at its end with the smaller bead id
-                auto nid_of = [&](int s) { return slot_bead_id(s >= c0 && s < c0 + cnt ? s_tag[s - c0] : bf.id[s]); };
 #pragma unroll
                 for (int k = 0; k < 2; ++k) {
                     const int s = k == 0 ? nb.x : nb.y;
@@ -562,7 +570,7 @@ __device__ __forceinline__ void bead_kernel_body(const BeadParams<T>& p, const B
                         fx -= p.k_bond * dx;
                         fy -= p.k_bond * dy;
                         fz -= p.k_bond * dz;
-                        if (MODE == kModeForce && sums && nid_of(s) > bid) add_squares(acc[0], dx, dy, dz, p.e_len);
+                        if (MODE == kModeForce && sums) add_squares(acc[0], dx, dy, dz, p.e_len);
                     }
                 }
                 for_each_extra_bond(nb, bf.ext, [&](int s) {
@@ -573,7 +581,7 @@ __device__ __forceinline__ void bead_kernel_body(const BeadParams<T>& p, const B
                     fx -= p.k_bond * dx;
                     fy -= p.k_bond * dy;
                     fz -= p.k_bond * dz;
-                    if (MODE == kModeForce && sums && nid_of(s) > bid) add_squares(acc[0], dx, dy, dz, p.e_len);
+                    if (MODE == kModeForce && sums) add_squares(acc[0], dx, dy, dz, p.e_len);
                 });
                 if (not_finite(fx, fy, fz)) atomicOr(bf.err, kErrNonFinite);
                 if (MODE == kModeForce) {
@@ -685,7 +693,7 @@ __global__ void __launch_bounds__(256, bead_ctas<P, T, false, 2>())
 // i.e. the adjoint of the spread (the same weights, differentiated) applied
 // to the potential field w_K, plus the bond term. `pot` holds
 // i (w_A + i w_B) per grid point. Output by bead id (null: none). The block's
-// sum of |bond|^2 (scaled, each bond once) goes to bf.partials[blockIdx.x], so
+// sum of |bond|^2 (scaled, each bond from both ends) goes to bf.partials[blockIdx.x], so
 // that the bond energy needs no force pass of its own.
 template <int P, typename T>
 __global__ void __launch_bounds__(256) adjoint_kernel(BeadParams<T> p, BeadBuffers<T> bf, const cplx_t<T>* __restrict__ pot,
@@ -708,16 +716,17 @@ __global__ void __launch_bounds__(256) adjoint_kernel(BeadParams<T> p, BeadBuffe
 #pragma unroll
             for (int c = 0; c < P; ++c)
 #pragma unroll
-                for (int b = 0; b < P; ++b)
+                for (int b = 0; b < P; ++b) {
+                    const cplx_t<T>* row = pot + (size_t)(species >> 1) * 4 * ((size_t)p.n * p.n * p.n) +
+                                           ((size_t)pwrap(st.jz + c, p.n) * p.n + pwrap(st.jy + b, p.n)) * p.n;
+                    RowGrad<T> r;
 #pragma unroll
                     for (int a = 0; a < P; ++a) {
-                        const size_t g = ((size_t)pwrap(st.jz + c, p.n) * p.n + pwrap(st.jy + b, p.n)) * p.n + pwrap(st.jx + a, p.n);
-                        const cplx_t<T> v = pot[(size_t)(species >> 1) * 4 * ((size_t)p.n * p.n * p.n) + g];
-                        const T w = (species & 1) ? -v.x : v.y;  // w_2p = Im, w_2p+1 = -Re of i (w_2p + i w_2p+1)
-                        gx += dx[a] * st.wy[b] * st.wz[c] * w;
-                        gy += st.wx[a] * dy[b] * st.wz[c] * w;
-                        gz += st.wx[a] * st.wy[b] * dz[c] * w;
+                        const cplx_t<T> v = row[pwrap(st.jx + a, p.n)];
+                        r.point(st.wx[a], dx[a], (species & 1) ? -v.x : v.y);  // w_2p = Im, w_2p+1 = -Re of i (w_2p + i w_2p+1)
                     }
+                    r.add_to(st.wy[b], st.wz[c], dy[b], dz[c], gx, gy, gz);
+                }
             gx *= p.inv_dx;
             gy *= p.inv_dx;
             gz *= p.inv_dx;
@@ -730,7 +739,7 @@ __global__ void __launch_bounds__(256) adjoint_kernel(BeadParams<T> p, BeadBuffe
             gx += p.k_bond * dx;
             gy += p.k_bond * dy;
             gz += p.k_bond * dz;
-            if (slot_bead_id(bf.id[s]) > bid) add_squares(acc[0], dx, dy, dz, p.e_len);
+            add_squares(acc[0], dx, dy, dz, p.e_len);
         };
         if (nb.x >= 0) bond(nb.x);
         if (nb.y >= 0) bond(nb.y);

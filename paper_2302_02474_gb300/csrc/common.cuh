@@ -64,26 +64,39 @@ template <> struct FixedPoint<float> {
     using patch_t = unsigned int;
     static constexpr double scale = 4194304.0;  // 2^22
     static constexpr int max_tile_beads = 1023;
-    // round(w 2^22) for w in [0, 1]: adding 1.5 2^23 rounds to nearest and leaves
-    // the integer in the low bits (the product is exact). The conversion
-    // instruction runs at a quarter of the rate of these two.
-    static __device__ __forceinline__ unsigned int to_patch(float w) {
-        return __float_as_uint(__fmaf_rn(w, 4194304.0f, 12582912.0f)) - 0x4B400000u;
+    // round(w 2^22) of a weight w = wx wyz in [0, 1], from wx and scaled(wyz):
+    // adding 1.5 2^23 rounds to nearest and leaves the integer in the low bits.
+    // The conversion instruction runs at a quarter of the rate.
+    static __device__ __forceinline__ float scaled(float wyz) { return wyz * 4194304.0f; }
+    static __device__ __forceinline__ unsigned int to_patch(float wx, float wyz_s) {
+        return __float_as_uint(__fmaf_rn(wx, wyz_s, 12582912.0f)) - 0x4B400000u;
     }
-    static __device__ __forceinline__ unsigned long long to_grid(float w) { return to_patch(w); }
+    static __device__ __forceinline__ unsigned long long to_grid(float wx, float wyz_s) { return to_patch(wx, wyz_s); }
 };
 // FP64: one 64-bit shared word per point and species.
 template <> struct FixedPoint<double> {
     using patch_t = unsigned long long;
     static constexpr double scale = 17592186044416.0;  // 2^44
     static constexpr int max_tile_beads = 0x7fffffff;
-    static __device__ __forceinline__ unsigned long long to_patch(double w) {
-        return (unsigned long long)__double2ll_rn(w * scale);
+    static __device__ __forceinline__ double scaled(double wyz) { return wyz * scale; }
+    static __device__ __forceinline__ unsigned long long to_patch(double wx, double wyz_s) {
+        return (unsigned long long)__double2ll_rn(wx * wyz_s);
     }
-    static __device__ __forceinline__ unsigned long long to_grid(double w) { return to_patch(w); }
+    static __device__ __forceinline__ unsigned long long to_grid(double wx, double wyz_s) { return to_patch(wx, wyz_s); }
 };
 // Fixed point -> density (scale = 2^-F / dV); no FP64 in the FP32 path.
-__device__ __forceinline__ float from_fixed(long long v, float scale) { return mul_rn(__ll2float_rn(v), scale); }
+// (FP32: the 64-bit conversion instruction is slow; the leading 32 bits of |v|
+// with a sticky bit for the rest round to the same float)
+__device__ __forceinline__ float ll_to_float(long long v) {
+    const unsigned long long a = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+    const unsigned hi = (unsigned)(a >> 32), lo = (unsigned)a;
+    const int s = __clz(hi);  // 32: |v| < 2^32
+    const unsigned top = s == 32 ? lo : __funnelshift_l(lo, hi, s) | ((lo << s) != 0u ? 1u : 0u);
+    const float f = __uint2float_rn(top);
+    const float r = s == 32 ? f : f * __int_as_float((127 + 32 - s) << 23);
+    return v < 0 ? -r : r;
+}
+__device__ __forceinline__ float from_fixed(long long v, float scale) { return mul_rn(ll_to_float(v), scale); }
 __device__ __forceinline__ double from_fixed(long long v, double scale) { return mul_rn((double)v, scale); }
 // The same for densities (v >= 0). A sum below 2^32 (a thousand beads on one
 // point) is converted from 32 bits: the 64-bit conversion runs at a small

@@ -267,7 +267,7 @@ template <typename T> class Engine final : public EngineBase {
         if (e) {
             const BeadParams<T> p = bead_params();
             const double el = p.e_len, ev = p.e_vel;
-            e->e_bond = 1.5 / (cfg_->b * cfg_->b) * h[5] / (el * el);
+            e->e_bond = 0.75 / (cfg_->b * cfg_->b) * h[5] / (el * el);  // every bond from both ends
             e->kinetic = 0.5 * cfg_->mass * h[6] / (ev * ev);
             for (int d = 0; d < 3; ++d) e->net_force[d] = h[7 + d];
             e->e_chi = e->e_kappa = e->e_elec = 0.0;
@@ -319,7 +319,7 @@ template <typename T> class Engine final : public EngineBase {
         for (int k = 0; k < 5; ++k) s[k] = host_sums()[k] / (er * er);
         s[2] *= kk * kk;  // summed with integer frequencies
         s[3] *= kk * kk;
-        const double eb = 1.5 / (cfg_->b * cfg_->b) * host_sums()[5] / ((double)p.e_len * p.e_len);
+        const double eb = 0.75 / (cfg_->b * cfg_->b) * host_sums()[5] / ((double)p.e_len * p.e_len);
         const double V = cfg_->L * cfg_->L * cfg_->L;
         const double dV = V / (double)M_;
         const double rho0 = cfg_->n_beads / V;

@@ -769,7 +769,7 @@ __global__ void __launch_bounds__(256) generic_bead_kernel(BeadParams<T> p, Bead
                 fx -= p.k_bond * dx;
                 fy -= p.k_bond * dy;
                 fz -= p.k_bond * dz;
-                if (MODE == kModeForce && sums && slot_bead_id(bf.id[s]) > bid) add_squares(acc[0], dx, dy, dz, p.e_len);
+                if (MODE == kModeForce && sums) add_squares(acc[0], dx, dy, dz, p.e_len);
             };
             if (nb.x >= 0) bond(nb.x);
             if (nb.y >= 0) bond(nb.y);
@@ -844,9 +844,9 @@ __global__ void __launch_bounds__(256) generic_bead_kernel(BeadParams<T> p, Bead
 #pragma unroll
                 for (int b = 0; b < P; ++b) {
                     const size_t oy = oz + (size_t)pwrap(st.jy + b, n) * n;
-                    const T wyz = st.wy[b] * wz;
+                    const T wyz = FP::scaled(st.wy[b] * wz);
 #pragma unroll
-                    for (int a = 0; a < P; ++a) atomicAdd(rk + oy + pwrap(st.jx + a, n), FP::to_grid(st.wx[a] * wyz));
+                    for (int a = 0; a < P; ++a) atomicAdd(rk + oy + pwrap(st.jx + a, n), FP::to_grid(st.wx[a], wyz));
                 }
             }
         }

@@ -42,11 +42,11 @@ __global__ void noalloc_spread(int64_t n_beads, const float* __restrict__ xyz, c
     for (int c = 0; c < P; ++c)
 #pragma unroll
         for (int b = 0; b < P; ++b) {
-            const float wyz = st.wy[b] * st.wz[c];
+            const float wyz = FixedPoint<float>::scaled(st.wy[b] * st.wz[c]);
 #pragma unroll
             for (int a = 0; a < P; ++a) {
                 const size_t g = ((size_t)((st.jz + c) & nm) * n + ((st.jy + b) & nm)) * n + ((st.jx + a) & nm);
-                atomicAdd(rho + K * M + g, FixedPoint<float>::to_grid(st.wx[a] * wyz));
+                atomicAdd(rho + K * M + g, FixedPoint<float>::to_grid(st.wx[a], wyz));
             }
         }
 }

@@ -440,17 +440,15 @@ __device__ __forceinline__ void vjp_gather_global(const Stencil<P, T>& st, const
 #pragma unroll
         for (int b = 0; b < P; ++b) {
             const size_t row = ((size_t)pwrap(st.jz + c, n) * n + pwrap(st.jy + b, n)) * n;
-            const T wyz = st.wy[b] * st.wz[c], dyz = dwy[b] * st.wz[c], ydz = st.wy[b] * dwz[c];
+            RowGrad<T> r;
 #pragma unroll
             for (int a = 0; a < P; ++a) {
                 const size_t g = row + pwrap(st.jx + a, n);
                 const cplx_t<T> f0 = fields[g], f1 = fields[M + g], f2 = fields[2 * M + g], f3 = __ldca(psi + g);
                 const T ldw = l[0] * (K ? f0.y : f0.x) + l[1] * (K ? f1.y : f1.x) + l[2] * (K ? f2.y : f2.x);
-                const T val = (K ? -f3.x : f3.y) * inv_dV - ldw;
-                o[0] += dwx[a] * wyz * val;
-                o[1] += st.wx[a] * dyz * val;
-                o[2] += st.wx[a] * ydz * val;
+                r.point(st.wx[a], dwx[a], (K ? -f3.x : f3.y) * inv_dV - ldw);
             }
+            r.add_to(st.wy[b], st.wz[c], dwy[b], dwz[c], o[0], o[1], o[2]);
         }
 }
 
@@ -543,15 +541,13 @@ __global__ void __launch_bounds__(256) vjp_beads_tiled(BeadParams<float> p, Bead
             for (int c = 0; c < P; ++c)
 #pragma unroll
                 for (int b = 0; b < P; ++b) {
-                    const float wyz = st.wy[b] * st.wz[c], dyz = dwy[b] * st.wz[c], ydz = st.wy[b] * dwz[c];
+                    RowGrad<float> r;
 #pragma unroll
                     for (int a = 0; a < P; ++a) {
                         const float4 f = base[(c * W + b) * W + a];
-                        const float val = f.w - (l[0] * f.x + l[1] * f.y + l[2] * f.z);
-                        o[0] += dwx[a] * wyz * val;
-                        o[1] += st.wx[a] * dyz * val;
-                        o[2] += st.wx[a] * ydz * val;
+                        r.point(st.wx[a], dwx[a], f.w - (l[0] * f.x + l[1] * f.y + l[2] * f.z));
                     }
+                    r.add_to(st.wy[b], st.wz[c], dwy[b], dwz[c], o[0], o[1], o[2]);
                 }
         } else {
             vjp_gather_global<P>(st, dwx, dwy, dwz, l, K, p.n, fields, psi, inv_dV, o);
@@ -588,14 +584,10 @@ __global__ void __launch_bounds__(256) density_vjp_kernel(BeadParams<T> p, BeadB
 #pragma unroll
         for (int b = 0; b < P; ++b) {
             const size_t row = ((size_t)pwrap(st.jz + c, n) * n + pwrap(st.jy + b, n)) * n;
-            const T wyz = st.wy[b] * st.wz[c], dyz = dwy[b] * st.wz[c], ydz = st.wy[b] * dwz[c];
+            RowGrad<T> r;
 #pragma unroll
-            for (int a = 0; a < P; ++a) {
-                const T v = f[row + pwrap(st.jx + a, n)];
-                ox += dwx[a] * wyz * v;
-                oy += st.wx[a] * dyz * v;
-                oz += st.wx[a] * ydz * v;
-            }
+            for (int a = 0; a < P; ++a) r.point(st.wx[a], dwx[a], f[row + pwrap(st.jx + a, n)]);
+            r.add_to(st.wy[b], st.wz[c], dwy[b], dwz[c], ox, oy, oz);
         }
     const T s = p.inv_dx * inv_dV;  // d/dr = (1/dx) d/ds
     out[3 * (size_t)bid] = ox * s;
@@ -654,10 +646,10 @@ __global__ void adjoint_step(size_t n3, const T* __restrict__ jt, double* __rest
     dependency_wait();
     if (i >= n3) return;
     const double r = rb[i] + (double)__ldcg(jt + i);
-    const double hb = sd * r + sh * ub[i], u = su * hb;
+    const double hb = sd * r + sh * ub[i], u = su == 1.0 ? hb : su * hb;
     rb[i] = r;
     ub[i] = u;
-    lam[i] = (T)(sf * hb + (at_start ? wf * u : 0.0));
+    lam[i] = at_start ? (T)(sf * hb + wf * u) : (T)(sf * hb);  // (FP64 operations are the cost here)
 }
 
 // Up to eight device-to-device copies in one launch (blockIdx.y = copy; 16-byte

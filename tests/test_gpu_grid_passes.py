@@ -63,3 +63,50 @@ def test_spectrum_and_gradients_match_numpy(B, n, prec):
         assert np.linalg.norm(got - zc) <= tol * np.linalg.norm(zc), s
         got = t.field_gradient(dtype=np.float64)
         assert np.linalg.norm(got - want) <= tol * np.linalg.norm(want), s
+
+
+ANY = [(3, n) for n in (4, 7, 17, 20, 26, 34, 45, 55)] + [(2, n) for n in (4, 13, 32, 65, 127, 300, 1500)]
+
+
+@pytest.mark.parametrize("species", [2, 3])
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("dim,n", ANY)
+def test_any_size_gradients_match_numpy(B, dim, n, prec, species):
+    """Factors in registers and through the second line buffer (primes), both
+    last axes, one and two species pairs, and lines too long for the fused
+    last pass. A factor of R points is a direct sum of R terms, so a line of
+    n1 n2 points has a relative error of at most about eps (n1 + n2); the
+    gradients take dim axes twice."""
+    mt = (I.MolType(120, 6, 3),)
+    L = 0.55 * n
+    draw = I.random_walk_positions_2d if dim == 2 else I.random_walk_positions
+    t = B.Tild(L, n, 1, prec, 5, dim=dim)
+    t.set_chains([(m.n_chains, m.N, m.n_a) for m in mt], 1.0)
+    chi = np.array([[0.0, 1.1, 0.6], [1.1, 0.0, 0.4], [0.6, 0.4, 0.0]])[:species, :species]
+    if species == 3:
+        t.set_species(3, np.arange(720) % 3)
+    t.set_interactions(1.1, 6.0, 0.5)
+    if species == 3:
+        t.set_chi_matrix(chi)
+    t.set_positions(draw(mt, L, 1.0, 7))
+    rho = t.density(dtype=np.float64)
+    axes = (1, 2, 3) if dim == 3 else (2, 3)
+    f = np.fft.fftfreq(n, 1.0 / n) * 2 * np.pi / L
+    g = f.copy()
+    if n % 2 == 0:
+        g[n // 2] = 0.0
+    kz = f if dim == 3 else np.zeros(1)
+    k2 = kz[:, None, None] ** 2 + f[None, :, None] ** 2 + f[None, None, :] ** 2
+    u = np.exp(-k2 * 0.5**2) / (720 / L**dim)
+    z = np.fft.fftn(rho, axes=axes)
+    w = [u * sum((chi[i, j] + 6.0) * z[j] for j in range(species)) for i in range(species)]
+    got = t.field_gradient(dtype=np.float64)
+    got = got[None] if species == 2 else got  # [pair, D, z, y, x, 2]
+    n1 = max(d for d in range(1, int(n**0.5) + 1) if n % d == 0)
+    tol = 2 * dim * np.finfo(np.float32 if prec == "fp32" else np.float64).eps * (n1 + n // n1)
+    ks = (g[None, None, :], g[None, :, None], g[:, None, None])[:dim]
+    for d in range(dim):
+        for s in range(species):
+            want = np.fft.ifftn(1j * ks[d] * w[s], axes=tuple(a - 1 for a in axes)).real
+            err = np.linalg.norm(got[s // 2, d, ..., s % 2] - want)
+            assert err <= tol * np.linalg.norm(want), (d, s)

@@ -50,6 +50,11 @@ template <typename T> class Engine final : public EngineBase {
         tiles_ = (n_ + kTile - 1) / kTile;
         P_ = cfg->pmeorder + 1;
         plane_fits_ = plane_fits(n_, sizeof(V));
+        // default launch shape of the planes (tild_set_launch_shapes, tild_autotune
+        // choose others): 512 threads; 128^3 FP32 1,024, which hide the latency of
+        // its one CTA per SM (step 146.9 -> 142.5 us); 64^3 FP64 the row and column
+        // passes, which spread over all SMs (320.8 -> 277.6; at 48^3 118 against 150)
+        plane_nt_ = sizeof(T) == 4 && n_ == 128 ? 1024 : sizeof(T) == 8 && n_ == 64 ? 0 : 512;
         C_ = std::min(n_, (int)(128 / sizeof(V)));  // y-column tiles of the split passes
         CZ_ = zpass_cols(n_);                          // column tiles of the z pass
         TILD_CUDA(cudaGetDevice(&device_));
@@ -1104,7 +1109,7 @@ template <typename T> class Engine final : public EngineBase {
         return (int)std::max(1L, std::min(32L, c));
     }
     size_t gaxis_smem() const { return ((size_t)n_ + 2 * (size_t)gaxis_lines() * (n_ + 1)) * sizeof(V); }
-    // blocks of the bead kernel (its FP64 partial sums)
+    // blocks of the bead kernel (its partial sums)
     size_t bead_blocks() const {
         return per_bead() ? ((size_t)cfg_->n_beads + bead_threads() - 1) / bead_threads() : (size_t)n_tiles_;
     }
@@ -1674,8 +1679,8 @@ template <typename T> class Engine final : public EngineBase {
     // default, at least 2
     static constexpr int zpass_cols_alt(int n) { return zpass_cols2(n); }
     size_t zpass_smem_cols(int c) const { return ((size_t)n_ + 4 * (size_t)n_ * c) * sizeof(V); }
-    // plane kernels with NT threads: stage B of the line transform keeps
-    // ceil(n N1 / NT) units of N2 values per thread; at most 32 complex.
+    // plane kernels with NT threads: 512, or for small planes (several per SM) 256
+    // or 128 with at most 32 complex values of a line transform's stage per thread.
     // 1024 threads where every thread has a stage-B unit (n N1 >= 1024).
     static constexpr bool plane_nt_ok(int n, int nt) {
         if (nt == 512) return true;

@@ -1,7 +1,7 @@
 // Grid and bead kernels for any grid size and for two-dimensional boxes
 // (Sec. "TILD Branch": periodic boxes in two or three dimensions; Listing
 // infile runs D = 2 on a 65 x 65 grid). The same method as the tiled path,
-// organised for generality rather than speed:
+// organised for any size:
 //   - beads: one thread per bead (no tiles or shared patches); the density
 //     is accumulated with 64-bit fixed-point global atomics, so it is as
 //     bit-reproducible as the tiled path's;

@@ -154,7 +154,8 @@ template <> struct Wide<float> {
     }
     __device__ __forceinline__ stored store() const { return {hi, lo}; }
     static __device__ __forceinline__ Wide load(stored s) { return {s.x, s.y}; }
-    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+    // an infinite sum stays infinite: its rounding errors (inf - inf) say nothing
+    __device__ __forceinline__ double value() const { return isfinite(hi) ? (double)hi + (double)lo : (double)hi; }
 };
 
 // acc += x^2

@@ -58,3 +58,20 @@ def test_density_float_readout(B, n_chains, n):
     d64, d32 = t.density(dtype=np.float64), t.density(dtype=np.float32)
     assert d64.max() > 0
     assert np.all(np.abs(d32 - d64) <= np.spacing(np.abs(d64).astype(np.float32)))
+
+
+@pytest.mark.parametrize("n", [16, 21])  # tiled and any-size kernels
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_an_infinite_velocity_gives_an_infinite_kinetic_energy(B, n, precision):
+    spec = I.small_system(n_chains=300, N=10, n_a=4, L=8.0, n=n, precision=precision)
+    t = B.Tild(spec.L, n, 1, precision, 3)
+    t.set_chains([(m.n_chains, m.N, m.n_a) for m in spec.moltypes], spec.b)
+    t.set_interactions(spec.chi, spec.kappa, spec.a)
+    t.set_integrator(0.005, 1.0, 1.0)
+    t.set_positions(I.initial_positions(spec))
+    v = np.zeros((3000, 3))
+    v[7, 1] = -np.inf
+    t.set_velocities(v)
+    _, e = t.compute(forces=False)
+    assert e["kinetic"] == np.inf
+    assert np.isfinite(e["bond"]) and np.isfinite(e["chi"]) and np.isfinite(e["kappa"])

@@ -40,7 +40,7 @@ __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(
 __device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
 template <class V> __device__ __forceinline__ V c_mul(V a, V b) {
-    return {fma_rn(a.x, b.x, -mul_rn(a.y, b.y)), fma_rn(a.x, b.y, mul_rn(a.y, b.x))};
+    return {fma_rn(a.x, b.x, -mul_rn(a.y, b.y)), fma_rn(a.y, b.x, mul_rn(a.x, b.y))};
 }
 template <class V> __device__ __forceinline__ V c_conj(V a) { return {a.x, -a.y}; }
 template <class V, typename T> __device__ __forceinline__ V c_scale(V a, T s) { return {a.x * s, a.y * s}; }
@@ -64,12 +64,13 @@ template <> struct FixedPoint<float> {
     using patch_t = unsigned int;
     static constexpr double scale = 4194304.0;  // 2^22
     static constexpr int max_tile_beads = 1023;
-    // round(w 2^22) of a weight w = wx wyz in [0, 1], from wx and scaled(wyz):
-    // adding 1.5 2^23 rounds to nearest and leaves the integer in the low bits.
-    // The conversion instruction runs at a quarter of the rate.
+    // round(w 2^22) of a weight w = wx wyz in [0, 1], from wx and scaled(wyz); w
+    // is the float product, so that the integers are those of every kernel that
+    // forms the weight first. Adding 1.5 2^23 rounds to nearest and leaves the
+    // integer in the low bits: the conversion instruction runs at a quarter of the rate.
     static __device__ __forceinline__ float scaled(float wyz) { return wyz * 4194304.0f; }
     static __device__ __forceinline__ unsigned int to_patch(float wx, float wyz_s) {
-        return __float_as_uint(__fmaf_rn(wx, wyz_s, 12582912.0f)) - 0x4B400000u;
+        return __float_as_uint(__fadd_rn(__fmul_rn(wx, wyz_s), 12582912.0f)) - 0x4B400000u;
     }
     static __device__ __forceinline__ unsigned long long to_grid(float wx, float wyz_s) { return to_patch(wx, wyz_s); }
 };

@@ -35,9 +35,13 @@ template <> struct fft_split<40> { static constexpr int N1 = 8, N2 = 5; };
 template <> struct fft_split<48> { static constexpr int N1 = 16, N2 = 3; };
 template <> struct fft_split<80> { static constexpr int N1 = 16, N2 = 5; };
 
-// Multiply v by W_16^m = exp(DIR * 2 pi i m / 16); m is a compile-time
-// constant after unrolling, so the branches fold away.
-template <int DIR, class V> __device__ __forceinline__ V w16_mul(int m, V v) {
+// Multiply v by W_16^m = exp(DIR * 2 pi i m / 16), a factor of the R-point
+// radix (R = 8, 16); m is a compile-time constant after unrolling, so the
+// branches fold away. Which product of a sum is rounded by itself is part of
+// the transform's definition here: sums that nearly cancel, as the parameter
+// derivatives of a force product do, show the last bits of a spectrum, and a
+// spectrum is the same bits whatever kernel computes it.
+template <int DIR, int R, class V> __device__ __forceinline__ V w16_mul(int m, V v) {
     using T = decltype(v.x);
     const T c1 = T(0.92387953251128675613), s1 = T(0.38268343236508977173);  // cos, sin(pi/8)
     const T h = T(0.70710678118654752440);                                    // cos(pi/4)
@@ -63,7 +67,11 @@ template <int DIR, class V> __device__ __forceinline__ V w16_mul(int m, V v) {
         default: cr = c1; ci = s1; break;  // 15
     }
     if (DIR > 0) ci = -ci;
-    return c_mul(v, V{cr, ci});
+    if (m % 4 != 2) return c_mul(v, V{cr, ci});
+    // odd multiples of pi/4
+    const bool x_first = R == 16 || m == 2, y_first = R == 16 ? m == 6 : m == 2;
+    return {x_first ? fma_rn(v.x, cr, -mul_rn(v.y, ci)) : fma_rn(-v.y, ci, mul_rn(v.x, cr)),
+            y_first ? fma_rn(v.x, ci, mul_rn(v.y, cr)) : fma_rn(v.y, cr, mul_rn(v.x, ci))};
 }
 
 // In-register DFT of R points (R = 1, 2, 4, 8, 16 by radix-2 decimation in
@@ -80,7 +88,7 @@ template <int R, int DIR, class V> struct reg_dft {
         reg_dft<R / 2, DIR, V>::run(o);
 #pragma unroll
         for (int k = 0; k < R / 2; ++k) {
-            const V t = w16_mul<DIR>(k * (16 / R), o[k]);
+            const V t = w16_mul<DIR, R>(k * (16 / R), o[k]);
             v[k] = c_add(e[k], t);
             v[k + R / 2] = c_sub(e[k], t);
         }
@@ -98,10 +106,9 @@ template <int DIR, class V> struct reg_dft<3, DIR, V> {
         const T c = T(-0.5), s = T(DIR) * T(0.86602540378443864676);  // DIR sin(2 pi / 3)
         const V t1 = c_add(v[1], v[2]), t3 = c_sub(v[1], v[2]);
         const V m = {fma_rn(c, t1.x, v[0].x), fma_rn(c, t1.y, v[0].y)};
-        const V it = {-mul_rn(s, t3.y), mul_rn(s, t3.x)};  // i s (x1 - x2)
         v[0] = c_add(v[0], t1);
-        v[1] = c_add(m, it);
-        v[2] = c_sub(m, it);
+        v[1] = {fma_rn(-s, t3.y, m.x), fma_rn(s, t3.x, m.y)};  // m +- i s (x1 - x2)
+        v[2] = {fma_rn(s, t3.y, m.x), fma_rn(-s, t3.x, m.y)};
     }
 };
 

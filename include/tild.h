@@ -138,7 +138,8 @@ typedef struct {
  *   dU/dchi   = (1/rho_0) int int rho_A u_G rho_B          (Eq. fh)
  *   dU/dkappa = (1/2rho_0) int int (rho_+ - rho_0) u_G (rho_+ - rho_0)
  *   dU/da     = sum over k of (d u_hat/d a) (...), d u_hat/d a = -2 a |k|^2 u_hat
- * (sigma^2 = 2 a^2, Eqs. fhF, HelfandF), all reduced in FP64 on the device. */
+ * (sigma^2 = 2 a^2, Eqs. fhF, HelfandF), all reduced on the device with the
+ * precision and range of FP64 sums. */
 typedef struct {
     double energy;
     double e_bond;

@@ -90,7 +90,7 @@ template <typename T> struct BeadBuffers {
     const T* __restrict__ v_in;   // SETVEL: velocities by id (null: Maxwell-Boltzmann)
     // FORCE (may be null): [blocks][5] sums of |bond|^2 (scaled by e_len^2, each
     // bond from both of its ends), |v|^2 (by e_vel^2) and F
-    typename Wide<T>::stored* __restrict__ partials;
+    double* __restrict__ partials;
 };
 
 template <typename T> __device__ __forceinline__ T wrap_coord(T x, T L, T inv_L) {
@@ -658,7 +658,7 @@ __device__ __forceinline__ void bead_kernel_body(const BeadParams<T>& p, const B
         }
     }
     if constexpr (MODE == kModeForce) {
-        if (sums) block_sum<5, T>(acc, [&](int k, const Wide<T>& v) { bf.partials[5 * (size_t)t + k] = v.store(); });
+        if (sums) block_sum<5, T>(acc, [&](int k, double v) { bf.partials[5 * (size_t)t + k] = v; });
     }
 }
 
@@ -751,7 +751,36 @@ __global__ void __launch_bounds__(256) adjoint_kernel(BeadParams<T> p, BeadBuffe
             grad_out[3 * (size_t)bid + 2] = gz;
         }
     }
-    block_sum<1, T>(acc, [&](int, const Wide<T>& v) { bf.partials[blockIdx.x] = v.store(); });
+    block_sum<1, T>(acc, [&](int, double v) { bf.partials[blockIdx.x] = v; });
+}
+
+// The bead sums of an observable in FP64, not scaled: |bond|^2 (each bond from
+// both ends) and, from the velocities and forces by id of a force pass (null:
+// none), |v|^2 and F. Takes the place of an FP32 context's Wide sums that left
+// the range of floats.
+template <typename T>
+__global__ void __launch_bounds__(256) bead_sums64(BeadParams<T> p, BeadBuffers<T> bf, const T* __restrict__ v,
+                                                   const T* __restrict__ f, double* __restrict__ partials) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    Wide<double> acc[5];
+    if (i < p.n_beads) {
+        const T x = bf.px[i], y = bf.py[i], z = bf.pz[i];
+        const int2 nb = bf.nbr[i];
+        auto bond = [&](int s) {
+            const double dx = min_image(x - bf.px[s], p.L, p.inv_L), dy = min_image(y - bf.py[s], p.L, p.inv_L);
+            const double dz = min_image(z - bf.pz[s], p.L, p.inv_L);
+            acc[0].add(dx * dx + dy * dy + dz * dz);
+        };
+        if (nb.x >= 0) bond(nb.x);
+        if (nb.y >= 0) bond(nb.y);
+        for_each_extra_bond(nb, bf.ext, bond);
+        if (v)
+            for (int d = 0; d < 3; ++d) {
+                acc[1].add_prod(v[3 * (size_t)i + d], v[3 * (size_t)i + d]);
+                acc[2 + d].add(f[3 * (size_t)i + d]);
+            }
+    }
+    block_sum<5, double>(acc, [&](int k, double s) { partials[5 * (size_t)blockIdx.x + k] = s; });
 }
 
 // ------------------------------------------------------------- binning

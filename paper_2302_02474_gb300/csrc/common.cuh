@@ -108,91 +108,129 @@ __device__ __forceinline__ float density_from_fixed(long long v, float scale) {
 }
 __device__ __forceinline__ double density_from_fixed(long long v, double scale) { return from_fixed(v, scale); }
 
-// Sums of observables (energies, forces) in more than the working precision.
-// FP64 contexts sum in FP64. FP32 contexts sum pairs (hi, lo) of floats: a sum
-// keeps its rounding errors exactly (Knuth's two-sum) and a product its own
-// (by a fused multiply-add; Dekker 1971), about 48 bits in all. The FP64 unit
-// of this part does two operations per clock and SM, and the FP64 form of
-// these sums took longer than the passes that feed them (bead forces of 1.6M
-// beads 151 -> 77 us, 128^3 z pass with energies 98 -> 24 us, isolated).
+// Sums of observables (energies, forces): at least the precision of FP64 sums.
+// FP64 contexts sum in FP64. The FP64 unit of this part does two operations per
+// clock and SM, and FP64 sums of float terms took longer than the passes that
+// feed them; FP32 contexts therefore sum triples of floats. A sum (hi, mid)
+// keeps the rounding errors of hi exactly in mid, and those of mid in lo
+// (Knuth's two-sum), and a product its own (by a fused multiply-add; Dekker
+// 1971): what is lost is below 2^-70 of the sum per term. Per block the
+// triples become doubles. The exponent range remains that of floats, so terms
+// are scaled to be near 1, and a sum that left the range (wide_in_range) is
+// taken again in FP64 by bead_sums64 and spectral_sums64. Forces, energies and
+// density of 1.6M beads on 128^3: 437 us with FP64 sums, 243 with these (218
+// with pairs of floats, which hold 48 bits at best and fewer where the terms
+// are uneven).
 template <typename T> struct Wide;
 template <> struct Wide<double> {
     using stored = double;
     double v = 0.0;
+    static __device__ __forceinline__ Wide prod(double a, double b) { return {a * b}; }
+    static __device__ __forceinline__ Wide sum(double a, double b) { return {a + b}; }
     __device__ __forceinline__ void add(double x) { v += x; }
     __device__ __forceinline__ void add_prod(double a, double b) { v = fma(a, b, v); }
     __device__ __forceinline__ void add(const Wide& o) { v += o.v; }
     __device__ __forceinline__ Wide times(double s) const { return {v * s}; }
+    __device__ __forceinline__ Wide square() const { return {v * v}; }
     __device__ __forceinline__ Wide shfl_down(int o) const { return {__shfl_down_sync(0xffffffffu, v, o)}; }
     __device__ __forceinline__ stored store() const { return v; }
     static __device__ __forceinline__ Wide load(stored s) { return {s}; }
     __device__ __forceinline__ double value() const { return v; }
 };
+// s + e = a + b, s the rounded sum
+__device__ __forceinline__ float two_sum(float a, float b, float& e) {
+    const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+    return s;
+}
 template <> struct Wide<float> {
-    using stored = float2;
-    float hi = 0.f, lo = 0.f;
-    __device__ __forceinline__ void add(float x) {
-        const float s = __fadd_rn(hi, x), b = __fsub_rn(s, hi);
-        const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b));
-        hi = s;
+    using stored = float3;
+    float hi = 0.f, mid = 0.f, lo = 0.f;
+    static __device__ __forceinline__ Wide prod(float a, float b) {
+        const float p = __fmul_rn(a, b);
+        return {p, __fmaf_rn(a, b, -p), 0.f};
+    }
+    static __device__ __forceinline__ Wide sum(float a, float b) {
+        Wide r;
+        r.hi = two_sum(a, b, r.mid);
+        return r;
+    }
+    __device__ __forceinline__ void add_mid(float x) {
+        float e;
+        mid = two_sum(mid, x, e);
         lo = __fadd_rn(lo, e);
+    }
+    __device__ __forceinline__ void add(float x) {
+        float e;
+        hi = two_sum(hi, x, e);
+        add_mid(e);
     }
     __device__ __forceinline__ void add_prod(float a, float b) {
         const float p = __fmul_rn(a, b);
-        lo = __fadd_rn(lo, __fmaf_rn(a, b, -p));
         add(p);
+        add_mid(__fmaf_rn(a, b, -p));
     }
     __device__ __forceinline__ void add(const Wide& o) {
-        lo = __fadd_rn(lo, o.lo);
         add(o.hi);
+        add_mid(o.mid);
+        lo = __fadd_rn(lo, o.lo);
     }
     __device__ __forceinline__ Wide times(float s) const {
-        const float p = __fmul_rn(hi, s);
-        return {p, __fmaf_rn(lo, s, __fmaf_rn(hi, s, -p))};
+        Wide r = prod(hi, s);
+        const float q = __fmul_rn(mid, s);
+        r.lo = __fmaf_rn(lo, s, __fmaf_rn(mid, s, -q));
+        r.add_mid(q);
+        return r;
+    }
+    __device__ __forceinline__ Wide square() const {
+        Wide r = prod(hi, hi);
+        const float h2 = __fadd_rn(hi, hi), q = __fmul_rn(h2, mid);
+        r.lo = __fmaf_rn(h2, lo, __fmaf_rn(mid, mid, __fmaf_rn(h2, mid, -q)));
+        r.add_mid(q);
+        return r;
     }
     __device__ __forceinline__ Wide shfl_down(int o) const {
-        return {__shfl_down_sync(0xffffffffu, hi, o), __shfl_down_sync(0xffffffffu, lo, o)};
+        return {__shfl_down_sync(0xffffffffu, hi, o), __shfl_down_sync(0xffffffffu, mid, o), __shfl_down_sync(0xffffffffu, lo, o)};
     }
-    __device__ __forceinline__ stored store() const { return {hi, lo}; }
-    static __device__ __forceinline__ Wide load(stored s) { return {s.x, s.y}; }
+    __device__ __forceinline__ stored store() const { return make_float3(hi, mid, lo); }
+    static __device__ __forceinline__ Wide load(stored s) { return {s.x, s.y, s.z}; }
     // an infinite sum stays infinite: its rounding errors (inf - inf) say nothing
-    __device__ __forceinline__ double value() const { return isfinite(hi) ? (double)hi + (double)lo : (double)hi; }
+    __device__ __forceinline__ double value() const { return isfinite(hi) ? (double)hi + ((double)mid + (double)lo) : (double)hi; }
 };
-
-// acc += x^2
-__device__ __forceinline__ void add_square(Wide<double>& acc, const Wide<double>& x) { acc.add_prod(x.v, x.v); }
-__device__ __forceinline__ void add_square(Wide<float>& acc, const Wide<float>& x) {
-    acc.add_prod(x.hi, x.hi);
-    acc.lo = __fmaf_rn(__fadd_rn(x.hi, x.hi), x.lo, acc.lo);
+// Whether the value of an FP32 context's Wide sum can be taken as it is: finite,
+// and so large that products below the range of floats (2^-149 each) are no
+// part of it. zero_ok: whether a zero is known to be no such loss.
+template <typename T> inline bool wide_in_range(double v, bool zero_ok) {
+    return sizeof(T) == 8 || (v - v == 0.0 && (v == 0.0 ? zero_ok : v > 0x1p-60 || v < -0x1p-60));
 }
 
-// Sums of the K values over a block of up to 1024 threads, in a fixed order;
-// thread 0 writes them to out[0 .. K - 1].
+// Sums of the K values over a block (whole warps, up to 32), in a fixed order;
+// out(k, sum) is called by one thread for each k.
 template <int K, typename T, class Out> __device__ __forceinline__ void block_sum(Wide<T> (&acc)[K], Out out) {
     __shared__ typename Wide<T>::stored red[K][32];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, warps = blockDim.x >> 5;
 #pragma unroll
     for (int k = 0; k < K; ++k) {
         for (int o = 16; o > 0; o >>= 1) acc[k].add(acc[k].shfl_down(o));
         if (lane == 0) red[k][wid] = acc[k].store();
     }
     __syncthreads();
-    if (threadIdx.x < K) {
+    for (int k = wid; k < K; k += warps) {
         Wide<T> s;
-        for (int w = 0; w < (int)blockDim.x / 32; ++w) s.add(Wide<T>::load(red[threadIdx.x][w]));
-        out(threadIdx.x, s);
+        if (lane < warps) s = Wide<T>::load(red[k][lane]);
+        for (int o = 16; o > 0; o >>= 1) s.add(s.shfl_down(o));
+        if (lane == 0) out(k, s.value());
     }
 }
 
 // out[k] = sum of component k = blockIdx.x of the K-component block sums.
-template <typename T>
-__global__ void __launch_bounds__(1024) sum_partials(const typename Wide<T>::stored* __restrict__ partials, int n_blocks, int K,
-                                                     double* __restrict__ out) {
-    Wide<T> acc[1];
+static __global__ void __launch_bounds__(1024) sum_partials(const double* __restrict__ partials, int n_blocks, int K,
+                                                            double* __restrict__ out) {
+    Wide<double> acc[1];
     const int k = blockIdx.x;
 #pragma unroll 4
-    for (int b = threadIdx.x; b < n_blocks; b += 1024) acc[0].add(Wide<T>::load(partials[(size_t)b * K + k]));
-    block_sum<1, T>(acc, [&](int, const Wide<T>& s) { out[k] = s.value(); });
+    for (int b = threadIdx.x; b < n_blocks; b += blockDim.x) acc[0].add(partials[(size_t)b * K + k]);
+    block_sum<1, double>(acc, [&](int, double s) { out[k] = s; });
 }
 
 // Tiles of the bead kernel: beads are binned by 8x8x8 grid cells.

@@ -257,7 +257,7 @@ template <typename T> class Engine final : public EngineBase {
         if ((st = enqueue_fields(want_e ? 1 : 0, partials_, nullptr))) return st;
         if (want_e && (st = reduce_partials(z_blocks(), 5, sums()))) return st;
         BeadBuffers<T> bf = bead_buffers();
-        if (e) bf.partials = (typename Wide<T>::stored*)partials_;
+        if (e) bf.partials = partials_;
         const size_t n3 = (size_t)3 * cfg_->n_beads;
         const bool direct = f && device_native(dtype, where);  // the kernel writes the caller's array
         if (f) {
@@ -268,10 +268,19 @@ template <typename T> class Engine final : public EngineBase {
         if (e && (st = reduce_partials(bead_blocks(), 5, sums() + 5))) return st;
         if (f && !direct && (st = stage_out_vec((T*)aux_, n3, f, dtype, where))) return st;
         if ((st = finish())) return st;
-        const double* h = host_sums();
+        const BeadParams<T> p = bead_params();
+        double h[10], el = p.e_len, ev = p.e_vel, er = spectral_params().e_rho;
+        std::copy(host_sums(), host_sums() + 10, h);
         if (e) {
-            const BeadParams<T> p = bead_params();
-            const double el = p.e_len, ev = p.e_vel;
+            const bool bead_ok = wide_in_range<T>(h[5], !has_bonds()) && wide_in_range<T>(h[6], p.vu == T(0) && p.vf == T(0) && p.vg == T(0)) &&
+                                 std::isfinite(h[7] + h[8] + h[9]);
+            const bool k_ok = !want_e || (wide_in_range<T>(h[0], true) && wide_in_range<T>(h[1], true) && wide_in_range<T>(h[4], true));
+            if (sizeof(T) == 4 && !(bead_ok && k_ok)) {
+                if ((st = sums_fp64(want_e, true, h))) return st;
+                el = ev = er = 1.0;
+            }
+        }
+        if (e) {
             e->e_bond = 0.75 / (cfg_->b * cfg_->b) * h[5] / (el * el);  // every bond from both ends
             e->kinetic = 0.5 * cfg_->mass * h[6] / (ev * ev);
             for (int d = 0; d < 3; ++d) e->net_force[d] = h[7 + d];
@@ -280,7 +289,7 @@ template <typename T> class Engine final : public EngineBase {
         if (want_e && e) {
             const double V = volume();
             const double dV = V / (double)M_;
-            const double rho0 = cfg_->n_beads / V, er = spectral_params().e_rho;
+            const double rho0 = cfg_->n_beads / V;
             // one pair: the z pass sums Re[conj(rho_A) rho_B]; two pairs: chi-weighted sums
             e->e_chi = (NP_ == 1 ? cfg_->chi : 1.0) / rho0 * dV * dV / V * (h[0] / (er * er));
             e->e_kappa = cfg_->kappa / (2.0 * rho0) * dV * dV / V * (h[1] / (er * er));
@@ -304,7 +313,7 @@ template <typename T> class Engine final : public EngineBase {
         if ((st = enqueue_fields(2, partials_, nullptr, kInvPot))) return st;
         if ((st = reduce_partials(n_z_blocks_, 5, sums()))) return st;
         BeadBuffers<T> bf = bead_buffers();
-        bf.partials = (typename Wide<T>::stored*)partials_;
+        bf.partials = partials_;
         const bool direct = dUdr && device_native(dtype, where);
         if (dUdr && !direct && (st = ensure_aux(3 * N * sizeof(T)))) return st;
         T* out = !dUdr ? nullptr : direct ? (T*)dUdr : (T*)aux_;
@@ -319,12 +328,19 @@ template <typename T> class Engine final : public EngineBase {
         if ((st = reduce_partials(blocks(N), 1, sums() + 5))) return st;
         if (dUdr && !direct && (st = stage_out_vec((T*)aux_, 3 * N, dUdr, dtype, where))) return st;
         if ((st = finish())) return st;
-        const double er = spectral_params().e_rho, kk = 2.0 * 3.14159265358979323846 / cfg_->L;
-        double s[5];
-        for (int k = 0; k < 5; ++k) s[k] = host_sums()[k] / (er * er);
+        const double kk = 2.0 * 3.14159265358979323846 / cfg_->L;
+        double s[6], el = p.e_len, er = spectral_params().e_rho;
+        std::copy(host_sums(), host_sums() + 6, s);
+        bool ok = wide_in_range<T>(s[5], !has_bonds());
+        for (int k = 0; k < 5; ++k) ok = ok && wide_in_range<T>(s[k], true);
+        if (sizeof(T) == 4 && !ok) {
+            if ((st = sums_fp64(true, false, s))) return st;
+            el = er = 1.0;
+        }
+        for (int k = 0; k < 5; ++k) s[k] /= er * er;
         s[2] *= kk * kk;  // summed with integer frequencies
         s[3] *= kk * kk;
-        const double eb = 0.75 / (cfg_->b * cfg_->b) * host_sums()[5] / ((double)p.e_len * p.e_len);
+        const double eb = 0.75 / (cfg_->b * cfg_->b) * s[5] / (el * el);
         const double V = cfg_->L * cfg_->L * cfg_->L;
         const double dV = V / (double)M_;
         const double rho0 = cfg_->n_beads / V;
@@ -1158,7 +1174,7 @@ template <typename T> class Engine final : public EngineBase {
         TILD_CUDA(cudaGetLastError());
         return TILD_OK;
     }
-    tild_status line_spectral(typename Wide<T>::stored* partials) {
+    tild_status line_spectral(double* partials) {
         const int lg = line_last_lg();
         const SpectralParams<T> sp = spectral_params();
         const LineArgs<T> a = line_args(lg, n_);
@@ -1364,8 +1380,48 @@ template <typename T> class Engine final : public EngineBase {
     const double* host_sums() const { return reinterpret_cast<const double*>(words_ + 4); }
     // sums()[k] of the K-component block sums in partials_
     tild_status reduce_partials(size_t n_blocks, int K, double* out) {
-        sum_partials<T><<<K, 1024, 0, stream_>>>((const typename Wide<T>::stored*)partials_, (int)n_blocks, K, out);
+        sum_partials<<<K, (unsigned)std::min<size_t>(1024, (n_blocks + 31) / 32 * 32), 0, stream_>>>(partials_, (int)n_blocks, K, out);
         TILD_CUDA(cudaGetLastError());
+        return TILD_OK;
+    }
+    bool has_bonds() const {
+        if (cfg_->explicit_bonds) return !cfg_->bond_pairs.empty();
+        for (int k = 0; k < cfg_->topo.n_types; ++k)
+            if (cfg_->topo.N[k] > 1) return true;
+        return false;
+    }
+    // The sums of an observable again in FP64 (an FP32 context's that left the
+    // range of floats), not scaled: s[0 .. 4] the spectral ones, s[5] of the
+    // bonds and, with velocities and forces, s[6 .. 9].
+    tild_status sums_fp64(bool spectral, bool forces, double* s) {
+        const size_t N = cfg_->n_beads;
+        tild_status st;
+        if ((st = device_buffer(&partials_, partials_bytes_, 5 * (size_t)blocks(std::max(N, M_)) * sizeof(double)))) return st;
+        T *v = nullptr, *f = nullptr;
+        if (forces) {  // (the fields at the beads are those of the call)
+            if ((st = ensure_aux(6 * N * sizeof(T)))) return st;
+            BeadBuffers<T> bf = bead_buffers();
+            bf.f_out = f = (T*)aux_;
+            bf.v_out = v = f + 3 * N;
+            if ((st = launch_bead(kModeForce, bf))) return st;
+        }
+        bead_sums64<T><<<blocks(N), 256, 0, stream_>>>(bead_params(), bead_buffers(), v, f, partials_);
+        TILD_CUDA(cudaGetLastError());
+        if ((st = reduce_partials(blocks(N), 5, sums() + 5))) return st;
+        if (spectral) {
+            if ((st = device_buffer(&spec_, spec_bytes_, NP_ * M_ * sizeof(V)))) return st;
+            if ((st = enqueue_forward(false, true)) || (st = enqueue_zpass(nullptr, spec_))) return st;
+            const SpectralParams<T> sp = spectral_params();
+            const int el = c_el_on() ? 1 : 0;
+            if (NP_ == 2)
+                spectral_sums64<T, 2><<<blocks(M_), 256, 0, stream_>>>(spec_, n_, nz_, sp, el, partials_);
+            else
+                spectral_sums64<T, 1><<<blocks(M_), 256, 0, stream_>>>(spec_, n_, nz_, sp, el, partials_);
+            TILD_CUDA(cudaGetLastError());
+            if ((st = reduce_partials(blocks(M_), 5, sums()))) return st;
+        }
+        if ((st = finish())) return st;
+        std::copy(host_sums() + (spectral ? 0 : 5), host_sums() + (forces ? 10 : 6), s + (spectral ? 0 : 5));
         return TILD_OK;
     }
     // whether the caller's array can be a kernel's own input or output
@@ -1744,7 +1800,7 @@ template <typename T> class Engine final : public EngineBase {
         return sp;
     }
 
-    template <int NN> tild_status zpass_n(typename Wide<T>::stored* partials, V* spec_out, bool g_only, int want_e) {
+    template <int NN> tild_status zpass_n(double* partials, V* spec_out, bool g_only, int want_e) {
         constexpr int CC = zpass_cols(NN);
         const SpectralParams<T> sp = spectral_params();
         const bool el = c_el_on();
@@ -1827,8 +1883,7 @@ template <typename T> class Engine final : public EngineBase {
         if (c_el_on() && (st = refresh(cfg_->charge_smear, kernel_ae_, kernel1d_ + n_))) return st;
         return TILD_OK;
     }
-    tild_status enqueue_zpass(double* partials_d, V* spec_out, bool g_only = false, int want_e = 1) {
-        auto* partials = (typename Wide<T>::stored*)partials_d;
+    tild_status enqueue_zpass(double* partials, V* spec_out, bool g_only = false, int want_e = 1) {
         tild_status st;
         if ((st = refresh_tables())) return st;
         if (generic_) {

@@ -156,7 +156,7 @@ __global__ void generic_load_density(size_t M, int np, unsigned long long* __res
 template <typename T, int NP>
 __global__ void __launch_bounds__(256) generic_spectral(const cplx_t<T>* __restrict__ Z, cplx_t<T>* __restrict__ out,
                                                         int n, int nz, SpectralParams<T> sp,
-                                                        typename Wide<T>::stored* __restrict__ partials) {
+                                                        double* __restrict__ partials) {
     using V = cplx_t<T>;
     const size_t M = (size_t)nz * n * n;
     const size_t g = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -210,7 +210,7 @@ __global__ void __launch_bounds__(256) generic_spectral(const cplx_t<T>* __restr
         }
     }
     if (partials) {
-        block_sum<5, T>(acc, [&](int k, const Wide<T>& v) { partials[5 * (size_t)blockIdx.x + k] = v.store(); });
+        block_sum<5, T>(acc, [&](int k, double v) { partials[5 * (size_t)blockIdx.x + k] = v; });
     }
 }
 
@@ -595,7 +595,7 @@ __global__ void __launch_bounds__(128) line_y(LineArgs<T> g, cplx_t<T>* __restri
 // i k_last Q, Q_p = w~_2p + i w~_2p+1 (as in the z pass of the tiled grids).
 template <typename T, int NP, int D>
 __global__ void __launch_bounds__(128) line_last(LineArgs<T> g, const cplx_t<T>* __restrict__ Z, cplx_t<T>* __restrict__ H,
-                                                 SpectralParams<T> sp, typename Wide<T>::stored* __restrict__ partials) {
+                                                 SpectralParams<T> sp, double* __restrict__ partials) {
     using V = cplx_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LineShared<T> sh(smem_raw, g);
@@ -708,7 +708,7 @@ __global__ void __launch_bounds__(128) line_last(LineArgs<T> g, const cplx_t<T>*
     }
     if (partials) {
         const size_t b = (size_t)blockIdx.y * gridDim.x + blockIdx.x;
-        block_sum<5, T>(acc, [&](int k, const Wide<T>& v) { partials[5 * b + k] = v.store(); });
+        block_sum<5, T>(acc, [&](int k, double v) { partials[5 * b + k] = v; });
     }
 }
 
@@ -852,7 +852,7 @@ __global__ void __launch_bounds__(256) generic_bead_kernel(BeadParams<T> p, Bead
         }
     }
     if (MODE == kModeForce && sums) {
-        block_sum<5, T>(acc, [&](int k, const Wide<T>& v) { bf.partials[5 * (size_t)blockIdx.x + k] = v.store(); });
+        block_sum<5, T>(acc, [&](int k, double v) { bf.partials[5 * (size_t)blockIdx.x + k] = v; });
     }
 }
 

@@ -659,19 +659,13 @@ template <typename T, int N> __device__ __forceinline__ T freq_sq(int i) {
 template <typename T, int WANT_E, class V>
 __device__ __forceinline__ void add_energies(Wide<T> (&acc)[5], V A, V B, T uh, T e_rho, T weight, bool zero, T m2) {
     const T ar = A.x * e_rho, ai = A.y * e_rho, br = B.x * e_rho, bi = B.y * e_rho;
-    Wide<T> f;
-    f.add_prod(ar, br);
+    Wide<T> f = Wide<T>::prod(ar, br);
     f.add_prod(ai, bi);
     f = f.times(uh * weight);
     acc[0].add(f);
     if (WANT_E > 1) acc[2].add(f.times(m2));
-    Wide<T> tr, ti, q;
-    tr.add(ar);
-    tr.add(br);
-    ti.add(ai);
-    ti.add(bi);
-    add_square(q, tr);
-    add_square(q, ti);
+    Wide<T> q = Wide<T>::sum(ar, br).square();
+    q.add(Wide<T>::sum(ai, bi).square());
     q = q.times(zero ? T(0) : uh * weight);
     acc[1].add(q);
     if (WANT_E > 1) acc[3].add(q.times(m2));
@@ -809,8 +803,7 @@ __device__ __forceinline__ void z_tile(cplx_t<T>* buf, cplx_t<T>* tw, const cplx
                     wB.x = fma_rn(cB2, rq.x, wB.x);
                     wB.y = fma_rn(cB2, rq.y, wB.y);
                     if (WANT_E) {
-                        Wide<T> f;
-                        f.add_prod(rq.x * sp.e_rho, rq.x * sp.e_rho);
+                        Wide<T> f = Wide<T>::prod(rq.x * sp.e_rho, rq.x * sp.e_rho);
                         f.add_prod(rq.y * sp.e_rho, rq.y * sp.e_rho);
                         acc[4].add(f.times(weight * gq));
                     }
@@ -871,7 +864,7 @@ template <typename T> struct ZArgs {
     cplx_t<T>* H;
     const cplx_t<T>* tw;
     SpectralParams<T> sp;
-    typename Wide<T>::stored* energy_partials;
+    double* energy_partials;
 };
 
 template <typename T, int N, int C, bool G_ONLY = false, bool EL = false, int WANT_E = 0>
@@ -901,7 +894,7 @@ __device__ __forceinline__ void z_spectral_body(const ZArgs<T>& args, int bx, in
         });
     if constexpr (WANT_E != 0) {
         const size_t b = (size_t)by * gdx + bx;
-        block_sum<5, T>(acc, [&](int k, const Wide<T>& v) { args.energy_partials[5 * b + k] = v.store(); });
+        block_sum<5, T>(acc, [&](int k, double v) { args.energy_partials[5 * b + k] = v; });
     }
 }
 
@@ -951,7 +944,7 @@ template <typename T, int N, int C> __host__ __device__ constexpr int z_ctas() {
 template <typename T, int N, int C, bool G_ONLY = false, bool EL = false, int WANT_E = 0>
 __global__ void __launch_bounds__(256, z_ctas<T, N, C>()) z_spectral(const cplx_t<T>* __restrict__ Zxy, cplx_t<T>* __restrict__ H,
                                                   const cplx_t<T>* __restrict__ tw_g, SpectralParams<T> sp,
-                                                  typename Wide<T>::stored* __restrict__ energy_partials) {
+                                                  double* __restrict__ energy_partials) {
     z_spectral_body<T, N, C, G_ONLY, EL, WANT_E>(ZArgs<T>{Zxy, H, tw_g, sp, energy_partials}, blockIdx.x, blockIdx.y,
                                                  gridDim.x);
 }
@@ -982,8 +975,7 @@ __device__ __forceinline__ void add_energies4(Wide<T> (&acc)[5], const V (&A)[2 
     for (int K = 0; K < 2 * NP; ++K) {
 #pragma unroll
         for (int K2 = K + 1; K2 < 2 * NP; ++K2) {
-            Wide<T> f;
-            f.add_prod(S[K].x, S[K2].x);
+            Wide<T> f = Wide<T>::prod(S[K].x, S[K2].x);
             f.add_prod(S[K].y, S[K2].y);
             fchi.add(f.times(sp.chi4[K][K2]));
         }
@@ -992,9 +984,8 @@ __device__ __forceinline__ void add_energies4(Wide<T> (&acc)[5], const V (&A)[2 
     }
     acc[0].add(fchi.times(uh));
     if (!zero) {
-        Wide<T> q;
-        add_square(q, tr);
-        add_square(q, ti);
+        Wide<T> q = tr.square();
+        q.add(ti.square());
         acc[1].add(q.times(uh));
     }
 }
@@ -1078,7 +1069,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 1) z_spectral_pairs(
                                                                                 cplx_t<T>* __restrict__ H,
                                                                                 const cplx_t<T>* __restrict__ tw_g,
                                                                                 SpectralParams<T> sp,
-                                                                                typename Wide<T>::stored* __restrict__ energy_partials) {
+                                                                                double* __restrict__ energy_partials) {
     using V = cplx_t<T>;
     constexpr int NP = 2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1115,7 +1106,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 1) z_spectral_pairs(
         z_tile_pairs<T, N, C, 2, G_ONLY>(buf, tw, e1, sp, p0, ky, want_e, acc);
     if (want_e) {
         const size_t b = (size_t)by * gridDim.x + bx;
-        block_sum<5, T>(acc, [&](int k, const Wide<T>& v) { energy_partials[5 * b + k] = v.store(); });
+        block_sum<5, T>(acc, [&](int k, double v) { energy_partials[5 * b + k] = v; });
     }
     // buffer b = (d NP + q) R + r: field 0 (G) or 2 (G_z) of pair q, row r
     const int nbuf = (G_ONLY ? 1 : 2) * NP * R * TS;
@@ -1125,6 +1116,55 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 1) z_spectral_pairs(
         const int z = rem / C, c = rem % C;
         H[(3 * q + 2 * d) * M + z * NN + (size_t)ky[r] * N + p0 + c] = buf[i];
     }
+}
+
+// The z pass's energy sums in FP64, not scaled, from the spectra Z in natural
+// order ([NP][nz][n][n]; any n, one layer in two dimensions): [0 .. 4] of
+// add_energies (one pair; the Coulomb sum with el) or add_energies4. Takes the
+// place of an FP32 context's Wide sums that left the range of floats.
+template <typename T, int NP>
+__global__ void __launch_bounds__(256) spectral_sums64(const cplx_t<T>* __restrict__ Z, int n, int nz, SpectralParams<T> sp, int el,
+                                                       double* __restrict__ partials) {
+    using V = cplx_t<T>;
+    const size_t M = (size_t)nz * n * n, g = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    Wide<double> acc[5];
+    if (g < M) {
+        const int i[3] = {(int)(g % n), (int)((g / n) % n), (int)(g / ((size_t)n * n))}, len[3] = {n, n, nz};
+        size_t gm = 0;
+        T uh = T(1), uc = T(1), k2 = T(0);
+        double m2 = 0.0;
+        for (int d = 2; d >= 0; --d) gm = gm * len[d] + (i[d] == 0 ? 0 : len[d] - i[d]);
+        for (int d = 0; d < (nz > 1 ? 3 : 2); ++d) {
+            const T m = (T)(2 * i[d] < len[d] ? i[d] : i[d] - len[d]), k = sp.two_pi_over_L * m;
+            uh *= sp.kernel1d[i[d]];
+            if (el) uc *= sp.kernel1d_el[i[d]];
+            k2 += k * k;
+            m2 += (double)m * m;
+        }
+        V A[2 * NP];
+        double tr = 0.0, ti = 0.0, chi = 0.0;
+        for (int q = 0; q < NP; ++q) {
+            const V Zk = Z[q * M + g], Zm = Z[q * M + gm];
+            A[2 * q] = {T(0.5) * (Zk.x + Zm.x), T(0.5) * (Zk.y - Zm.y)};
+            A[2 * q + 1] = {T(0.5) * (Zk.y + Zm.y), -T(0.5) * (Zk.x - Zm.x)};
+        }
+        for (int K = 0; K < 2 * NP; ++K) {
+            tr += A[K].x;
+            ti += A[K].y;
+            for (int K2 = K + 1; K2 < 2 * NP; ++K2)
+                chi += (NP == 1 ? 1.0 : (double)sp.chi4[K][K2]) * ((double)A[K].x * A[K2].x + (double)A[K].y * A[K2].y);
+        }
+        const double fchi = uh * chi, fkap = g == 0 ? 0.0 : uh * (tr * tr + ti * ti);
+        acc[0].add(fchi);
+        acc[1].add(fkap);
+        acc[2].add(m2 * fchi);
+        acc[3].add(m2 * fkap);
+        if (el && k2 > T(0)) {
+            const double rx = sp.qA * A[0].x + sp.qB * A[1].x, ry = sp.qA * A[0].y + sp.qB * A[1].y;
+            acc[4].add((double)(uc * recip(k2)) * (rx * rx + ry * ry));
+        }
+    }
+    block_sum<5, double>(acc, [&](int k, double s) { partials[5 * (size_t)blockIdx.x + k] = s; });
 }
 
 }  // namespace tild

@@ -58,7 +58,7 @@ template <typename T> struct BeadParams {
     T vu, vf, vg, wu, wf, wg;
     int noise_lag;
     T sigma_v;        // sqrt(kT / m) (initial velocities)
-    T mass;
+    int species;      // of the density and field arrays (2 or 4)
     // powers of two near 1/L and near 1/sigma_v: bond vectors and velocities are
     // scaled by them before their squares are summed, so that no unit system
     // takes the squares out of the range of floats (1 in FP64)
@@ -173,6 +173,19 @@ template <int P, typename T> struct Stencil {
         dh_weights<P>(z * inv_dx, jz, wz);
     }
 };
+
+// Debug build: whether a bead's id, species and stencil index nothing outside the
+// context's arrays (pwrap brings points within one period back to the grid).
+template <int P, typename T>
+__device__ __forceinline__ bool bead_ok(const BeadParams<T>& p, const BeadBuffers<T>& bf, const Stencil<P, T>& st, int bid, int species) {
+    return debug_check(bid < p.n_beads && species < p.species && min(st.jx, min(st.jy, st.jz)) >= -p.n &&
+                           max(st.jx, max(st.jy, st.jz)) + P <= 2 * p.n,
+                       bf.err);
+}
+// the same of a neighbour's slot
+template <typename T> __device__ __forceinline__ bool slot_ok(const BeadParams<T>& p, const BeadBuffers<T>& bf, int s) {
+    return debug_check(s >= 0 && s < p.n_beads, bf.err);
+}
 
 // Gradient of a gathered scalar: per stencil row (b, c) the sums s = sum_a
 // w_x[a] f and ds = sum_a w_x'[a] f, two products per point instead of six.
@@ -574,7 +587,7 @@ __device__ __forceinline__ void bead_kernel_body(const BeadParams<T>& p, const B
                     }
                 }
                 for_each_extra_bond(nb, bf.ext, [&](int s) {
-                    if (!debug_check(s >= 0 && s < p.n_beads, bf.err)) return;
+                    if (!slot_ok(p, bf, s)) return;
                     const T dx = min_image(x - bf.px[s], p.L, p.inv_L);
                     const T dy = min_image(y - bf.py[s], p.L, p.inv_L);
                     const T dz = min_image(z - bf.pz[s], p.L, p.inv_L);
@@ -706,9 +719,10 @@ __global__ void __launch_bounds__(256) adjoint_kernel(BeadParams<T> p, BeadBuffe
         const int bid = slot_bead_id(tag);
         const int species = slot_species(tag);
         T gx = 0, gy = 0, gz = 0;
-        if (grad_out) {
-            Stencil<P, T> st;
-            st.set(x, y, z, p.inv_dx);
+        Stencil<P, T> st;
+        st.set(x, y, z, p.inv_dx);
+        const bool ok = bead_ok(p, bf, st, bid, species);
+        if (grad_out && ok) {
             T dx[P], dy[P], dz[P];
             dh_weight_derivs<P>(x * p.inv_dx, dx);
             dh_weight_derivs<P>(y * p.inv_dx, dy);
@@ -733,6 +747,7 @@ __global__ void __launch_bounds__(256) adjoint_kernel(BeadParams<T> p, BeadBuffe
         }
         const int2 nb = bf.nbr[i];
         auto bond = [&](int s) {
+            if (!slot_ok(p, bf, s)) return;
             const T dx = min_image(x - bf.px[s], p.L, p.inv_L);
             const T dy = min_image(y - bf.py[s], p.L, p.inv_L);
             const T dz = min_image(z - bf.pz[s], p.L, p.inv_L);
@@ -745,7 +760,7 @@ __global__ void __launch_bounds__(256) adjoint_kernel(BeadParams<T> p, BeadBuffe
         if (nb.y >= 0) bond(nb.y);
         for_each_extra_bond(nb, bf.ext, bond);
         if (not_finite(gx, gy, gz)) atomicOr(bf.err, kErrNonFinite);
-        if (grad_out) {
+        if (grad_out && ok) {
             grad_out[3 * (size_t)bid + 0] = gx;
             grad_out[3 * (size_t)bid + 1] = gy;
             grad_out[3 * (size_t)bid + 2] = gz;
@@ -767,6 +782,7 @@ __global__ void __launch_bounds__(256) bead_sums64(BeadParams<T> p, BeadBuffers<
         const T x = bf.px[i], y = bf.py[i], z = bf.pz[i];
         const int2 nb = bf.nbr[i];
         auto bond = [&](int s) {
+            if (!slot_ok(p, bf, s)) return;
             const double dx = min_image(x - bf.px[s], p.L, p.inv_L), dy = min_image(y - bf.py[s], p.L, p.inv_L);
             const double dz = min_image(z - bf.pz[s], p.L, p.inv_L);
             acc[0].add(dx * dx + dy * dy + dz * dz);

@@ -435,8 +435,8 @@ constexpr unsigned kErrNonFinite = 1u;
 constexpr unsigned kErrBounds = 2u;  // a bounds check of the debug build failed
 
 // Debug build (compiled with -DTILD_DEBUG=1, `_build.build(debug=True)`):
-// the bead kernels check slot and grid indices before they use them; a
-// failed check records kErrBounds in the context's error word and the access
+// the bead kernels, tiled and per bead, and the adjoint kernels check bead ids,
+// slots, species and grid indices before they use them; a failed check records kErrBounds in the context's error word and the access
 // is skipped (no trap), and the next synchronising call returns
 // TILD_EDEVICE. In the normal build every check is the constant true.
 #ifndef TILD_DEBUG

@@ -2018,7 +2018,7 @@ template <typename T> class Engine final : public EngineBase {
         p.k_bond = (T)(3.0 / (c.b * c.b));
         integrator_constants(c, p);
         p.sigma_v = (T)std::sqrt(c.kT / c.mass);
-        p.mass = (T)c.mass;
+        p.species = NS_;
         p.e_len = power_of_two(1.0 / c.L);
         p.e_vel = power_of_two(c.kT > 0 ? std::sqrt(c.mass / c.kT) : 1.0);
         p.seed = c.seed;

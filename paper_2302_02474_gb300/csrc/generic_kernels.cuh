@@ -733,7 +733,7 @@ __global__ void __launch_bounds__(256) generic_bead_kernel(BeadParams<T> p, Bead
         Stencil<P, T> st;
         st.set(x, y, z, p.inv_dx);
         constexpr int PZ = D == 3 ? P : 1;
-        if (MODE != kModeSpread) {
+        if (MODE != kModeSpread && bead_ok(p, bf, st, bid, species)) {
             // field force: -sum_g W(r - g) grad w_K(g)
             const cplx_t<T>* gp = bf.grad + (size_t)(species >> 1) * 4 * M;
             const int comp = species & 1;
@@ -763,6 +763,7 @@ __global__ void __launch_bounds__(256) generic_bead_kernel(BeadParams<T> p, Bead
             T fx = -gx, fy = -gy, fz = -gz;
             const int2 nb = bf.nbr[i];
             auto bond = [&](int s) {
+                if (!slot_ok(p, bf, s)) return;
                 const T dx = min_image(x - bf.px[s], p.L, p.inv_L);
                 const T dy = min_image(y - bf.py[s], p.L, p.inv_L);
                 const T dz = D == 3 ? min_image(z - bf.pz[s], p.L, p.inv_L) : T(0);
@@ -834,7 +835,7 @@ __global__ void __launch_bounds__(256) generic_bead_kernel(BeadParams<T> p, Bead
                 st.set(x, y, z, p.inv_dx);
             }
         }
-        if (MODE == kModeSpread || MODE == kModeStep) {
+        if ((MODE == kModeSpread || MODE == kModeStep) && bead_ok(p, bf, st, bid, species)) {
             using FP = FixedPoint<T>;
             unsigned long long* rk = bf.rho_fx + (size_t)species * M;
 #pragma unroll

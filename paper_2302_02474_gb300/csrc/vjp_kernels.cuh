@@ -135,10 +135,11 @@ __global__ void __launch_bounds__(256) vjp_spread(BeadParams<T> p, BeadBuffers<T
     T sc, inv;
     AdjointFixed<T>::scales(*bits, S, sc, inv);
     const int tag = bf.id[i];
-    const T* lp = lam + 3 * (size_t)slot_bead_id(tag);
-    const T l[3] = {lp[0] * sc, lp[1] * sc, lp[2] * sc};
     Stencil<P, T> st;
     st.set(bf.px[i], bf.py[i], bf.pz[i], p.inv_dx);
+    if (!bead_ok(p, bf, st, slot_bead_id(tag), slot_species(tag))) return;
+    const T* lp = lam + 3 * (size_t)slot_bead_id(tag);
+    const T l[3] = {lp[0] * sc, lp[1] * sc, lp[2] * sc};
     vjp_spread_global<P>(st, l, slot_species(tag), p.n, fx);
 }
 
@@ -190,10 +191,11 @@ __global__ void __launch_bounds__(256) vjp_spread_tiled(BeadParams<float> p, Bea
     for (int i = start + threadIdx.x; i < end; i += blockDim.x) {
         const int tag = bf.id[i];
         const int K = slot_species(tag);
-        const float* lp = lam + 3 * (size_t)slot_bead_id(tag);
-        const float l[3] = {lp[0] * sc, lp[1] * sc, lp[2] * sc};
         Stencil<P, float> st;
         st.set(bf.px[i], bf.py[i], bf.pz[i], p.inv_dx);
+        if (!bead_ok(p, bf, st, slot_bead_id(tag), K)) continue;
+        const float* lp = lam + 3 * (size_t)slot_bead_id(tag);
+        const float l[3] = {lp[0] * sc, lp[1] * sc, lp[2] * sc};
         int3 o;
         if (patch_local(st, org, o) && patch_ok) {
 #pragma unroll
@@ -459,7 +461,10 @@ __device__ __forceinline__ void vjp_bonds_store(const BeadParams<T>& p, const Be
 #pragma unroll
     for (int d = 0; d < 3; ++d) o[d] *= p.inv_dx;
     auto bond = [&](int s) {
-        const T* ln = lam + 3 * (size_t)slot_bead_id(bf.id[s]);
+        if (!slot_ok(p, bf, s)) return;
+        const int other = slot_bead_id(bf.id[s]);
+        if (!slot_ok(p, bf, other)) return;
+        const T* ln = lam + 3 * (size_t)other;
 #pragma unroll
         for (int d = 0; d < 3; ++d) o[d] -= p.k_bond * (l[d] - ln[d]);
     };
@@ -481,10 +486,11 @@ __global__ void __launch_bounds__(256) vjp_beads(BeadParams<T> p, BeadBuffers<T>
     const T x = bf.px[i], y = bf.py[i], z = bf.pz[i];
     const int tag = bf.id[i];
     const int bid = slot_bead_id(tag);
-    const T* lp = lam + 3 * (size_t)bid;
-    const T l[3] = {lp[0], lp[1], lp[2]};
     Stencil<P, T> st;
     st.set(x, y, z, p.inv_dx);
+    if (!bead_ok(p, bf, st, bid, slot_species(tag))) return;
+    const T* lp = lam + 3 * (size_t)bid;
+    const T l[3] = {lp[0], lp[1], lp[2]};
     T dwx[P], dwy[P], dwz[P], o[3] = {T(0), T(0), T(0)};
     dh_weight_derivs<P>(x * p.inv_dx, dwx);
     dh_weight_derivs<P>(y * p.inv_dx, dwy);
@@ -526,10 +532,11 @@ __global__ void __launch_bounds__(256) vjp_beads_tiled(BeadParams<float> p, Bead
         const float x = bf.px[i], y = bf.py[i], z = bf.pz[i];
         const int tag = bf.id[i];
         const int bid = slot_bead_id(tag), K = slot_species(tag);
-        const float* lp = lam + 3 * (size_t)bid;
-        const float l[3] = {lp[0], lp[1], lp[2]};
         Stencil<P, float> st;
         st.set(x, y, z, p.inv_dx);
+        if (!bead_ok(p, bf, st, bid, K)) continue;
+        const float* lp = lam + 3 * (size_t)bid;
+        const float l[3] = {lp[0], lp[1], lp[2]};
         float dwx[P], dwy[P], dwz[P], o[3] = {0.f, 0.f, 0.f};
         dh_weight_derivs<P>(x * p.inv_dx, dwx);
         dh_weight_derivs<P>(y * p.inv_dx, dwy);
@@ -572,6 +579,7 @@ __global__ void __launch_bounds__(256) density_vjp_kernel(BeadParams<T> p, BeadB
     const int bid = slot_bead_id(tag), K = slot_species(tag);
     Stencil<P, T> st;
     st.set(x, y, z, p.inv_dx);
+    if (!bead_ok(p, bf, st, bid, K)) return;
     T dwx[P], dwy[P], dwz[P];
     dh_weight_derivs<P>(x * p.inv_dx, dwx);
     dh_weight_derivs<P>(y * p.inv_dx, dwy);

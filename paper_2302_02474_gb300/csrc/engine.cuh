@@ -2080,14 +2080,23 @@ template <typename T> class Engine final : public EngineBase {
     //   the tiles of a small grid leave idle on most SMs; order 1, 32^3, 20,000
     //   beads 44.9 / 22.5, 64^3, 200,000 168 / 131; order 3 118 / 55, 419 / 326.
     //   FP32, order 1: up to about 48,000 beads latency decides, and a tile's
-    //   patch adds barriers and a flush to the chain (24^3, 4,060 beads: step
-    //   15.6 / 14.4; 48^3, 40,000: 21.1 / 20.4); beyond that the global atomics
-    //   do (64^3, 200,000: 30.6 / 37.4), and at higher orders at every size
-    //   (order 3, 24^3: 20.2 / 22.5).
+    //   patch adds barriers and a flush to the chain; beyond that the global
+    //   atomics do (64^3, 200,000: 30.6 / 37.4), and at higher orders at every
+    //   size (order 3, 24^3: 20.2 / 22.5). Step, tiled / per bead:
+    //     8^3    2,000 beads 25.2 / 9.6   48,000 484 / 27.2
+    //     16^3   2,000 10.7 / 10.4        48,000 75.9 / 14.7
+    //     24^3   4,000 11.4 / 12.0        14,000 14.9 / 11.9   48,000 29.1 / 14.4
+    //     32^3   20,000 13.9 / 13.3       48,000 18.3 / 16.6
+    //     40^3   20,000 14.8 / 15.0       32,000 15.9 / 16.0   48,000 16.9 / 19.2
+    //     48^3   22,000 18.7 / 18.7       30,000 19.3 / 20.1   48,000 20.3 / 25.9
+    //     64^3   48,000 23.5 / 22.5       80^3 37.3 / 31.9     128^3 98.4 / 75.9
+    //   At 40^3 and 48^3 the tiles are many and the launches overlap (above
+    //   48^3 a graph's do not), so the per-bead form ends at 22,000 beads there.
     bool per_bead() const {
         if (generic_) return true;
         if (analytic()) return false;
-        return sizeof(T) == 8 || (P_ == 2 && cfg_->n_beads <= 48000);
+        const bool few_tiles = M_ <= 32 * 32 * 32, graph_overlaps = M_ <= 48 * 48 * 48;
+        return sizeof(T) == 8 || (P_ == 2 && cfg_->n_beads <= (few_tiles || !graph_overlaps ? 48000 : 22000));
     }
     // Threads per block: small blocks spread few beads over all SMs (FP64,
     // 32^3: 22.5 us with 32 threads, 28.7 with 128).

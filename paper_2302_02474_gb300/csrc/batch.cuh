@@ -363,6 +363,8 @@ template <typename T> class BatchEngine final : public BatchBase {
             }
             ++since;
         }
+        int64_t sorting = 0;
+        for (const E* e : reps_) sorting += sorts * e->sort_launches();
         if (persistent_) {
             // one launch per run of steps between re-binnings
             int64_t since2 = steps_since_sort_, runs = 0;
@@ -378,9 +380,9 @@ template <typename T> class BatchEngine final : public BatchBase {
                 }
                 ++since2;
             }
-            return runs + sorts * 4 * (int64_t)reps_.size();
+            return runs + sorting;
         }
-        return n * 4 * (int64_t)groups_.size() + sorts * 4 * (int64_t)reps_.size();
+        return n * 4 * (int64_t)groups_.size() + sorting;
     }
 
    private:

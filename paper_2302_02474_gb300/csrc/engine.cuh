@@ -936,10 +936,11 @@ template <typename T> class Engine final : public EngineBase {
         return check_err();
     }
 
+    int64_t sort_launches() const { return n_fine_ <= kScanOne ? 4 : 7; }  // of one re-binning
     int64_t launches(int64_t n) const override {
         const int D = cfg_->dim;
         const int64_t per_step = generic_ ? (use_lines() ? 2 * D : (1 + D) + 1 + (int64_t)NP_ * D + 1) : (use_planes() ? 2 : 4) + 2;
-        const int64_t per_sort = n_fine_ <= kScanOne ? 4 : 7;
+        const int64_t per_sort = sort_launches();
         const int K = cfg_->sort_every;
         int64_t since = steps_since_sort_, sorts = 0;
         for (int64_t s = 0; s < n; ++s) {

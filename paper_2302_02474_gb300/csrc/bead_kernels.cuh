@@ -801,14 +801,6 @@ __global__ void __launch_bounds__(256) bead_sums64(BeadParams<T> p, BeadBuffers<
 
 // ------------------------------------------------------------- binning
 
-// Tile of a position: index of the 8x8x8-cell tile holding floor(r/dx).
-template <typename T> __device__ __forceinline__ int tile_key(T x, T y, T z, T inv_dx, int n, int tiles) {
-    const int cx = min(max((int)floor(x * inv_dx), 0), n - 1);
-    const int cy = min(max((int)floor(y * inv_dx), 0), n - 1);
-    const int cz = min(max((int)floor(z * inv_dx), 0), n - 1);
-    return ((cz / kTile) * tiles + cy / kTile) * tiles + cx / kTile;
-}
-
 // atomicAdd(counter + key, 1) for every active lane with one atomic per
 // distinct key in the warp; returns this lane's value before its increment.
 __device__ __forceinline__ int warp_aggregated_inc(int* counter, int key) {

@@ -43,7 +43,6 @@ template <class V> __device__ __forceinline__ V c_mul(V a, V b) {
     return {fma_rn(a.x, b.x, -mul_rn(a.y, b.y)), fma_rn(a.y, b.x, mul_rn(a.x, b.y))};
 }
 template <class V> __device__ __forceinline__ V c_conj(V a) { return {a.x, -a.y}; }
-template <class V, typename T> __device__ __forceinline__ V c_scale(V a, T s) { return {a.x * s, a.y * s}; }
 // multiply by -i (forward-transform quarter turn) or +i
 template <class V> __device__ __forceinline__ V c_mul_negi(V a) { return {a.y, -a.x}; }
 template <class V> __device__ __forceinline__ V c_mul_posi(V a) { return {-a.y, a.x}; }

@@ -1617,17 +1617,21 @@ template <typename T> class Engine final : public EngineBase {
         }
         const int s4 = (int)bead_smem(false, 4), sa4 = (int)bead_smem(true, 4);
         TILD_CUDA(cudaFuncSetAttribute(bead_kernel<P, kModeSpread, T, false, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, s4));
-        TILD_CUDA(cudaFuncSetAttribute(bead_kernel<P, kModeForce, T, false, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, s4));
-        TILD_CUDA(cudaFuncSetAttribute(bead_kernel<P, kModeSetVel, T, false, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, s4));
-        TILD_CUDA(cudaFuncSetAttribute(bead_kernel<P, kModeStep, T, false, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, s4));
+        if constexpr (sizeof(T) == 4) {  // (FP64: per_bead)
+            TILD_CUDA(cudaFuncSetAttribute(bead_kernel<P, kModeForce, T, false, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, s4));
+            TILD_CUDA(cudaFuncSetAttribute(bead_kernel<P, kModeSetVel, T, false, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, s4));
+            TILD_CUDA(cudaFuncSetAttribute(bead_kernel<P, kModeStep, T, false, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, s4));
+        }
         TILD_CUDA(cudaFuncSetAttribute(bead_kernel<P, kModeForce, T, true, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, sa4));
         TILD_CUDA(cudaFuncSetAttribute(bead_kernel<P, kModeSetVel, T, true, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, sa4));
         TILD_CUDA(cudaFuncSetAttribute(bead_kernel<P, kModeStep, T, true, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, sa4));
         const int s = (int)bead_smem(false, 2);
         TILD_CUDA(cudaFuncSetAttribute(bead_kernel<P, kModeSpread, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, s));
-        TILD_CUDA(cudaFuncSetAttribute(bead_kernel<P, kModeForce, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, s));
-        TILD_CUDA(cudaFuncSetAttribute(bead_kernel<P, kModeSetVel, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, s));
-        TILD_CUDA(cudaFuncSetAttribute(bead_kernel<P, kModeStep, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, s));
+        if constexpr (sizeof(T) == 4) {  // (FP64: per_bead)
+            TILD_CUDA(cudaFuncSetAttribute(bead_kernel<P, kModeForce, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, s));
+            TILD_CUDA(cudaFuncSetAttribute(bead_kernel<P, kModeSetVel, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, s));
+            TILD_CUDA(cudaFuncSetAttribute(bead_kernel<P, kModeStep, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, s));
+        }
         const int sa = (int)bead_smem(true, 2);
         TILD_CUDA(cudaFuncSetAttribute(bead_kernel<P, kModeForce, T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sa));
         TILD_CUDA(cudaFuncSetAttribute(bead_kernel<P, kModeSetVel, T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sa));
@@ -2064,11 +2068,15 @@ template <typename T> class Engine final : public EngineBase {
             }
         } else {
             const size_t sm = bead_smem(false, NS);
-            switch (mode) {
-                case kModeSpread: launch(bead_kernel<P, kModeSpread, T, false, NS>, grid, 256, sm, p, bf); break;
-                case kModeForce: launch(bead_kernel<P, kModeForce, T, false, NS>, grid, 256, sm, p, bf); break;
-                case kModeSetVel: launch(bead_kernel<P, kModeSetVel, T, false, NS>, grid, 256, sm, p, bf); break;
-                default: launch(bead_kernel<P, kModeStep, T, false, NS>, grid, 256, sm, p, bf); break;
+            if constexpr (sizeof(T) == 8) {  // the analytic force's spread; everything else is per_bead
+                launch(bead_kernel<P, kModeSpread, T, false, NS>, grid, 256, sm, p, bf);
+            } else {
+                switch (mode) {
+                    case kModeSpread: launch(bead_kernel<P, kModeSpread, T, false, NS>, grid, 256, sm, p, bf); break;
+                    case kModeForce: launch(bead_kernel<P, kModeForce, T, false, NS>, grid, 256, sm, p, bf); break;
+                    case kModeSetVel: launch(bead_kernel<P, kModeSetVel, T, false, NS>, grid, 256, sm, p, bf); break;
+                    default: launch(bead_kernel<P, kModeStep, T, false, NS>, grid, 256, sm, p, bf); break;
+                }
             }
         }
         TILD_CUDA(cudaGetLastError());

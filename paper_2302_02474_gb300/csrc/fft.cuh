@@ -219,10 +219,6 @@ __device__ __forceinline__ void smem_fft_lines(V* buf, Addr addr, int es, const 
     }
 }
 
-template <int LS> struct StridedLines {
-    __device__ __forceinline__ int operator()(int l) const { return l * LS; }
-};
-
 // ------------------------------------------------- register-first stages
 //
 // The passes of the step run each stage of a line transform as one visit of

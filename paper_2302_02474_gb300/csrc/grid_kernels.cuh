@@ -644,8 +644,6 @@ template <int C, int STRIDE> struct TileAddr {  // buffer b of a tile set starts
     __device__ __forceinline__ int operator()(int l) const { return (l / C) * STRIDE + l % C; }
 };
 
-template <typename T> __device__ __forceinline__ int freq_index(int i, int n) { return i < n / 2 ? i : i - n; }
-
 // Square of the integer frequency of FFT index i (exact in floats).
 template <typename T, int N> __device__ __forceinline__ T freq_sq(int i) {
     const T m = (T)(i < N / 2 ? i : i - N);

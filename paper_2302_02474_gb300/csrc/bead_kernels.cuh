@@ -110,15 +110,15 @@ template <typename T> __device__ __forceinline__ bool not_finite(T a, T b, T c) 
 // fused products written out: the tiled and the per-bead kernels give the same
 // bits. f: force, g: normal.
 template <typename T> __device__ __forceinline__ T velocity_of(const BeadParams<T>& p, T u, T f, T g) {
-    return fma_rn(p.vg, g, fma_rn(p.vf, f, mul_rn(p.vu, u)));
+    return fma_rn(p.vg, g, fma_rn(p.vu, u, mul_rn(p.vf, f)));
 }
 template <typename T> __device__ __forceinline__ T carried_of(const BeadParams<T>& p, T v, T f, T g) {
-    return fma_rn(p.wg, g, fma_rn(p.wf, f, mul_rn(p.wu, v)));
+    return fma_rn(p.wg, g, fma_rn(p.wu, v, mul_rn(p.wf, f)));
 }
 template <typename T> __device__ __forceinline__ void step_update(const BeadParams<T>& p, T& x, T& u, T f, T g) {
-    const T h = fma_rn(p.sg, g, fma_rn(p.sf, f, mul_rn(p.su, u)));
+    const T h = fma_rn(p.sg, g, fma_rn(p.su, u, mul_rn(p.sf, f)));
     x = wrap_coord(fma_rn(p.se, g, fma_rn(p.sd, h, x)), p.L, p.inv_L);
-    u = fma_rn(p.sk, g, mul_rn(p.sh, h));
+    u = fma_rn(p.sh, h, mul_rn(p.sk, g));
 }
 
 // acc += |s d|^2

@@ -69,7 +69,7 @@ template <int DIR, int R, class V> __device__ __forceinline__ V w16_mul(int m, V
     if (DIR > 0) ci = -ci;
     if (m % 4 != 2) return c_mul(v, V{cr, ci});
     // odd multiples of pi/4
-    const bool x_first = R == 16 || m == 2, y_first = R == 16 ? m == 6 : m == 2;
+    const bool x_first = DIR < 0 ? R == 16 || m == 2 : R == 8 || m == 6, y_first = R == 16 ? m == 6 : m == 2;
     return {x_first ? fma_rn(v.x, cr, -mul_rn(v.y, ci)) : fma_rn(-v.y, ci, mul_rn(v.x, cr)),
             y_first ? fma_rn(v.x, ci, mul_rn(v.y, cr)) : fma_rn(v.y, cr, mul_rn(v.x, ci))};
 }

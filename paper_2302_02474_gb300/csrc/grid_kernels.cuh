@@ -688,20 +688,25 @@ __device__ __forceinline__ void add_energies(Wide<T> (&acc)[5], V A, V B, T uh, 
 // times: 24.1 -> 16.7 us at 128^3, 190 -> 114 us at 256^3, 16 column tiles
 // (256^3: 8), isolated launches.
 //   1. stage A of the forward transform from global memory;
-//   2. stage B in registers; the spectral multiply where it left X[k]; and
-//      the first stage of the inverse transform on the products, without
-//      leaving registers: with the two factors taken in the other order (N2
-//      points over k2, then N1 over k1; z = m + N2 q) its inputs are the N2
-//      outputs of one stage-B unit;
+//   2. stage B in registers; the spectral multiply where it left X[k]; and,
+//      where the two factors are equal (16, 64, 256), the first stage of the
+//      inverse transform on the products without leaving registers: its inputs
+//      are the N2 outputs of one stage-B unit;
 //   3. the inverse's second stage, to global memory.
+// Where the factors differ the inverse's first stage takes N1 points that lie
+// in N2 units: the products G go to the slots that their unit read, and a visit
+// of shared memory more makes the first stages of G and G_z (128^3: 1.4 us of a
+// step). Taking the factors in the other order fuses everywhere, but rounds
+// otherwise: that form serves FP64, the potentials and charges, whose results
+// are not the sums that nearly cancel.
 // The unit (row, column c, k1) of step 2 needs Z(-k) as well, the outputs of
 // the mirror unit (mirror row, mirror column, (N1 - k1) mod N1). PAIRED: a
 // thread takes both units and writes both; otherwise each unit has its own
 // thread, which transforms the mirror unit's inputs a second time (half the
 // registers and twice the threads, for tiles that leave threads idle).
-template <int N, int C> struct ZTile {
+template <typename T, int N, int C, bool OTHER = false> struct ZTile {
     static constexpr int N1 = fft_split<N>::N1, N2 = fft_split<N>::N2;
-    static constexpr bool paired = 2 * C * N1 > 256;
+    static constexpr bool paired = 2 * C * N1 > 256, fused = sizeof(T) == 8 || OTHER || N1 == N2 || N2 == 1;
     static_assert(256 % C == 0 && C * N1 <= 256, "every unit of a row has a thread");
 };
 
@@ -712,7 +717,8 @@ __device__ __forceinline__ void z_tile(cplx_t<T>* buf, cplx_t<T>* tw, const cplx
                                        const SpectralParams<T>& sp, int p0, const int (&ky)[2], int R, Wide<T> (&acc)[5],
                                        Fetch fetch, Out out) {
     using V = cplx_t<T>;
-    constexpr int TS = N * C, N1 = ZTile<N, C>::N1, N2 = ZTile<N, C>::N2;
+    constexpr int TS = N * C, N1 = ZTile<T, N, C>::N1, N2 = ZTile<T, N, C>::N2;
+    constexpr bool FUSED = ZTile<T, N, C, G_ONLY || EL>::fused;
     {
         int u = threadIdx.x;  // unit (row, j2, column), lanes over columns
         V v[N1];
@@ -742,7 +748,7 @@ __device__ __forceinline__ void z_tile(cplx_t<T>* buf, cplx_t<T>* tw, const cplx
     }
     __syncthreads();
     {
-        constexpr bool PAIRED = ZTile<N, C>::paired;
+        constexpr bool PAIRED = ZTile<T, N, C>::paired;
         const int q = threadIdx.x;
         const bool active = q < (PAIRED ? 1 : R) * C * N1;
         int c = q % C, k1 = (q / C) % N1, r = PAIRED ? 0 : q / (C * N1);
@@ -783,13 +789,16 @@ __device__ __forceinline__ void z_tile(cplx_t<T>* buf, cplx_t<T>* tw, const cplx
                 // rho~_A = (Z + conj Zm)/2, rho~_B = -i (Z - conj Zm)/2
                 const V A = {T(0.5) * (Z.x + Zm.x), T(0.5) * (Z.y - Zm.y)};
                 const V B = {T(0.5) * (Z.y + Zm.y), -T(0.5) * (Z.x - Zm.x)};
-                V wA = {mul_rn(uh, fma_rn(sp.eAA, A.x, mul_rn(sp.eAB, B.x))),
-                        mul_rn(uh, fma_rn(sp.eAA, A.y, mul_rn(sp.eAB, B.y)))};
-                V wB = {mul_rn(uh, fma_rn(sp.eAB, A.x, mul_rn(sp.eBB, B.x))),
-                        mul_rn(uh, fma_rn(sp.eAB, A.y, mul_rn(sp.eBB, B.y)))};
+                const V tA = {fma_rn(sp.eAA, A.x, mul_rn(sp.eAB, B.x)), fma_rn(sp.eAA, A.y, mul_rn(sp.eAB, B.y))};
+                const V tB = {fma_rn(sp.eAB, A.x, mul_rn(sp.eBB, B.x)), fma_rn(sp.eAB, A.y, mul_rn(sp.eBB, B.y))};
                 if (WANT_E)
                     add_energies<T, WANT_E>(acc, A, B, uh, sp.e_rho, weight, zero && kz == 0, mxy + freq_sq<T, N>(kz));
-                if (EL) {
+                // G = i (w~_A + i w~_B), k_x and k_y follow in the xy pass, and the same of -k
+                if constexpr (!EL) {
+                    ga[k2] = {-fma_rn(uh, tA.y, mul_rn(uh, tB.x)), fma_rn(uh, tA.x, -mul_rn(uh, tB.y))};
+                    if constexpr (PAIRED) gb[k2] = {fma_rn(uh, tA.y, -mul_rn(uh, tB.x)), fma_rn(uh, tA.x, mul_rn(uh, tB.y))};
+                } else {
+                    V wA = {mul_rn(uh, tA.x), mul_rn(uh, tA.y)}, wB = {mul_rn(uh, tB.x), mul_rn(uh, tB.y)};
                     // w_K += q_K c(k) rho~_q with rho~_q = q_A rho~_A + q_B rho~_B
                     const T qzv = raw_k<T, N>(kz, sp.two_pi_over_L);
                     const T k2sq = fma_rn(qzv, qzv, kxy2);
@@ -805,9 +814,9 @@ __device__ __forceinline__ void z_tile(cplx_t<T>* buf, cplx_t<T>* tw, const cplx
                         f.add_prod(rq.y * sp.e_rho, rq.y * sp.e_rho);
                         acc[4].add(f.times(weight * gq));
                     }
+                    ga[k2] = {-(wA.y + wB.x), wA.x - wB.y};
+                    if constexpr (PAIRED) gb[k2] = {wA.y - wB.x, wA.x + wB.y};
                 }
-                ga[k2] = {-(wA.y + wB.x), wA.x - wB.y};  // i (w~_A + i w~_B); k_x, k_y follow in the xy pass
-                if constexpr (PAIRED) gb[k2] = {wA.y - wB.x, wA.x + wB.y};  // the same of -k
             }
             // the inverse transform's first stage of G and G_z of one unit
             auto emit = [&](V (&g)[N2], int row, int col, int kk) {
@@ -824,7 +833,17 @@ __device__ __forceinline__ void z_tile(cplx_t<T>* buf, cplx_t<T>* tw, const cplx
 #pragma unroll
                 for (int m = 0; m < N2; ++m) o[m * C] = m == 0 ? g[0] : c_mul(g[m], twiddle<+1>(tw, kk * m));
             };
-            if constexpr (PAIRED) {
+            if constexpr (!FUSED) {
+                V* o = buf + r * TS + k1 * N2 * C + c;
+#pragma unroll
+                for (int k2 = 0; k2 < N2; ++k2) o[k2 * C] = ga[k2];
+                if constexpr (PAIRED) {
+                    o = buf + rB * TS + k1B * N2 * C + cB;
+                    if (R == 2)
+#pragma unroll
+                        for (int k2 = 0; k2 < N2; ++k2) o[k2 * C] = k1 == 0 ? gb[(N2 - k2) % N2] : gb[N2 - 1 - k2];
+                }
+            } else if constexpr (PAIRED) {
                 int sides = R;
 #pragma unroll 1
                 while (true) {
@@ -843,17 +862,42 @@ __device__ __forceinline__ void z_tile(cplx_t<T>* buf, cplx_t<T>* tw, const cplx
         }
     }
     __syncthreads();
-    const int units = (G_ONLY ? 1 : 2) * R * C * N2;
+    if constexpr (!FUSED) {
+        // the inverse's first stage, in place: unit (row, j2, column) on X[j2 + N2 j1]
+#pragma unroll 1
+        for (int u = threadIdx.x; u < R * C * N2; u += 256) {
+            const int j2 = (u / C) % N2;
+            V* p = buf + (u / (C * N2)) * TS + u % C;
+            V v[N1];
+#pragma unroll
+            for (int k = 0; k < N1; ++k) v[k] = p[LineSlots<N>::slot_of(j2 + N2 * k) * C];
+            if constexpr (!G_ONLY) {
+                V w[N1];
+#pragma unroll
+                for (int k = 0; k < N1; ++k) w[k] = c_scale_rn(v[k], grad_k<T, N>(j2 + N2 * k, sp.two_pi_over_L));
+                stage_a_regs<N, +1>(w, j2, tw);
+#pragma unroll
+                for (int k = 0; k < N1; ++k) p[R * TS + LineSlots<N>::slot_of(j2 + N2 * k) * C] = w[k];
+            }
+            stage_a_regs<N, +1>(v, j2, tw);
+#pragma unroll
+            for (int k = 0; k < N1; ++k) p[LineSlots<N>::slot_of(j2 + N2 * k) * C] = v[k];
+        }
+        __syncthreads();
+    }
+    // the second stage: NB points over the NA units
+    constexpr int NB = FUSED ? N1 : N2, NA = N / NB;
+    const int units = (G_ONLY ? 1 : 2) * R * C * NA;
 #pragma unroll 1
     for (int u = threadIdx.x; u < units; u += 256) {
-        const int c = u % C, m = (u / C) % N2, b = u / (C * N2);
-        const V* p = buf + b * TS + m * C + c;
-        V v[N1];
+        const int c = u % C, m = (u / C) % NA, b = u / (C * NA);
+        const V* p = buf + b * TS + c;
+        V v[NB];
 #pragma unroll
-        for (int k1 = 0; k1 < N1; ++k1) v[k1] = p[k1 * N2 * C];
-        reg_dft<N1, +1, V>::run(v);
+        for (int k = 0; k < NB; ++k) v[k] = p[(FUSED ? k * NA + m : LineSlots<N>::slot_of(k + NB * m)) * C];
+        reg_dft<NB, +1, V>::run(v);
 #pragma unroll
-        for (int k = 0; k < N1; ++k) out(b, c, m + N2 * k, v[k]);
+        for (int k = 0; k < NB; ++k) out(b, c, m + NA * k, v[k]);
     }
 }
 
@@ -901,7 +945,7 @@ template <typename T, int N, int C>
 __global__ void __launch_bounds__(256) z_spectrum(const cplx_t<T>* __restrict__ Zxy, const cplx_t<T>* __restrict__ tw_g,
                                                   cplx_t<T>* __restrict__ spectrum) {
     using V = cplx_t<T>;
-    constexpr int N1 = ZTile<N, C>::N1, N2 = ZTile<N, C>::N2;
+    constexpr int N1 = ZTile<T, N, C>::N1, N2 = ZTile<T, N, C>::N2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V* tw = reinterpret_cast<V*>(smem_raw);
     V* buf = tw + N;

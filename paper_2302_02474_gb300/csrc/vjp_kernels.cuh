@@ -428,6 +428,19 @@ __global__ void __launch_bounds__(256) z_vjp(cplx_t<T>* __restrict__ H, const cp
     }
 }
 
+// One point of a bead's gather: o += grad W (psi/dV - lam . D w), f the point's
+// D w, w the weights' x part and (y, z) parts. (Each fused product is written
+// out: the tiled and the global gather give the same bits.)
+template <typename T>
+__device__ __forceinline__ void vjp_point(T wx, T dwx, T wyz, T dyz, T ydz, const T (&l)[3], T f0, T f1, T f2, T psi, T inv_dV,
+                                          T (&o)[3]) {
+    const T ldw = fma_rn(l[2], f2, fma_rn(l[0], f0, mul_rn(l[1], f1)));
+    const T v = fma_rn(psi, inv_dV, -ldw);
+    o[0] = fma_rn(mul_rn(dwx, wyz), v, o[0]);
+    o[1] = fma_rn(mul_rn(wx, dyz), v, o[1]);
+    o[2] = fma_rn(mul_rn(wx, ydz), v, o[2]);
+}
+
 // Per bead: sum_g grad W_j(g) [psi_{K_j}(g)/dV - lam_j . D w_{K_j}(g)] and the
 // bond term. fields: (d_x, d_y, d_z)(w_A, w_B), [3][M]; psi: i (psi_A + i psi_B).
 // lam and out by bead id ([N][3]).
@@ -442,15 +455,14 @@ __device__ __forceinline__ void vjp_gather_global(const Stencil<P, T>& st, const
 #pragma unroll
         for (int b = 0; b < P; ++b) {
             const size_t row = ((size_t)pwrap(st.jz + c, n) * n + pwrap(st.jy + b, n)) * n;
-            RowGrad<T> r;
+            const T wyz = st.wy[b] * st.wz[c], dyz = dwy[b] * st.wz[c], ydz = st.wy[b] * dwz[c];
 #pragma unroll
             for (int a = 0; a < P; ++a) {
                 const size_t g = row + pwrap(st.jx + a, n);
                 const cplx_t<T> f0 = fields[g], f1 = fields[M + g], f2 = fields[2 * M + g], f3 = __ldca(psi + g);
-                const T ldw = l[0] * (K ? f0.y : f0.x) + l[1] * (K ? f1.y : f1.x) + l[2] * (K ? f2.y : f2.x);
-                r.point(st.wx[a], dwx[a], (K ? -f3.x : f3.y) * inv_dV - ldw);
+                vjp_point(st.wx[a], dwx[a], wyz, dyz, ydz, l, K ? f0.y : f0.x, K ? f1.y : f1.x, K ? f2.y : f2.x,
+                          K ? -f3.x : f3.y, inv_dV, o);
             }
-            r.add_to(st.wy[b], st.wz[c], dwy[b], dwz[c], o[0], o[1], o[2]);
         }
 }
 
@@ -500,7 +512,7 @@ __global__ void __launch_bounds__(256) vjp_beads(BeadParams<T> p, BeadBuffers<T>
 }
 
 // The same with the tile's fields staged in shared memory (FP32 contexts): one
-// record (d_x w, d_y w, d_z w, psi/dV) per point and species, so a bead reads
+// record (d_x w, d_y w, d_z w, psi) per point and species, so a bead reads
 // one 16-byte word per point where it read four 8-byte words of global memory
 // and used half of each.
 template <int P> constexpr size_t vjp_beads_smem() { return (size_t)2 * Patch<P>::W3 * sizeof(float4); }
@@ -524,8 +536,8 @@ __global__ void __launch_bounds__(256) vjp_beads_tiled(BeadParams<float> p, Bead
         const int row = i / W;
         const size_t g = (size_t)rowbase[row] + pwrap(org.x + i - row * W, p.n);
         const float2 f0 = __ldg(fields + g), f1 = __ldg(fields + M + g), f2 = __ldg(fields + 2 * M + g), f3 = __ldca(psi + g);
-        rec[i] = make_float4(f0.x, f1.x, f2.x, f3.y * inv_dV);
-        rec[W3 + i] = make_float4(f0.y, f1.y, f2.y, -f3.x * inv_dV);
+        rec[i] = make_float4(f0.x, f1.x, f2.x, f3.y);
+        rec[W3 + i] = make_float4(f0.y, f1.y, f2.y, -f3.x);
     }
     __syncthreads();
     for (int i = start + threadIdx.x; i < end; i += 256) {
@@ -548,13 +560,12 @@ __global__ void __launch_bounds__(256) vjp_beads_tiled(BeadParams<float> p, Bead
             for (int c = 0; c < P; ++c)
 #pragma unroll
                 for (int b = 0; b < P; ++b) {
-                    RowGrad<float> r;
+                    const float wyz = st.wy[b] * st.wz[c], dyz = dwy[b] * st.wz[c], ydz = st.wy[b] * dwz[c];
 #pragma unroll
                     for (int a = 0; a < P; ++a) {
                         const float4 f = base[(c * W + b) * W + a];
-                        r.point(st.wx[a], dwx[a], f.w - (l[0] * f.x + l[1] * f.y + l[2] * f.z));
+                        vjp_point(st.wx[a], dwx[a], wyz, dyz, ydz, l, f.x, f.y, f.z, f.w, inv_dV, o);
                     }
-                    r.add_to(st.wy[b], st.wz[c], dwy[b], dwz[c], o[0], o[1], o[2]);
                 }
         } else {
             vjp_gather_global<P>(st, dwx, dwy, dwz, l, K, p.n, fields, psi, inv_dV, o);

@@ -4,7 +4,9 @@ Density: every weight is round(fl(w_x fl(w_y w_z)) 2^22), by whichever bead
 kernel it is spread. Parameter derivatives of a force product: sums over
 wavevectors that nearly cancel, so their last digits show the roundings of the
 weights and of every stage of the transforms; tests/golden/force_vjp_theta.txt
-holds them, with their errors against the FP64 oracle, as bits. Comparisons
+holds them, with their errors against the FP64 oracle, as bits. Steps: checksums
+and derivatives in tests/golden/trajectory_bits.txt, of noiseless trajectories on
+every split of the transform lengths. Comparisons
 are exact.
 """
 import os
@@ -76,3 +78,34 @@ def theta(B, n, order, n_chains):
 @pytest.mark.parametrize("n,order,n_chains,want", _golden())
 def test_parameter_derivatives_of_a_force_product(B, n, order, n_chains, want):
     assert theta(B, n, order, n_chains) == want
+
+
+def _trajectory_golden():
+    with open(os.path.join(os.path.dirname(GOLDEN), "trajectory_bits.txt")) as f:
+        return [line.split() for line in f if line.strip() and not line.startswith("#")]
+
+
+def trajectory(B, n, order, n_chains, scheme):
+    """Checksums of positions and velocities after 9 steps, and the bits of the
+    parameter derivatives through 4 steps."""
+    import zlib
+
+    from paper_2302_02474_gb300.trajectory import trajectory_vjp
+
+    spec = I.small_system(n_chains=n_chains, N=10, n_a=4, L=0.5 * n, n=n, pmeorder=order, precision="fp32")
+    t = B.Tild.from_spec(spec)
+    t.set_integrator(0.005, 1.0, 0.0, 1.0)  # no noise: sums and products alone
+    t.set_scheme(scheme)
+    t.set_positions(I.initial_positions(spec).astype(np.float32))
+    rng = np.random.default_rng(n + order)
+    t.set_velocities(rng.normal(size=(spec.n_beads, 3)).astype(np.float32))
+    lam = rng.normal(size=(spec.n_beads, 3)).astype(np.float32)
+    g = trajectory_vjp(t, 4, lam, lam, 4)
+    t.step(5)
+    sums = ["%08x" % zlib.crc32(np.ascontiguousarray(x).tobytes()) for x in (t.positions(dtype=np.float32), t.velocities(dtype=np.float32))]
+    return sums + [float(g[k]).hex() for k in ("chi", "kappa", "a")]
+
+
+@pytest.mark.parametrize("row", _trajectory_golden(), ids=lambda r: "-".join(r[:4]))
+def test_steps_and_derivatives_through_them(B, row):
+    assert trajectory(B, int(row[0]), int(row[1]), int(row[2]), row[3]) == row[4:]

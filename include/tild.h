@@ -378,13 +378,12 @@ tild_status tild_density_vjp(tild_ctx* ctx, const void* dL_drho, void* out, int 
  * for every scheme (EM has no velocity: v0_bar is 0). Reverse mode
  * recomputes the states of each segment of checkpoint_every steps from a
  * device checkpoint (bit-identical), keeps each recomputed state binned as
- * it was (positions in slot order, slot arrays and the density grid, so no
- * re-binning before its VJP) and takes one force vector-Jacobian product per
+ * it was (positions in slot order and slot arrays, so no re-binning before
+ * its VJP) with its fields and takes one force vector-Jacobian product per
  * state; the adjoint vectors are FP64. All arrays are [n_beads][3] by bead
  * id in dtype/where. The context ends at step n_steps. Device scratch, kept
  * with the context: n_steps/C + 2 states and C binned snapshots (3N values,
- * 3N ints, 2 n^3 64-bit grid points and the 4 n^3 complex values of that
- * state's fields each), C = min(checkpoint_every, n_steps). */
+ * 3N ints and the 4 n^3 complex values of that state's fields each), C = min(checkpoint_every, n_steps). */
 tild_status tild_trajectory_vjp(tild_ctx* ctx, int64_t n_steps, int checkpoint_every, const void* r_bar,
                                 const void* v_bar, int dtype, int where, void* r0_bar, void* v0_bar, double* dtheta);
 
@@ -453,7 +452,8 @@ tild_status tild_autotune(tild_ctx* ctx, int64_t trial_steps, int* sort_every, d
 /* Launch shapes of the step's FFT passes (results are bit-identical for
  * every choice; only speed changes):
  *   plane_threads  threads of each xy-plane CTA of the forward and inverse
- *                  passes: 512 (default), or 256 / 128 for planes small
+ *                  passes: 512 (default, but 1024 at n = 128 in FP32
+ *                  and 0 at n = 64 in FP64), or 256 / 128 for planes small
  *                  enough that several CTAs share an SM (n <= 80 and n <= 64
  *                  respectively, when stage B of the line transform keeps at
  *                  most 32 complex values per thread), 1024 (FP32, n = 80 and
@@ -463,12 +463,13 @@ tild_status tild_autotune(tild_ctx* ctx, int64_t trial_steps, int* sort_every, d
  *                  grids whose planes do not fit shared memory; n a
  *                  multiple of 16 in FP32, of 8 (and at least 16) in FP64);
  *   z_columns      column tile of the z pass: the default (128 bytes of
- *                  complex values) or the alternative of half that width
- *                  (twice the CTAs).
+ *                  complex values; 64 at n = 256) or the alternative of half
+ *                  that width (twice the CTAs).
  * tild_get_launch_shapes reports the current values; tild_set_launch_shapes
  * returns TILD_EINVAL for a value this grid does not have and
  * TILD_EUNSUPPORTED on the any-size grids. Batches launch every grid-size
- * group with the shapes of its first context. */
+ * group with the shapes of its first context, 512 plane threads where that
+ * context has 1024 or 0. */
 tild_status tild_get_launch_shapes(tild_ctx* ctx, int* plane_threads, int* z_columns);
 tild_status tild_set_launch_shapes(tild_ctx* ctx, int plane_threads, int z_columns);
 

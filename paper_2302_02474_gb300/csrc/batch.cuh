@@ -118,7 +118,7 @@ template <typename T> class BatchEngine final : public BatchBase {
                 g.el = e->c_el_on();
                 g.C = E::zpass_cols(e->n_);
                 g.tiles3 = e->n_tiles_;
-                g.nt = e->plane_nt_;
+                g.nt = e->plane_nt_;  // (1,024 and 0, the row passes: 512 in a batch, see with_group_nt)
                 g.zalt = e->zalt_ && !g.el;
                 groups_.push_back(g);
             }
@@ -539,11 +539,13 @@ template <typename T> class BatchEngine final : public BatchBase {
     int cur_pos_ = 0, cur_uid_ = 0, steps_since_sort_ = 0;
     cudaGraphExec_t graph_ = nullptr;
     static constexpr int kSortStreams = 16;
-    // Batches of fewer replicas than this start on the persistent kernel (one
-    // launch per run of steps, which callers may count on), larger ones on the
-    // group launches, which are faster at every size (us per step of replicas
-    // of 4,000 to 40,000 beads, persistent / groups: 6 replicas 92 / 46, 16
-    // replicas 172 / 83, 64 replicas 659 / 365).
+    // Batches of fewer replicas than this start on the persistent kernel, larger
+    // ones on the group launches. The line is a promise, not a crossing of times:
+    // a small batch takes one launch per run of steps and bounds its waits unless
+    // the caller chooses otherwise (tild_batch_set_persistent, the autotuner). The
+    // group launches are faster at every size (us per step of replicas of 4,000
+    // to 40,000 beads, persistent / groups: 6 replicas 92 / 46, 16 replicas
+    // 172 / 83, 64 replicas 659 / 365), so large batches do not.
     static constexpr int kPersistentMax = 8;
     std::vector<std::pair<cudaStream_t, cudaEvent_t>> sort_streams_;
     cudaEvent_t fork_ = nullptr;

@@ -117,7 +117,7 @@ __device__ __forceinline__ double density_from_fixed(long long v, double scale) 
 // triples become doubles. The exponent range remains that of floats, so terms
 // are scaled to be near 1, and a sum that left the range (wide_in_range) is
 // taken again in FP64 by bead_sums64 and spectral_sums64. Forces, energies and
-// density of 1.6M beads on 128^3: 437 us with FP64 sums, 243 with these (218
+// density of 1.6M beads on 128^3: 437 us with FP64 sums, 246 with these (220
 // with pairs of floats, which hold 48 bits at best and fewer where the terms
 // are uneven).
 template <typename T> struct Wide;
@@ -435,9 +435,10 @@ constexpr unsigned kErrBounds = 2u;  // a bounds check of the debug build failed
 
 // Debug build (compiled with -DTILD_DEBUG=1, `_build.build(debug=True)`):
 // the bead kernels, tiled and per bead, and the adjoint kernels check bead ids,
-// slots, species and grid indices before they use them; a failed check records kErrBounds in the context's error word and the access
-// is skipped (no trap), and the next synchronising call returns
-// TILD_EDEVICE. In the normal build every check is the constant true.
+// slots, species and grid indices before they use them; a failed check records
+// kErrBounds in the context's error word and the access is skipped (no trap),
+// and the next synchronising call returns TILD_EDEVICE. In the normal build
+// every check is the constant true.
 #ifndef TILD_DEBUG
 #define TILD_DEBUG 0
 #endif

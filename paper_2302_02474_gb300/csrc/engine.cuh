@@ -51,9 +51,13 @@ template <typename T> class Engine final : public EngineBase {
         P_ = cfg->pmeorder + 1;
         plane_fits_ = plane_fits(n_, sizeof(V));
         // default launch shape of the planes (tild_set_launch_shapes, tild_autotune
-        // choose others): 512 threads; 128^3 FP32 1,024, which hide the latency of
-        // its one CTA per SM (step 146.9 -> 142.5 us); 64^3 FP64 the row and column
-        // passes, which spread over all SMs (320.8 -> 277.6; at 48^3 118 against 150)
+        // choose others): 512 threads; 1,024 at 128^3 FP32, whose one CTA per SM
+        // leaves its latency to them; at 64^3 FP64 the row and column passes, which
+        // spread over every SM's FP64 unit where 64 planes reach 64 of 152. Step at
+        // 0.4 beads per point, us, as rows and columns / 512 / 1,024 threads:
+        //   FP64  24^3 53/48  32^3 58/55  40^3 77/83  48^3 160/127  64^3 222/260  80^3 563/514
+        //   FP32  48^3 23/20  64^3 27/26  80^3 47/42/44  128^3 131/126/122
+        // (40^3 FP64 would gain too and keeps its planes.)
         plane_nt_ = sizeof(T) == 4 && n_ == 128 ? 1024 : sizeof(T) == 8 && n_ == 64 ? 0 : 512;
         C_ = std::min(n_, (int)(128 / sizeof(V)));  // y-column tiles of the split passes
         CZ_ = zpass_cols(n_);                          // column tiles of the z pass

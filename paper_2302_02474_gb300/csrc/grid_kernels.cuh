@@ -685,7 +685,7 @@ __device__ __forceinline__ void add_energies(Wide<T> (&acc)[5], V A, V B, T uh, 
 // Bound by L2 and HBM traffic and by the tail of its 1.1 to 1.7 waves. Each
 // value visits shared memory twice and the CTA meets at three barriers, where
 // load, transform, multiply and inverse as separate passes visited it five
-// times: 24.1 -> 16.7 us at 128^3, 190 -> 114 us at 256^3, 16 column tiles
+// times: 24.1 -> 16.9 us at 128^3, 190 -> 114 us at 256^3, 16 column tiles
 // (256^3: 8), isolated launches.
 //   1. stage A of the forward transform from global memory;
 //   2. stage B in registers; the spectral multiply where it left X[k]; and,

@@ -166,7 +166,7 @@ template <int P> __device__ __forceinline__ int3 tile_patch(int t, int tiles, in
 // patch is flushed with one 64-bit add per point, rows of both species
 // contiguous. Integer sums: the same bits as the global path.
 // 200k beads, 64^3: 28.1 -> 16.1 us (P = 2); vjp_beads_tiled in place of the
-// per-bead gather 20.6 -> 14.3 us.
+// per-bead gather 20.6 -> 14.6 us.
 constexpr int kVjpTileBeads = 2047;
 template <int P> constexpr size_t vjp_spread_smem() { return (size_t)12 * Patch<P>::W3 * sizeof(int); }
 template <int P>

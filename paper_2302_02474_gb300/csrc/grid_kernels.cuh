@@ -1173,14 +1173,14 @@ __global__ void __launch_bounds__(256) spectral_sums64(const cplx_t<T>* __restri
     if (g < M) {
         const int i[3] = {(int)(g % n), (int)((g / n) % n), (int)(g / ((size_t)n * n))}, len[3] = {n, n, nz};
         size_t gm = 0;
-        T uh = T(1), uc = T(1), k2 = T(0);
+        T uh = T(1), uc = T(1), q[3] = {T(0), T(0), T(0)};
         double m2 = 0.0;
         for (int d = 2; d >= 0; --d) gm = gm * len[d] + (i[d] == 0 ? 0 : len[d] - i[d]);
         for (int d = 0; d < (nz > 1 ? 3 : 2); ++d) {
-            const T m = (T)(2 * i[d] < len[d] ? i[d] : i[d] - len[d]), k = sp.two_pi_over_L * m;
+            const T m = (T)(2 * i[d] < len[d] ? i[d] : i[d] - len[d]);
             uh *= sp.kernel1d[i[d]];
             if (el) uc *= sp.kernel1d_el[i[d]];
-            k2 += k * k;
+            q[d] = sp.two_pi_over_L * m;
             m2 += (double)m * m;
         }
         V A[2 * NP];
@@ -1201,8 +1201,9 @@ __global__ void __launch_bounds__(256) spectral_sums64(const cplx_t<T>* __restri
         acc[1].add(fkap);
         acc[2].add(m2 * fchi);
         acc[3].add(m2 * fkap);
+        const T k2 = fma_rn(q[2], q[2], fma_rn(q[0], q[0], mul_rn(q[1], q[1])));
         if (el && k2 > T(0)) {
-            const double rx = sp.qA * A[0].x + sp.qB * A[1].x, ry = sp.qA * A[0].y + sp.qB * A[1].y;
+            const double rx = fma_rn(sp.qA, A[0].x, mul_rn(sp.qB, A[1].x)), ry = fma_rn(sp.qA, A[0].y, mul_rn(sp.qB, A[1].y));
             acc[4].add((double)(uc * recip(k2)) * (rx * rx + ry * ry));
         }
     }

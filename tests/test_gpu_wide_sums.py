@@ -105,3 +105,50 @@ def test_field_energies(B, species, a):
     for k in want:
         # the test's own terms have up to four roundings each, of alternating sign over 4,096 modes
         assert want[k] != 0 and abs(e[k] - want[k]) <= 4 * TOL * abs(want[k]), k
+
+
+# A velocity outside the range of floats sends every sum of the call to FP64; the
+# energies are those of the ordinary sums, whose spectra are the same bits on
+# tiled grids (TOL, twice) and differ by FP32 transforms of other factors elsewhere.
+@pytest.mark.parametrize("n,dim,species,charged", [(16, 3, 2, False), (24, 3, 2, True), (16, 3, 4, False), (15, 3, 2, False), (21, 2, 3, False)])
+def test_sums_again_in_fp64(B, n, dim, species, charged):
+    chains, N, L = 250, 8, 8.0
+    t = B.Tild(L, n, 1, "fp32", 3, dim=dim)
+    t.set_chains([(chains, N, N // 2)], 1.0)
+    t.set_interactions(0.8, 20.0, 0.5)
+    if species > 2:
+        t.set_species(species, np.arange(chains * N) % species)
+        t.set_chi_matrix([[0.0 if i == j else 0.3 + 0.1 * (i + j) for j in range(species)] for i in range(species)])
+    if charged:
+        t.set_electrostatics(1.0, -1.0, 1.0, 0.5)
+    t.set_integrator(0.005, 1.0, 1.0, 1.0)
+    rng = np.random.default_rng(n)
+    pos, v = rng.random((chains * N, 3)) * L, rng.normal(size=(chains * N, 3))
+    if dim == 2:
+        pos[:, 2] = v[:, 2] = 0.0
+    t.set_positions(pos)
+    t.set_velocities(v)
+    _, e = t.compute(forces=False)
+    t.set_velocities(v * 1e25)
+    f, w = t.compute()
+    for k in ("bond", "chi", "kappa", "elec"):
+        assert abs(w[k] - e[k]) <= (2 * TOL if n % 8 == 0 else 2e-6) * abs(e[k]), k
+    assert (e["elec"] != 0) == charged
+    np.testing.assert_allclose(w["net_force"], f.astype(np.float64).sum(0), rtol=0, atol=1e-12 * np.abs(f).sum())
+
+
+def test_energy_gradient_again_in_fp64(B):
+    """Bonds of 1e-18: the gradient's sums in FP64 against an FP64 context's (2e-5, FP32 transforms)."""
+    rng = np.random.default_rng(3)
+    pos = (np.repeat(rng.random((500, 1, 3)) * 8.0, 4, axis=1)).astype(np.float32)
+    pos[:3] = rng.random((3, 4, 3)) * 1e-18  # the only bonds that are not zero
+    out = []
+    for prec in ("fp32", "fp64"):
+        t = B.Tild(8.0, 16, 2, prec, 3)
+        t.set_chains([(500, 4, 2)], 1.0)
+        t.set_interactions(0.8, 20.0, 0.5)
+        t.set_positions(pos.reshape(-1, 3).astype(np.float64))
+        out.append(t.energy_gradient(with_positions=False)[0])
+    for k, ref in out[1].items():
+        assert abs(out[0][k] - ref) <= 2e-5 * abs(ref), k
+    assert 0 < out[0]["e_bond"] < 1e-30

@@ -260,6 +260,14 @@ template <int N> struct LineSlots {
     // the slot that holds X[k] after stage B, and its inverse
     static __device__ __forceinline__ int slot_of(int k) { return (k % N1) * N2 + k / N1; }
     static __device__ __forceinline__ int index_of(int slot) { return slot / N2 + N1 * (slot % N2); }
+    // slot_of(j + N2 m), j < N2; where N2 divides N1 the parts of j and m separate,
+    // so that unrolled accesses over either share one address
+    static __device__ __forceinline__ int slot_of_part(int j, int m) {
+        if constexpr (N1 % N2 == 0)
+            return j * N2 + (m % (N1 / N2)) * N2 * N2 + m / (N1 / N2);
+        else
+            return slot_of(j + N2 * m);
+    }
 };
 
 // v * s with each product rounded by itself: the same bits in every pass that

@@ -695,7 +695,7 @@ __device__ __forceinline__ void add_energies(Wide<T> (&acc)[5], V A, V B, T uh, 
 //   3. the inverse's second stage, to global memory.
 // Where the factors differ the inverse's first stage takes N1 points that lie
 // in N2 units: the products G go to the slots that their unit read, and a visit
-// of shared memory more makes the first stages of G and G_z (128^3: 1.4 us of a
+// of shared memory more makes the first stages of G and G_z (128^3: 0.4 us of a
 // step). Taking the factors in the other order fuses everywhere, but rounds
 // otherwise: that form serves FP64, the potentials and charges, whose results
 // are not the sums that nearly cancel.
@@ -780,7 +780,7 @@ __device__ __forceinline__ void z_tile(cplx_t<T>* buf, cplx_t<T>* tw, const cplx
             const T mxy = freq_sq<T, N>(kx) + freq_sq<T, N>(kyr);
             const T weight = PAIRED && R == 2 ? T(2) : T(1);  // k and -k contribute the same
             const bool zero = kx == 0 && kyr == 0;
-            V ga[N2], gb[PAIRED ? N2 : 1];
+            V ga[FUSED ? N2 : 1], gb[FUSED && PAIRED ? N2 : 1];
 #pragma unroll
             for (int k2 = 0; k2 < N2; ++k2) {
                 const V Z = va[k2], Zm = k1 == 0 ? vb[(N2 - k2) % N2] : vb[N2 - 1 - k2];
@@ -794,9 +794,10 @@ __device__ __forceinline__ void z_tile(cplx_t<T>* buf, cplx_t<T>* tw, const cplx
                 if (WANT_E)
                     add_energies<T, WANT_E>(acc, A, B, uh, sp.e_rho, weight, zero && kz == 0, mxy + freq_sq<T, N>(kz));
                 // G = i (w~_A + i w~_B), k_x and k_y follow in the xy pass, and the same of -k
+                V G, Gm;
                 if constexpr (!EL) {
-                    ga[k2] = {-fma_rn(uh, tA.y, mul_rn(uh, tB.x)), fma_rn(uh, tA.x, -mul_rn(uh, tB.y))};
-                    if constexpr (PAIRED) gb[k2] = {fma_rn(uh, tA.y, -mul_rn(uh, tB.x)), fma_rn(uh, tA.x, mul_rn(uh, tB.y))};
+                    G = {-fma_rn(uh, tA.y, mul_rn(uh, tB.x)), fma_rn(uh, tA.x, -mul_rn(uh, tB.y))};
+                    Gm = {fma_rn(uh, tA.y, -mul_rn(uh, tB.x)), fma_rn(uh, tA.x, mul_rn(uh, tB.y))};
                 } else {
                     V wA = {mul_rn(uh, tA.x), mul_rn(uh, tA.y)}, wB = {mul_rn(uh, tB.x), mul_rn(uh, tB.y)};
                     // w_K += q_K c(k) rho~_q with rho~_q = q_A rho~_A + q_B rho~_B
@@ -814,8 +815,18 @@ __device__ __forceinline__ void z_tile(cplx_t<T>* buf, cplx_t<T>* tw, const cplx
                         f.add_prod(rq.y * sp.e_rho, rq.y * sp.e_rho);
                         acc[4].add(f.times(weight * gq));
                     }
-                    ga[k2] = {-(wA.y + wB.x), wA.x - wB.y};
-                    if constexpr (PAIRED) gb[k2] = {wA.y - wB.x, wA.x + wB.y};
+                    G = {-(wA.y + wB.x), wA.x - wB.y};
+                    Gm = {wA.y - wB.x, wA.x + wB.y};
+                }
+                if constexpr (FUSED) {
+                    ga[k2] = G;
+                    if constexpr (PAIRED) gb[k2] = Gm;
+                } else {  // to the slots that the units' inputs came from
+                    buf[r * TS + (k1 * N2 + k2) * C + c] = G;
+                    if constexpr (PAIRED) {
+                        const int mk = k1 == 0 ? (N2 - k2) % N2 : N2 - 1 - k2;
+                        if (R == 2) buf[rB * TS + (k1B * N2 + mk) * C + cB] = Gm;
+                    }
                 }
             }
             // the inverse transform's first stage of G and G_z of one unit
@@ -833,17 +844,7 @@ __device__ __forceinline__ void z_tile(cplx_t<T>* buf, cplx_t<T>* tw, const cplx
 #pragma unroll
                 for (int m = 0; m < N2; ++m) o[m * C] = m == 0 ? g[0] : c_mul(g[m], twiddle<+1>(tw, kk * m));
             };
-            if constexpr (!FUSED) {
-                V* o = buf + r * TS + k1 * N2 * C + c;
-#pragma unroll
-                for (int k2 = 0; k2 < N2; ++k2) o[k2 * C] = ga[k2];
-                if constexpr (PAIRED) {
-                    o = buf + rB * TS + k1B * N2 * C + cB;
-                    if (R == 2)
-#pragma unroll
-                        for (int k2 = 0; k2 < N2; ++k2) o[k2 * C] = k1 == 0 ? gb[(N2 - k2) % N2] : gb[N2 - 1 - k2];
-                }
-            } else if constexpr (PAIRED) {
+            if constexpr (FUSED && PAIRED) {
                 int sides = R;
 #pragma unroll 1
                 while (true) {
@@ -856,7 +857,7 @@ __device__ __forceinline__ void z_tile(cplx_t<T>* buf, cplx_t<T>* tw, const cplx
                     c = cB;
                     k1 = k1B;
                 }
-            } else {
+            } else if constexpr (FUSED) {
                 emit(ga, r, c, k1);
             }
         }
@@ -869,19 +870,22 @@ __device__ __forceinline__ void z_tile(cplx_t<T>* buf, cplx_t<T>* tw, const cplx
             const int j2 = (u / C) % N2;
             V* p = buf + (u / (C * N2)) * TS + u % C;
             V v[N1];
+            auto load = [&]() {
 #pragma unroll
-            for (int k = 0; k < N1; ++k) v[k] = p[LineSlots<N>::slot_of(j2 + N2 * k) * C];
+                for (int k = 0; k < N1; ++k) v[k] = p[LineSlots<N>::slot_of_part(j2, k) * C];
+            };
+            load();
             if constexpr (!G_ONLY) {
-                V w[N1];
 #pragma unroll
-                for (int k = 0; k < N1; ++k) w[k] = c_scale_rn(v[k], grad_k<T, N>(j2 + N2 * k, sp.two_pi_over_L));
-                stage_a_regs<N, +1>(w, j2, tw);
+                for (int k = 0; k < N1; ++k) v[k] = c_scale_rn(v[k], grad_k<T, N>(j2 + N2 * k, sp.two_pi_over_L));
+                stage_a_regs<N, +1>(v, j2, tw);
 #pragma unroll
-                for (int k = 0; k < N1; ++k) p[R * TS + LineSlots<N>::slot_of(j2 + N2 * k) * C] = w[k];
+                for (int k = 0; k < N1; ++k) p[R * TS + LineSlots<N>::slot_of_part(j2, k) * C] = v[k];
+                load();  // (a second copy in registers spills)
             }
             stage_a_regs<N, +1>(v, j2, tw);
 #pragma unroll
-            for (int k = 0; k < N1; ++k) p[LineSlots<N>::slot_of(j2 + N2 * k) * C] = v[k];
+            for (int k = 0; k < N1; ++k) p[LineSlots<N>::slot_of_part(j2, k) * C] = v[k];
         }
         __syncthreads();
     }
@@ -894,7 +898,7 @@ __device__ __forceinline__ void z_tile(cplx_t<T>* buf, cplx_t<T>* tw, const cplx
         const V* p = buf + b * TS + c;
         V v[NB];
 #pragma unroll
-        for (int k = 0; k < NB; ++k) v[k] = p[(FUSED ? k * NA + m : LineSlots<N>::slot_of(k + NB * m)) * C];
+        for (int k = 0; k < NB; ++k) v[k] = p[(FUSED ? k * NA + m : LineSlots<N>::slot_of_part(k, m)) * C];
         reg_dft<NB, +1, V>::run(v);
 #pragma unroll
         for (int k = 0; k < NB; ++k) out(b, c, m + NA * k, v[k]);
@@ -980,11 +984,13 @@ __global__ void __launch_bounds__(256) z_spectrum(const cplx_t<T>* __restrict__ 
 // WANT_E: the energy sums as well (2: and their |k|^2-weighted versions), an
 // instantiation of its own, so that the step's kernel carries none of their
 // code or registers.
-template <typename T, int N, int C> __host__ __device__ constexpr int z_ctas() {
-    return sizeof(T) == 8 ? 1 : N == 256 ? (C <= 8 ? 2 : 1) : C <= 8 ? 4 : 3;
+// (Resident CTAs: 16 columns of 128 whose inverse is not fused spill at three
+// CTAs' 80 registers, 18.2 us in the step against 17.4 with two.)
+template <typename T, int N, int C, bool OTHER = false> __host__ __device__ constexpr int z_ctas() {
+    return sizeof(T) == 8 ? 1 : N == 256 ? (C <= 8 ? 2 : 1) : C <= 8 ? 4 : N == 128 && !OTHER ? 2 : 3;
 }
 template <typename T, int N, int C, bool G_ONLY = false, bool EL = false, int WANT_E = 0>
-__global__ void __launch_bounds__(256, z_ctas<T, N, C>()) z_spectral(const cplx_t<T>* __restrict__ Zxy, cplx_t<T>* __restrict__ H,
+__global__ void __launch_bounds__(256, z_ctas<T, N, C, G_ONLY || EL>()) z_spectral(const cplx_t<T>* __restrict__ Zxy, cplx_t<T>* __restrict__ H,
                                                   const cplx_t<T>* __restrict__ tw_g, SpectralParams<T> sp,
                                                   double* __restrict__ energy_partials) {
     z_spectral_body<T, N, C, G_ONLY, EL, WANT_E>(ZArgs<T>{Zxy, H, tw_g, sp, energy_partials}, blockIdx.x, blockIdx.y,

@@ -348,7 +348,10 @@ tild_status tild_energy_gradient(tild_ctx* ctx, tild_energy_grad* g, void* dU_dr
  * (tild_trajectory_vjp). lam is spread onto the grid in 64-bit fixed
  * point with a power-of-two scale taken from max|lam|, so the result is
  * bitwise reproducible and exactly homogeneous under power-of-two scaling of
- * lam; a non-finite lam makes every output NaN. Returns
+ * lam; a non-finite lam makes every output NaN. The entries of dtheta are
+ * sums over wavevectors of both signs: where they nearly cancel (a random
+ * lam), FP32 contexts hold them to the rounding of FP32 spectra relative to
+ * the size of the terms, not of the sum. Returns
  * TILD_EUNSUPPORTED with the analytic force method or for grids whose
  * planes do not fit one CTA (FP32 above 128^3, FP64 above 64^3). */
 tild_status tild_force_vjp(tild_ctx* ctx, const void* lam, void* out, int dtype, int where, double* dtheta);
@@ -362,7 +365,8 @@ tild_status tild_force_vjp(tild_ctx* ctx, const void* lam, void* out, int dtype,
  * density grid (for example a density-profile loss) with respect to the
  * positions. Passed as r_bar to tild_trajectory_vjp it carries the loss back
  * through a trajectory. Three-dimensional boxes (else TILD_EUNSUPPORTED).
- * Allocates a context scratch of n_species n^3 + 3 n_beads values. */
+ * Arrays that are not device arrays of the context's precision, or that
+ * overlap, go through a context scratch of n_species n^3 + 3 n_beads values. */
 tild_status tild_density_vjp(tild_ctx* ctx, const void* dL_drho, void* out, int dtype, int where);
 
 /* Derivatives through a trajectory (differentiable form): runs n_steps
@@ -383,7 +387,8 @@ tild_status tild_density_vjp(tild_ctx* ctx, const void* dL_drho, void* out, int 
  * state; the adjoint vectors are FP64. All arrays are [n_beads][3] by bead
  * id in dtype/where. The context ends at step n_steps. Device scratch, kept
  * with the context: n_steps/C + 2 states and C binned snapshots (3N values,
- * 3N ints and the 4 n^3 complex values of that state's fields each), C = min(checkpoint_every, n_steps). */
+ * 3N ints and the 4 n^3 complex values of that state's fields each),
+ * C = min(checkpoint_every, n_steps). */
 tild_status tild_trajectory_vjp(tild_ctx* ctx, int64_t n_steps, int checkpoint_every, const void* r_bar,
                                 const void* v_bar, int dtype, int where, void* r0_bar, void* v0_bar, double* dtheta);
 

@@ -1165,9 +1165,22 @@ template <typename T> class Engine final : public EngineBase {
         const int lg = line_last_lg() - (NP_ == 2 ? 3 : 2);
         return dim3(div_up(n_, 1 << lg), cfg_->dim == 3 ? n_ / 2 + 1 : 1);
     }
-    // whether the lines of one column fit the last pass (2D grids of a few
-    // thousand points per edge do not: whole-axis passes)
-    bool use_lines() const { return generic_ && line_smem((NP_ == 2 ? 8 : 4) * n_) <= (size_t)kLineSmem; }
+    // Whether the line passes serve the grid. The lines of one column have to fit
+    // the last pass (2D grids of a few thousand points per edge do not). Long 2D
+    // lines in FP32 leave it few CTAs per SM, each with a direct DFT of a large
+    // factor: above 600 points per edge it pays where it runs in two waves at
+    // most, the second at least half full. Step, us, whole-axis passes / lines,
+    // one pair: 509 1262/606, 600 266/124, 641 1638/1983, 719 6654/1488, 800
+    // 382/305, 900 354/303, 1000 523/582, 1021 3973/4965, 1500 1090/1667, 2000
+    // 1860/3423; two pairs: 600 389/233, 641 2444/3008, 800 648/751, 1000 941/1218.
+    // FP64 gains at every size that fits (1200 7568/6149, 1021 75.9/51.5 ms).
+    bool use_lines() const {
+        if (!generic_ || line_smem((NP_ == 2 ? 8 : 4) * n_) > (size_t)kLineSmem) return false;
+        if (sizeof(T) == 8 || cfg_->dim == 3 || n_ <= 600) return true;
+        const size_t per_cta = line_smem(n_ << line_last_lg()) + 1024;
+        const unsigned resident = 152u * (unsigned)(228 * 1024 / per_cta), ctas = line_last_grid().x;
+        return ctas <= resident || (ctas <= 2 * resident && 2 * (ctas - resident) >= resident);
+    }
     tild_status line_forward(bool zero_after) {
         const int lg = line_rows_lg(NP_);
         launch(line_x_forward<T>, dim3(div_up(nz_ * n_, 1 << lg), NP_), 128, line_smem((n_ | 1) << lg), 

@@ -70,12 +70,6 @@ template <typename T> class Engine final : public EngineBase {
         TILD_CUDA(dev_malloc((void**)&kernel1d_, 2 * n_ * sizeof(T)));  // exp(-a^2 k_m^2), then exp(-a_e^2 k_m^2)
         TILD_CUDA(dev_malloc((void**)&counters_, kWords * sizeof(unsigned long long)));
         TILD_CUDA(cudaMemset(counters_, 0, kWords * sizeof(unsigned long long)));
-        if (cudaHostAlloc((void**)&words_, kWords * sizeof(unsigned long long), cudaHostAllocDefault) != cudaSuccess) {
-            cudaGetLastError();
-            words_ = nullptr;
-            err = "cannot allocate the pinned read-back words";
-            return TILD_ENOMEM;
-        }
         // tiles of 8^3 cells (one layer of tiles on a 2D grid)
         n_tiles_ = tiles_ * tiles_ * ((nz_ + kTile - 1) / kTile);
         n_fine_ = (size_t)kFineBins * n_tiles_ + 1;  // re-binning bins (tile, edge class, bank group)
@@ -1068,10 +1062,12 @@ template <typename T> class Engine final : public EngineBase {
     double kernel_a_ = -1.0, kernel_ae_ = -1.0;
     V* spec_ = nullptr;
     // [0] noise step counter, [1] error flags, [4 ..] sums of one call (FP64);
-    // words_: their pinned host copy, one transfer per synchronising call
+    // words_: their host copy, one transfer per synchronising call (pageable: a
+    // pinned one cost a context 350 us of its 570 to create and free, and saved
+    // nothing: an empty synchronising call takes 13.5 us either way)
     static constexpr int kWords = 16;
     unsigned long long* counters_ = nullptr;
-    unsigned long long* words_ = nullptr;
+    unsigned long long words_[kWords] = {};
     double* partials_ = nullptr;
     size_t n_partials_ = 0, n_z_blocks_ = 0;
     // beads
@@ -1382,8 +1378,6 @@ template <typename T> class Engine final : public EngineBase {
                         sp_of_id_, adj_, ext_ids_, ext_slots_, io_};
         for (void* p : ptrs) dev_free(p);
         rho_fx_ = nullptr;
-        if (words_) cudaFreeHost(words_);
-        words_ = nullptr;
         if (own_stream_) cudaStreamDestroy(own_stream_);
         own_stream_ = nullptr;
     }
